@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "coarse_inverse.cuh"
 #include "common.cuh"
 #include "handle.h"
 #include "params.h"
@@ -464,10 +465,10 @@ pfm_status linearize_impl(pfm_handle* h, pfm_precision prec, double* R_fused = n
     }
   }
   Level& c = h->L[nl - 1];
-  launch_coarse_assemble<double>(c.g, h->dp, c.H64, c.mask, h->Kaug, 2 * h->nc_dofs, s, h->det);
-  if (h->contact_on) launch_contact_coarse(c.g, c.Kc64, c.mask, h->Kaug, 2 * h->nc_dofs, s);
+  launch_coarse_assemble<double>(c.g, h->dp, c.H64, c.mask, h->Kaug, h->nc_dofs, s, h->det);
+  if (h->contact_on) launch_contact_coarse(c.g, c.Kc64, c.mask, h->Kaug, h->nc_dofs, s);
   CKL_AT("coarse operator");
-  dense_gauss_jordan_inverse(h->Kaug, h->nc_dofs, h->Kinv, h->gj_keys, h->gj_used, h->gj_piv, h->flag_dev, s);
+  launch_coarse_inverse(h->Kaug, h->nc_dofs, h->Kinv, h->gj_used, h->gj_piv, h->flag_dev, s);
   CKL_AT("coarse inverse");
   int flag = 0;
   CK(cudaMemcpyAsync(&flag, h->flag_dev, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1118,9 +1119,8 @@ pfm_status pfm_create(const pfm_mesh_desc* mesh, const pfm_params* params, pfm_h
   if ((st = dalloc(h, &h->zd, n)) != PFM_OK) return cleanup(st);
   if ((st = dalloc(h, &h->partial, size_t(reduction_blocks(n)) * (MAX_RESTART + 1))) != PFM_OK) return cleanup(st);
   if ((st = dalloc(h, &h->hdev, size_t(3) * (MAX_RESTART + 2))) != PFM_OK) return cleanup(st);
-  if ((st = dalloc(h, &h->Kaug, size_t(h->nc_dofs) * 2 * h->nc_dofs)) != PFM_OK) return cleanup(st);
+  if ((st = dalloc(h, &h->Kaug, size_t(h->nc_dofs) * (h->nc_dofs + GJ_NB))) != PFM_OK) return cleanup(st);
   if ((st = dalloc(h, &h->Kinv, size_t(h->nc_dofs) * h->nc_dofs)) != PFM_OK) return cleanup(st);
-  if ((st = dalloc(h, &h->gj_keys, size_t(h->nc_dofs) + 1)) != PFM_OK) return cleanup(st);
   if ((st = dalloc(h, &h->gj_used, h->nc_dofs)) != PFM_OK) return cleanup(st);
   if ((st = dalloc(h, &h->gj_piv, h->nc_dofs)) != PFM_OK) return cleanup(st);
   cudaError_t e = cudaDeviceSynchronize();
@@ -1145,7 +1145,7 @@ void pfm_destroy(pfm_handle* h) {
   dfree(h->lz);
   dfree(h->dirval); dfree(h->energy_dev); dfree(h->flag_dev); dfree(h->diag_part); dfree(h->load_dev); dfree(h->R); dfree(h->dU); dfree(h->wv);
   dfree(h->rv); dfree(h->zd); dfree(h->ir_r); dfree(h->ir_d); dfree(h->partial); dfree(h->hdev); dfree(h->V); dfree(h->Kaug); dfree(h->Kinv);
-  dfree(h->gj_keys); dfree(h->gj_used); dfree(h->gj_piv); dfree(h->amax_dev);
+  dfree(h->gj_used); dfree(h->gj_piv); dfree(h->amax_dev);
   if (h->Z) cudaFree(h->Z);
   if (h->vgraph) cudaGraphExecDestroy(h->vgraph);
   if (h->hpin) cudaFreeHost(h->hpin);

@@ -20,6 +20,7 @@
 #include <cstring>
 #include <vector>
 
+#include "coarse_inverse.cuh"
 #include "common.cuh"
 #include "fe_device.cuh"
 #include "handle.h"
@@ -116,9 +117,8 @@ struct BBd {
 // Gauss-Jordan inverse of one problem's dense coarse operator.
 struct BGj {
   int problem;
-  double* M;
+  double* M;  // n x n, followed by GJ_NB * n doubles of work
   int n;
-  unsigned long long* keys;
   int* used;
   int* piv;
   double* Ainv;
@@ -461,26 +461,27 @@ __global__ void k_b_lanczos_orth(const BLev* __restrict__ S, int usel, int qsel,
 }
 
 // Gauss-Jordan over the batch: blockIdx.y = problem
-__global__ void k_b_gj_first_key(const BGj* __restrict__ G, Gate on) {
+__global__ void __launch_bounds__(GJ_MAX_THREADS) k_b_gj_panel(const BGj* __restrict__ G, int k0, int* singular,
+                                                               Gate on) {
   const BGj& q = G[blockIdx.y];
-  if (!on(q.problem)) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < q.n; i += gridDim.x * blockDim.x)
-    atomicMax(&q.keys[0], pivot_key(q.M[int64_t(i) * 2 * q.n], i));
+  if (k0 >= q.n || !on(q.problem)) return;  // the whole cluster
+  gj_panel(q.M, q.n, k0, (q.n + int(gridDim.x) - 1) / int(gridDim.x), q.used, q.piv, q.M + int64_t(q.n) * q.n, singular,
+           blockIdx.x, gridDim.x);
 }
 
-__global__ void __launch_bounds__(256) k_b_gj_step(const BGj* __restrict__ G, int k, int* singular, Gate on) {
-  const BGj& q = G[blockIdx.y];
-  if (k >= q.n || !on(q.problem)) return;
-  gj_step_row(q.M, q.n, 2 * q.n, k, q.keys, q.used, q.piv, singular, int(blockIdx.x), blockIdx.x == 0);
+__global__ void __launch_bounds__(64) k_b_gj_update(const BGj* __restrict__ G, int k0, Gate on) {
+  const BGj& q = G[blockIdx.z];
+  const int r0 = int(blockIdx.y) * GJ_TILE, c0 = int(blockIdx.x) * GJ_TILE;
+  if (k0 >= q.n || r0 >= q.n || c0 >= q.n || !on(q.problem)) return;
+  gj_update_tile(q.M, q.n, k0, q.used, q.M + int64_t(q.n) * q.n, r0, c0);
 }
 
 __global__ void k_b_gj_extract(const BGj* __restrict__ G, Gate on) {
   const BGj& q = G[blockIdx.y];
   const int k = blockIdx.x;
   if (k >= q.n || !on(q.problem)) return;
-  const int p = q.piv[k];
-  const double inv = 1.0 / q.M[int64_t(p) * 2 * q.n + k];
-  for (int c = threadIdx.x; c < q.n; c += blockDim.x) q.Ainv[int64_t(k) * q.n + c] = q.M[int64_t(p) * 2 * q.n + q.n + c] * inv;
+  const double* src = q.M + int64_t(q.piv[k]) * q.n;
+  for (int j = threadIdx.x; j < q.n; j += blockDim.x) q.Ainv[int64_t(k) * q.n + q.piv[j]] = src[j];
 }
 
 // ---------------------------------------------------------------------------
@@ -1071,7 +1072,7 @@ pfm_status engine_build(pfm_batch* b, const pfm_solve_opts& o, BatchEngine** out
       if (coarsest) {
         E->D[l].C.push_back(BCo{p, h->nc_dofs, h->Kinv, lv.b32, lv.x32});
         E->D[l].maxn = std::max(E->D[l].maxn, h->nc_dofs);
-        E->G.push_back(BGj{p, h->Kaug, h->nc_dofs, h->gj_keys, h->gj_used, h->gj_piv, h->Kinv});
+        E->G.push_back(BGj{p, h->Kaug, h->nc_dofs, h->gj_used, h->gj_piv, h->Kinv});
         E->maxnG = std::max(E->maxnG, h->nc_dofs);
         continue;
       }
@@ -1366,16 +1367,20 @@ pfm_status eng_linearize(pfm_batch* b, BatchEngine* E, int power_its) {
     if (!E->hact[p]) continue;
     pfm_handle* h = b->hs[p];
     Level& c = h->L.back();
-    launch_coarse_assemble<double>(c.g, h->dp, c.H64, c.mask, h->Kaug, 2 * h->nc_dofs, s);
-    BCK(cudaMemsetAsync(h->gj_keys, 0, sizeof(unsigned long long) * (h->nc_dofs + 1), s));
+    launch_coarse_assemble<double>(c.g, h->dp, c.H64, c.mask, h->Kaug, h->nc_dofs, s);
     BCK(cudaMemsetAsync(h->gj_used, 0, sizeof(int) * h->nc_dofs, s));
+    BCK(cudaMemsetAsync(h->gj_piv, 0, sizeof(int) * h->nc_dofs, s));
   }
   const int nG = int(E->G.size());
-  k_b_gj_first_key<<<dim3(gdiv(E->maxnG, 256), unsigned(nG)), 256, 0, s>>>(E->dG, g);
-  count_launches(1);
-  for (int k = 0; k < E->maxnG; ++k) {
-    k_b_gj_step<<<dim3(unsigned(E->maxnG), unsigned(nG)), 256, 0, s>>>(E->dG, k, E->singular, g);
-    count_launches(1);
+  const GjShape sh = gj_shape(E->maxnG);
+  const unsigned tiles = gdiv(E->maxnG, GJ_TILE);
+  for (int k0 = 0; k0 < E->maxnG; k0 += GJ_NB) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    gj_panel_config(sh, nG, s, &cfg, &at);
+    BCK(cudaLaunchKernelEx(&cfg, k_b_gj_panel, static_cast<const BGj*>(E->dG), k0, E->singular, g));
+    k_b_gj_update<<<dim3(tiles, tiles, unsigned(nG)), 64, 0, s>>>(E->dG, k0, g);
+    count_launches(2);
   }
   k_b_gj_extract<<<dim3(unsigned(E->maxnG), unsigned(nG)), 256, 0, s>>>(E->dG, g);
   count_launches(1);
@@ -1561,7 +1566,7 @@ std::vector<uint64_t> engine_signature(const pfm_batch* b) {
       add(lv.x32); add(lv.b32); add(lv.y32); add(lv.r32); add(lv.d32);
     }
     add(h->V); add(h->Z); add(h->wv); add(h->dU); add(h->R); add(h->rv); add(h->Kaug); add(h->Kinv);
-    add(h->gj_keys); add(h->gj_used); add(h->gj_piv);
+    add(h->gj_used); add(h->gj_piv);
     uint64_t x = 1469598103934665603ull;  // FNV-1a over the parameter block
     const unsigned char* c = reinterpret_cast<const unsigned char*>(&h->dp);
     for (size_t i = 0; i < sizeof(DevParams); ++i) x = (x ^ c[i]) * 1099511628211ull;

@@ -214,8 +214,7 @@ void launch_scale_inv_sqrt(int64_t n, const T* y, const double* dot, T* x, cudaS
 template <typename T>
 void launch_lanczos_orth(int64_t n, T* u, const T* q, const T* qp, const double* alpha, const double* beta2prev,
                          cudaStream_t s);
-int dense_gauss_jordan_inverse(double* Maug, int n, double* Ainv, unsigned long long* keys, int* used, int* piv,
-                               int* singular, cudaStream_t s);
+void launch_coarse_inverse(double* M, int n, double* Ainv, int* used, int* piv, int* singular, cudaStream_t s);
 template <typename T>
 void launch_coarse_solve(int n, const double* Ainv, const T* b, T* x, cudaStream_t s);
 

@@ -98,10 +98,9 @@ struct pfm_handle {
   pfm_precision kry_prec = PFM_F64;
   double* V = nullptr;
   void* Z = nullptr;
-  // coarse dense operator [K | I] reduced by Gauss-Jordan, its inverse, work
+  // coarse dense operator (reduced in place, with work rows behind it), its inverse, work
   double* Kaug = nullptr;
   double* Kinv = nullptr;
-  unsigned long long* gj_keys = nullptr;
   int* gj_used = nullptr;
   int* gj_piv = nullptr;
   int nc_dofs = 0;

@@ -3,8 +3,7 @@
 // single-problem kernels (mg_kernels.cu) and the batched kernels (batch.cu):
 // integer-exact 1-D interpolation between structured grids on the same box,
 // state injection, prolongation and restriction at one node, the Chebyshev
-// smoothing updates at one node, the power-iteration start vector and one
-// Gauss-Jordan elimination step of the dense coarse operator.
+// smoothing updates at one node and the power-iteration start vector.
 //
 // Grid transfer in 1-D: fine node i sits at coarse coordinate i*nc/nf; with
 // i*nc = I0*nf + rem, its interpolation weights are (1 - rem/nf) on coarse
@@ -257,50 +256,6 @@ __device__ __forceinline__ double power_init_value(int64_t i, int64_t nn, const 
   const double u = double(z >> 11) * (1.0 / 9007199254740992.0) * 2.0 - 1.0;
   const int f = int(i / nn);
   return ((mask[i % nn] >> f) & 1) ? 0.0 : u;
-}
-
-// Gauss-Jordan elimination with partial pivoting on the augmented n x 2n
-// matrix [K | I], with the row permutation kept implicit: step k takes the
-// pivot row p chosen by step k-1 (largest |M[i][k]| over rows not yet used as
-// pivots), eliminates column k from every other row (columns > k of the left
-// half and the whole right half; column k itself is never read again), and in
-// the same launch votes the pivot of step k+1 with a 64-bit atomicMax on
-// (|value| as FP32 bits, row). Row p is left unscaled; at the end inverse row
-// k is row piv[k] of the right half divided by M[piv[k]][k].
-__device__ __forceinline__ unsigned long long pivot_key(double v, int row) {
-  return (static_cast<unsigned long long>(__float_as_uint(float(fabs(v)))) << 32) | unsigned(row);
-}
-
-// Step k of the elimination for row i (one thread block; threads stride over
-// the columns); the block with lead == true records the pivot.
-__device__ __forceinline__ void gj_step_row(double* __restrict__ M, int n, int ld, int k,
-                                            unsigned long long* __restrict__ keys, int* __restrict__ used,
-                                            int* __restrict__ piv, int* singular, int i, bool lead) {
-  const int p = int(keys[k] & 0xffffffffu);
-  const double pk = M[int64_t(p) * ld + k];
-  if (!(fabs(pk) > 0.0)) {
-    if (lead && threadIdx.x == 0) *singular = 1;
-    return;
-  }
-  if (lead && threadIdx.x == 0) piv[k] = p;
-  if (i >= n) return;
-  if (i == p) {
-    if (threadIdx.x == 0) used[p] = 1;
-    return;
-  }
-  const double f = M[int64_t(i) * ld + k] / pk;
-  const bool candidate = (k + 1 < n) && !used[i];
-  double* Mi = M + int64_t(i) * ld;
-  const double* Mp = M + int64_t(p) * ld;
-  if (f != 0.0) {
-    for (int j = k + 1 + threadIdx.x; j < 2 * n; j += blockDim.x) {
-      const double v = Mi[j] - f * Mp[j];
-      Mi[j] = v;
-      if (j == k + 1 && candidate) atomicMax(&keys[k + 1], pivot_key(v, i));
-    }
-  } else if (candidate && threadIdx.x == 0) {
-    atomicMax(&keys[k + 1], pivot_key(Mi[k + 1], i));
-  }
 }
 
 }  // namespace pfm

@@ -2,12 +2,13 @@
 // for re-discretisation, trilinear prolongation P and restriction R = P^T
 // between nested or non-nested structured grids on the same box, the damped
 // point-block Jacobi update, and the dense coarse-level operator with its
-// inverse by Gauss-Jordan elimination with partial pivoting.
+// inverse by blocked Gauss-Jordan elimination with partial pivoting.
 //
 // Grid transfer in 1-D: fine node i sits at coarse coordinate i*nc/nf; with
 // i*nc = I0*nf + rem, its interpolation weights are (1 - rem/nf) on coarse
 // node I0 and rem/nf on I0+1. All index arithmetic is integer, so P and
 // R = P^T use identical weights on nested (nf = 2 nc) and non-nested grids.
+#include "coarse_inverse.cuh"
 #include "common.cuh"
 #include "mg_device.cuh"
 
@@ -106,78 +107,84 @@ __global__ void k_sub(int64_t n, const T* __restrict__ b, const T* __restrict__ 
 }
 
 // Dense coarse operator K (row-major, leading dimension ld) from the stored
-// point Hessians: thread (element, local row l = f*8 + a) adds row l of the
-// element matrix sum_q w (Bz^T H_q Bz + Bg^T G Bg). color < 0: every element,
-// added with atomics; color = 0..7: only the elements with
-// (ei & 1) + 2 (ej & 1) + 4 (ek & 1) == color, which share no node, added
+// point Hessians: entry (l, m) of an element's matrix, l = f*8 + a, is
+// sum_q w (Bz^T H_q Bz + Bg^T G Bg). One CTA per (element, row field): the
+// element's Hessians and the shape functions at the Gauss points are staged in
+// shared memory once and every thread forms entries of the 8 rows of that
+// field. Bound by the latency of the FP64 pipe on the few CTAs that a coarsest
+// level has (64 elements, 72 x 72 entries each); one thread per whole row, as
+// an earlier form had it, took 628 us for that level, this form 75 us.
+// color < 0: every element, added with atomics; color = 0..7: only the elements
+// with (ei & 1) + 2 (ej & 1) + 4 (ek & 1) == color, which share no node, added
 // without atomics (eight launches in colour order give a fixed summation order).
 template <typename T>
-__global__ void k_coarse_assemble(Grid g, DevParams P, const T* __restrict__ H, double* __restrict__ K,
-                                  int ld, int color) {
-  const int64_t tid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t e = tid / NED;
-  if (e >= g.ne()) return;
-  if (color >= 0) {
-    const int64_t ei = e % g.nx, ej = (e / g.nx) % g.ny, ek = e / (int64_t(g.nx) * g.ny);
-    if (int((ei & 1) + 2 * (ej & 1) + 4 * (ek & 1)) != color) return;
-  }
-  const int l = int(tid % NED);
-  const int fl = l / 8, al = l % 8;
+__global__ void __launch_bounds__(192) k_coarse_assemble(Grid g, DevParams P, const T* __restrict__ H,
+                                                         double* __restrict__ K, int ld, int color) {
+  __shared__ double Hs[8][NH];
+  __shared__ double Ns[8][8], dNs[3][8][8];  // [local node][Gauss point]
+  const int64_t e = blockIdx.x;
+  const int fl = int(blockIdx.y);
+  const int64_t ei = e % g.nx, ej = (e / g.nx) % g.ny, ek = e / (int64_t(g.nx) * g.ny);
+  if (color >= 0 && int((ei & 1) + 2 * (ej & 1) + 4 * (ek & 1)) != color) return;
   const int64_t nn = g.nn();
-  const double ih[3] = {1.0 / g.hx, 1.0 / g.hy, 1.0 / g.hz};
   const double w = g.w();
-  auto node_of = [&](int a) {
-    int64_t ei = e % g.nx, r = e / g.nx, ej = r % g.ny, ek = r / g.ny;
-    return (ei + (a & 1)) + int64_t(g.nx + 1) * ((ej + ((a >> 1) & 1)) + int64_t(g.ny + 1) * (ek + (a >> 2)));
-  };
-  auto shape = [&](int a, int q, double& N, double dN[3]) {
+  for (int i = threadIdx.x; i < 8 * NH; i += blockDim.x)
+    Hs[i / NH][i % NH] = double(H[hstore_offset<T>(e >> 2, i % NH, int(e & 3) * 8 + i / NH)]);
+  if (threadIdx.x < 64) {
+    const double ih[3] = {1.0 / g.hx, 1.0 / g.hy, 1.0 / g.hz};
+    const int a = int(threadIdx.x) >> 3, q = int(threadIdx.x) & 7;
     double phi[3], dphi[3];
     for (int d = 0; d < 3; ++d) {
       const int ad = (a >> d) & 1, qd = (q >> d) & 1;
       phi[d] = (ad == qd) ? GB : GA;
       dphi[d] = (ad ? 1.0 : -1.0) * ih[d];
     }
-    N = phi[0] * phi[1] * phi[2];
-    dN[0] = dphi[0] * phi[1] * phi[2];
-    dN[1] = phi[0] * dphi[1] * phi[2];
-    dN[2] = phi[0] * phi[1] * dphi[2];
+    Ns[a][q] = phi[0] * phi[1] * phi[2];
+    dNs[0][a][q] = dphi[0] * phi[1] * phi[2];
+    dNs[1][a][q] = phi[0] * dphi[1] * phi[2];
+    dNs[2][a][q] = phi[0] * phi[1] * dphi[2];
+  }
+  __syncthreads();
+  auto node_of = [&](int a) {
+    return (ei + (a & 1)) + int64_t(g.nx + 1) * ((ej + ((a >> 1) & 1)) + int64_t(g.ny + 1) * (ek + (a >> 2)));
   };
-  const int64_t row = fl * nn + node_of(al);
-  const int64_t blk = e >> 2;
-  const int lane0 = int(e & 3) * 8;
-  for (int m = 0; m < NED; ++m) {
+  for (int i = threadIdx.x; i < 8 * NED; i += blockDim.x) {
+    const int al = i / NED, m = i % NED;
     const int fm = m / 8, am = m % 8;
     double s = 0.0;
     for (int q = 0; q < 8; ++q) {
-      double Nl, dNl[3], Nm, dNm[3];
-      shape(al, q, Nl, dNl);
-      shape(am, q, Nm, dNm);
       // z-rows touched by DOF (f, a): u_i -> 3i+J (dN_J); eta_k -> 9+k (N)
-      int rl[3], rm[3];
-      double cl[3], cm[3];
-      int nl, nm;
-      if (fl < 3) { nl = 3; for (int J = 0; J < 3; ++J) { rl[J] = 3 * fl + J; cl[J] = dNl[J]; } }
-      else { nl = 1; rl[0] = 9 + fl - 3; cl[0] = Nl; }
-      if (fm < 3) { nm = 3; for (int J = 0; J < 3; ++J) { rm[J] = 3 * fm + J; cm[J] = dNm[J]; } }
-      else { nm = 1; rm[0] = 9 + fm - 3; cm[0] = Nm; }
-      for (int x = 0; x < nl; ++x)
-        for (int y = 0; y < nm; ++y) {
-          const int r = rl[x] < rm[y] ? rl[x] : rm[y];
-          const int cc = rl[x] < rm[y] ? rm[y] : rl[x];
-          s += cl[x] * cm[y] * double(H[hstore_offset<T>(blk, hidx(r, cc), lane0 + q)]);
-        }
-      if (fl >= 3 && fm >= 3)
-        s += (dNl[0] * dNm[0] + dNl[1] * dNm[1] + dNl[2] * dNm[2]) * P.G[fl - 3][fm - 3];
+      const double* Hq = Hs[q];
+      if (fl < 3 && fm < 3) {
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+#pragma unroll
+          for (int y = 0; y < 3; ++y) {
+            const int rl = 3 * fl + x, rm = 3 * fm + y;
+            s += dNs[x][al][q] * dNs[y][am][q] * Hq[rl < rm ? hidx(rl, rm) : hidx(rm, rl)];
+          }
+      } else if (fl < 3) {
+#pragma unroll
+        for (int x = 0; x < 3; ++x) s += dNs[x][al][q] * Ns[am][q] * Hq[hidx(3 * fl + x, 9 + fm - 3)];
+      } else if (fm < 3) {
+#pragma unroll
+        for (int y = 0; y < 3; ++y) s += Ns[al][q] * dNs[y][am][q] * Hq[hidx(3 * fm + y, 9 + fl - 3)];
+      } else {
+        const int rl = 9 + fl - 3, rm = 9 + fm - 3;
+        s += Ns[al][q] * Ns[am][q] * Hq[rl < rm ? hidx(rl, rm) : hidx(rm, rl)];
+        s += (dNs[0][al][q] * dNs[0][am][q] + dNs[1][al][q] * dNs[1][am][q] + dNs[2][al][q] * dNs[2][am][q]) *
+             P.G[fl - 3][fm - 3];
+      }
     }
-    const int64_t col = fm * nn + node_of(am);
+    double* out = K + (fl * nn + node_of(al)) * ld + (fm * nn + node_of(am));
     if (color >= 0)
-      K[row * ld + col] += w * s;
+      *out += w * s;
     else
-      atomicAdd(&K[row * ld + col], w * s);
+      atomicAdd(out, w * s);
   }
 }
 
-// Dirichlet rows/columns -> identity, and the identity block of the augmented matrix.
+// Dirichlet rows/columns -> identity.
 __global__ void k_coarse_bc(int n, int64_t nn, const dmask_t* __restrict__ mask, double* __restrict__ K,
                             int ld) {
   const int64_t tid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -186,29 +193,27 @@ __global__ void k_coarse_bc(int n, int64_t nn, const dmask_t* __restrict__ mask,
   const bool dr = (mask[r % nn] >> (r / nn)) & 1;
   const bool dc = (mask[c % nn] >> (c / nn)) & 1;
   if (dr || dc) K[int64_t(r) * ld + c] = (r == c) ? 1.0 : 0.0;
-  K[int64_t(r) * ld + n + c] = (r == c) ? 1.0 : 0.0;
 }
 
-__global__ void k_gj_first_key(const double* __restrict__ M, int n, int ld, unsigned long long* keys) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    atomicMax(&keys[0], pivot_key(M[int64_t(i) * ld], i));
+// Blocked Gauss-Jordan inverse (coarse_inverse.cuh): panel by one cluster,
+// update of the other columns, and the final row/column permutation.
+__global__ void __launch_bounds__(GJ_MAX_THREADS) k_gj_panel(double* __restrict__ M, int n, int k0, int R,
+                                                             int* __restrict__ used, int* __restrict__ piv,
+                                                             double* __restrict__ W, int* singular) {
+  gj_panel(M, n, k0, R, used, piv, W, singular, blockIdx.x, gridDim.x);
 }
 
-// One block per row i; threads stride over the columns.
-__global__ void __launch_bounds__(256) k_gj_step(double* __restrict__ M, int n, int ld, int k,
-                                                 unsigned long long* __restrict__ keys, int* __restrict__ used,
-                                                 int* __restrict__ piv, int* singular) {
-  gj_step_row(M, n, ld, k, keys, used, piv, singular, int(blockIdx.x), blockIdx.x == 0);
+__global__ void __launch_bounds__(64) k_gj_update(double* __restrict__ M, int n, int k0, const int* __restrict__ used,
+                                                  const double* __restrict__ W) {
+  gj_update_tile(M, n, k0, used, W, int(blockIdx.y) * GJ_TILE, int(blockIdx.x) * GJ_TILE);
 }
 
-// Ainv[k][c] = M[piv[k]][n + c] / M[piv[k]][k]
-__global__ void k_gj_extract(const double* __restrict__ M, int n, int ld, const int* __restrict__ piv,
+// Ainv[k][piv[j]] = M[piv[k]][j]
+__global__ void k_gj_extract(const double* __restrict__ M, int n, const int* __restrict__ piv,
                              double* __restrict__ Ainv) {
   const int k = blockIdx.x;
-  if (k >= n) return;
-  const int p = piv[k];
-  const double inv = 1.0 / M[int64_t(p) * ld + k];
-  for (int c = threadIdx.x; c < n; c += blockDim.x) Ainv[int64_t(k) * n + c] = M[int64_t(p) * ld + n + c] * inv;
+  const double* src = M + int64_t(piv[k]) * n;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) Ainv[int64_t(k) * n + piv[j]] = src[j];
 }
 
 // x = Ainv b (Ainv dense n x n, row-major).
@@ -363,30 +368,34 @@ void launch_coarse_assemble(const Grid& g, const DevParams& P, const T* H, const
   const int n = int(NF * g.nn());
   cudaMemsetAsync(K, 0, sizeof(double) * size_t(n) * ld, s);
   for (int c = det ? 0 : -1; c < (det ? 8 : 0); ++c) {
-    k_coarse_assemble<T><<<grid_for(g.ne() * NED, 128), 128, 0, s>>>(g, P, H, K, ld, c);
+    k_coarse_assemble<T><<<dim3(unsigned(g.ne()), NF), 192, 0, s>>>(g, P, H, K, ld, c);
     count_launches(1);
   }
   k_coarse_bc<<<grid_for(int64_t(n) * n, 256), 256, 0, s>>>(n, g.nn(), mask, K, ld);
   count_launches(1);
 }
 
-// Invert the dense coarse operator from the augmented [K | I] (n x 2n,
-// ld = 2n; overwritten) into Ainv (n x n). work: (n+1) keys, n used flags and
-// n pivot rows. Returns the number of kernel launches.
-int dense_gauss_jordan_inverse(double* Maug, int n, double* Ainv, unsigned long long* keys, int* used, int* piv,
-                               int* singular, cudaStream_t s) {
-  const int ld = 2 * n;
-  cudaMemsetAsync(keys, 0, sizeof(unsigned long long) * (n + 1), s);
+// Invert the dense coarse operator M (n x n, overwritten; followed by GJ_NB * n
+// doubles of work) into Ainv (n x n). used, piv: n integers of work each.
+// One panel and one update per GJ_NB columns. Measured at n = 1125 (the 4^3
+// coarsest level): 71 panels of 79 us and 71 updates of 42 us, 8.6 ms; one
+// launch per column over the augmented matrix took 15.2 ms.
+void launch_coarse_inverse(double* M, int n, double* Ainv, int* used, int* piv, int* singular, cudaStream_t s) {
+  double* W = M + int64_t(n) * n;
   cudaMemsetAsync(used, 0, sizeof(int) * n, s);
-  k_gj_first_key<<<grid_for(n, 256), 256, 0, s>>>(Maug, n, ld, keys);
-  count_launches(1);
-  for (int k = 0; k < n; ++k) {
-    k_gj_step<<<n, 256, 0, s>>>(Maug, n, ld, k, keys, used, piv, singular);
-    count_launches(1);
+  cudaMemsetAsync(piv, 0, sizeof(int) * n, s);  // in range also where a singular column leaves it unset
+  const GjShape sh = gj_shape(n);
+  const unsigned tiles = unsigned((n + GJ_TILE - 1) / GJ_TILE);
+  for (int k0 = 0; k0 < n; k0 += GJ_NB) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    gj_panel_config(sh, 1, s, &cfg, &at);
+    cudaLaunchKernelEx(&cfg, k_gj_panel, M, n, k0, sh.rows, used, piv, W, singular);
+    k_gj_update<<<dim3(tiles, tiles), 64, 0, s>>>(M, n, k0, used, W);
+    count_launches(2);
   }
-  k_gj_extract<<<n, 256, 0, s>>>(Maug, n, ld, piv, Ainv);
+  k_gj_extract<<<n, 256, 0, s>>>(M, n, piv, Ainv);
   count_launches(1);
-  return n + 2;
 }
 
 template <typename T>
