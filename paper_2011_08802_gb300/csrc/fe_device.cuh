@@ -16,6 +16,7 @@
 #include <cuda_fp16.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -170,6 +171,33 @@ struct NoLinTail {
   __device__ void operator()(const TC*, const TC*, TC, int64_t, bool, int) const {}
 };
 
+// Receives the Hessian entries of one Gauss point as they become final and
+// writes them to the requested stores (null stores are skipped; lanes without
+// an element write zeros).
+template <typename TC>
+struct HessStore {
+  static constexpr bool want = true;
+  double* H64;
+  float* H32;
+  float* H32lo;
+  int64_t blk;
+  int lane;
+  bool valid;
+  __device__ __forceinline__ void operator()(int j, TC v) const {
+    if constexpr (std::is_same<TC, float>::value) {
+      const float h = valid ? v : 0.f;
+      if (H64) H64[hstore_offset<double>(blk, j, lane)] = double(h);
+      if (H32) H32[hstore_offset<float>(blk, j, lane)] = h;
+      if (H32lo) H32lo[hstore_offset<float>(blk, j, lane)] = 0.f;
+    } else {
+      const double h = valid ? double(v) : 0.0;
+      if (H64) H64[hstore_offset<double>(blk, j, lane)] = h;
+      if (H32) H32[hstore_offset<float>(blk, j, lane)] = float(h);
+      if (H32lo) H32lo[hstore_offset<float>(blk, j, lane)] = float(h - double(float(h)));
+    }
+  }
+};
+
 // Gauss-point Hessians of element block blk (this warp; lane = 8 e + q),
 // computed in TC (FP64 for the finest and the coarsest level, FP32 for the
 // intermediate levels of an FP32 preconditioner) and stored in the requested
@@ -192,15 +220,11 @@ __device__ __forceinline__ void linearize_lane(const Grid& g, const DevParams& P
   gather_state<TC>(U, nn, node, valid, l8, ihx, ihy, ihz, F, eh, ge);
 #pragma unroll
   for (int k = 0; k < NV; ++k) ehn[k] = q1_value(valid ? TC(Un[(3 + k) * nn + node]) : TC(0));
-  TC W, gr[NZ], Hp[NH];
-  qp_local<TC, true>(P, F, eh, ehn, &W, gr, Hp);
+  TC W, gr[NZ];
+  const HessStore<TC> store{H64, H32, H32lo, blk, lane, valid};
+  qp_point<TC>(P, F, eh, ehn, &W, gr, store);
+  for (int j = NH; j < NHP; ++j) store(j, TC(0));  // padding entries are stored as zeros
   tail(ge, gr, W, node, valid, l8);
-  for (int j = 0; j < NHP; ++j) {  // padding entries NH..NHP-1 are stored as zeros
-    const double h = (valid && j < NH) ? double(Hp[j < NH ? j : 0]) : 0.0;
-    if (H64) H64[hstore_offset<double>(blk, j, lane)] = h;
-    if (H32) H32[hstore_offset<float>(blk, j, lane)] = float(h);
-    if (H32lo) H32lo[hstore_offset<float>(blk, j, lane)] = float(h - double(float(h)));
-  }
 }
 
 // Nodal NF x NF diagonal blocks (9 x 9 for N = 6). For local node a of the

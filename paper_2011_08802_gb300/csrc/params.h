@@ -18,26 +18,33 @@ namespace pfm {
 // Ahat_ii = 0, and T the 7x6 map eta = e_0 + T eta_hat.
 inline void make_dev_params(const pfm_params& in, DevParams& out) {
   const double pi = 3.14159265358979323846;
+  const int si[6] = {0, 1, 2, 1, 0, 0}, sj[6] = {0, 1, 2, 2, 2, 1};  // Voigt slots
+  for (int v = 0; v < 6; ++v) out.U0[v] = in.Ut[0][3 * si[v] + sj[v]];
+  for (int k = 0; k < NV; ++k)
+    for (int v = 0; v < 6; ++v) out.dU[k][v] = in.Ut[k + 1][3 * si[v] + sj[v]] - out.U0[v];
   for (int p = 0; p < NPH; ++p) {
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) out.U[p][i][j] = in.Ut[p][3 * i + j];
     for (int I = 0; I < 6; ++I)
       for (int J = 0; J < 6; ++J) out.Lv[p][I][J] = in.Lvoigt[p][6 * I + J];
-    out.F0[p] = in.F0[p];
     out.inv_mtau[p] = 1.0 / (in.mobility[p] * in.tau);
   }
-  double Ahat[NPH][NPH];
+  double cobst[NPH][NPH], Ahat[NPH][NPH];
   for (int i = 0; i < NPH; ++i)
     for (int j = 0; j < NPH; ++j) {
       if (i == j) {
-        out.cobst[i][j] = 0.0;
+        cobst[i][j] = 0.0;
         Ahat[i][j] = 0.0;
       } else {
         double c = 4.0 * in.gamma_scale * in.gamma[i][j] / (pi * in.ell[i][j]);
-        out.cobst[i][j] = c;
+        cobst[i][j] = c;
         Ahat[i][j] = -c * in.ell[i][j] * in.ell[i][j];
       }
     }
+  // chemical and obstacle energy with eta = e_0 + T eta_hat
+  out.W0 = in.F0[0];
+  for (int k = 0; k < NV; ++k) {
+    out.lin[k] = cobst[0][k + 1] + in.F0[k + 1] - in.F0[0];
+    for (int l = 0; l < NV; ++l) out.Cc[k][l] = cobst[k + 1][l + 1] - cobst[k + 1][0] - cobst[0][l + 1];
+  }
   for (int k = 0; k < NV; ++k)
     for (int l = 0; l < NV; ++l)
       out.G[k][l] = Ahat[k + 1][l + 1] - Ahat[0][l + 1] - Ahat[k + 1][0] + Ahat[0][0];

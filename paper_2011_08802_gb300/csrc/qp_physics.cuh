@@ -12,18 +12,35 @@
 // interface energy is a constant quadratic form handled by the element
 // kernels.
 //
-// Derivatives. With A = (F^t)^-1, M = F A, E = C^e = M^T M and the energy
-// written as g(E, eta) = 1/2 J_t h(E):L(eta):h(E), J_t = det F^t, the chain
-// rule gives first and second derivatives from those of E and of h = 1/2 log.
-// The derivatives of the matrix logarithm use the spectral decomposition of
-// E (cyclic Jacobi) and the Daleckii-Krein formulas: in the eigenbasis,
-// Dlog[X]_ab = f1(l_a,l_b) X_ab and
+// Derivatives. With A = (F^t)^-1, M = F^e = F A and E = C^e = M^T M, the elastic
+// energy is J_t g(M), g = 1/2 h:L:h, h = 1/2 log E, J_t = det F^t. Every
+// direction moves M along a rank-one matrix l A_c^T (A_c: column c of A): F_pc
+// along l = e_p, an entry (i, c) of F^t along l = -M e_i, so with q = Q^T M^T l
+// and a_c = Q^T A_c (Q: eigenvectors of E) the rotated change of E is
+// a_c q^T + q a_c^T. The second derivative along two such directions is
+// q^T R_cc' q' with six 3x3 matrices R_cc' per Gauss point (the spectral second
+// derivative of g contracted with a_c and a_c', plus the stress term
+// (A 2S A)_cc' diag(1/lambda), because l . l' = q^T Lambda^-1 q'). The
+// order parameters enter only through the six entries of the symmetric F^t:
+// rows and columns of the Hessian are formed for those six entries and turned
+// into the eta_hat_k by the constant matrix of dU_k = U_k - U_0.
+// The point physics is bound by the FP64 pipe (about 2 multiply-adds per clock
+// and SM), so what counts is the number of FP64 instructions; FP32 ones are
+// nearly free. The eigenvectors start from FP32 Jacobi rotations of the
+// deviator of E and two FP64 corrections by small rotations follow
+// (quadratic convergence from 1e-7); the rotation is held as a quaternion, so it
+// is orthonormal to rounding without a Gram-Schmidt pass. The divided
+// differences of log use the series of 2 atanh((a-b)/(a+b)) when a and b are
+// close, which needs one reciprocal and no logarithm. Measured against the form
+// with one direction per unknown, a Jacobi eigensolve in FP64 and a 120-entry
+// array of the Hessian: linearisation with residual of 80x72x56 elements 37.8 ->
+// 23.6 ms (stack per thread 5.9 -> 1.6 KB), residual of 97x65x50 10.1 -> 7.0 ms.
+//
+// The matrix logarithm's derivatives are the Daleckii-Krein formulas: in the
+// eigenbasis Dlog[X]_ab = f1(l_a,l_b) X_ab and
 // D2log[X,Y]_ab = sum_c f2(l_a,l_c,l_b) (X_ac Y_cb + Y_ac X_cb), with f1, f2
-// the first and second divided differences of log. These are exact for
-// repeated eigenvalues as long as the divided differences are evaluated
-// without cancellation, which dd1_log / dd2_log do (log1p quotient; Taylor
-// series of the second divided difference about the mean when all three
-// arguments are close).
+// the first and second divided differences of log, exact for repeated
+// eigenvalues because no difference quotient of nearly equal values is formed.
 //
 // Pade modes (Sec. 2.4, Eqs. pade11, pade22, pade33). The paper's (m,m)
 // approximant of H^e is the primary matrix function h = 1/2 r_m(C^e), r_m the
@@ -40,8 +57,10 @@
 #ifdef __CUDACC__
 #define PFM_HD __host__ __device__ __forceinline__
 #define PFM_HD_BIG __host__ __device__
+#define PFM_HD_COLD static __host__ __device__ __noinline__
 #else
 #define PFM_HD_BIG inline
+#define PFM_HD_COLD static inline
 #include <cmath>
 #define PFM_HD inline
 using std::sqrt;
@@ -138,14 +157,16 @@ constexpr int NHP = (NH + 7) / 8 * 8;
 
 // Physical parameters, passed by value to kernels (constant bank).
 struct DevParams {
-  double U[NPH][3][3];      // transformation stretches U_i (U_0 = I)
+  double U0[6];             // transformation stretch U_0 (Voigt slots 00, 11, 22, 12, 02, 01)
+  double dU[NV][6];         // U_k - U_0, the derivative of F^t with respect to eta_hat_k
   double Lv[NPH][6][6];     // stiffness L_i in Voigt form (engineering shear)
-  double F0[NPH];           // chemical energies F_i^0
   double inv_mtau[NPH];     // 1 / (m_i tau)
-  double cobst[NPH][NPH];   // 4 gamma_ij / (pi ell_ij), zero diagonal
+  // chemical and obstacle energy in the condensed unknowns (eta_0 = 1 - sum eta_hat):
+  // W0 + sum_k lin_k eta_hat_k + 1/2 sum_kl Cc_kl eta_hat_k eta_hat_l
+  double W0, lin[NV], Cc[NV][NV];
   double G[NV][NV];         // gradient-energy matrix in eta_hat (per direction)
   double eps_eta;           // penalty parameter
-  int same_L;               // 1 when every phase has the same stiffness (then L(eta) = L sum eta)
+  int same_L;               // 1 when every phase has the same stiffness (then L(eta) = L, as sum eta = 1)
   int cubic;                // 1 when that stiffness is cubic in the frame of the data:
   double cub_lambda, cub_mu, cub_delta;  // L = lambda I x I + 2 mu I_sym + delta sum_n e_n^4
   int hencky;               // 0: exact log; m = 1, 2, 3: Pade (m,m) (Gauss-Legendre form below)
@@ -157,21 +178,24 @@ PFM_HD int hidx(int r, int c) { return r * NZ - (r * (r - 1)) / 2 + (c - r); }
 
 template <typename T> struct Tol;
 template <> struct Tol<double> {
-  static constexpr double dd2_gap = 1e-3;    // relative spread below which f2 uses its Taylor series
+  static constexpr float f2_gap = 2e-2f;     // relative spread up to which f2 of three values uses its series
   static constexpr double jacobi_off = 1e-17;
 };
 #ifdef __CUDACC__
 template <> struct Tol<df64> {
-  static constexpr double dd2_gap = 1e-3;
+  static constexpr float f2_gap = 2e-2f;
   static constexpr double jacobi_off = 1e-14;  // the double-float resolution
 };
 #endif
 template <> struct Tol<float> {
-  static constexpr float dd2_gap = 3e-2f;
+  static constexpr float f2_gap = 1e-1f;
   static constexpr float jacobi_off = 1e-8f;
 };
 
-template <typename T> PFM_HD T tmin(T a, T b) { return a < b ? a : b; }
+template <typename T> PFM_HD float to_f32(T a) { return float(a); }
+#ifdef __CUDACC__
+template <> PFM_HD float to_f32<df64>(df64 a) { return a.hi; }
+#endif
 
 // ---------------------------------------------------------------------------
 // 3x3 helpers (full storage)
@@ -201,56 +225,22 @@ PFM_HD void rot_in(const T Q[3][3], const T a[3][3], T c[3][3]) {
   mtm3(Q, t, c);
 }
 
+// Inverse (packed) and determinant of a packed symmetric 3x3 matrix.
 template <typename T>
-PFM_HD T tr_ab(const T a[3][3], const T b[3][3]) {  // tr(a b)
-  T s = 0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) s += a[i][j] * b[j][i];
-  return s;
-}
-
-template <typename T>
-PFM_HD T ddot3(const T a[3][3], const T b[3][3]) {  // a : b
-  T s = 0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) s += a[i][j] * b[i][j];
-  return s;
-}
-
-// Inverse and determinant of a symmetric positive-definite 3x3 matrix.
-template <typename T>
-PFM_HD T inv_sym3(const T a[3][3], T r[3][3]) {
-  T c00 = a[1][1] * a[2][2] - a[1][2] * a[2][1];
-  T c01 = a[1][2] * a[2][0] - a[1][0] * a[2][2];
-  T c02 = a[1][0] * a[2][1] - a[1][1] * a[2][0];
-  T det = a[0][0] * c00 + a[0][1] * c01 + a[0][2] * c02;
-  T id = T(1) / det;
-  r[0][0] = c00 * id;
-  r[0][1] = r[1][0] = c01 * id;
-  r[0][2] = r[2][0] = c02 * id;
-  r[1][1] = (a[0][0] * a[2][2] - a[0][2] * a[2][0]) * id;
-  r[1][2] = r[2][1] = (a[0][2] * a[1][0] - a[0][0] * a[1][2]) * id;
-  r[2][2] = (a[0][0] * a[1][1] - a[0][1] * a[1][0]) * id;
+PFM_HD T inv_sym6(const T a[6], T r[6]) {
+  const T c00 = a[1] * a[2] - a[3] * a[3];
+  const T c01 = a[3] * a[4] - a[5] * a[2];
+  const T c02 = a[5] * a[3] - a[1] * a[4];
+  const T det = a[0] * c00 + a[5] * c01 + a[4] * c02;
+  const T id = T(1) / det;
+  r[0] = c00 * id;
+  r[5] = c01 * id;
+  r[4] = c02 * id;
+  r[1] = (a[0] * a[2] - a[4] * a[4]) * id;
+  r[3] = (a[5] * a[4] - a[0] * a[3]) * id;
+  r[2] = (a[0] * a[1] - a[5] * a[5]) * id;
   return det;
 }
-
-// Voigt vector with engineering shear: (a00, a11, a22, 2a12, 2a02, 2a01).
-template <typename T>
-PFM_HD void voigt_strain(const T a[3][3], T v[6]) {
-  v[0] = a[0][0]; v[1] = a[1][1]; v[2] = a[2][2];
-  v[3] = a[1][2] + a[2][1]; v[4] = a[0][2] + a[2][0]; v[5] = a[0][1] + a[1][0];
-}
-// Symmetric tensor from a Voigt stress vector (no shear factor).
-template <typename T>
-PFM_HD void from_voigt_stress(const T v[6], T a[3][3]) {
-  a[0][0] = v[0]; a[1][1] = v[1]; a[2][2] = v[2];
-  a[1][2] = a[2][1] = v[3]; a[0][2] = a[2][0] = v[4]; a[0][1] = a[1][0] = v[5];
-}
-
 
 // Packed symmetric 3x3 storage (00, 11, 22, 12, 02, 01), the Voigt order.
 PFM_HD int sym_i(int v) { return v < 3 ? v : (v == 3 ? 1 : 0); }
@@ -263,12 +253,6 @@ PFM_HD T symget(const T* X, int a, int b) {
 }
 // Voigt slot (00, 11, 22, 12, 02, 01) of the symmetric pair (a, c).
 PFM_HD int voigt_slot(int a, int c) { return a == c ? a : 6 - a - c; }
-
-template <typename T>
-PFM_HD void load_U(const DevParams& P, int p, T U[3][3]) {
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) U[i][j] = T(P.U[p][i][j]);
-}
 
 // ---------------------------------------------------------------------------
 // Symmetric 3x3 eigen-decomposition by cyclic Jacobi rotations:
@@ -319,42 +303,165 @@ PFM_HD void jacobi_eig3(T a[3][3], T lam[3], T Q[3][3]) {
 }
 
 
-// Eigen-decomposition used by the point physics: in FP32 directly; in FP64
-// the Jacobi rotations are first run in FP32 (cheap square roots and
-// divisions), the matrix is rotated into that approximate eigenbasis in FP64
-// and FP64 Jacobi sweeps finish it (quadratic convergence from ~1e-7).
+// Rotation matrix of a quaternion (w, x, y, z) of any length.
 template <typename T>
-PFM_HD void eig_sym3(T a[3][3], T lam[3], T Q[3][3]) {
-  jacobi_eig3(a, lam, Q);
+PFM_HD void quat_rot(const T q[4], T R[3][3]) {
+  const T s = T(2) / (q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
+  const T xs = q[1] * s, ys = q[2] * s, zs = q[3] * s;
+  const T wx = q[0] * xs, wy = q[0] * ys, wz = q[0] * zs;
+  const T xx = q[1] * xs, xy = q[1] * ys, xz = q[1] * zs;
+  const T yy = q[2] * ys, yz = q[2] * zs, zz = q[3] * zs;
+  R[0][0] = T(1) - (yy + zz);
+  R[0][1] = xy - wz;
+  R[0][2] = xz + wy;
+  R[1][0] = xy + wz;
+  R[1][1] = T(1) - (xx + zz);
+  R[1][2] = yz - wx;
+  R[2][0] = xz - wy;
+  R[2][1] = yz + wx;
+  R[2][2] = T(1) - (xx + yy);
 }
-template <>
-PFM_HD void eig_sym3<double>(double a[3][3], double lam[3], double Q[3][3]) {
-  float af[3][3], lf[3], Qf[3][3];
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) af[i][j] = float(a[i][j]);
-  jacobi_eig3(af, lf, Qf);
-  double Q0[3][3], b[3][3], Q1[3][3];
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) Q0[i][j] = double(Qf[i][j]);
-  // re-orthonormalise the FP32 eigenvectors in FP64 (modified Gram-Schmidt)
-  for (int c = 0; c < 3; ++c) {
-    for (int pc = 0; pc < c; ++pc) {
-      double d = Q0[0][c] * Q0[0][pc] + Q0[1][c] * Q0[1][pc] + Q0[2][c] * Q0[2][pc];
-      for (int i = 0; i < 3; ++i) Q0[i][c] -= d * Q0[i][pc];
+
+// q <- q (1, x, y, z) (Hamilton product): R(q) <- R(q) R(1, x, y, z)
+template <typename T>
+PFM_HD void quat_mul_unit(T q[4], T x, T y, T z) {
+  const T w = q[0], a = q[1], b = q[2], c = q[3];
+  q[0] = w - (a * x + b * y + c * z);
+  q[1] = a + (w * x + b * z - c * y);
+  q[2] = b + (w * y + c * x - a * z);
+  q[3] = c + (w * z + a * y - b * x);
+}
+
+// Cyclic Jacobi on the packed symmetric matrix a (FP32): on return a is
+// diagonal to rounding and q the quaternion of the rotation Q with
+// a_in = Q diag(a) Q^T. A rotation by the angle phi in the plane (p, r) that
+// keeps axis n multiplies the quaternion by (1, -+ tan(phi/2) e_n).
+PFM_HD void jacobi_quat(float a[6], float q[4]) {
+  q[0] = 1.f;
+  q[1] = q[2] = q[3] = 0.f;
+  for (int sweep = 0; sweep < 16; ++sweep) {
+    const float off = fabsf(a[3]) + fabsf(a[4]) + fabsf(a[5]);
+    const float dia = fabsf(a[0]) + fabsf(a[1]) + fabsf(a[2]);
+    if (off <= Tol<float>::jacobi_off * dia) break;
+#pragma unroll
+    for (int n = 2; n >= 0; --n) {  // planes (0,1), (0,2), (1,2)
+      const int p = n == 0 ? 1 : 0, r = n == 2 ? 1 : 2;
+      const float apr = a[3 + n];
+      if (fabsf(apr) <= Tol<float>::jacobi_off * (fabsf(a[p]) + fabsf(a[r]))) {
+        a[3 + n] = 0.f;
+        continue;
+      }
+      const float theta = (a[r] - a[p]) / (2.f * apr);
+      float t = 1.f / (fabsf(theta) + sqrtf(theta * theta + 1.f));
+      if (theta < 0.f) t = -t;
+      const float c = 1.f / sqrtf(t * t + 1.f);
+      const float sn = t * c;
+      const float tau = sn / (1.f + c);
+      a[p] -= t * apr;
+      a[r] += t * apr;
+      a[3 + n] = 0.f;
+      // the entries that couple axis n to p and r are the slots 3 + r and 3 + p
+      const float anp = a[3 + r], anr = a[3 + p];
+      a[3 + r] = anp - sn * (anr + tau * anp);
+      a[3 + p] = anr + sn * (anp - tau * anr);
+      const float v = n == 1 ? tau : -tau;
+      const float w = q[0], x = q[1], y = q[2], z = q[3];
+      if (n == 0) {
+        q[0] = w - x * v; q[1] = x + w * v; q[2] = y + z * v; q[3] = z - y * v;
+      } else if (n == 1) {
+        q[0] = w - y * v; q[1] = x - z * v; q[2] = y + w * v; q[3] = z + x * v;
+      } else {
+        q[0] = w - z * v; q[1] = x + y * v; q[2] = y - x * v; q[3] = z + w * v;
+      }
     }
-    double nrm = sqrt(Q0[0][c] * Q0[0][c] + Q0[1][c] * Q0[1][c] + Q0[2][c] * Q0[2][c]);
-    const double inrm = 1.0 / nrm;
-    for (int i = 0; i < 3; ++i) Q0[i][c] *= inrm;
   }
-  rot_in(Q0, a, b);
-  jacobi_eig3(b, lam, Q1);
-  mm3(Q0, Q1, Q);
+}
+
+// b = R^T X R (packed)
+template <typename T>
+PFM_HD void rot_sym6(const T R[3][3], const T X[6], T b[6]) {
+  T t[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      t[i][j] = symget(X, i, 0) * R[0][j] + symget(X, i, 1) * R[1][j] + symget(X, i, 2) * R[2][j];
+#pragma unroll
+  for (int v = 0; v < 6; ++v) {
+    const int i = sym_i(v), j = sym_j(v);
+    b[v] = R[0][i] * t[0][j] + R[1][i] * t[1][j] + R[2][i] * t[2][j];
+  }
+}
+
+// Nearly equal eigenvalues (a gap below about 1e-4 of the deviator): Jacobi
+// rotations with exact angles on the rotated matrix. Rare, and out of line so
+// that it takes no registers from the common path.
+PFM_HD_COLD void eig_finish_jacobi(const double b[6], double lam[3], double R[3][3]) {
+  double a[3][3] = {{b[0], b[5], b[4]}, {b[5], b[1], b[3]}, {b[4], b[3], b[2]}};
+  double Q1[3][3], Q[3][3];
+  jacobi_eig3(a, lam, Q1);
+  mm3(R, Q1, Q);
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) R[i][j] = Q[i][j];
+}
+
+// Eigen-decomposition E = Q diag(1 + x) Q^T of the packed symmetric matrix E. The
+// deviator is rotated and x = (mean - 1) + its eigenvalues, so that neither x
+// nor the differences of eigenvalues carry the rounding of numbers near 1.
+PFM_HD void eig_sym6(const float E[6], float x[3], float Q[3][3]) {
+  const float m = (E[0] + E[1] + E[2]) * (1.f / 3.f);
+  float a[6] = {E[0] - m, E[1] - m, E[2] - m, E[3], E[4], E[5]}, q[4];
+  jacobi_quat(a, q);
+  quat_rot(q, Q);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) x[i] = (m - 1.f) + a[i];
+}
+// FP64: eigenvectors from FP32 Jacobi, then twice b = R^T X R and the
+// simultaneous small rotation tan(phi/2) = b_pr / (2 (b_rr - b_pp)) in the three
+// planes, its angles in FP32 (the error left after the first correction is the
+// square of the angles, about 1e-13 of the deviator, and nothing after the
+// second). Angles above 1e-3 in the first correction mean nearly equal
+// eigenvalues, where Jacobi with exact angles takes over.
+PFM_HD void eig_sym6(const double E[6], double x[3], double Q[3][3]) {
+  const double m = (E[0] + E[1] + E[2]) * (1.0 / 3.0);
+  const double X[6] = {E[0] - m, E[1] - m, E[2] - m, E[3], E[4], E[5]};
+  float a[6], qf[4];
+#pragma unroll
+  for (int v = 0; v < 6; ++v) a[v] = float(X[v]);
+  jacobi_quat(a, qf);
+  double q[4] = {double(qf[0]), double(qf[1]), double(qf[2]), double(qf[3])};
+  double b[6];
+#pragma unroll
+  for (int pass = 0; pass < 2; ++pass) {
+    quat_rot(q, Q);
+    rot_sym6(Q, X, b);
+    float tau[3], big = 0.f;  // tau[n]: the plane that keeps axis n
+    const float num[3] = {float(b[3]), float(b[4]), float(b[5])};
+    const float den[3] = {float(b[2] - b[1]), float(b[2] - b[0]), float(b[1] - b[0])};
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+      tau[n] = num[n] == 0.f ? 0.f : 0.5f * num[n] / den[n];
+      const float t = fabsf(tau[n]);
+      big = t <= big ? big : t;  // a NaN stays
+    }
+    if (pass == 0 && !(big <= 1e-3f)) {
+      eig_finish_jacobi(b, x, Q);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) x[i] += m - 1.0;
+      return;
+    }
+    quat_mul_unit(q, double(-tau[0]), double(tau[1]), double(-tau[2]));
+  }
+  quat_rot(q, Q);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) x[i] = (m - 1.0) + b[i];
 }
 
 #ifdef __CUDACC__
 // Double-float version of the FP64 eigen-decomposition: FP32 Jacobi seed,
 // re-orthonormalisation and the finishing sweeps in double-float.
-__device__ __forceinline__ void eig_sym3(df64 a[3][3], df64 lam[3], df64 Q[3][3]) {
+__device__ __forceinline__ void eig_sym6(const df64 E[6], df64 x[3], df64 Q[3][3]) {
+  df64 a[3][3] = {{E[0], E[5], E[4]}, {E[5], E[1], E[3]}, {E[4], E[3], E[2]}};
   float af[3][3], lf[3], Qf[3][3];
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j) af[i][j] = a[i][j].hi;
@@ -371,522 +478,606 @@ __device__ __forceinline__ void eig_sym3(df64 a[3][3], df64 lam[3], df64 Q[3][3]
     for (int i = 0; i < 3; ++i) Q0[i][c] *= inrm;
   }
   rot_in(Q0, a, b);
+  df64 lam[3];
   jacobi_eig3(b, lam, Q1);
+  for (int i = 0; i < 3; ++i) x[i] = lam[i] - df64(1.0);
   mm3(Q0, Q1, Q);
 }
 #endif
 
-// First divided difference of log: (log a - log b)/(a - b), 1/a if a == b.
-template <typename T>
-PFM_HD T dd1_log(T a, T b) {
-  if (a < b) { T t = a; a = b; b = t; }
-  T d = a - b;
-  if (d == T(0)) return T(1) / a;
-  return log1p(d / b) / d;
-}
-
-// Second divided difference of log, symmetric in its arguments.
-template <typename T>
-PFM_HD T dd2_log(T x0, T x1, T x2) {
-  // sort descending: a >= b >= c
-  T a = x0, b = x1, c = x2, t;
-  if (a < b) { t = a; a = b; b = t; }
-  if (b < c) { t = b; b = c; c = t; }
-  if (a < b) { t = a; a = b; b = t; }
-  T gap = a - c;
-  if (gap > Tol<T>::dd2_gap * a) return (dd1_log(a, b) - dd1_log(b, c)) / gap;
-  // f[x0,x1,x2] = sum_j f^(2+j)(m)/(2+j)! h_j(x - m); for log this is
-  // (1/m^2) sum_j (-1)^(j+1) h_j(u)/(j+2), u = (x - m)/m, h_j the complete
-  // homogeneous symmetric polynomial of degree j, built one variable at a
-  // time: h_j(u_0..u_i) = h_j(u_0..u_(i-1)) + u_i h_(j-1)(u_0..u_i).
-  const T m = (a + b + c) / T(3);
-  const T im = T(1) / m;
-  const T u[3] = {(a - m) * im, (b - m) * im, (c - m) * im};
-  T hh[6] = {T(1), T(0), T(0), T(0), T(0), T(0)};
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 1; j < 6; ++j) hh[j] = (i == 0 ? T(0) : hh[j]) + u[i] * hh[j - 1];
-  // alternating weights -1/2, 1/3, -1/4, 1/5, -1/6, 1/7
-  const T wj[6] = {T(-0.5), T(1.0 / 3.0), T(-0.25), T(0.2), T(-1.0 / 6.0), T(1.0 / 7.0)};
-  T sum = T(0);
-#pragma unroll
-  for (int j = 0; j < 6; ++j) sum += wj[j] * hh[j];
-  return sum * im * im;
-}
-
-// Second divided difference of log at (x, y, z) from the first ones
-// fxy = f[x,y], fyz = f[y,z], fxz = f[x,z]. On a wide spread it is the
-// quotient over the largest gap with the middle value as pivot, which is the
-// quotient dd2_log forms after sorting (the same operands up to signs, so the
-// same result); on a narrow spread, dd2_log's series.
-template <typename T>
-PFM_HD T dd2_log_f1(T x, T y, T z, T fxy, T fyz, T fxz) {
-  const T dxz = x - z, dxy = x - y, dyz = y - z;
-  const T axz = fabs(dxz), axy = fabs(dxy), ayz = fabs(dyz);
-  T num, den, gap;
-  if (axz >= axy && axz >= ayz) {  // y in the middle
-    num = fxy - fyz;
-    den = dxz;
-    gap = axz;
-  } else if (axy >= ayz) {  // z in the middle
-    num = fxz - fyz;
-    den = dxy;
-    gap = axy;
-  } else {  // x in the middle
-    num = fxy - fxz;
-    den = dyz;
-    gap = ayz;
+// First divided difference f1 = (log a - log b)/(a - b) of log and, with PAIR,
+// the second ones f2(a,a,b) and f2(a,b,b) (d = a - b, ia = 1/a, ib = 1/b). With
+// z = (a - b)/(a + b): f1 = 2/(a+b) sum_n z^2n/(2n+1) and
+// f2(a,a,b), f2(a,b,b) = -1/(2ab) +- 2/(a+b)^2 sum_{n>=1} 2n/(2n+1) z^(2n-1)
+// (their mean is (1/a - 1/b)/(2(a-b)); the odd part of the series is the rest).
+// Seven terms give 1e-18 for |z| <= 1/16, that is a/b within 13 per cent;
+// wider pairs take the quotients, which lose nothing there.
+template <bool PAIR, typename T>
+PFM_HD T dd_log(T a, T b, T d, T ia, T ib, T* faab, T* fabb) {
+  const T r = T(1) / (a + b);
+  const T z = d * r;
+  if (fabsf(to_f32(z)) <= 0.0625f) {
+    const T y = z * z;
+    const T r2 = r + r;
+    T p = T(1.0 / 13.0);
+    p = p * y + T(1.0 / 11.0);
+    p = p * y + T(1.0 / 9.0);
+    p = p * y + T(1.0 / 7.0);
+    p = p * y + T(1.0 / 5.0);
+    p = p * y + T(1.0 / 3.0);
+    p = p * y + T(1);
+    if (PAIR) {
+      T c = T(14.0 / 15.0);
+      c = c * y + T(12.0 / 13.0);
+      c = c * y + T(10.0 / 11.0);
+      c = c * y + T(8.0 / 9.0);
+      c = c * y + T(6.0 / 7.0);
+      c = c * y + T(4.0 / 5.0);
+      c = c * y + T(2.0 / 3.0);
+      const T odd = r2 * r * z * c;
+      const T even = T(-0.5) * ia * ib;
+      *faab = even + odd;
+      *fabb = even - odd;
+    }
+    return r2 * p;
   }
-  const T top = x > y ? (x > z ? x : z) : (y > z ? y : z);
-  if (gap > Tol<T>::dd2_gap * top) return num / den;
-  return dd2_log(x, y, z);
+  const T f1 = d < T(0) ? log1p(-d / a) / -d : log1p(d / b) / d;
+  if (PAIR) {
+    const T id = T(1) / d;
+    *faab = (ia - f1) * id;
+    *fabb = (f1 - ib) * id;
+  }
+  return f1;
+}
+
+// Second divided difference of log at three values from their first ones
+// (f12 = f[l1,l2] and so on; x = l - 1). Narrow spread (the whole spread at most
+// Tol::f2_gap of the mean m): f^(2+j)(m)/(2+j)! h_j(x - m) summed over j, for log
+// (1/m^2) sum_j (-1)^(j+1) h_j(u)/(j+2), u = (x - m)/m, with the complete
+// homogeneous symmetric polynomials h_j; the u sum to zero, so
+// h_j = -e2 h_(j-2) + e3 h_(j-3). Otherwise the quotient over the largest gap.
+template <typename T>
+PFM_HD T dd2_log(const T x[3], T f12, T f02, T f01) {
+  const float g01 = fabsf(to_f32(x[0] - x[1])), g02 = fabsf(to_f32(x[0] - x[2])), g12 = fabsf(to_f32(x[1] - x[2]));
+  const float gap = fmaxf(g01, fmaxf(g02, g12));
+  const T m = (x[0] + x[1] + x[2]) * T(1.0 / 3.0);
+  if (gap <= Tol<T>::f2_gap * fabsf(1.f + to_f32(m))) {
+    const T im = T(1) / (T(1) + m);
+    const T u0 = (x[0] - m) * im, u1 = (x[1] - m) * im, u2 = (x[2] - m) * im;
+    const T ne2 = u0 * u0 + u1 * (u0 + u1);  // -e2 = u0^2 + u0 u1 + u1^2
+    const T e3 = u0 * u1 * u2;
+    const T h4 = ne2 * ne2, h5 = T(2) * ne2 * e3;
+    const T h6 = ne2 * h4 + e3 * e3, h7 = ne2 * h5 + e3 * h4, h8 = ne2 * h6 + e3 * h5;
+    const T s = T(-0.5) - T(0.25) * ne2 + T(0.2) * e3 - T(1.0 / 6.0) * h4 + T(1.0 / 7.0) * h5 - T(0.125) * h6 +
+                T(1.0 / 9.0) * h7 - T(0.1) * h8;
+    return s * im * im;
+  }
+  if (g02 >= g01 && g02 >= g12) return (f01 - f12) / (x[0] - x[2]);
+  if (g01 >= g12) return (f02 - f12) / (x[0] - x[1]);
+  return (f01 - f02) / (x[1] - x[2]);
 }
 
 // ---------------------------------------------------------------------------
 // Local energy density with gradient and (optionally) packed Hessian.
 //
 // Fin: F row-major; eh, ehn: eta_1..eta_6 at t_{n+1} and t_n.
-// Outputs: *W, g[15] = dW/dz, Hp[120] = packed d^2W/dz^2 (if Hp != nullptr).
-template <typename T, bool WANT_HESS>
-PFM_HD_BIG void qp_local(const DevParams& P, const T Fin[9], const T eh[NV], const T ehn[NV], T* W,
-                     T g[NZ], T* Hp) {
-  T eta[NPH], etan[NPH];
-  {
-    T s = 0, sn = 0;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) { eta[k + 1] = eh[k]; etan[k + 1] = ehn[k]; s += eh[k]; sn += ehn[k]; }
-    eta[0] = T(1) - s;
-    etan[0] = T(1) - sn;
-  }
-  // sum of the eta_i as the same floating-point sum the per-phase loops form
-  T esum = T(0);
-#pragma unroll
-  for (int p = 0; p < NPH; ++p) esum += eta[p];
-  T F[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) F[i][j] = Fin[3 * i + j];
+// Outputs: *W, g[15] = dW/dz; with Emit::want every entry of the packed Hessian
+// d^2W/dz^2 is handed once to emit(index, value) when it is final (no order), so
+// no array of the whole Hessian is kept.
+template <typename T>
+struct NoHess {
+  static constexpr bool want = false;
+  PFM_HD void operator()(int, T) const {}
+};
+template <typename T>
+struct HessArray {
+  static constexpr bool want = true;
+  T* Hp;
+  PFM_HD void operator()(int i, T v) const { Hp[i] = v; }
+};
 
-  // transformation stretch, its inverse and determinant
-  T Ft[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+template <typename T, typename Emit>
+PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T ehn[NV], T* W, T g[NZ],
+                     const Emit& emit) {
+  // transformation stretch F^t = U_0 + sum eta_hat_k dU_k, its inverse and determinant
+  T A[6];
+  T Jt;
+  {
+    T Ft[6];
 #pragma unroll
-  for (int p = 0; p < NPH; ++p)
+    for (int v = 0; v < 6; ++v) {
+      T s = eh[0] * T(P.dU[0][v]);
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) Ft[i][j] += eta[p] * T(P.U[p][i][j]);
-  T A[3][3];
-  const T Jt = inv_sym3(Ft, A);
+      for (int k = 1; k < NV; ++k) s += eh[k] * T(P.dU[k][v]);
+      Ft[v] = T(P.U0[v]) + s;  // one rounding near 1
+    }
+    Jt = inv_sym6(Ft, A);
+  }
   T M[3][3];  // F^e = F A
-  mm3(F, A, M);
-  T E[3][3];  // C^e = M^T M
-  mtm3(M, M, E);
-
-  // spectral decomposition of C^e and the Hencky strain h = 1/2 log C^e
-  T lam[3], Q[3][3];
-  {
-    T tmp[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) tmp[i][j] = E[i][j];
-    eig_sym3(tmp, lam, Q);
-  }
-  // f = log (exact mode) or the Pade approximant r_m, at the eigenvalues, and
-  // its first divided differences
-  T loglam[3];
-  T f1[3][3];
-  T rp[3][3];  // Pade modes: rp[k][a] = 1 / p_k(lam_a)
-  const int npade = P.hencky;
-  if (npade == 0) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) loglam[a] = log(lam[a]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = a; b < 3; ++b) f1[a][b] = f1[b][a] = (a == b) ? T(1) / lam[a] : dd1_log(lam[a], lam[b]);
-  } else {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      loglam[a] = T(0);
-#pragma unroll
-      for (int b = 0; b < 3; ++b) f1[a][b] = T(0);
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      if (k < npade) {
-        const T sk = T(P.pade_s[k]), wk = T(P.pade_w[k]);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          rp[k][a] = T(1) / (T(1) + sk * (lam[a] - T(1)));
-          loglam[a] += wk * (lam[a] - T(1)) * rp[k][a];
-        }
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-          for (int b = 0; b < 3; ++b) f1[a][b] += wk * rp[k][a] * rp[k][b];
-      }
-    }
-  }
-  T h[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      h[i][j] = T(0.5) * (Q[i][0] * loglam[0] * Q[j][0] + Q[i][1] * loglam[1] * Q[j][1] +
-                          Q[i][2] * loglam[2] * Q[j][2]);
-
-  // stress-like T = L(eta) : h and the per-phase L_i : h
-  T hv[6];
-  voigt_strain(h, hv);
-  T Tv[6] = {0, 0, 0, 0, 0, 0};
-  T hLh[NPH];  // h : L_i : h
-  if (P.same_L) {
-    T s = 0;
+      M[i][j] = Fin[3 * i] * symget(A, 0, j) + Fin[3 * i + 1] * symget(A, 1, j) + Fin[3 * i + 2] * symget(A, 2, j);
+  T x[3], lam[3], Q[3][3];  // eigenvalues lam = 1 + x
+  {
+    T E[6];  // C^e = M^T M
 #pragma unroll
-    for (int I = 0; I < 6; ++I) {
-      T li = 0;
-#pragma unroll
-      for (int J = 0; J < 6; ++J) li += T(P.Lv[0][I][J]) * hv[J];
-      Tv[I] = esum * li;
-      s += hv[I] * li;
+    for (int v = 0; v < 6; ++v) {
+      const int i = sym_i(v), j = sym_j(v);
+      E[v] = M[0][i] * M[0][j] + M[1][i] * M[1][j] + M[2][i] * M[2][j];
     }
+    eig_sym6(E, x, Q);
 #pragma unroll
-    for (int p = 0; p < NPH; ++p) hLh[p] = s;
+    for (int a = 0; a < 3; ++a) lam[a] = T(1) + x[a];
+  }
+  // h = log (exact mode) or the Pade approximant r_m at the eigenvalues (halved:
+  // the Hencky strain), and its divided differences: f1 in the Voigt slots,
+  // f2d[a] = f2(a,a,a), f2p[n] = {f2(p,p,r), f2(p,r,r)} for the pair (p, r), p < r,
+  // without n, and f2t = f2(0,1,2)
+  T h[3], f1[6], f2d[3], f2p[3][2], f2t = T(0);
+  if (P.hencky == 0) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) f1[a] = T(1) / lam[a];
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+      const int p = n == 0 ? 1 : 0, r = n == 2 ? 1 : 2;
+      f1[3 + n] = dd_log<Emit::want>(lam[p], lam[r], x[p] - x[r], f1[p], f1[r], &f2p[n][0], &f2p[n][1]);
+    }
+    // log at one eigenvalue, the others through the divided differences
+    const T l0 = x[0] * dd_log<false>(lam[0], T(1), x[0], T(0), T(0), (T*)nullptr, (T*)nullptr);
+    h[0] = T(0.5) * l0;
+    h[1] = T(0.5) * (l0 + (x[1] - x[0]) * f1[5]);
+    h[2] = T(0.5) * (l0 + (x[2] - x[0]) * f1[4]);
+    if (Emit::want) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) f2d[a] = T(-0.5) * f1[a] * f1[a];
+      f2t = dd2_log(x, f1[3], f1[4], f1[5]);
+    }
   } else {
 #pragma unroll
-    for (int p = 0; p < NPH; ++p) {
-      T s = 0;
+    for (int a = 0; a < 3; ++a) h[a] = f2d[a] = f2p[a][0] = f2p[a][1] = T(0);
+#pragma unroll
+    for (int v = 0; v < 6; ++v) f1[v] = T(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (k < P.hencky) {
+        const T sk = T(P.pade_s[k]), wk = T(P.pade_w[k]);
+        T rp[3];  // 1 / p_k(lam_a)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          rp[a] = T(1) / (T(1) + sk * x[a]);
+          h[a] += T(0.5) * wk * x[a] * rp[a];
+        }
+#pragma unroll
+        for (int v = 0; v < 6; ++v) f1[v] += wk * rp[sym_i(v)] * rp[sym_j(v)];
+        if (Emit::want) {
+          const T ws = wk * sk;
+#pragma unroll
+          for (int a = 0; a < 3; ++a) f2d[a] -= ws * rp[a] * rp[a] * rp[a];
+#pragma unroll
+          for (int n = 0; n < 3; ++n) {
+            const int p = n == 0 ? 1 : 0, r = n == 2 ? 1 : 2;
+            const T wpr = ws * rp[p] * rp[r];
+            f2p[n][0] -= wpr * rp[p];
+            f2p[n][1] -= wpr * rp[r];
+          }
+          f2t -= ws * rp[0] * rp[1] * rp[2];
+        }
+      }
+    }
+  }
+
+  // products of the rows of Q: w[n][v] = Q_na Q_nb for the slot v = (a, b)
+  T w[3][6];
+#pragma unroll
+  for (int n = 0; n < 3; ++n)
+#pragma unroll
+    for (int v = 0; v < 6; ++v) w[n][v] = Q[n][sym_i(v)] * Q[n][sym_j(v)];
+
+  // rotated stress-like T~ = Q^T (L(eta):h) Q, times J_t
+  T TJ[6];
+  T hv[6];             // general stiffness: lab-frame Hencky strain (Voigt, engineering shear)
+  T hLh[NPH];          // and h : L_i : h
+  if (P.cubic) {
+    // lambda I x I + 2 mu I_sym is the same in every basis; delta sum_n e_n^4
+    // becomes delta sum_n w_n w_n^T
+    const T tr = h[0] + h[1] + h[2];
+    const T lt = T(P.cub_lambda) * tr;
+    T c[3];
+#pragma unroll
+    for (int n = 0; n < 3; ++n) c[n] = T(P.cub_delta) * (w[n][0] * h[0] + w[n][1] * h[1] + w[n][2] * h[2]);
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      T t = c[0] * w[0][v] + c[1] * w[1][v] + c[2] * w[2][v];
+      if (v < 3) t += lt + T(2.0 * P.cub_mu) * h[v];
+      TJ[v] = Jt * t;
+    }
+  } else {
+    T hm[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      const int i = sym_i(v), j = sym_j(v);
+      hm[v] = Q[i][0] * h[0] * Q[j][0] + Q[i][1] * h[1] * Q[j][1] + Q[i][2] * h[2] * Q[j][2];
+      hv[v] = v < 3 ? hm[v] : T(2) * hm[v];
+    }
+    T Tv[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+    T se = eh[0];
+#pragma unroll
+    for (int k = 1; k < NV; ++k) se += eh[k];
+    const T eta0 = T(1) - se;
+    const int np = P.same_L ? 1 : NPH;
+    for (int p = 0; p < np; ++p) {
+      const T ep = P.same_L ? T(1) : (p == 0 ? eta0 : eh[p - 1]);
+      T s = T(0);
 #pragma unroll
       for (int I = 0; I < 6; ++I) {
-        T li = 0;
+        T li = T(0);
 #pragma unroll
         for (int J = 0; J < 6; ++J) li += T(P.Lv[p][I][J]) * hv[J];
-        Tv[I] += eta[p] * li;
+        Tv[I] += ep * li;
         s += hv[I] * li;
       }
       hLh[p] = s;
     }
+    T Tt[6];
+    rot_sym6(Q, Tv, Tt);
+#pragma unroll
+    for (int v = 0; v < 6; ++v) TJ[v] = Jt * Tt[v];
   }
-  T hT = 0;
-#pragma unroll
-  for (int I = 0; I < 6; ++I) hT += hv[I] * Tv[I];
-  T Tm[3][3];
-  from_voigt_stress(Tv, Tm);
+  const T cW = T(0.5) * (h[0] * TJ[0] + h[1] * TJ[1] + h[2] * TJ[2]);  // elastic energy 1/2 J_t h:L:h
 
-  // S = dW_el/dE = J_t Dh[T] = 1/2 J_t Dlog[T]; in the eigenbasis S~ = 1/2 J_t f1 o T~
-  T Tt[3][3];
-  rot_in(Q, Tm, Tt);
-  T St[3][3], S[3][3];
+  // twice the rotated stress S~ = dW_el/dE = 1/2 J_t f1 o T~, and the rotated
+  // columns of A and rows of M
+  T S2[6], Aq[3][3], Mq[3][3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
+  for (int v = 0; v < 6; ++v) S2[v] = f1[v] * TJ[v];
 #pragma unroll
-    for (int b = 0; b < 3; ++b) St[a][b] = T(0.5) * Jt * f1[a][b] * Tt[a][b];
-  {
-    T t[3][3];
+  for (int c = 0; c < 3; ++c)
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int a = 0; a < 3; ++a) {
+      Aq[c][a] = symget(A, c, 0) * Q[0][a] + symget(A, c, 1) * Q[1][a] + symget(A, c, 2) * Q[2][a];
+      Mq[c][a] = M[c][0] * Q[0][a] + M[c][1] * Q[1][a] + M[c][2] * Q[2][a];
+    }
+  // dW_el/dF = 2 M S A = (M Q) 2S~ (A Q)^T
+  T Pf[3][3];
 #pragma unroll
-      for (int b = 0; b < 3; ++b) t[i][b] = Q[i][0] * St[0][b] + Q[i][1] * St[1][b] + Q[i][2] * St[2][b];
+  for (int p = 0; p < 3; ++p) {
+    T n[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int a = 0; a < 3; ++a)
+      n[a] = Mq[p][0] * symget(S2, 0, a) + Mq[p][1] * symget(S2, 1, a) + Mq[p][2] * symget(S2, 2, a);
 #pragma unroll
-      for (int j = 0; j < 3; ++j) S[i][j] = t[i][0] * Q[j][0] + t[i][1] * Q[j][1] + t[i][2] * Q[j][2];
-  }
-
-  // energy
-  T Wloc = T(0.5) * Jt * hT;
-  // With eta_0 = 1 - sum eta_hat (Sec. 3.1) the elastic energy depends on
-  // eta_hat_k through U(eta) = sum eta_i U_i and L(eta) = sum eta_i L_i, i.e.
-  // along dU_k = U_k - U_0 and dL_k = L_k - L_0.
-  // dU_k is symmetric (a difference of stretches), so tr(X dU_k) = <X^T, dU_k>.
-  T trAdU[NV];  // tr(A dU_k) = (d J_t / d eta_hat_k) / J_t
-  T gel[NV];    // dW_el / d eta_hat_k
-  {
-    T ES[3][3], ESA[3][3];  // E S, E S A
-    mm3(E, S, ES);
-    mm3(ES, A, ESA);
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      T ta = 0, te = 0;
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          const T d = T(P.U[k + 1][i][j]) - T(P.U[0][i][j]);
-          ta += A[i][j] * d;
-          te += ESA[j][i] * d;
-        }
-      trAdU[k] = ta;
-      // S : dE/d eta_hat_k = -2 tr(S A dU_k E) = -2 tr(E S A dU_k)
-      gel[k] = T(0.5) * Jt * trAdU[k] * hT + T(0.5) * Jt * (hLh[k + 1] - hLh[0]) + T(-2) * te;
+    for (int c = 0; c < 3; ++c) {
+      Pf[p][c] = n[0] * Aq[c][0] + n[1] * Aq[c][1] + n[2] * Aq[c][2];
+      g[3 * p + c] = Pf[p][c];
     }
   }
-  // chemical, obstacle, dissipation, penalty: dW/d eta_i per phase
-  T geta[NPH];
+  // dW_el/dF^t = cW A - Zs with Zs the symmetric part of 2 E S A = M^T dW_el/dF
+  T Zs[6];
 #pragma unroll
-  for (int i = 0; i < NPH; ++i) {
-    T d = eta[i] - etan[i];
-    T neg = eta[i] < T(0) ? eta[i] : T(0);
-    Wloc += eta[i] * T(P.F0[i]) + T(0.5) * T(P.inv_mtau[i]) * d * d + T(0.5) * T(P.eps_eta) * neg * neg;
-    T go = 0;
+  for (int v = 0; v < 6; ++v) {
+    const int i = sym_i(v), j = sym_j(v);
+    T z = M[0][i] * Pf[0][j] + M[1][i] * Pf[1][j] + M[2][i] * Pf[2][j];
+    if (v >= 3) z = T(0.5) * (z + (M[0][j] * Pf[0][i] + M[1][j] * Pf[1][i] + M[2][j] * Pf[2][i]));
+    Zs[v] = z;
+  }
+  T gU[6];
 #pragma unroll
-    for (int j = 0; j < NPH; ++j) {
-      if (j > i) Wloc += T(P.cobst[i][j]) * eta[i] * eta[j];
-      go += T(P.cobst[i][j]) * eta[j];
-    }
-    geta[i] = T(P.F0[i]) + go + T(P.inv_mtau[i]) * d + T(P.eps_eta) * neg;
+  for (int v = 0; v < 6; ++v) {
+    const T t = cW * A[v] - Zs[v];
+    gU[v] = v < 3 ? t : t + t;
+  }
+  // order parameters: elastic part along dU_k, chemical and obstacle energy,
+  // dissipation and penalty (eta_0 = 1 - sum eta_hat, Sec. 3.1)
+  T se = eh[0], d0 = ehn[0] - eh[0];
+#pragma unroll
+  for (int k = 1; k < NV; ++k) {
+    se += eh[k];
+    d0 += ehn[k] - eh[k];
+  }
+  const T eta0 = T(1) - se;
+  const T neg0 = eta0 < T(0) ? eta0 : T(0);
+  T Wloc = cW + T(P.W0);
+  const T g0 = T(P.inv_mtau[0]) * d0 + T(P.eps_eta) * neg0;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    T qk = T(0);
+#pragma unroll
+    for (int l = 0; l < NV; ++l) qk += T(P.Cc[k][l]) * eh[l];
+    const T d = eh[k] - ehn[k];
+    const T neg = eh[k] < T(0) ? eh[k] : T(0);
+    const T dis = T(P.inv_mtau[k + 1]) * d, pen = T(P.eps_eta) * neg;
+    Wloc += eh[k] * (T(P.lin[k]) + T(0.5) * qk) + T(0.5) * (dis * d + pen * neg);
+    T gk = T(P.lin[k]) + qk;
+#pragma unroll
+    for (int v = 0; v < 6; ++v) gk += gU[v] * T(P.dU[k][v]);
+    g[9 + k] = gk + ((dis + pen) - g0);  // the penalty, by far the largest, last
+  }
+  Wloc += T(0.5) * (T(P.inv_mtau[0]) * d0 * d0 + T(P.eps_eta) * neg0 * neg0);
+  if (!P.same_L) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) g[9 + k] += T(0.5) * Jt * (hLh[k + 1] - hLh[0]);
   }
   *W = Wloc;
-
-  // gradient: P_el = 2 M S A, then eta_hat_k = eta_k - eta_0 (Sec. 3.1)
-  {
-    T MS[3][3], Pm[3][3];
-    mm3(M, S, MS);
-    mm3(MS, A, Pm);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) g[3 * i + j] = T(2) * Pm[i][j];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) g[9 + k] = gel[k] + (geta[k + 1] - geta[0]);
-  }
-  if (!WANT_HESS) return;
-  // the direction eta_hat_k carries dU_k = U_k - U_0; A dU_k enters below
-  T dU[NV][3][3], AdU[NV][3][3];
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) dU[k][i][j] = T(P.U[k + 1][i][j]) - T(P.U[0][i][j]);
-    mm3(A, dU[k], AdU[k]);
-  }
+  if (!Emit::want) return;
 
   // ---------------------------------------------------------------------
-  // Hessian in the 9 + N unknowns z = (F_pQ: 0..8, eta_hat_1..N: 9..8+N), packed
-  // into Hp[hidx(r, c)], r <= c. With eta_0 = 1 - sum eta_hat (Sec. 3.1) every
-  // eta-dependence enters through U(eta) = sum eta_i U_i and L(eta) =
-  // sum eta_i L_i, so the direction eta_hat_k carries dU_k = U_k - U_0 and
-  // dL_k = L_k - L_0 (dU_k, A dU_k and tr(A dU_k) from above) and the
-  // elimination of eta_0 holds term by term.
-  constexpr int ND = NZ;
-  // Rotated directions X~_k = Q^T dE_k Q, symmetric, stored as 6 values
-  // (00, 11, 22, 12, 02, 01).
-  T Xs[ND][6];
+  // Spectral second derivative: J_t (Dh[X]:L~:Dh[Y] + h''-part) as a symmetric
+  // form Mb in the Voigt slots of X~, the diagonal slots holding half of X~_aa
+  // (X~ = a q^T + q a^T has 2 a_a q_a there)
+  T Mb[21];  // packed upper triangle, hm6(I, J)
+  auto hm6 = [](int I, int J) { return I <= J ? I * 6 - (I * (I - 1)) / 2 + (J - I) : J * 6 - (J * (J - 1)) / 2 + (I - J); };
   {
-    T Aq[3][3], Mq[3][3];  // Aq[c] = Q^T (column c of A), Mq[p] = Q^T (row p of M)
-    for (int c = 0; c < 3; ++c)
-      for (int a = 0; a < 3; ++a) {
-        Aq[c][a] = Q[0][a] * A[0][c] + Q[1][a] * A[1][c] + Q[2][a] * A[2][c];
-        Mq[c][a] = Q[0][a] * M[c][0] + Q[1][a] * M[c][1] + Q[2][a] * M[c][2];
+    T fJ[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) fJ[v] = Jt * f1[v];
+    if (P.cubic) {
+      T dw[3][6];
+#pragma unroll
+      for (int n = 0; n < 3; ++n)
+#pragma unroll
+        for (int v = 0; v < 6; ++v) dw[n][v] = T(P.cub_delta) * w[n][v];
+#pragma unroll
+      for (int I = 0; I < 6; ++I)
+#pragma unroll
+        for (int J = I; J < 6; ++J) {
+          T v = dw[0][I] * w[0][J] + dw[1][I] * w[1][J] + dw[2][I] * w[2][J];
+          if (I < 3 && J < 3) v += T(P.cub_lambda);
+          if (I == J) v += I < 3 ? T(2.0 * P.cub_mu) : T(P.cub_mu);
+          Mb[hm6(I, J)] = fJ[I] * f1[J] * v;
+        }
+    } else {
+      T Nv[6][6];  // v(Q X~ Q^T) = Nv v(X~), engineering shear
+      for (int I = 0; I < 6; ++I) {
+        const int i = sym_i(I), j = sym_j(I);
+        const T cI = (I < 3) ? T(1) : T(2);
+        for (int B = 0; B < 6; ++B) {
+          const int a = sym_i(B), b = sym_j(B);
+          Nv[I][B] = (B < 3) ? cI * Q[i][a] * Q[j][a] : cI * T(0.5) * (Q[i][a] * Q[j][b] + Q[i][b] * Q[j][a]);
+        }
       }
-    for (int p = 0; p < 3; ++p)
+      T LN[6][6];
+      for (int I = 0; I < 6; ++I) {
+        T Le[6];  // row I of L(eta)
+        for (int J = 0; J < 6; ++J) {
+          T l = T(P.Lv[0][I][J]);
+          if (!P.same_L) {
+            l = eta0 * l;
+            for (int k = 0; k < NV; ++k) l += eh[k] * T(P.Lv[k + 1][I][J]);
+          }
+          Le[J] = l;
+        }
+        for (int B = 0; B < 6; ++B) {
+          T s = T(0);
+          for (int J = 0; J < 6; ++J) s += Le[J] * Nv[J][B];
+          LN[I][B] = s;
+        }
+      }
+#pragma unroll
+      for (int I = 0; I < 6; ++I)
+#pragma unroll
+        for (int J = I; J < 6; ++J) {
+          T s = T(0);
+          for (int K = 0; K < 6; ++K) s += Nv[K][I] * LN[K][J];
+          Mb[hm6(I, J)] = fJ[I] * f1[J] * s;
+        }
+    }
+    // sum over a, b, c of f2(a,b,c) T~_ab into the slots (a,c), (b,c)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      Mb[hm6(a, a)] += T(4) * f2d[a] * TJ[a];
+#pragma unroll
       for (int c = 0; c < 3; ++c) {
-        T* X = Xs[3 * p + c];
-        for (int v = 0; v < 6; ++v) {
-          const int a = sym_i(v), b = sym_j(v);
-          X[v] = Aq[c][a] * Mq[p][b] + Mq[p][a] * Aq[c][b];
-        }
+        if (c == a) continue;
+        const int n = 3 - a - c, sl = 3 + n;
+        Mb[hm6(sl, sl)] += (a < c ? f2p[n][0] : f2p[n][1]) * TJ[a];
       }
+    }
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+      const int p = n == 0 ? 1 : 0, r = n == 2 ? 1 : 2, sl = 3 + n;
+      const T t2 = T(2) * TJ[sl];
+      Mb[hm6(p, sl)] += f2p[n][0] * t2;
+      Mb[hm6(r, sl)] += f2p[n][1] * t2;
+      Mb[hm6(3 + r, 3 + p)] += f2t * TJ[sl];  // slots (p, n) and (r, n)
+    }
   }
-  for (int k = 0; k < NV; ++k) {
-    T B[3][3];
-    rot_in(Q, AdU[k], B);  // B = Q^T A dU_k Q ; dE~ = -(B Lambda + Lambda B^T)
+  // left vectors of the directions in the eigenbasis: Mq[p] (F_p.) and
+  // Uq[i] = -Lambda Q^T e_i (entry (i, .) of F^t)
+  T Uq[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) Uq[i][a] = -(lam[a] * Q[i][a]);
+  T il[3];  // 1 / lambda
+#pragma unroll
+  for (int a = 0; a < 3; ++a) il[a] = P.hencky == 0 ? f1[a] : T(1) / lam[a];
+  T FU[9][6], K[21];
+#pragma unroll
+  for (int r = 0; r < 9; ++r)
+#pragma unroll
+    for (int v = 0; v < 6; ++v) FU[r][v] = T(0);
+#pragma unroll
+  for (int v = 0; v < 21; ++v) K[v] = T(0);
+#pragma unroll
+  for (int c2 = 0; c2 < 3; ++c2) {
+    T Y[6][3];  // Mb N_c2: change of slot v along (column c2, left vector e_b)
+#pragma unroll
+    for (int v = 0; v < 6; ++v)
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+        Y[v][b] = Mb[hm6(v, voigt_slot(b, 0))] * Aq[c2][0] + Mb[hm6(v, voigt_slot(b, 1))] * Aq[c2][1] +
+                  Mb[hm6(v, voigt_slot(b, 2))] * Aq[c2][2];
+    T sa[3];  // 2S~ a_c2
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      sa[a] = symget(S2, a, 0) * Aq[c2][0] + symget(S2, a, 1) * Aq[c2][1] + symget(S2, a, 2) * Aq[c2][2];
+#pragma unroll
+    for (int c = 0; c <= c2; ++c) {
+      T R[3][3];
+      const T asa = Aq[c][0] * sa[0] + Aq[c][1] * sa[1] + Aq[c][2] * sa[2];
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          if (c == c2 && b < e) {
+            R[e][b] = R[b][e];
+            continue;
+          }
+          T s = Aq[c][0] * Y[voigt_slot(e, 0)][b] + Aq[c][1] * Y[voigt_slot(e, 1)][b] + Aq[c][2] * Y[voigt_slot(e, 2)][b];
+          if (e == b) s += asa * il[e];
+          R[e][b] = s;
+        }
+      T Zf[3][3], Zu[3][3];  // left vectors times R
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          Zf[p][b] = Mq[p][0] * R[0][b] + Mq[p][1] * R[1][b] + Mq[p][2] * R[2][b];
+          Zu[p][b] = Uq[p][0] * R[0][b] + Uq[p][1] * R[1][b] + Uq[p][2] * R[2][b];
+        }
+      auto dot = [](const T* x, const T* y) { return x[0] * y[0] + x[1] * y[1] + x[2] * y[2]; };
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          // F_pc with F_rc2 (final)
+          if (c < c2 || p <= r) {
+            const int i = 3 * p + c, j = 3 * r + c2;
+            emit(i <= j ? hidx(i, j) : hidx(j, i), dot(Zf[p], Mq[r]));
+          }
+          // F_pc with F^t_(r, c2), and F_pc2 with F^t_(r, c)
+          FU[3 * p + c][voigt_slot(r, c2)] += dot(Zf[p], Uq[r]);
+          if (c < c2) FU[3 * p + c2][voigt_slot(r, c)] += dot(Zu[r], Mq[p]);
+          // F^t_(p, c) with F^t_(r, c2)
+          if (c < c2 || p <= r) {
+            const T u = dot(Zu[p], Uq[r]);
+            const int v = voigt_slot(p, c), x = voigt_slot(r, c2);
+            K[hm6(v, x)] += (v == x && !(p == r && c == c2)) ? u + u : u;
+          }
+        }
+    }
+  }
+  // second derivatives of F^e along F and F^t, and of J_t
+#pragma unroll
+  for (int p = 0; p < 3; ++p)
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int v = 0; v < 6; ++v) {
+        const int i = sym_i(v), j = sym_j(v);
+        T s = A[v] * Pf[p][c];
+        if (v >= 3) s += s;
+        s -= symget(A, c, i) * Pf[p][j];
+        if (v >= 3) s -= symget(A, c, j) * Pf[p][i];
+        FU[3 * p + c][v] += s;
+      }
+  // K += 2 tr(Z' dU A dU') - tr(A dU) tr(Z' dU') - tr(Z' dU) tr(A dU'), Z' = Zs - cW/2 A
+  {
+    T Z[6], At[6], Zt[6];
+#pragma unroll
     for (int v = 0; v < 6; ++v) {
-      const int a = sym_i(v), b = sym_j(v);
-      Xs[9 + k][v] = -(B[a][b] * lam[b] + lam[a] * B[b][a]);
+      Z[v] = Zs[v] - T(0.5) * cW * A[v];
+      At[v] = v < 3 ? A[v] : A[v] + A[v];
+      Zt[v] = v < 3 ? Z[v] : Z[v] + Z[v];
     }
-  }
-  // d~_k = Dh~[X~_k] = 1/2 f1 o X~_k as Voigt strain vectors (engineering
-  // shear): d~_k[v] = c[v] X~_k[v]
-  T cv[6];
-  for (int v = 0; v < 6; ++v) cv[v] = T(0.5) * f1[sym_i(v)][sym_j(v)] * (v < 3 ? T(1) : T(2));
-  // L~ = Nv^T L(eta) Nv with v(Q d~ Q^T) = Nv v(d~)
-  T Lt[6][6];
-  if (P.cubic) {
-    // cubic stiffness: the isotropic part lambda I x I + 2 mu I_sym is the
-    // same in every basis, and the cubic part delta sum_n e_n^4 turns into
-    // delta sum_n w_n w_n^T with w_n[A] = r_a r_b for the slot A = (a, b) and
-    // r = row n of Q (e_n in the eigenbasis); all scaled by sum eta
-    const T lam_c = T(P.cub_lambda) * esum, mu_c = T(P.cub_mu) * esum, del_c = T(P.cub_delta) * esum;
-    T w[3][6];
 #pragma unroll
-    for (int n = 0; n < 3; ++n)
+    for (int v = 0; v < 6; ++v)
 #pragma unroll
-      for (int A_ = 0; A_ < 6; ++A_) w[n][A_] = Q[n][sym_i(A_)] * Q[n][sym_j(A_)];
-#pragma unroll
-    for (int A_ = 0; A_ < 6; ++A_)
-#pragma unroll
-      for (int B = A_; B < 6; ++B) {
-        T v = del_c * (w[0][A_] * w[0][B] + w[1][A_] * w[1][B] + w[2][A_] * w[2][B]);
-        if (A_ < 3 && B < 3) v += lam_c;
-        if (A_ == B) v += A_ < 3 ? T(2) * mu_c : mu_c;
-        Lt[A_][B] = Lt[B][A_] = v;
-      }
-  } else {
-    T Nv[6][6];
-    for (int I = 0; I < 6; ++I) {
-      const int i = sym_i(I), j = sym_j(I);
-      const T cI = (I < 3) ? T(1) : T(2);
-      for (int B = 0; B < 6; ++B) {
-        const int a = sym_i(B), b = sym_j(B);
-        Nv[I][B] = (B < 3) ? cI * Q[i][a] * Q[j][a] : cI * T(0.5) * (Q[i][a] * Q[j][b] + Q[i][b] * Q[j][a]);
-      }
-    }
-    T Le[6][6];  // L(eta) = sum_p eta_p L_p
-    for (int I = 0; I < 6; ++I)
-      for (int J = 0; J < 6; ++J) {
-        T lij = 0;
-        if (P.same_L) {
-          lij = T(P.Lv[0][I][J]) * esum;
-        } else {
-          for (int p = 0; p < NPH; ++p) lij += eta[p] * T(P.Lv[p][I][J]);
+      for (int x = v; x < 6; ++x) {
+        const int i = sym_i(v), j = sym_j(v), k = sym_i(x), l = sym_j(x);
+        // tr(Z E A E') over the entries (i,j), (j,i) of E and (k,l), (l,k) of E'
+        T s = symget(Z, l, i) * symget(A, j, k);
+        if (x >= 3) s += symget(Z, k, i) * symget(A, j, l);
+        if (v >= 3) {
+          s += symget(Z, l, j) * symget(A, i, k);
+          if (x >= 3) s += symget(Z, k, j) * symget(A, i, l);
         }
-        Le[I][J] = lij;
-      }
-    T LN[6][6];
-    for (int I = 0; I < 6; ++I)
-      for (int B = 0; B < 6; ++B) {
-        T s = 0;
-        for (int J = 0; J < 6; ++J) s += Le[I][J] * Nv[J][B];
-        LN[I][B] = s;
-      }
-    for (int A_ = 0; A_ < 6; ++A_)
-      for (int B = 0; B < 6; ++B) {
-        T s = 0;
-        for (int I = 0; I < 6; ++I) s += Nv[I][A_] * LN[I][B];
-        Lt[A_][B] = s;
+        K[hm6(v, x)] += s + s - (At[v] * Zt[x] + Zt[v] * At[x]);
       }
   }
-  // The second-order part of the elastic energy along directions k, l,
-  // J_t (d~_k . L~ d~_l + K(k,l)) with K(k,l) = sum_abc f2_abc T~_ab X~_k[a][c]
-  // X~_l[b][c] (f2: second divided differences, symmetric), is one symmetric
-  // bilinear form in the 6 stored entries of X~: X~_k^T Mb X~_l with
-  // Mb[v][w] = J_t (c[v] L~[v][w] c[w] + sum of f2_abc T~_ab over the (a, b, c)
-  // whose pairs (a, c) and (b, c) have the Voigt slots v and w).
-  T f2[3][3][3];
-  for (int a = 0; a < 3; ++a)
-    for (int b = a; b < 3; ++b)
-      for (int c = b; c < 3; ++c) {
-        T v;
-        if (npade == 0) {
-          // one eigenvalue: f'' / 2 = -1 / (2 lam^2)
-          v = (a == c) ? T(-0.5) * f1[a][a] * f1[a][a]
-                       : dd2_log_f1(lam[a], lam[b], lam[c], f1[a][b], f1[b][c], f1[a][c]);
-        } else {
-          v = T(0);
-          for (int k = 0; k < 3; ++k)
-            if (k < npade) v -= T(P.pade_w[k]) * T(P.pade_s[k]) * rp[k][a] * rp[k][b] * rp[k][c];
-        }
-        f2[a][b][c] = f2[a][c][b] = f2[b][a][c] = f2[b][c][a] = f2[c][a][b] = f2[c][b][a] = v;
-      }
-  T Mb[6][6];
-  for (int I = 0; I < 6; ++I)
-    for (int J = 0; J < 6; ++J) Mb[I][J] = cv[I] * Lt[I][J] * cv[J];
-  for (int a = 0; a < 3; ++a)
-    for (int b = 0; b < 3; ++b)
-      for (int c = 0; c < 3; ++c) Mb[voigt_slot(a, c)][voigt_slot(b, c)] += f2[a][b][c] * Tt[a][b];
-  for (int I = 0; I < 6; ++I)
-    for (int J = 0; J < 6; ++J) Mb[I][J] *= Jt;
-  // (dL_k h) rotated and scaled by c, so that (dL_k h)~ : d~_l = LhT[k] . X~_l;
-  // zero when every phase has the same stiffness
-  T LhT[NV][6];
+  // per-phase stiffness: (dL_k h) along the directions, LX[k][v] for F^t
+  T LX[NV][6];
   if (!P.same_L) {
     for (int k = 0; k < NV; ++k) {
-      T lv[6], lm[3][3], lr[3][3];
+      T lv[6], lr[6];
       for (int I = 0; I < 6; ++I) {
-        T s = 0;
+        T s = T(0);
         for (int J = 0; J < 6; ++J) s += (T(P.Lv[k + 1][I][J]) - T(P.Lv[0][I][J])) * hv[J];
         lv[I] = s;
       }
-      from_voigt_stress(lv, lm);
-      rot_in(Q, lm, lr);
-      for (int v = 0; v < 6; ++v) LhT[k][v] = cv[v] * lr[sym_i(v)][sym_j(v)];
+      rot_sym6(Q, lv, lr);
+      for (int v = 0; v < 6; ++v) lr[v] = Jt * f1[v] * lr[v];
+      for (int v = 0; v < 6; ++v) LX[k][v] = T(0);
+      for (int c = 0; c < 3; ++c) {
+        T t[3];
+        for (int a = 0; a < 3; ++a)
+          t[a] = symget(lr, a, 0) * Aq[c][0] + symget(lr, a, 1) * Aq[c][1] + symget(lr, a, 2) * Aq[c][2];
+        for (int p = 0; p < 3; ++p) {
+          T fk = t[0] * Mq[p][0] + t[1] * Mq[p][1] + t[2] * Mq[p][2];
+          for (int v = 0; v < 6; ++v) fk += FU[3 * p + c][v] * T(P.dU[k][v]);
+          emit(hidx(3 * p + c, 9 + k), fk);
+          LX[k][voigt_slot(p, c)] += t[0] * Uq[p][0] + t[1] * Uq[p][1] + t[2] * Uq[p][2];
+        }
+      }
+    }
+  } else {
+#pragma unroll 1
+    for (int k = 0; k < NV; ++k) {
+      T d[6];
+#pragma unroll
+      for (int v = 0; v < 6; ++v) d[v] = T(P.dU[k][v]);
+#pragma unroll
+      for (int r = 0; r < 9; ++r) {
+        T s = FU[r][0] * d[0];
+#pragma unroll
+        for (int v = 1; v < 6; ++v) s += FU[r][v] * d[v];
+        emit(hidx(r, 9 + k), s);
+      }
     }
   }
-  // second-order part X~_k^T Mb X~_l, and the first-order terms
-  // g_{E eta_p}[X_k] = tr(A dU_p) S~:X~_k + J_t (dL_p h)~ : d~_k, added to the
-  // F-eta and eta-eta entries (the latter for both index orders).
-  for (int k = 0; k < ND; ++k) {
-    T Y[6];
-    for (int I = 0; I < 6; ++I) {
-      T s = 0;
-      for (int J = 0; J < 6; ++J) s += Mb[I][J] * Xs[k][J];
-      Y[I] = s;
+  // eta-eta: K along the dU_k, and the local terms
+  // Cc_kl + d_0 + delta_kl d_k, d_i = 1/(m_i tau) + eps [eta_i < 0]
+  const T dd0 = T(P.inv_mtau[0]) + (eta0 < T(0) ? T(P.eps_eta) : T(0));
+#pragma unroll 1
+  for (int q = 0; q < NV; ++q) {
+    T t[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      T s = K[hm6(v, 0)] * T(P.dU[q][0]);
+#pragma unroll
+      for (int x = 1; x < 6; ++x) s += K[hm6(v, x)] * T(P.dU[q][x]);
+      t[v] = s;
     }
-    for (int l = k; l < ND; ++l) {
-      T acc = 0;
-      for (int I = 0; I < 6; ++I) acc += Xs[l][I] * Y[I];
-      Hp[hidx(k, l)] = acc;
-    }
-    // S~ : X~_k (tensor double contraction of symmetric matrices)
-    T SX = 0;
-    for (int v = 0; v < 6; ++v) SX += (v < 3 ? T(1) : T(2)) * St[sym_i(v)][sym_j(v)] * Xs[k][v];
-    for (int p = 0; p < NV; ++p) {
-      T ge = trAdU[p] * SX;
+    for (int p = 0; p <= q; ++p) {
+      T s = T(P.Cc[p][q]);
+#pragma unroll
+      for (int v = 0; v < 6; ++v) s += t[v] * T(P.dU[p][v]);
+      T loc = dd0;
+      if (p == q) loc += T(P.inv_mtau[p + 1]) + (eh[p] < T(0) ? T(P.eps_eta) : T(0));
       if (!P.same_L) {
-        T d = 0;
-        for (int v = 0; v < 6; ++v) d += LhT[p][v] * Xs[k][v];
-        ge += Jt * d;
+        T ap = T(0), aq = T(0);  // tr(A dU_p), tr(A dU_q)
+        for (int v = 0; v < 6; ++v) {
+          const T a2 = v < 3 ? A[v] : A[v] + A[v];
+          ap += a2 * T(P.dU[p][v]);
+          aq += a2 * T(P.dU[q][v]);
+          s += LX[p][v] * T(P.dU[q][v]) + LX[q][v] * T(P.dU[p][v]);
+        }
+        s += T(0.5) * Jt * (ap * (hLh[q + 1] - hLh[0]) + aq * (hLh[p + 1] - hLh[0]));
       }
-      if (k < 9) {
-        Hp[hidx(k, 9 + p)] += ge;
-      } else {
-        const int q = k - 9;
-        const int lo = p < q ? p : q, hi = p < q ? q : p;
-        Hp[hidx(9 + lo, 9 + hi)] += (p == q) ? T(2) * ge : ge;
-      }
+      emit(hidx(9 + p, 9 + q), s + loc);
     }
   }
-  // S : d^2E, F-F block: delta_pr 2 (A S A)_QS
-  T ASA[3][3];
-  {
-    T t[3][3];
-    mm3(S, A, t);
-    mm3(A, t, ASA);
-  }
-  for (int p = 0; p < 3; ++p)
-    for (int q = 0; q < 3; ++q)
-      for (int s2 = q; s2 < 3; ++s2) Hp[hidx(3 * p + q, 3 * p + s2)] += T(2) * ASA[q][s2];
-  // per direction: Y_k = A dU_k A, S Y_k, C Y_k, S E dU_k
-  T C[3][3], SE[3][3];
-  mtm3(F, F, C);
-  mm3(S, E, SE);
-  T Yk[NV][3][3], SY[NV][3][3], CY[NV][3][3], SEU[NV][3][3];
-  for (int k = 0; k < NV; ++k) {
-    mm3(AdU[k], A, Yk[k]);
-    mm3(S, Yk[k], SY[k]);
-    mm3(C, Yk[k], CY[k]);
-    mm3(SE, dU[k], SEU[k]);
-  }
-  // F-eta block: -2 (F N_k)_rQ with N_k = ASA dU_k A + A dU_k ASA, where
-  // F ASA dU_k A = M (S Y_k) and F A dU_k ASA = (M dU_k) ASA
-  for (int k = 0; k < NV; ++k) {
-    T MdU[3][3], t1[3][3], t2[3][3];
-    mm3(M, SY[k], t1);
-    mm3(M, dU[k], MdU);
-    mm3(MdU, ASA, t2);
-    for (int r = 0; r < 9; ++r) Hp[hidx(r, 9 + k)] += T(-2) * (t1[r / 3][r % 3] + t2[r / 3][r % 3]);
-  }
-  // eta-eta block: S:d2E + explicit eta derivatives of g + local terms
-  // (obstacle, dissipation, penalty), the last written in eta_hat:
-  // c_kl - c_k0 - c_0l + c_00 + d_0 + delta_kl d_k, d_i = 1/(m_i tau) + eps [eta_i < 0]
-  const T d0 = T(P.inv_mtau[0]) + (eta[0] < T(0) ? T(P.eps_eta) : T(0));
-  for (int p = 0; p < NV; ++p) {
-    const T hLp = hLh[p + 1] - hLh[0];
-    for (int q = p; q < NV; ++q) {
-      const T hLq = hLh[q + 1] - hLh[0];
-      T sd2E = T(2) * (tr_ab(SEU[p], Yk[q]) + tr_ab(SEU[q], Yk[p]) + tr_ab(SY[p], CY[q]));
-      T Jpq = Jt * (trAdU[p] * trAdU[q] - tr_ab(AdU[p], AdU[q]));
-      T gee = T(0.5) * Jpq * hT + T(0.5) * Jt * trAdU[p] * hLq + T(0.5) * Jt * trAdU[q] * hLp;
-      T loc = T(P.cobst[p + 1][q + 1]) - T(P.cobst[p + 1][0]) - T(P.cobst[0][q + 1]) + T(P.cobst[0][0]) + d0;
-      if (p == q) loc += T(P.inv_mtau[p + 1]) + (eta[p + 1] < T(0) ? T(P.eps_eta) : T(0));
-      Hp[hidx(9 + p, 9 + q)] += sd2E + gee + loc;
-    }
-  }
+}
+
+// qp_point with the packed Hessian (if wanted) in an array.
+template <typename T, bool WANT_HESS>
+PFM_HD_BIG void qp_local(const DevParams& P, const T Fin[9], const T eh[NV], const T ehn[NV], T* W, T g[NZ], T* Hp) {
+  if constexpr (WANT_HESS)
+    qp_point<T>(P, Fin, eh, ehn, W, g, HessArray<T>{Hp});
+  else
+    qp_point<T>(P, Fin, eh, ehn, W, g, NoHess<T>{});
 }
 
 }  // namespace pfm
