@@ -22,7 +22,7 @@
 // one row per thread, the row's nb entries in registers; per column every CTA
 // sends its best candidate (value, row and the row scaled by the pivot) to all
 // CTAs through distributed shared memory and one cluster barrier follows, so a
-// column costs about 5 microseconds of latency and no launch (times at
+// column costs about 4 microseconds of latency and no launch (times at
 // launch_coarse_inverse).
 #pragma once
 
@@ -55,6 +55,19 @@ __device__ __forceinline__ unsigned long long gj_key(double v) {
   return (static_cast<unsigned long long>(__double_as_longlong(v)) & 0x7fffffffffffffffull) + 1ull;
 }
 
+// Largest key of the warp with its index (ties: the lowest index).
+__device__ __forceinline__ void gj_best(unsigned long long& key, int& r) {
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) {
+    const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, m);
+    const int orow = __shfl_xor_sync(0xffffffffu, r, m);
+    if (ok > key || (ok == key && orow < r)) {
+      key = ok;
+      r = orow;
+    }
+  }
+}
+
 // Panel step (see above) by one cluster of `csize` CTAs, this CTA of rank
 // `rank`; R = rows per CTA (<= blockDim.x). used[row] = 1 + the column the row
 // was the pivot of (0: not yet). A column without a non-zero pivot sets
@@ -84,39 +97,28 @@ __device__ __forceinline__ void gj_panel(double* __restrict__ M, int n, int k0, 
     // best row of the CTA
     unsigned long long key = u == 0 ? gj_key(a[j]) : 0ull;
     int r = row;
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1) {
-      const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, m);
-      const int orow = __shfl_xor_sync(0xffffffffu, r, m);
-      if (ok > key || (ok == key && orow < r)) {
-        key = ok;
-        r = orow;
-      }
-    }
+    gj_best(key, r);
     if (lane == 0) {
       wkey[wid] = key;
       wrow[wid] = r;
     }
     __syncthreads();
-    unsigned long long bk = wkey[0];
-    int br = wrow[0];
-    for (int w = 1; w < nwarp; ++w)
-      if (wkey[w] > bk) {  // rows grow with the warp: the first of equals is the lowest
-        bk = wkey[w];
-        br = wrow[w];
-      }
+    unsigned long long bk = lane < nwarp ? wkey[lane] : 0ull;
+    int br = lane < nwarp ? wrow[lane] : 0;
+    gj_best(bk, br);
     // the warp that holds it sends the candidate to every CTA
     const int owner = bk == 0 ? 0 : br - int(rank) * R;
     if (wid == (owner >> 5)) {
       const int src = owner & 31;
       const double pv = __shfl_sync(0xffffffffu, a[j], src);
       const double ip = 1.0 / pv;
-      double val = 0.0;
+      double val = 1.0;
 #pragma unroll
       for (int c = 0; c < GJ_NB; ++c) {
         const double x = __shfl_sync(0xffffffffu, a[c], src);
-        if (lane == c) val = c == j ? ip : x * ip;
+        if (lane == c && c != j) val = x;
       }
+      val *= ip;
       for (unsigned t = 0; t < csize; ++t) {
         GjCandidate* m = cl.map_shared_rank(&mail[j & 1][rank], t);
         if (lane < GJ_NB) m->row[lane] = val;
@@ -127,9 +129,9 @@ __device__ __forceinline__ void gj_panel(double* __restrict__ M, int n, int k0, 
     }
     cl.sync();
     // the same choice in every CTA
-    int best = 0;
-    for (unsigned t = 1; t < csize; ++t)
-      if (mail[j & 1][t].key > mail[j & 1][best].key) best = int(t);
+    unsigned long long mk = lane < int(csize) ? mail[j & 1][lane].key : 0ull;
+    int best = lane;
+    gj_best(mk, best);
     const GjCandidate& p = mail[j & 1][best];
     if (p.key == 0 || !(fabs(p.pivot) > 0.0)) {
       if (rank == 0 && tid == 0) *singular = 1;

@@ -378,7 +378,7 @@ void launch_coarse_assemble(const Grid& g, const DevParams& P, const T* H, const
 // Invert the dense coarse operator M (n x n, overwritten; followed by GJ_NB * n
 // doubles of work) into Ainv (n x n). used, piv: n integers of work each.
 // One panel and one update per GJ_NB columns. Measured at n = 1125 (the 4^3
-// coarsest level): 71 panels of 79 us and 71 updates of 42 us, 8.6 ms; one
+// coarsest level): 71 panels of 60 us and 71 updates of 42 us, 7.3 ms; one
 // launch per column over the augmented matrix took 15.2 ms.
 void launch_coarse_inverse(double* M, int n, double* Ainv, int* used, int* piv, int* singular, cudaStream_t s) {
   double* W = M + int64_t(n) * n;
