@@ -336,7 +336,6 @@ pfm_status residual_impl(pfm_handle* h, double* R, double* energy_host) {
   Level& f = h->L[0];
   cudaStream_t s = h->stream;
   TRY(det_ready(h));
-  if (!h->det) CK(cudaMemsetAsync(R, 0, sizeof(double) * ndof(f), s));  // the atomic form adds into R
   CK(cudaMemsetAsync(h->energy_dev, 0, sizeof(double), s));
   {
     ProfScope ps(h, PFM_PROF_RESIDUAL);
@@ -416,7 +415,6 @@ pfm_status linearize_impl(pfm_handle* h, pfm_precision prec, double* R_fused = n
       const bool fp32_compute = !fine && !coarsest && prec == PFM_F32;
       const int arith = fp32_compute ? LIN_F32 : (h->lin_df ? LIN_DF : LIN_F64);
       if (fine && R_fused) {
-        if (!h->det) CK(cudaMemsetAsync(R_fused, 0, sizeof(double) * ndof(lv), s));
         CK(cudaMemsetAsync(h->energy_dev, 0, sizeof(double), s));
         const LinResidual res{lv.mask, R_fused, h->energy_dev, det_W<double>(h)};
         launch_linearize(lv.g, h->dp, lv.U, lv.Un, need64 ? lv.H64 : nullptr, need32 ? lv.H32 : nullptr,
@@ -1590,7 +1588,6 @@ pfm_status pfm_param_grad(pfm_handle* h, const double* w_dev, double* dPi, doubl
     make_dev_params(q, dq);
     for (int ph = 0; ph < NPH; ++ph) dq.inv_mtau[ph] = 0.0;  // no dissipation
     if (dR_dev) Rk = dR_dev + int64_t(k) * n;
-    CK(cudaMemsetAsync(Rk, 0, sizeof(double) * n, s));
     CK(cudaMemsetAsync(h->energy_dev, 0, sizeof(double), s));
     TRY(det_ready(h));
     launch_residual(f.g, dq, f.U, f.Un, f.mask, Rk, h->energy_dev, s, det_W<double>(h));

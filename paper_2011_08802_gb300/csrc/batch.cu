@@ -23,6 +23,7 @@
 #include "coarse_inverse.cuh"
 #include "common.cuh"
 #include "fe_device.cuh"
+#include "grad_energy.cuh"
 #include "handle.h"
 #include "mg_device.cuh"
 
@@ -130,6 +131,8 @@ struct BOut {
   int64_t n;  // 9 * nodes
   DfConst dk;
   JParams<double> jp64;
+  GradEDf ged;            // nodal gradient energy in double-float and FP64
+  GradE<double> ge64;
   const float* Hhi;
   const float* Hlo;
   const double* H64;
@@ -201,7 +204,7 @@ __global__ void __launch_bounds__(256) k_b_japply(const BLev* __restrict__ S, in
       if constexpr (H16)
         japply_block_h16<false>(L.g, L.jp, L.wh, L.H16, L.mask, L.vec[vsel], L.vec[ysel], blk - L.blk0, lane);
       else
-        japply_block<float>(L.g, L.jp, L.H, L.mask, L.vec[vsel], L.vec[ysel], blk - L.blk0, lane);
+        japply_block<float, true>(L.g, L.jp, L.H, L.mask, L.vec[vsel], L.vec[ysel], blk - L.blk0, lane);
     }
   }
 }
@@ -496,17 +499,27 @@ __global__ void k_b_cast_in(const BOut* __restrict__ O, const BFgm* __restrict__
     o.b32[i] = float(v[i]);
 }
 
-// Z_j = x32 (the V-cycle output) and w = Z_j at Dirichlet DOFs, 0 elsewhere
+// Z_j = x32 (the V-cycle output)
 __global__ void k_b_store_z(const BOut* __restrict__ O, const BFgm* __restrict__ F, int j) {
   const int p = blockIdx.y;
   if (!F[p].active) return;
   const BOut& o = O[p];
-  const int64_t nn = o.g.nn();
   float* z = o.Z + int64_t(j) * o.n;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < o.n; i += int64_t(gridDim.x) * blockDim.x) {
-    const float v = o.x32[i];
-    z[i] = v;
-    o.w[i] = ((o.mask[i % nn] >> int(i / nn)) & 1) ? double(v) : 0.0;
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < o.n; i += int64_t(gridDim.x) * blockDim.x)
+    z[i] = o.x32[i];
+}
+
+// first pass of w = J Z_j: identity rows and the nodal gradient energy
+// (grad_energy.cuh) of every active problem
+__global__ void __launch_bounds__(GE_COLS * NV) k_b_grad_energy_df(const BOut* __restrict__ O, const BFgm* __restrict__ F, int j) {
+  const int p = blockIdx.y;
+  if (!F[p].active) return;
+  const BOut& o = O[p];
+  const int64_t ncol = grad_energy_columns(o.g);
+  __shared__ GradESmem<df64> sm;
+  for (int64_t t = int64_t(blockIdx.x) * GE_COLS; t < ncol; t += int64_t(gridDim.x) * GE_COLS) {
+    grad_energy_block<df64, GE_APPLY>(o.g, o.ged, o.mask, o.Z + int64_t(j) * o.n, o.w, t, ncol, sm, false);
+    __syncthreads();
   }
 }
 
@@ -537,7 +550,7 @@ __global__ void __launch_bounds__(256) k_b_japply64(const BOut* __restrict__ O, 
     if (!F[p].restart) continue;
     const BOut& o = O[p];
     const int64_t b = blk - o.blk0;
-    if (b < o.g.nblk()) japply_block<double>(o.g, o.jp64, o.H64, o.mask, o.x, o.w, b, lane);
+    if (b < o.g.nblk()) japply_block<double, false>(o.g, o.jp64, o.H64, o.mask, o.x, o.w, b, lane);
   }
 }
 
@@ -706,14 +719,17 @@ __global__ void k_b_count(const BFgm* __restrict__ F, int np, int* out) {
   if (threadIdx.x < 2) out[threadIdx.x] = cnt[threadIdx.x];
 }
 
-// Restart, step 1: w = J x at Dirichlet DOFs (identity), 0 elsewhere.
-__global__ void k_b_restart_init(const BOut* __restrict__ O, const BFgm* __restrict__ F) {
+// Restart, step 1: first pass of w = J x (identity rows, nodal gradient energy).
+__global__ void __launch_bounds__(GE_COLS * NV) k_b_restart_init(const BOut* __restrict__ O, const BFgm* __restrict__ F) {
   const int p = blockIdx.y;
   if (!F[p].restart) return;
   const BOut& o = O[p];
-  const int64_t nn = o.g.nn();
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < o.n; i += int64_t(gridDim.x) * blockDim.x)
-    o.w[i] = ((o.mask[i % nn] >> int(i / nn)) & 1) ? o.x[i] : 0.0;
+  const int64_t ncol = grad_energy_columns(o.g);
+  __shared__ GradESmem<double> sm;
+  for (int64_t t = int64_t(blockIdx.x) * GE_COLS; t < ncol; t += int64_t(gridDim.x) * GE_COLS) {
+    grad_energy_block<double, GE_APPLY>(o.g, o.ge64, o.mask, o.x, o.w, t, ncol, sm, false);
+    __syncthreads();
+  }
 }
 
 // Restart, step 2: r = b - w
@@ -883,7 +899,7 @@ struct BatchEngine {
   int maxnG = 0;
   std::vector<BOut> O;
   BOut* dO = nullptr;
-  int64_t nblkO = 0, maxnO = 0;
+  int64_t nblkO = 0, maxnO = 0, maxcolO = 0;
   DevParams* dP = nullptr;
   BFgm* dF = nullptr;
   double *partial = nullptr, *h1 = nullptr, *h2 = nullptr, *hn = nullptr, *dots = nullptr;
@@ -1124,8 +1140,11 @@ pfm_status engine_build(pfm_batch* b, const pfm_solve_opts& o, BatchEngine** out
     BOut ob{};
     ob.g = f.g;
     ob.n = ndof(f);
-    ob.dk = make_dfconst(f.g, h->dp);
+    ob.dk = make_dfconst(f.g);
     ob.jp64 = make_jparams<double>(f.g, h->dp);
+    grad_energy_const(f.g, h->dp, ob.ged);
+    grad_energy_const(f.g, h->dp, ob.ge64);
+    E->maxcolO = std::max(E->maxcolO, grad_energy_columns(f.g));
     ob.Hhi = f.H32;
     ob.Hlo = f.H32lo;
     ob.H64 = f.H64;
@@ -1430,8 +1449,9 @@ void eng_iteration(BatchEngine* E, int j) {
   count_launches(1);
   eng_vcycle(E, 0, g);
   k_b_store_z<<<gv, BT, 0, s>>>(E->dO, E->dF, j);
+  k_b_grad_energy_df<<<dim3(gdiv(E->maxcolO, GE_COLS), unsigned(np)), dim3(GE_COLS, NV), 0, s>>>(E->dO, E->dF, j);
   k_b_japply_df<<<E->grid_df, 256, 0, s>>>(E->dO, E->dF, np, E->nblkO, j);
-  count_launches(2);
+  count_launches(3);
   const dim3 gc(BCH, unsigned(np));
   for (double* h : {E->h1, E->h2}) {
     for (int j0 = 0; j0 <= j; j0 += BMDOT) {
@@ -1463,7 +1483,7 @@ void eng_cycle_start(BatchEngine* E, bool first) {
     k_b_begin<<<gv, BT, 0, s>>>(E->dO, E->dF, E->dact);
     count_launches(1);
   }
-  k_b_restart_init<<<gv, BT, 0, s>>>(E->dO, E->dF);
+  k_b_restart_init<<<dim3(gdiv(E->maxcolO, GE_COLS), unsigned(np)), dim3(GE_COLS, NV), 0, s>>>(E->dO, E->dF);
   count_launches(1);
   if (!first) {
     k_b_japply64<<<E->grid_j64, 256, 0, s>>>(E->dO, E->dF, np, E->nblkO);
@@ -1542,7 +1562,6 @@ pfm_status eng_residual_norms(pfm_batch* b, BatchEngine* E) {
     if (!E->hact[p]) continue;
     pfm_handle* h = b->hs[p];
     Level& f = h->L[0];
-    BCK(cudaMemsetAsync(h->R, 0, sizeof(double) * ndof(f), s));
     launch_residual(f.g, h->dp, f.U, f.Un, f.mask, h->R, nullptr, s);
   }
   k_b_res_norm2<<<dim3(BCH, unsigned(E->np)), BT, 0, s>>>(E->dO, E->dact, E->partial);

@@ -130,6 +130,7 @@ void count_launches(int n);
 // non-null = the atomic-free two-pass form (per-(element, node) contributions
 // in W, summed per node in a fixed order; bitwise reproducible). W holds
 // 9 * 32 * nblk entries of the output type (+ nblk for the residual's energy).
+// R is written in full, *energy is added to.
 // df: the point physics in double-float arithmetic (FP32 pipes) instead of FP64
 void launch_residual(const Grid& g, const DevParams& P, const double* U, const double* Un,
                      const dmask_t* mask, double* R, double* energy, cudaStream_t s, double* W = nullptr,
@@ -137,8 +138,8 @@ void launch_residual(const Grid& g, const DevParams& P, const double* U, const d
 // arithmetic of the point physics in the linearisation
 enum { LIN_F64 = 0, LIN_F32 = 1, LIN_DF = 2 };
 // optional residual of the same state formed in the linearisation pass
-// (arith == LIN_F64 only; ignored otherwise): R (zeroed by the caller unless W
-// is set), energy (optional), W the atomic-free scratch as for launch_residual
+// (arith == LIN_F64 only; ignored otherwise): R (every entry written), energy
+// (optional, added to), W the atomic-free scratch as for launch_residual
 struct LinResidual {
   const dmask_t* mask;
   double* R;

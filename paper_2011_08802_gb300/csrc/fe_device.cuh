@@ -46,7 +46,8 @@ __device__ __forceinline__ void q1_gather(T v, int l8, T ihx, T ihy, T ihz, T& v
   gx = gb * dxy + ga * t3;
 }
 
-// Nodal value -> value at this lane's point.
+// Nodal value -> value at this lane's point; also its transpose (point weights
+// for N_a -> this lane's node), because N_a(q) is symmetric in a and q.
 template <typename T>
 __device__ __forceinline__ T q1_value(T v) {
   const T ga = T(GA), gb = T(GB);
@@ -105,11 +106,13 @@ __device__ __forceinline__ int64_t elem_node(const Grid& g, int64_t e, int a) {
   return (ei + (a & 1)) + int64_t(g.nx + 1) * ((ej + ((a >> 1) & 1)) + int64_t(g.ny + 1) * (ek + (a >> 2)));
 }
 
-// Gather F = I + grad u, eta_hat and grad eta_hat at this lane's point.
+// Gather F = I + grad u and eta_hat at this lane's point (the gradients of
+// eta_hat enter only the gradient energy, an operator on the nodes:
+// grad_energy.cuh).
 template <typename T, typename Src>
 __device__ __forceinline__ void gather_state(const Src* __restrict__ U, int64_t nn, int64_t node,
                                              bool valid, int l8, T ihx, T ihy, T ihz, T F[9],
-                                             T eh[NV], T ge[3 * NV]) {
+                                             T eh[NV]) {
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     T v = valid ? T(U[i * nn + node]) : T(0);
@@ -125,7 +128,7 @@ __device__ __forceinline__ void gather_state(const Src* __restrict__ U, int64_t 
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     T v = valid ? T(U[(3 + k) * nn + node]) : T(0);
-    q1_gather(v, l8, ihx, ihy, ihz, eh[k], ge[3 * k], ge[3 * k + 1], ge[3 * k + 2]);
+    eh[k] = q1_value(v);
   }
 }
 
@@ -168,7 +171,7 @@ struct JParams {
 
 struct NoLinTail {
   template <typename TC>
-  __device__ void operator()(const TC*, const TC*, TC, int64_t, bool, int) const {}
+  __device__ void operator()(const TC*, TC, int64_t, bool, int) const {}
 };
 
 // Receives the Hessian entries of one Gauss point as they become final and
@@ -201,10 +204,9 @@ struct HessStore {
 // Gauss-point Hessians of element block blk (this warp; lane = 8 e + q),
 // computed in TC (FP64 for the finest and the coarsest level, FP32 for the
 // intermediate levels of an FP32 preconditioner) and stored in the requested
-// precisions (null stores are skipped). tail(ge, gr, W, node, valid, l8)
-// sees the point's eta gradients, energy gradient and energy density (the
-// residual of the same state can be formed from them without a second
-// evaluation of the point physics).
+// precisions (null stores are skipped). tail(gr, W, node, valid, l8) sees the
+// point's energy gradient and energy density (the residual of the same state
+// can be formed from them without a second evaluation of the point physics).
 template <typename TC, typename Tail = NoLinTail>
 __device__ __forceinline__ void linearize_lane(const Grid& g, const DevParams& P, const double* __restrict__ U,
                                                const double* __restrict__ Un, double* __restrict__ H64,
@@ -216,15 +218,15 @@ __device__ __forceinline__ void linearize_lane(const Grid& g, const DevParams& P
   const int64_t nn = g.nn();
   const int64_t node = valid ? elem_node(g, e, l8) : 0;
   const TC ihx = TC(1.0 / g.hx), ihy = TC(1.0 / g.hy), ihz = TC(1.0 / g.hz);
-  TC F[9], eh[NV], ge[3 * NV], ehn[NV];
-  gather_state<TC>(U, nn, node, valid, l8, ihx, ihy, ihz, F, eh, ge);
+  TC F[9], eh[NV], ehn[NV];
+  gather_state<TC>(U, nn, node, valid, l8, ihx, ihy, ihz, F, eh);
 #pragma unroll
   for (int k = 0; k < NV; ++k) ehn[k] = q1_value(valid ? TC(Un[(3 + k) * nn + node]) : TC(0));
   TC W, gr[NZ];
   const HessStore<TC> store{H64, H32, H32lo, blk, lane, valid};
   qp_point<TC>(P, F, eh, ehn, &W, gr, store);
   for (int j = NH; j < NHP; ++j) store(j, TC(0));  // padding entries are stored as zeros
-  tail(ge, gr, W, node, valid, l8);
+  tail(gr, W, node, valid, l8);
 }
 
 // Nodal NF x NF diagonal blocks (9 x 9 for N = 6). For local node a of the
@@ -375,9 +377,10 @@ __device__ __forceinline__ void scatter_row(TY* __restrict__ y, TW* __restrict__
 // ---- BEGIN tangent application kernel
 // y += J v on the 4 elements of block blk (this warp; lane = 0..31): gather v
 // at the element nodes (Dirichlet DOFs read as 0), dz = (grad du, d eta_hat)
-// at the Gauss points, sigma = H dz from the packed symmetric store, plus the
-// constant gradient-energy term, scattered back with atomics.
-template <typename T>
+// at the Gauss points, sigma = H dz from the packed symmetric store, scattered
+// back with atomics. GE: with the constant gradient-energy term (else it is the
+// nodal operator of grad_energy.cuh, which initialises y).
+template <typename T, bool GE>
 __device__ __forceinline__ void japply_block(const Grid& g, const JParams<T>& jp, const T* __restrict__ H,
                                              const dmask_t* __restrict__ mask, const T* __restrict__ v,
                                              T* __restrict__ y, int64_t blk, int lane) {
@@ -389,7 +392,8 @@ __device__ __forceinline__ void japply_block(const Grid& g, const JParams<T>& jp
   const bool valid = e < g.ne();
   const int64_t node = valid ? elem_node(g, e, l8) : 0;
   const dmask_t dm = valid ? mask[node] : MASK_ALL;
-  T dz[NZ], ge[3 * NV];
+  T dz[NZ];
+  [[maybe_unused]] T ge[GE ? 3 * NV : 1];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     T x = ((dm >> i) & 1) ? T(0) : v[i * nn + node];
@@ -399,7 +403,10 @@ __device__ __forceinline__ void japply_block(const Grid& g, const JParams<T>& jp
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     T x = ((dm >> (3 + k)) & 1) ? T(0) : v[(3 + k) * nn + node];
-    q1_gather(x, l8, jp.ihx, jp.ihy, jp.ihz, dz[9 + k], ge[3 * k], ge[3 * k + 1], ge[3 * k + 2]);
+    if constexpr (GE)
+      q1_gather(x, l8, jp.ihx, jp.ihy, jp.ihz, dz[9 + k], ge[3 * k], ge[3 * k + 1], ge[3 * k + 2]);
+    else
+      dz[9 + k] = q1_value(x);
   }
   // sigma = H dz from the packed symmetric store
   T sg[NZ];
@@ -429,15 +436,20 @@ __device__ __forceinline__ void japply_block(const Grid& g, const JParams<T>& jp
   }
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-    T gf[3];
+    T r;
+    if constexpr (GE) {
+      T gf[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      T s = T(0);
+      for (int d = 0; d < 3; ++d) {
+        T s = T(0);
 #pragma unroll
-      for (int l = 0; l < NV; ++l) s += jp.G[k][l] * ge[3 * l + d];
-      gf[d] = w * s;
+        for (int l = 0; l < NV; ++l) s += jp.G[k][l] * ge[3 * l + d];
+        gf[d] = w * s;
+      }
+      r = q1_scatter(w * sg[9 + k], gf[0], gf[1], gf[2], l8, jp.ihx, jp.ihy, jp.ihz);
+    } else {
+      r = q1_value(w * sg[9 + k]);
     }
-    T r = q1_scatter(w * sg[9 + k], gf[0], gf[1], gf[2], l8, jp.ihx, jp.ihy, jp.ihz);
     if (valid && !((dm >> (3 + k)) & 1)) atomicAdd(&y[(3 + k) * nn + node], r);
   }
 }
@@ -449,7 +461,7 @@ __device__ __forceinline__ void japply_block(const Grid& g, const JParams<T>& jp
 // at the element nodes (Dirichlet DOFs read as 0), dz = (grad du, d eta_hat)
 // at the Gauss points, sigma = H dz from the packed symmetric store, plus the
 // constant gradient-energy term, scattered back with atomics.
-template <typename T>
+template <typename T, bool GE>
 __device__ __forceinline__ void japply_block_det(const Grid& g, const JParams<T>& jp, const T* __restrict__ H,
                                                  const dmask_t* __restrict__ mask, const T* __restrict__ v,
                                                  T* __restrict__ W, int64_t ws, int64_t blk, int lane) {
@@ -461,7 +473,8 @@ __device__ __forceinline__ void japply_block_det(const Grid& g, const JParams<T>
   const bool valid = e < g.ne();
   const int64_t node = valid ? elem_node(g, e, l8) : 0;
   const dmask_t dm = valid ? mask[node] : MASK_ALL;
-  T dz[NZ], ge[3 * NV];
+  T dz[NZ];
+  [[maybe_unused]] T ge[GE ? 3 * NV : 1];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     T x = ((dm >> i) & 1) ? T(0) : v[i * nn + node];
@@ -471,7 +484,10 @@ __device__ __forceinline__ void japply_block_det(const Grid& g, const JParams<T>
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     T x = ((dm >> (3 + k)) & 1) ? T(0) : v[(3 + k) * nn + node];
-    q1_gather(x, l8, jp.ihx, jp.ihy, jp.ihz, dz[9 + k], ge[3 * k], ge[3 * k + 1], ge[3 * k + 2]);
+    if constexpr (GE)
+      q1_gather(x, l8, jp.ihx, jp.ihy, jp.ihz, dz[9 + k], ge[3 * k], ge[3 * k + 1], ge[3 * k + 2]);
+    else
+      dz[9 + k] = q1_value(x);
   }
   // sigma = H dz from the packed symmetric store
   T sg[NZ];
@@ -501,15 +517,20 @@ __device__ __forceinline__ void japply_block_det(const Grid& g, const JParams<T>
   }
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-    T gf[3];
+    T r;
+    if constexpr (GE) {
+      T gf[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      T s = T(0);
+      for (int d = 0; d < 3; ++d) {
+        T s = T(0);
 #pragma unroll
-      for (int l = 0; l < NV; ++l) s += jp.G[k][l] * ge[3 * l + d];
-      gf[d] = w * s;
+        for (int l = 0; l < NV; ++l) s += jp.G[k][l] * ge[3 * l + d];
+        gf[d] = w * s;
+      }
+      r = q1_scatter(w * sg[9 + k], gf[0], gf[1], gf[2], l8, jp.ihx, jp.ihy, jp.ihz);
+    } else {
+      r = q1_value(w * sg[9 + k]);
     }
-    T r = q1_scatter(w * sg[9 + k], gf[0], gf[1], gf[2], l8, jp.ihx, jp.ihy, jp.ihz);
     scatter_row<true>(static_cast<T*>(nullptr), W, ws, 3 + k, blk, lane, (3 + k) * nn + node, r, valid && !((dm >> (3 + k)) & 1));
   }
 }
@@ -846,37 +867,43 @@ __device__ __forceinline__ dfl df_shx(dfl v, int m) { return {shx(v.hi, m), shx(
 
 struct DfConst {
   dfl ga, gb, ihx, ihy, ihz, w;
-  dfl G[NV][NV];
 };
 inline dfl df_host(double x) {
   const float hi = float(x);
   return {hi, float(x - double(hi))};
 }
 
-__device__ __forceinline__ void q1_gather_df(dfl v, int l8, const DfConst& k, dfl& val, dfl& gx, dfl& gy,
-                                             dfl& gz) {
-  dfl s = df_shx(v, 1);
-  dfl vx = df_add(df_mul(k.gb, v), df_mul(k.ga, s));
-  dfl dx = df_mul((l8 & 1) ? df_sub(v, s) : df_sub(s, v), k.ihx);
-  dfl s1 = df_shx(vx, 2), s2 = df_shx(dx, 2);
-  dfl vxy = df_add(df_mul(k.gb, vx), df_mul(k.ga, s1));
-  dfl vdy = df_mul((l8 & 2) ? df_sub(vx, s1) : df_sub(s1, vx), k.ihy);
-  dfl dxy = df_add(df_mul(k.gb, dx), df_mul(k.ga, s2));
-  dfl t1 = df_shx(vxy, 4), t2 = df_shx(vdy, 4), t3 = df_shx(dxy, 4);
-  val = df_add(df_mul(k.gb, vxy), df_mul(k.ga, t1));
-  gz = df_mul((l8 & 4) ? df_sub(vxy, t1) : df_sub(t1, vxy), k.ihz);
+// Double-float form of the gather of gradients: with ga + gb = 1 the value at a
+// point is v + ga (s - v), so the difference is shared with the derivative.
+// The nodal values are FP32 numbers, whose differences are exact sums.
+__device__ __forceinline__ dfl df_scale_add(dfl a, dfl k, dfl b) { return df_add(a, df_mul(k, b)); }  // a + k b
+__device__ __forceinline__ void q1_gather_grad_df(float v, int l8, const DfConst& k, dfl& gx, dfl& gy, dfl& gz) {
+  const float s = shx(v, 1);
+  const dfl d0 = df_two_sum(s, -v);
+  const dfl vx = df_scale_add(dfl{v, 0.f}, k.ga, d0);
+  const dfl dx = df_mul((l8 & 1) ? df_neg(d0) : d0, k.ihx);
+  const dfl s1 = df_shx(vx, 2), s2 = df_shx(dx, 2);
+  const dfl d1 = df_sub(s1, vx);
+  const dfl vxy = df_scale_add(vx, k.ga, d1);
+  const dfl vdy = df_mul((l8 & 2) ? df_neg(d1) : d1, k.ihy);
+  const dfl dxy = df_add(df_mul(k.gb, dx), df_mul(k.ga, s2));
+  const dfl t1 = df_shx(vxy, 4), t2 = df_shx(vdy, 4), t3 = df_shx(dxy, 4);
+  const dfl d2 = df_sub(t1, vxy);
+  gz = df_mul((l8 & 4) ? df_neg(d2) : d2, k.ihz);
   gy = df_add(df_mul(k.gb, vdy), df_mul(k.ga, t2));
   gx = df_add(df_mul(k.gb, dxy), df_mul(k.ga, t3));
 }
 
-__device__ __forceinline__ dfl q1_scatter_df(dfl val, dfl gx, dfl gy, dfl gz, bool has_val, int l8,
-                                             const DfConst& k) {
+// value at this lane's point, and its transpose (q1_value)
+__device__ __forceinline__ dfl q1_value_df(dfl v, const DfConst& k) {
+#pragma unroll
+  for (int m = 1; m <= 4; m <<= 1) v = df_add(df_mul(k.gb, v), df_mul(k.ga, df_shx(v, m)));
+  return v;
+}
+
+__device__ __forceinline__ dfl q1_scatter_grad_df(dfl gx, dfl gy, dfl gz, int l8, const DfConst& k) {
   dfl sz = df_shx(gz, 4), sx = df_shx(gx, 4), sy = df_shx(gy, 4);
   dfl A = df_mul((l8 & 4) ? df_add(gz, sz) : df_neg(df_add(gz, sz)), k.ihz);
-  if (has_val) {
-    dfl sv = df_shx(val, 4);
-    A = df_add(A, df_add(df_mul(k.gb, val), df_mul(k.ga, sv)));
-  }
   dfl Bx = df_add(df_mul(k.gb, gx), df_mul(k.ga, sx));
   dfl By = df_add(df_mul(k.gb, gy), df_mul(k.ga, sy));
   dfl sA = df_shx(A, 2), sBy = df_shx(By, 2), sBx = df_shx(Bx, 2);
@@ -888,7 +915,7 @@ __device__ __forceinline__ dfl q1_scatter_df(dfl val, dfl gx, dfl gy, dfl gz, bo
                 df_mul((l8 & 1) ? df_add(Dx, sD) : df_neg(df_add(Dx, sD)), k.ihx));
 }
 
-inline DfConst make_dfconst(const Grid& g, const DevParams& P) {
+inline DfConst make_dfconst(const Grid& g) {
   DfConst k;
   k.ga = df_host(GA);
   k.gb = df_host(GB);
@@ -896,8 +923,6 @@ inline DfConst make_dfconst(const Grid& g, const DevParams& P) {
   k.ihy = df_host(1.0 / g.hy);
   k.ihz = df_host(1.0 / g.hz);
   k.w = df_host(g.w());
-  for (int a = 0; a < NV; ++a)
-    for (int b = 0; b < NV; ++b) k.G[a][b] = df_host(P.G[a][b]);
   return k;
 }
 
@@ -949,17 +974,16 @@ __device__ __forceinline__ void japply_df_block(const Grid& g, const DfConst& k,
   const bool valid = e < g.ne();
   const int64_t node = valid ? elem_node(g, e, l8) : 0;
   const dmask_t dm = valid ? mask[node] : MASK_ALL;
-  dfl dz[NZ], ge[3 * NV];
+  dfl dz[NZ];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const float x = ((dm >> i) & 1) ? 0.f : v[i * nn + node];
-    dfl val;
-    q1_gather_df(dfl{x, 0.f}, l8, k, val, dz[3 * i], dz[3 * i + 1], dz[3 * i + 2]);
+    q1_gather_grad_df(x, l8, k, dz[3 * i], dz[3 * i + 1], dz[3 * i + 2]);
   }
 #pragma unroll
   for (int kk = 0; kk < NV; ++kk) {
     const float x = ((dm >> (3 + kk)) & 1) ? 0.f : v[(3 + kk) * nn + node];
-    q1_gather_df(dfl{x, 0.f}, l8, k, dz[9 + kk], ge[3 * kk], ge[3 * kk + 1], ge[3 * kk + 2]);
+    dz[9 + kk] = q1_value_df(dfl{x, 0.f}, k);
   }
   cacc acc[NZ];
 #pragma unroll
@@ -986,21 +1010,12 @@ __device__ __forceinline__ void japply_df_block(const Grid& g, const DfConst& k,
   for (int r = 0; r < NZ; ++r) sg[r] = cacc_value(acc[r]);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    dfl r = q1_scatter_df(dfl{0.f, 0.f}, df_mul(k.w, sg[3 * i]), df_mul(k.w, sg[3 * i + 1]),
-                          df_mul(k.w, sg[3 * i + 2]), false, l8, k);
+    const dfl r = df_mul(k.w, q1_scatter_grad_df(sg[3 * i], sg[3 * i + 1], sg[3 * i + 2], l8, k));
     scatter_row<DET>(y, W, ws, i, blk, lane, i * nn + node, double(r.hi) + double(r.lo), valid && !((dm >> i) & 1));
   }
 #pragma unroll
   for (int kk = 0; kk < NV; ++kk) {
-    dfl gf[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      cacc s = cacc{0.f, 0.f};
-#pragma unroll
-      for (int l = 0; l < NV; ++l) cacc_add(s, k.G[kk][l].hi, k.G[kk][l].lo, ge[3 * l + d]);
-      gf[d] = df_mul(k.w, cacc_value(s));
-    }
-    dfl r = q1_scatter_df(df_mul(k.w, sg[9 + kk]), gf[0], gf[1], gf[2], true, l8, k);
+    const dfl r = df_mul(k.w, q1_value_df(sg[9 + kk], k));
     scatter_row<DET>(y, W, ws, 3 + kk, blk, lane, (3 + kk) * nn + node, double(r.hi) + double(r.lo),
                      valid && !((dm >> (3 + kk)) & 1));
   }

@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "fe_device.cuh"
+#include "grad_energy.cuh"
 
 namespace pfm {
 namespace {
@@ -35,44 +36,31 @@ namespace {
 #define PFM_RES_MINB 2
 #endif
 // Residual rows and energy of one Gauss point (lane = 8 e + q of block blk)
-// from its eta gradients ge, energy gradient gr and energy density Wd: the
-// gradient-energy flux G grad eta, the nodal rows scattered (DET: to the
-// scratch W) with Dirichlet rows left out, the energy summed per warp.
+// from its energy gradient gr and energy density Wd: the nodal rows scattered
+// (DET: to the scratch W) with Dirichlet rows left out, the energy summed per
+// warp. The gradient energy is the nodal operator of grad_energy.cuh.
 template <typename TC, bool DET>
-__device__ __forceinline__ void residual_tail(const Grid& g, const DevParams& P, const TC* ge, const TC* gr, TC Wd,
-                                              int64_t node, bool valid, int l8, int64_t blk, int lane,
-                                              const dmask_t* __restrict__ mask, double* __restrict__ R,
-                                              double* energy, double* __restrict__ W, int64_t ws) {
+__device__ __forceinline__ void residual_tail(const Grid& g, const TC* gr, TC Wd, int64_t node, bool valid, int l8,
+                                              int64_t blk, int lane, const dmask_t* __restrict__ mask,
+                                              double* __restrict__ R, double* energy, double* __restrict__ W,
+                                              int64_t ws) {
   const int64_t nn = g.nn();
   const TC ihx = TC(1.0 / g.hx), ihy = TC(1.0 / g.hy), ihz = TC(1.0 / g.hz);
-  TC gf[3 * NV];
-  TC Wg = TC(0.0);
-#pragma unroll
-  for (int k = 0; k < NV; ++k)
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      TC s = TC(0.0);
-#pragma unroll
-      for (int l = 0; l < NV; ++l) s += TC(P.G[k][l]) * ge[3 * l + d];
-      gf[3 * k + d] = s;
-      Wg += TC(0.5) * ge[3 * k + d] * s;
-    }
   const TC w = TC(g.w());
   const dmask_t dm = valid ? mask[node] : dmask_t(0);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    TC r = q1_scatter_grad(w * gr[3 * i], w * gr[3 * i + 1], w * gr[3 * i + 2], l8, ihx, ihy, ihz);
+    TC r = w * q1_scatter_grad(gr[3 * i], gr[3 * i + 1], gr[3 * i + 2], l8, ihx, ihy, ihz);
     scatter_row<DET>(R, W, ws, i, blk, lane, i * nn + node, double(r), valid && !((dm >> i) & 1));
   }
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-    TC r = q1_scatter(w * gr[9 + k], w * gf[3 * k], w * gf[3 * k + 1], w * gf[3 * k + 2], l8, ihx,
-                      ihy, ihz);
+    TC r = w * q1_value(gr[9 + k]);
     scatter_row<DET>(R, W, ws, 3 + k, blk, lane, (3 + k) * nn + node, double(r),
                      valid && !((dm >> (3 + k)) & 1));
   }
   if (energy) {
-    double en = warp_sum(valid ? double(w * (Wd + Wg)) : 0.0);
+    double en = warp_sum(valid ? double(w * Wd) : 0.0);
     if constexpr (DET) {
       if (lane == 0) W[NF * ws + blk] = en;
     } else {
@@ -84,11 +72,11 @@ __device__ __forceinline__ void residual_tail(const Grid& g, const DevParams& P,
 // Out-of-line copy for the linearisation pass, so that the register
 // allocation of its point physics does not see the residual's scatter.
 template <typename TC, bool DET>
-__device__ __noinline__ void residual_tail_call(const Grid& g, const DevParams& P, const TC* ge, const TC* gr, TC Wd,
-                                                int64_t node, bool valid, int l8, int64_t blk, int lane,
-                                                const dmask_t* __restrict__ mask, double* __restrict__ R,
-                                                double* energy, double* __restrict__ W, int64_t ws) {
-  residual_tail<TC, DET>(g, P, ge, gr, Wd, node, valid, l8, blk, lane, mask, R, energy, W, ws);
+__device__ __noinline__ void residual_tail_call(const Grid& g, const TC* gr, TC Wd, int64_t node, bool valid, int l8,
+                                                int64_t blk, int lane, const dmask_t* __restrict__ mask,
+                                                double* __restrict__ R, double* energy, double* __restrict__ W,
+                                                int64_t ws) {
+  residual_tail<TC, DET>(g, gr, Wd, node, valid, l8, blk, lane, mask, R, energy, W, ws);
 }
 
 template <typename TC, bool DET>
@@ -106,13 +94,13 @@ __global__ void __launch_bounds__(128, PFM_RES_MINB) k_residual(Grid g, DevParam
   const int64_t nn = g.nn();
   const int64_t node = valid ? elem_node(g, e, l8) : 0;
   const TC ihx = TC(1.0 / g.hx), ihy = TC(1.0 / g.hy), ihz = TC(1.0 / g.hz);
-  TC F[9], eh[NV], ge[3 * NV], ehn[NV];
-  gather_state<TC>(U, nn, node, valid, l8, ihx, ihy, ihz, F, eh, ge);
+  TC F[9], eh[NV], ehn[NV];
+  gather_state<TC>(U, nn, node, valid, l8, ihx, ihy, ihz, F, eh);
 #pragma unroll
   for (int k = 0; k < NV; ++k) ehn[k] = q1_value(valid ? TC(Un[(3 + k) * nn + node]) : TC(0.0));
   TC Wd, gr[NZ];
   qp_local<TC, false>(P, F, eh, ehn, &Wd, gr, nullptr);
-  residual_tail<TC, DET>(g, P, ge, gr, Wd, node, valid, l8, blk, lane, mask, R, energy, W, ws);
+  residual_tail<TC, DET>(g, gr, Wd, node, valid, l8, blk, lane, mask, R, energy, W, ws);
 }
 
 // Node pass of the atomic-free scatter (node_gather) over all nodes.
@@ -165,13 +153,13 @@ __global__ void __launch_bounds__(128) k_linearize(Grid g, DevParams P, const do
       static_assert(std::is_same<TC, double>::value, "residual pass in FP64 only");
       const int64_t ws = g.nblk() * 32;
       linearize_lane<TC>(g, P, U, Un, H64, H32, H32lo, blk, lane,
-                         [&](const TC* ge, const TC* gr, TC Wd, int64_t node, bool valid, int l8) {
+                         [&](const TC* gr, TC Wd, int64_t node, bool valid, int l8) {
                            if (RW)
-                             residual_tail_call<TC, true>(g, P, ge, gr, Wd, node, valid, l8, blk, lane, mask, R,
-                                                          energy, RW, ws);
+                             residual_tail_call<TC, true>(g, gr, Wd, node, valid, l8, blk, lane, mask, R, energy, RW,
+                                                          ws);
                            else
-                             residual_tail_call<TC, false>(g, P, ge, gr, Wd, node, valid, l8, blk, lane, mask,
-                                                           R, energy, nullptr, 0);
+                             residual_tail_call<TC, false>(g, gr, Wd, node, valid, l8, blk, lane, mask, R, energy,
+                                                           nullptr, 0);
                          });
     } else {
       linearize_lane<TC>(g, P, U, Un, H64, H32, H32lo, blk, lane);
@@ -215,7 +203,7 @@ __global__ void __launch_bounds__(256, PFM_JAPPLY_MINB) k_japply(Grid g, JParams
   static_assert(BLK_BYTES % 16 == 0, "bulk prefetch size");
   for (int64_t blk = wg; blk < nblk; blk += nw) {
     if (lane == 0) prefetch_l2(H + blk * HBLK, BLK_BYTES);
-    japply_block<T>(g, jp, H, mask, v, y, blk, lane);
+    japply_block<T, sizeof(T) == 4>(g, jp, H, mask, v, y, blk, lane);
   }
 }
 
@@ -233,7 +221,7 @@ __global__ void __launch_bounds__(256, PFM_JAPPLY_MINB) k_japply_det(Grid g, JPa
   constexpr unsigned BLK_BYTES = unsigned(HBLK * sizeof(T));
   for (int64_t blk = wg; blk < nblk; blk += nw) {
     if (lane == 0) prefetch_l2(H + blk * HBLK, BLK_BYTES);
-    japply_block_det<T>(g, jp, H, mask, v, W, ws, blk, lane);
+    japply_block_det<T, sizeof(T) == 4>(g, jp, H, mask, v, W, ws, blk, lane);
   }
 }
 
@@ -369,7 +357,7 @@ __global__ void __launch_bounds__(32 * WPC, (staged_minb<S, D, WPC>())) k_japply
 // y += J v with v in FP32 (exact input), the tangent as Hhi + Hlo (two FP32
 // stores of the FP64 Hessians) and double-float arithmetic throughout; the
 // element contributions are added to the FP64 output y (initialised by
-// k_japply_init_df). Same persistent warp mapping as k_japply.
+// the nodal gradient energy). Same persistent warp mapping as k_japply.
 #ifndef PFM_DF_MINB
 #define PFM_DF_MINB (PFM_NV == 6 ? 2 : 8)
 #endif
@@ -386,14 +374,30 @@ __global__ void __launch_bounds__(256, PFM_DF_MINB) k_japply_df(Grid g, DfConst 
   for (int64_t blk = wg; blk < nblk; blk += nw) japply_df_block<DET>(g, k, Hhi, Hlo, mask, v, y, blk, lane, W, ws);
 }
 
-// y = v at Dirichlet DOFs, 0 elsewhere (FP32 input, FP64 output).
-__global__ void k_japply_init_df(int64_t nn, const dmask_t* __restrict__ mask, const float* __restrict__ v,
-                                 double* __restrict__ y) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < NF * nn;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t node = i % nn;
-    const int f = int(i / nn);
-    y[i] = ((mask[node] >> f) & 1) ? double(v[i]) : 0.0;
+// Nodal gradient energy (grad_energy.cuh): first pass of an application or a
+// residual, or added after the node pass of the atomic-free forms. The energy
+// goes to *energy with one atomic per block, or as one partial per block to
+// part (summed in a fixed order by k_sum_fixed).
+template <typename TA, int MODE, typename TV, typename TY>
+__global__ void __launch_bounds__(GE_COLS * NV) k_grad_energy(Grid g, typename GeArith<TA>::C c, int64_t ncol,
+                                                              const dmask_t* __restrict__ mask,
+                                                              const TV* __restrict__ v, TY* __restrict__ y,
+                                                              double* energy, double* __restrict__ part) {
+  __shared__ GradESmem<TA> sm;
+  __shared__ double red[NV];
+  const bool want = energy != nullptr || part != nullptr;
+  double en = grad_energy_block<TA, MODE>(g, c, mask, v, y, int64_t(blockIdx.x) * GE_COLS, ncol, sm, want);
+  if (!want) return;
+  en = warp_sum(en);  // a warp holds the columns of one order parameter
+  if (threadIdx.x == 0) red[threadIdx.y] = en;
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    double s = 0.0;
+    for (int k = 0; k < NV; ++k) s += red[k];
+    if (part)
+      part[blockIdx.x] = s;
+    else
+      atomicAdd(energy, s);
   }
 }
 
@@ -539,7 +543,7 @@ __global__ void __launch_bounds__(256, PFM_JAPPLY_MINB) k_japply_range(Grid g, J
   constexpr unsigned BLK_BYTES = unsigned(HBLK * sizeof(T));
   for (int64_t blk = b0 + wg; blk < b1; blk += nw) {
     if (lane == 0) prefetch_l2(H + blk * HBLK, BLK_BYTES);
-    japply_block<T>(g, jp, H, mask, v, y, blk, lane);
+    japply_block<T, true>(g, jp, H, mask, v, y, blk, lane);
   }
 }
 
@@ -560,10 +564,43 @@ __global__ void k_identity_rows(int64_t nn, const dmask_t* __restrict__ mask, co
 
 int sm_count();
 
+// Launch of the nodal gradient energy over all columns of g; returns the blocks.
+template <typename TA, int MODE, typename TV, typename TY>
+unsigned launch_grad_energy(const Grid& g, const DevParams& P, const dmask_t* mask, const TV* v, TY* y, cudaStream_t s,
+                            double* energy = nullptr, double* part = nullptr) {
+  typename GeArith<TA>::C c;
+  grad_energy_const(g, P, c);
+  const int64_t ncol = grad_energy_columns(g);
+  const unsigned blocks = grid_for(ncol, GE_COLS);
+  k_grad_energy<TA, MODE, TV, TY><<<blocks, dim3(GE_COLS, NV), 0, s>>>(g, c, ncol, mask, v, y, energy, part);
+  count_launches(1);
+  return blocks;
+}
+
+// Passes after the element pass of an atomic-free residual: the node sums, the
+// nodal gradient energy and the energy's partial sums.
+void residual_det_tail(const Grid& g, const DevParams& P, const double* U, const dmask_t* mask, double* R,
+                       double* energy, double* W, cudaStream_t s) {
+  const int64_t ws = g.nblk() * 32;
+  k_node_gather<double, double, double><<<grid_for(g.nn(), 128), 128, 0, s>>>(g, W, ws, mask, nullptr, R);
+  count_launches(1);
+  if (energy) {
+    k_sum_fixed<<<1, 1024, 0, s>>>(g.nblk(), W + NF * ws, energy);
+    count_launches(1);
+  }
+  // the node sums are done with W, so the block partials can go there
+  const unsigned nb = launch_grad_energy<double, GE_ADD>(g, P, mask, U, R, s, nullptr, energy ? W : nullptr);
+  if (energy) {
+    k_sum_fixed<<<1, 1024, 0, s>>>(nb, W, energy);
+    count_launches(1);
+  }
+}
+
 void launch_residual(const Grid& g, const DevParams& P, const double* U, const double* Un,
                      const dmask_t* mask, double* R, double* energy, cudaStream_t s, double* W, bool df) {
   const int64_t threads = g.nblk() * 32;
   if (!W) {
+    launch_grad_energy<double, GE_RES>(g, P, mask, U, R, s, energy);
     if (df)
       k_residual<df64, false><<<grid_for(threads, 128), 128, 0, s>>>(g, P, U, Un, mask, R, energy, nullptr, 0);
     else
@@ -576,12 +613,8 @@ void launch_residual(const Grid& g, const DevParams& P, const double* U, const d
     k_residual<df64, true><<<grid_for(threads, 128), 128, 0, s>>>(g, P, U, Un, mask, R, energy, W, ws);
   else
     k_residual<double, true><<<grid_for(threads, 128), 128, 0, s>>>(g, P, U, Un, mask, R, energy, W, ws);
-  k_node_gather<double, double, double><<<grid_for(g.nn(), 128), 128, 0, s>>>(g, W, ws, mask, nullptr, R);
-  count_launches(2);
-  if (energy) {
-    k_sum_fixed<<<1, 1024, 0, s>>>(g.nblk(), W + NF * ws, energy);
-    count_launches(1);
-  }
+  count_launches(1);
+  residual_det_tail(g, P, U, mask, R, energy, W, s);
 }
 
 void launch_linearize(const Grid& g, const DevParams& P, const double* U, const double* Un,
@@ -598,6 +631,7 @@ void launch_linearize(const Grid& g, const DevParams& P, const double* U, const 
   double* R = with_res ? res->R : nullptr;
   double* energy = with_res ? res->energy : nullptr;
   double* RW = with_res ? res->W : nullptr;
+  if (with_res && !RW) launch_grad_energy<double, GE_RES>(g, P, mask, U, R, s, energy);
   if (arith == LIN_F32)
     k_linearize<float><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, nullptr, nullptr, nullptr, nullptr);
   else if (arith == LIN_DF)
@@ -607,15 +641,7 @@ void launch_linearize(const Grid& g, const DevParams& P, const double* U, const 
   else
     k_linearize<double><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, nullptr, nullptr, nullptr, nullptr);
   count_launches(1);
-  if (RW) {  // node pass of the atomic-free form, as in launch_residual
-    const int64_t ws = g.nblk() * 32;
-    k_node_gather<double, double, double><<<grid_for(g.nn(), 128), 128, 0, s>>>(g, RW, ws, mask, nullptr, R);
-    count_launches(1);
-    if (energy) {
-      k_sum_fixed<<<1, 1024, 0, s>>>(g.nblk(), RW + NF * ws, energy);
-      count_launches(1);
-    }
-  }
+  if (RW) residual_det_tail(g, P, U, mask, R, energy, RW, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -812,12 +838,20 @@ inline const void* japply_elem_fn(const __half*) { return reinterpret_cast<const
 // only; the atomic-free form and FP64 use the register-fed kernel (with the
 // default shape when the tuned one is staged).
 template <typename T, typename S = T>
-void japply_launch_shape(const Grid& g, const JParams<T>& jp, float wh, const S* H, const dmask_t* mask, const T* v,
+void japply_launch_shape(const Grid& g, const DevParams& P, const JParams<T>& jp, float wh, const S* H, const dmask_t* mask, const T* v,
                          T* y, const JShape& js, cudaStream_t s, T* W = nullptr, const JStaged* jst = nullptr) {
   const int64_t nn = g.nn();
+  // FP32 arithmetic keeps the gradient energy in its element kernel (bound by
+  // reading the store, or, with the binary16 store, faster than another pass);
+  // FP64 takes the nodal operator as its first pass
+  constexpr bool GE = std::is_same<T, float>::value;
   if (!W) {
-    k_japply_init<T><<<grid_for(NF * nn, 256) < 4096 ? grid_for(NF * nn, 256) : 4096, 256, 0, s>>>(nn, mask, v, y);
-    count_launches(1);
+    if constexpr (GE) {
+      k_japply_init<T><<<grid_for(NF * nn, 256) < 4096 ? grid_for(NF * nn, 256) : 4096, 256, 0, s>>>(nn, mask, v, y);
+      count_launches(1);
+    } else {
+      launch_grad_energy<T, GE_APPLY>(g, P, mask, v, y, s);
+    }
   }
   if constexpr (std::is_same<T, float>::value) {
     if (js.stages > 0 && !W && jst) {
@@ -835,11 +869,12 @@ void japply_launch_shape(const Grid& g, const JParams<T>& jp, float wh, const S*
   if (W) {
     k_node_gather<T, T, T><<<grid_for(nn, 128), 128, 0, s>>>(g, W, g.nblk() * 32, mask, v, y);
     count_launches(1);
+    if constexpr (!GE) launch_grad_energy<T, GE_ADD>(g, P, mask, v, y, s);
   }
 }
 
 template <typename T, typename S = T>
-JShape japply_tune(const Grid& g, const JParams<T>& jp, float wh, const S* H, const dmask_t* mask, const T* v, T* y,
+JShape japply_tune(const Grid& g, const DevParams& P, const JParams<T>& jp, float wh, const S* H, const dmask_t* mask, const T* v, T* y,
                    cudaStream_t s, const JStaged* jst = nullptr) {
   const int pr = sizeof(S) == 2 ? 2 : (sizeof(T) == 4 ? 0 : 1);
   int cl = 0;
@@ -870,13 +905,13 @@ JShape japply_tune(const Grid& g, const JParams<T>& jp, float wh, const S* H, co
       }
   }
   for (const JShape& js : cand) {
-    japply_launch_shape<T, S>(g, jp, wh, H, mask, v, y, js, s, nullptr, jst);  // warm
+    japply_launch_shape<T, S>(g, P, jp, wh, H, mask, v, y, js, s, nullptr, jst);  // warm
     // best of three timings of three applications each (the shapes differ
     // by a few per cent, about the run-to-run spread of one timing)
     float ms = 1e30f;
     for (int t = 0; t < 3; ++t) {
       cudaEventRecord(a, s);
-      for (int r = 0; r < 3; ++r) japply_launch_shape<T, S>(g, jp, wh, H, mask, v, y, js, s, nullptr, jst);
+      for (int r = 0; r < 3; ++r) japply_launch_shape<T, S>(g, P, jp, wh, H, mask, v, y, js, s, nullptr, jst);
       cudaEventRecord(b, s);
       cudaEventSynchronize(b);
       float m = 0.f;
@@ -902,11 +937,11 @@ void launch_japply(const Grid& g, const DevParams& P, const T* H, const dmask_t*
   const JParams<T> jp = make_jparams<T>(g, P);
   if constexpr (std::is_same<T, float>::value) {
     const JStaged jst = make_jstaged(g, P, g.w());
-    const JShape js = japply_tune<T>(g, jp, 0.f, H, mask, v, y, s, &jst);
-    japply_launch_shape<T>(g, jp, 0.f, H, mask, v, y, js, s, W, &jst);
+    const JShape js = japply_tune<T>(g, P, jp, 0.f, H, mask, v, y, s, &jst);
+    japply_launch_shape<T>(g, P, jp, 0.f, H, mask, v, y, js, s, W, &jst);
   } else {
-    const JShape js = japply_tune<T>(g, jp, 0.f, H, mask, v, y, s);
-    japply_launch_shape<T>(g, jp, 0.f, H, mask, v, y, js, s, W);
+    const JShape js = japply_tune<T>(g, P, jp, 0.f, H, mask, v, y, s);
+    japply_launch_shape<T>(g, P, jp, 0.f, H, mask, v, y, js, s, W);
   }
 }
 
@@ -915,8 +950,8 @@ void launch_japply_h16(const Grid& g, const DevParams& P, const __half* H, float
   const JParams<float> jp = make_jparams<float>(g, P);
   const float wh = jp.w * inv_scale;
   const JStaged jst = make_jstaged(g, P, g.w() * double(inv_scale));
-  const JShape js = japply_tune<float, __half>(g, jp, wh, H, mask, v, y, s, &jst);
-  japply_launch_shape<float, __half>(g, jp, wh, H, mask, v, y, js, s, W, &jst);
+  const JShape js = japply_tune<float, __half>(g, P, jp, wh, H, mask, v, y, s, &jst);
+  japply_launch_shape<float, __half>(g, P, jp, wh, H, mask, v, y, js, s, W, &jst);
 }
 
 int take_wait_timeouts() {
@@ -957,12 +992,9 @@ float launch_store_to_half(const Grid& g, const float* H32, __half* H16, unsigne
 
 void launch_japply_df(const Grid& g, const DevParams& P, const float* Hhi, const float* Hlo, const dmask_t* mask,
                       const float* v, double* y, cudaStream_t s, double* W) {
-  const DfConst k = make_dfconst(g, P);
+  const DfConst k = make_dfconst(g);
   const int64_t nn = g.nn();
-  if (!W) {
-    k_japply_init_df<<<grid_for(NF * nn, 256) < 4096 ? grid_for(NF * nn, 256) : 4096, 256, 0, s>>>(nn, mask, v, y);
-    count_launches(1);
-  }
+  if (!W) launch_grad_energy<df64, GE_APPLY>(g, P, mask, v, y, s);
   static int per_sm = 0;
   if (per_sm == 0) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_japply_df<false>, 256, 0);
@@ -976,6 +1008,7 @@ void launch_japply_df(const Grid& g, const DevParams& P, const float* Hhi, const
     k_japply_df<true><<<blocks, 256, 0, s>>>(g, k, Hhi, Hlo, mask, v, y, W, ws);
     k_node_gather<double, float, double><<<grid_for(nn, 128), 128, 0, s>>>(g, W, ws, mask, v, y);
     count_launches(2);
+    launch_grad_energy<df64, GE_ADD>(g, P, mask, v, y, s);
     return;
   }
   k_japply_df<false><<<blocks, 256, 0, s>>>(g, k, Hhi, Hlo, mask, v, y, nullptr, 0);

@@ -95,11 +95,9 @@ pfm_status pfm_residual_noalloc(const pfm_mesh_desc* mesh, const pfm_params* par
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   DevParams dp;
   make_dev_params(*params, dp);
-  const int64_t n = int64_t(NF) * g.nn();
   // the scratch keeps the previous call's contents: clear what accumulates
   cudaError_t e = cudaMemsetAsync(energy, 0, sizeof(double), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(R_dev, 0, sizeof(double) * n, s);
   if (e != cudaSuccess) {
     g_noalloc_error = std::string("cudaMemsetAsync: ") + cudaGetErrorString(e);
     return PFM_ERR_CUDA;
