@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(128, PFM_RES_MINB) k_residual(Grid g, DevParam
   const int64_t e = tid >> 3;
   const int l8 = int(tid & 7);
   const int64_t blk = tid >> 5;
+  if (blk >= g.nblk()) return;  // padding warps of the last block own no part of W
   const int lane = int(tid & 31);
   const bool valid = e < g.ne();
   const int64_t nn = g.nn();
