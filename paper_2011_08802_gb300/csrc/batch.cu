@@ -277,17 +277,27 @@ __global__ void k_b_sub(const BLev* __restrict__ S, int asel, int bsel, int osel
 __global__ void k_b_restrict(const BTr* __restrict__ T, Gate on) {
   const BTr& t = T[blockIdx.y];
   if (!on(t.problem)) return;
-  const int64_t nnc = t.c.nn();
-  for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < nnc; idx += int64_t(gridDim.x) * blockDim.x)
-    restrict_node<float>(t.f, t.c, t.rf, t.mc, t.bc, idx);
+  const bool wide = !transfer_integer(t.f);  // numerators of the weights beyond FP32 integers
+  const int64_t n = wide ? t.c.nn() : NF * t.c.nn();
+  for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < n; idx += int64_t(gridDim.x) * blockDim.x) {
+    if (wide)
+      restrict_node<float>(t.f, t.c, t.rf, t.mc, t.bc, idx);
+    else
+      restrict_entry_int(t.f, t.c, t.rf, t.mc, t.bc, idx);
+  }
 }
 
 __global__ void k_b_prolong(const BTr* __restrict__ T, Gate on) {
   const BTr& t = T[blockIdx.y];
   if (!on(t.problem)) return;
-  const int64_t nnf = t.f.nn();
-  for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < nnf; idx += int64_t(gridDim.x) * blockDim.x)
-    prolong_node<float>(t.f, t.c, t.xc, t.mf, t.xf, idx);
+  const bool wide = !transfer_integer(t.f);
+  const int64_t n = wide ? t.f.nn() : NF * t.f.nn();
+  for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < n; idx += int64_t(gridDim.x) * blockDim.x) {
+    if (wide)
+      prolong_node<float>(t.f, t.c, t.xc, t.mf, t.xf, idx);
+    else
+      prolong_entry_int(t.f, t.c, t.xc, t.mf, t.xf, idx);
+  }
 }
 
 // x = Kinv b, one warp per row; blockIdx.y = problem.
@@ -1267,10 +1277,10 @@ void eng_vcycle(BatchEngine* E, int d, Gate g) {
   const int nu_post = E->nu_post > 0 ? std::max(1, int(std::lround(E->nu_post * gl))) : 0;
   const int ns = int(Ds.S.size());
   eng_smooth(E, d, true, nu_pre, true, g);
-  k_b_restrict<<<grid2(Ds.maxnnc, ns), BT, 0, E->s>>>(Ds.dT, g);
+  k_b_restrict<<<grid2(NF * Ds.maxnnc, ns), BT, 0, E->s>>>(Ds.dT, g);
   count_launches(1);
   eng_vcycle(E, d + 1, g);
-  k_b_prolong<<<grid2(Ds.maxnnf, ns), BT, 0, E->s>>>(Ds.dT, g);
+  k_b_prolong<<<grid2(NF * Ds.maxnnf, ns), BT, 0, E->s>>>(Ds.dT, g);
   count_launches(1);
   if (nu_post > 0) eng_smooth(E, d, false, nu_post, false, g);
 }

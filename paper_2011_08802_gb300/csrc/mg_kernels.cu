@@ -8,6 +8,8 @@
 // i*nc = I0*nf + rem, its interpolation weights are (1 - rem/nf) on coarse
 // node I0 and rem/nf on I0+1. All index arithmetic is integer, so P and
 // R = P^T use identical weights on nested (nf = 2 nc) and non-nested grids.
+#include <type_traits>
+
 #include "coarse_inverse.cuh"
 #include "common.cuh"
 #include "mg_device.cuh"
@@ -50,6 +52,18 @@ __global__ void k_prolong_add(Grid f, Grid c, const T* __restrict__ xc, const dm
   for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < nnf;
        idx += int64_t(gridDim.x) * blockDim.x)
     prolong_node<T>(f, c, xc, mf, xf, idx);
+}
+
+// FP32 vectors between non-nested grids: one thread per (node, field).
+__global__ void __launch_bounds__(128) k_prolong_add_int(Grid f, Grid c, const float* __restrict__ xc,
+                                                         const dmask_t* __restrict__ mf, float* __restrict__ xf) {
+  const int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (idx < NF * f.nn()) prolong_entry_int(f, c, xc, mf, xf, idx);
+}
+__global__ void __launch_bounds__(128) k_restrict_int(Grid f, Grid c, const float* __restrict__ rf,
+                                                      const dmask_t* __restrict__ mc, float* __restrict__ rc) {
+  const int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (idx < NF * c.nn()) restrict_entry_int(f, c, rf, mc, rc, idx);
 }
 
 // Nested grids: one thread per fine node (i over x-blocks and threads, j and
@@ -332,9 +346,17 @@ void launch_prolong_add(const Grid& fine, const Grid& coarse, const T* xc, const
   if (nested(fine, coarse) && grid3_ok(fine)) {
     const dim3 grid(unsigned((fine.nx + 1 + 127) / 128), unsigned(fine.ny + 1), unsigned(fine.nz + 1));
     k_prolong_add_nested<T><<<grid, 128, 0, s>>>(fine, coarse, xc, mf, xf);
-  } else {
-    k_prolong_add<T><<<grid_for(fine.nn(), 256), 256, 0, s>>>(fine, coarse, xc, mf, xf);
+    count_launches(1);
+    return;
   }
+  if constexpr (std::is_same<T, float>::value) {
+    if (transfer_integer(fine)) {
+      k_prolong_add_int<<<grid_for(NF * fine.nn(), 128), 128, 0, s>>>(fine, coarse, xc, mf, xf);
+      count_launches(1);
+      return;
+    }
+  }
+  k_prolong_add<T><<<grid_for(fine.nn(), 256), 256, 0, s>>>(fine, coarse, xc, mf, xf);
   count_launches(1);
 }
 
@@ -344,9 +366,17 @@ void launch_restrict(const Grid& fine, const Grid& coarse, const T* rf, const dm
   if (nested(fine, coarse) && grid3_ok(coarse)) {
     const dim3 grid(unsigned((coarse.nx + 1 + 127) / 128), unsigned(coarse.ny + 1), unsigned(coarse.nz + 1));
     k_restrict_nested<T><<<grid, 128, 0, s>>>(fine, coarse, rf, mc, rc);
-  } else {
-    k_restrict<T><<<grid_for(coarse.nn(), 128), 128, 0, s>>>(fine, coarse, rf, mc, rc);
+    count_launches(1);
+    return;
   }
+  if constexpr (std::is_same<T, float>::value) {
+    if (transfer_integer(fine)) {
+      k_restrict_int<<<grid_for(NF * coarse.nn(), 128), 128, 0, s>>>(fine, coarse, rf, mc, rc);
+      count_launches(1);
+      return;
+    }
+  }
+  k_restrict<T><<<grid_for(coarse.nn(), 128), 128, 0, s>>>(fine, coarse, rf, mc, rc);
   count_launches(1);
 }
 
