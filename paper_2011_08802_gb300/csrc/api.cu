@@ -99,21 +99,31 @@ T* det_W(pfm_handle* h) {
 // Tangent application inside the preconditioner on level l: from the level's
 // store, or from its binary16 copy when that is enabled and current (FP32);
 // timed on the finest level unless `timed` is false.
+// y_ready: y already holds the identity rows of x and zeros elsewhere (written by
+// the smoothing step before), for the paths that start from that.
 template <typename T>
-void precond_apply(pfm_handle* h, size_t l, const T* x, T* y, bool timed = true) {
+void precond_apply(pfm_handle* h, size_t l, const T* x, T* y, bool timed = true, bool y_ready = false) {
   Level& lv = h->L[l];
   const bool on = timed && l == 0;
   if constexpr (sizeof(T) == 4) {
     if (lv.H16 && lv.h16_scale > 0.f) {
       ProfScope ps(h, PFM_PROF_JAPPLY_F16, on);
-      launch_japply_h16(lv.g, h->dp, lv.H16, 1.f / lv.h16_scale, lv.mask, x, y, h->stream, det_W<float>(h));
+      launch_japply_h16(lv.g, h->dp, lv.H16, 1.f / lv.h16_scale, lv.mask, x, y, h->stream, det_W<float>(h), y_ready);
       if (h->contact_on) launch_contact_apply<T, T, T>(lv.g, LvVec<T>::Kc(lv), lv.mask, x, y, h->stream);
       return;
     }
   }
   ProfScope ps(h, sizeof(T) == 4 ? PFM_PROF_JAPPLY_F32 : PFM_PROF_JAPPLY_F64, on);
-  launch_japply<T>(lv.g, h->dp, LvVec<T>::H(lv), lv.mask, x, y, h->stream, det_W<T>(h));
+  launch_japply<T>(lv.g, h->dp, LvVec<T>::H(lv), lv.mask, x, y, h->stream, det_W<T>(h), y_ready);
   if (h->contact_on) launch_contact_apply<T, T, T>(lv.g, LvVec<T>::Kc(lv), lv.mask, x, y, h->stream);
+}
+
+// Whether an application in the precision T starts from identity rows and zeros
+// in y: FP32 arithmetic with atomics (FP64 begins with the nodal gradient energy,
+// the atomic-free forms write y in a node pass).
+template <typename T>
+bool starts_from_rows(const pfm_handle* h) {
+  return sizeof(T) == 4 && !h->det;
 }
 
 // ---------------------------------------------------------------------------
@@ -179,21 +189,25 @@ pfm_status smooth(pfm_handle* h, size_t l, bool zero_x, int nu, bool want_res, c
   const double hi = c.hi * lv.lam, lo = c.lo * lv.lam;
   const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta;
   double rho = 1.0 / sigma;
+  // each step also writes the identity rows and zeros that the next
+  // application starts from (null: that application initialises y itself)
+  const bool rows = starts_from_rows<T>(h);
+  T* yn = rows && (nu > 1 || want_res) ? y : nullptr;
   if (zero_x) {
-    launch_cheb_first<T>(lv.nn, D, b, T(1.0 / theta), true, true, r, d, x, s);
+    launch_cheb_first<T>(lv.nn, D, b, nullptr, T(1.0 / theta), true, r, d, x, lv.mask, yn, s);
   } else {
     precond_apply<T>(h, l, x, y);
-    launch_sub<T>(n, b, y, r, s);
-    launch_cheb_first<T>(lv.nn, D, r, T(1.0 / theta), false, false, r, d, x, s);
+    launch_cheb_first<T>(lv.nn, D, b, y, T(1.0 / theta), false, r, d, x, lv.mask, yn, s);
   }
   for (int k = 1; k < nu; ++k) {
-    precond_apply<T>(h, l, d, y);
+    precond_apply<T>(h, l, d, y, true, rows);
     const double rho_n = 1.0 / (2.0 * sigma - rho);
-    launch_cheb_step<T>(lv.nn, D, y, T(rho_n * rho), T(2.0 * rho_n / delta), r, d, x, s);
+    yn = rows && (k + 1 < nu || want_res) ? y : nullptr;
+    launch_cheb_step<T>(lv.nn, D, y, T(rho_n * rho), T(2.0 * rho_n / delta), r, d, x, lv.mask, yn, s);
     rho = rho_n;
   }
   if (want_res) {
-    precond_apply<T>(h, l, d, y);
+    precond_apply<T>(h, l, d, y, true, rows);
     launch_sub<T>(n, r, y, r, s);
   }
   CKL();
@@ -278,13 +292,8 @@ pfm_status estimate_lambda(pfm_handle* h, size_t l) {
   T* u = LvVec<T>::y(lv);
   T* w = LvVec<T>::r(lv);
   const T* D = LvVec<T>::D(lv);
-  auto dinv = [&](const T* src, T* dst) {  // dst = D^-1 src
-    CK(cudaMemsetAsync(dst, 0, sizeof(T) * n, s));
-    launch_smooth<T>(lv.nn, D, src, nullptr, T(1), dst, s);
-    return PFM_OK;
-  };
   launch_power_init<T>(lv.nn, lv.mask, q, s);
-  TRY(dinv(q, z));
+  launch_dinv<T>(lv.nn, D, q, z, s);
   launch_dot<T>(n, q, z, h->partial, nrm, s);
   launch_scale_inv_sqrt<T>(n, q, nrm, q, s);
   launch_scale_inv_sqrt<T>(n, z, nrm, z, s);
@@ -295,7 +304,7 @@ pfm_status estimate_lambda(pfm_handle* h, size_t l) {
     CKL_AT("eigenvalue estimate: tangent application");
     launch_dot<T>(n, z, u, h->partial, al + j, s);
     launch_lanczos_orth<T>(n, u, q, qp, al + j, j > 0 ? be + j - 1 : nullptr, s);
-    TRY(dinv(u, w));
+    launch_dinv<T>(lv.nn, D, u, w, s);
     launch_dot<T>(n, u, w, h->partial, be + j, s);
     if (j + 1 < K) {
       std::swap(q, qp);
@@ -441,7 +450,7 @@ pfm_status linearize_impl(pfm_handle* h, pfm_precision prec, double* R_fused = n
     CKL();
     if (coarsest) continue;
     if (prec == PFM_F32) {
-      TRY(dalloc(h, &lv.D32, size_t(NF2) * lv.nn));
+      TRY(dalloc(h, &lv.D32, size_t(NBD) * lv.nn));
       TRY(bd_scratch(h, size_t(NBD) * 32 * lv.nblk * sizeof(float)));
       launch_blockdiag<float>(lv.g, h->dp, lv.H32, lv.mask, lv.D32, static_cast<float*>(h->bd_scratch), s);
       if (h->contact_on) launch_contact_blockdiag<float>(lv.g, lv.Kc32, lv.D32, s);
@@ -451,7 +460,7 @@ pfm_status linearize_impl(pfm_handle* h, pfm_precision prec, double* R_fused = n
       TRY(ensure_level_vectors<float>(h));
       TRY(estimate_lambda<float>(h, l));
     } else {
-      TRY(dalloc(h, &lv.D64, size_t(NF2) * lv.nn));
+      TRY(dalloc(h, &lv.D64, size_t(NBD) * lv.nn));
       TRY(bd_scratch(h, size_t(NBD) * 32 * lv.nblk * sizeof(double)));
       launch_blockdiag<double>(lv.g, h->dp, lv.H64, lv.mask, lv.D64, static_cast<double*>(h->bd_scratch), s);
       if (h->contact_on) launch_contact_blockdiag<double>(lv.g, lv.Kc64, lv.D64, s);
@@ -1648,9 +1657,9 @@ pfm_status pfm_get_block_inverses(pfm_handle* h, int level, int64_t n0, int64_t 
   if (count == 0) return PFM_OK;
   const bool f32 = h->lin_prec == PFM_F32;
   if ((f32 && !lv.D32) || (!f32 && !lv.D64)) return h->fail(PFM_ERR_STATE, "no block inverses on this level");
-  std::vector<double> buf(size_t(NF2) * count);
+  std::vector<double> buf(size_t(NBD) * count);
   std::vector<float> b32(f32 ? size_t(count) : 0);
-  for (int e = 0; e < NF2; ++e) {
+  for (int e = 0; e < NBD; ++e) {
     if (f32) {
       CK(cudaMemcpyAsync(b32.data(), lv.D32 + int64_t(e) * lv.nn + n0, sizeof(float) * count,
                          cudaMemcpyDeviceToHost, h->stream));
@@ -1663,7 +1672,7 @@ pfm_status pfm_get_block_inverses(pfm_handle* h, int level, int64_t n0, int64_t 
   }
   CK(cudaStreamSynchronize(h->stream));
   for (int64_t i = 0; i < count; ++i)
-    for (int e = 0; e < NF2; ++e) inv_host[i * NF2 + e] = buf[size_t(e) * count + i];
+    for (int e = 0; e < NF2; ++e) inv_host[i * NF2 + e] = buf[size_t(bidx(e / NF, e % NF)) * count + i];
   return PFM_OK;
 }
 

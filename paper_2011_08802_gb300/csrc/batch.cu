@@ -182,7 +182,7 @@ __device__ __forceinline__ int find_entry(const S* __restrict__ set, int ns, int
 // from the FP32 stores or (H16) from their binary16 copies.
 // Each warp caches the descriptor of its current problem in shared memory.
 template <bool H16>
-__global__ void __launch_bounds__(256) k_b_japply(const BLev* __restrict__ S, int ns, int64_t nblk, int vsel,
+__global__ void __launch_bounds__(256, 2) k_b_japply(const BLev* __restrict__ S, int ns, int64_t nblk, int vsel,
                                                   int ysel, Gate on) {
   __shared__ BLev cache[8];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -203,8 +203,10 @@ __global__ void __launch_bounds__(256) k_b_japply(const BLev* __restrict__ S, in
     if (on(L.problem) && blk - L.blk0 < L.g.nblk()) {
       if constexpr (H16)
         japply_block_h16<false>(L.g, L.jp, L.wh, L.H16, L.mask, L.vec[vsel], L.vec[ysel], blk - L.blk0, lane);
-      else
+      else {
+        if (lane == 0) prefetch_l2(L.H + (blk - L.blk0) * HBLK, unsigned(HBLK * sizeof(float)));
         japply_block<float, true>(L.g, L.jp, L.H, L.mask, L.vec[vsel], L.vec[ysel], blk - L.blk0, lane);
+      }
     }
   }
 }
@@ -245,21 +247,24 @@ __global__ void k_b_init(const BLev* __restrict__ S, int vsel, int ysel, Gate on
     y[i] = ((L.mask[i % nn] >> int(i / nn)) & 1) ? v[i] : 0.f;
 }
 
-__global__ void k_b_cheb_first(const BLev* __restrict__ S, int srcsel, bool copy_r, bool zero_x, Gate on) {
+// rows: write the identity rows and zeros that the next application starts from
+__global__ void k_b_cheb_first(const BLev* __restrict__ S, bool zero_x, bool rows, Gate on) {
   const BLev& L = S[blockIdx.y];
   if (!on(L.problem)) return;
   const int64_t nn = L.g.nn();
   for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn; node += int64_t(gridDim.x) * blockDim.x)
-    cheb_first_node<float>(nn, L.D, L.vec[srcsel], L.inv_theta, copy_r, zero_x, L.vec[VR], L.vec[VD], L.vec[VX], node);
+    cheb_first_node<float>(nn, L.D, L.vec[VB], zero_x ? nullptr : L.vec[VY], L.inv_theta, zero_x, L.vec[VR], L.vec[VD],
+                           L.vec[VX], L.mask, rows ? L.vec[VY] : nullptr, node);
 }
 
-__global__ void k_b_cheb_step(const BLev* __restrict__ S, float a, float c, Gate on) {
+__global__ void k_b_cheb_step(const BLev* __restrict__ S, float a, float c, bool rows, Gate on) {
   const BLev& L = S[blockIdx.y];
   if (!on(L.problem)) return;
   const int64_t nn = L.g.nn();
   const float cp = c * L.inv_delta;
   for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn; node += int64_t(gridDim.x) * blockDim.x)
-    cheb_step_node<float>(nn, L.D, L.vec[VY], a, cp, L.vec[VR], L.vec[VD], L.vec[VX], node);
+    cheb_step_node<float>(nn, L.D, L.vec[VY], a, cp, L.vec[VR], L.vec[VD], L.vec[VX], L.mask,
+                          rows ? L.vec[VY] : nullptr, node);
 }
 
 // out = vec[asel] - vec[bsel]
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(128) k_b_linearize(const BLin* __restrict__ S,
 __global__ void k_b_zero_D(const BBd* __restrict__ S, Gate on) {
   const BBd& L = S[blockIdx.y];
   if (!on(L.problem)) return;
-  const int64_t n = NF2 * L.g.nn();
+  const int64_t n = NBD * L.g.nn();
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
     L.D[i] = 0.f;
 }
@@ -366,12 +371,12 @@ __global__ void __launch_bounds__(128) k_b_blockdiag(const BBd* __restrict__ S, 
   blockdiag_elem_node<float>(L.g, L.jp, L.H, L.D, e - L.e0, int(tid & 7));
 }
 
-__global__ void k_b_block_invert(const BBd* __restrict__ S, int* singular, Gate on) {
+__global__ void __launch_bounds__(16 * BI_NODES) k_b_block_invert(const BBd* __restrict__ S, int* singular, Gate on) {
+  __shared__ BlockInvertSmem sm;
   const BBd& L = S[blockIdx.y];
-  if (!on(L.problem)) return;
-  const int64_t nn = L.g.nn();
-  for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn; node += int64_t(gridDim.x) * blockDim.x)
-    block_invert_node<float>(nn, L.mask, L.D, singular, node);
+  const int64_t nn = L.g.nn(), n0 = int64_t(blockIdx.x) * BI_NODES;
+  if (n0 >= nn || !on(L.problem)) return;
+  block_invert_lanes(nn, L.mask, L.D, singular, n0, sm);
 }
 
 // power iteration: x = start vector
@@ -392,16 +397,12 @@ __global__ void k_b_dinv(const BLev* __restrict__ S, int src, int dst, Gate on) 
   const float* y = L.vec[src];
   float* r = L.vec[dst];
   for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn; node += int64_t(gridDim.x) * blockDim.x) {
-    float yv[NF];
+    float yv[NF], z[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) yv[f] = y[f * nn + node];
+    dinv_node<float>(nn, L.D, yv, z, node);
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      float s = 0.f;
-#pragma unroll
-      for (int c = 0; c < NF; ++c) s += L.D[(f * NF + c) * nn + node] * yv[c];
-      r[f * nn + node] = s;
-    }
+    for (int f = 0; f < NF; ++f) r[f * nn + node] = z[f];
   }
 }
 
@@ -440,8 +441,13 @@ __global__ void k_b_scale(const BLev* __restrict__ S, int src, int dst, const do
   const BLev& L = S[blockIdx.y];
   if (!on(L.problem)) return;
   const int64_t n = NF * L.g.nn();
-  const double d = dot[blockIdx.y];
-  const float sc = d > 0.0 ? float(1.0 / sqrt(d)) : 0.f;
+  __shared__ float scale;  // one FP64 square root and division per block, not per thread
+  if (threadIdx.x == 0) {
+    const double d = dot[blockIdx.y];
+    scale = d > 0.0 ? float(1.0 / sqrt(d)) : 0.f;
+  }
+  __syncthreads();
+  const float sc = scale;
   const float* a = L.vec[src];
   float* x = L.vec[dst];
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
@@ -464,8 +470,13 @@ __global__ void k_b_lanczos_orth(const BLev* __restrict__ S, int usel, int qsel,
   const BLev& L = S[blockIdx.y];
   if (!on(L.problem)) return;
   const int64_t n = NF * L.g.nn();
-  const float a = float(alpha[blockIdx.y]);
-  const float bq = beta2prev ? float(sqrt(beta2prev[blockIdx.y])) : 0.f;
+  __shared__ float ab[2];
+  if (threadIdx.x == 0) {
+    ab[0] = float(alpha[blockIdx.y]);
+    ab[1] = beta2prev ? float(sqrt(beta2prev[blockIdx.y])) : 0.f;
+  }
+  __syncthreads();
+  const float a = ab[0], bq = ab[1];
   float* u = L.vec[usel];
   const float* q = L.vec[qsel];
   const float* qp = L.vec[qpsel];
@@ -1008,7 +1019,7 @@ pfm_status engine_buffers(pfm_handle* h, int m) {
     if (fine || !coarsest) TRY(dalloc(h, &lv.H32, hsz));
     if (fine) TRY(dalloc(h, &lv.H32lo, hsz));
     if (h->pre_h16 && !coarsest) TRY(dalloc(h, &lv.H16, hsz));
-    if (!coarsest) TRY(dalloc(h, &lv.D32, size_t(NF2) * lv.nn));
+    if (!coarsest) TRY(dalloc(h, &lv.D32, size_t(NBD) * lv.nn));
     TRY(dalloc(h, &lv.x32, ndof(lv)));
     TRY(dalloc(h, &lv.b32, ndof(lv)));
     TRY(dalloc(h, &lv.y32, ndof(lv)));
@@ -1224,15 +1235,20 @@ pfm_status engine_build(pfm_batch* b, const pfm_solve_opts& o, BatchEngine** out
   return PFM_OK;
 }
 
-// y = J v on every level of a set (identity rows first, then the elements)
-void eng_japply(BatchEngine* E, const BLev* dS, int ns, int64_t nblk, int64_t maxnn, int v, int y, Gate g) {
-  k_b_init<<<grid2(NF * maxnn, ns), BT, 0, E->s>>>(dS, v, y, g);
+// y = J v on every level of a set (first pass, then the elements); y_ready: the
+// smoothing step before has written the identity rows and zeros
+void eng_japply(BatchEngine* E, const BLev* dS, int ns, int64_t nblk, int64_t maxnn, int v, int y, Gate g,
+                bool y_ready = false) {
+  if (!y_ready) {
+    k_b_init<<<grid2(NF * maxnn, ns), BT, 0, E->s>>>(dS, v, y, g);
+    count_launches(1);
+  }
   const int blocks = std::max(1, std::min<int>(E->grid_japply, int(gdiv(nblk * 32, 256))));
   if (E->h16)
     k_b_japply<true><<<blocks, 256, 0, E->s>>>(dS, ns, nblk, v, y, g);
   else
     k_b_japply<false><<<blocks, 256, 0, E->s>>>(dS, ns, nblk, v, y, g);
-  count_launches(2);
+  count_launches(1);
 }
 
 // nu Chebyshev steps on depth d (the single-problem smoother, every problem at once)
@@ -1242,24 +1258,19 @@ void eng_smooth(BatchEngine* E, int d, bool zero_x, int nu, bool want_res, Gate 
   const dim3 gn = grid2(Ds.maxnn, ns), gv = grid2(NF * Ds.maxnn, ns);
   const double sigma = (E->hi + E->lo) / (E->hi - E->lo);
   double rho = 1.0 / sigma;
-  if (zero_x) {
-    k_b_cheb_first<<<gn, BT, 0, E->s>>>(Ds.dS, VB, true, true, g);
-    count_launches(1);
-  } else {
-    eng_japply(E, Ds.dS, ns, Ds.nblk, Ds.maxnn, VX, VY, g);
-    k_b_sub<<<gv, BT, 0, E->s>>>(Ds.dS, VB, VY, VR, g);
-    k_b_cheb_first<<<gn, BT, 0, E->s>>>(Ds.dS, VR, false, false, g);
-    count_launches(2);
-  }
+  if (!zero_x) eng_japply(E, Ds.dS, ns, Ds.nblk, Ds.maxnn, VX, VY, g);
+  k_b_cheb_first<<<gn, BT, 0, E->s>>>(Ds.dS, zero_x, nu > 1 || want_res, g);
+  count_launches(1);
   for (int k = 1; k < nu; ++k) {
-    eng_japply(E, Ds.dS, ns, Ds.nblk, Ds.maxnn, VD, VY, g);
+    eng_japply(E, Ds.dS, ns, Ds.nblk, Ds.maxnn, VD, VY, g, true);
     const double rho_n = 1.0 / (2.0 * sigma - rho);
-    k_b_cheb_step<<<gn, BT, 0, E->s>>>(Ds.dS, float(rho_n * rho), float(2.0 * rho_n), g);
+    k_b_cheb_step<<<gn, BT, 0, E->s>>>(Ds.dS, float(rho_n * rho), float(2.0 * rho_n),
+                                       k + 1 < nu || want_res, g);
     count_launches(1);
     rho = rho_n;
   }
   if (want_res) {
-    eng_japply(E, Ds.dS, ns, Ds.nblk, Ds.maxnn, VD, VY, g);
+    eng_japply(E, Ds.dS, ns, Ds.nblk, Ds.maxnn, VD, VY, g, true);
     k_b_sub<<<gv, BT, 0, E->s>>>(Ds.dS, VR, VY, VR, g);
     count_launches(1);
   }
@@ -1341,9 +1352,9 @@ pfm_status eng_linearize(pfm_batch* b, BatchEngine* E, int power_its) {
     count_launches(1);
   }
   if (nA > 0) {
-    k_b_zero_D<<<grid2(NF2 * E->maxnnBd, nA), BT, 0, s>>>(E->dBd, g);
+    k_b_zero_D<<<grid2(NBD * E->maxnnBd, nA), BT, 0, s>>>(E->dBd, g);
     k_b_blockdiag<<<gdiv(E->neBd * 8, 128), 128, 0, s>>>(E->dBd, nA, E->neBd, g);
-    k_b_block_invert<<<grid2(E->maxnnBd, nA), BT, 0, s>>>(E->dBd, E->singular, g);
+    k_b_block_invert<<<dim3(gdiv(E->maxnnBd, BI_NODES), unsigned(nA)), 16 * BI_NODES, 0, s>>>(E->dBd, E->singular, g);
     count_launches(3);
     // Lanczos estimate of lambda_max(D^-1 J) on every non-coarsest level at
     // once (the single-problem estimate_lambda, entry by entry): q = VX / VB

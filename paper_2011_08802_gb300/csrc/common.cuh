@@ -15,6 +15,11 @@ namespace pfm {
 constexpr int NF = 3 + NV;          // unknowns per node: u (3) + eta_hat (N): 9 for N = 6
 constexpr int NBD = NF * (NF + 1) / 2;  // packed upper triangle of a nodal NF x NF block (45)
 constexpr int NF2 = NF * NF;            // entries of a nodal block (81)
+// packed index of (r, c), any order, in the upper triangle of a nodal block:
+// nodal blocks and their inverses are symmetric and stored as [NBD][n_nodes]
+__host__ __device__ constexpr int bidx(int r, int c) {
+  return r <= c ? r * NF - (r * (r - 1)) / 2 + (c - r) : c * NF - (c * (c - 1)) / 2 + (r - c);
+}
 constexpr int NED = 8 * NF;             // unknowns of one element (72)
 
 // Gauss points of the 2-point rule mapped to [0,1]: (1 -+ 1/sqrt(3)) / 2.
@@ -151,15 +156,16 @@ void launch_linearize(const Grid& g, const DevParams& P, const double* U, const 
                       const LinResidual* res = nullptr);
 void launch_japply_df(const Grid& g, const DevParams& P, const float* Hhi, const float* Hlo, const dmask_t* mask,
                       const float* v, double* y, cudaStream_t s, double* W = nullptr);
+// y_ready (FP32 without W): y already holds v at prescribed DOFs and 0 elsewhere
 template <typename T>
 void launch_japply(const Grid& g, const DevParams& P, const T* H, const dmask_t* mask, const T* v,
-                   T* y, cudaStream_t s, T* W = nullptr);
+                   T* y, cudaStream_t s, T* W = nullptr, bool y_ready = false);
 // y = J v from a binary16 copy of the FP32 store holding s H (FP32 arithmetic;
 // inv_scale = 1/s), and the conversion that makes that copy: returns s, a
 // power of two putting max |H| in [2^14, 2^15), or 0 on failure (scratch: one
 // device word).
 void launch_japply_h16(const Grid& g, const DevParams& P, const __half* H, float inv_scale, const dmask_t* mask,
-                       const float* v, float* y, cudaStream_t s, float* W = nullptr);
+                       const float* v, float* y, cudaStream_t s, float* W = nullptr, bool y_ready = false);
 float launch_store_to_half(const Grid& g, const float* H32, __half* H16, unsigned* scratch, cudaStream_t s);
 // power-of-two scale s of the binary16 copy for a store whose largest entry
 // has magnitude amax (finite)
@@ -201,11 +207,17 @@ void launch_sub(int64_t n, const T* b, const T* y, T* r, cudaStream_t s);
 template <typename T>
 void launch_coarse_assemble(const Grid& g, const DevParams& P, const T* H, const dmask_t* mask,
                             double* K, int ld, cudaStream_t s, bool det = false);
+// r = b - y (y null: b), d = c D^-1 r, x = d (first) or x += d; and r -= y,
+// d = a d + c D^-1 r, x += d. yn (optional) receives d at prescribed DOFs and 0
+// elsewhere, what an application to d starts from (yn may be y).
 template <typename T>
-void launch_cheb_first(int64_t nn, const T* D, const T* src, T c, bool copy_r, bool zero_x, T* r, T* d, T* x,
-                       cudaStream_t s);
+void launch_cheb_first(int64_t nn, const T* D, const T* b, const T* y, T c, bool zero_x, T* r, T* d, T* x,
+                       const dmask_t* mask, T* yn, cudaStream_t s);
 template <typename T>
-void launch_cheb_step(int64_t nn, const T* D, const T* y, T a, T c, T* r, T* d, T* x, cudaStream_t s);
+void launch_cheb_step(int64_t nn, const T* D, const T* y, T a, T c, T* r, T* d, T* x, const dmask_t* mask, T* yn,
+                      cudaStream_t s);
+template <typename T>
+void launch_dinv(int64_t nn, const T* D, const T* src, T* dst, cudaStream_t s);  // dst = D^-1 src
 template <typename T>
 void launch_power_init(int64_t nn, const dmask_t* mask, T* x, cudaStream_t s);
 template <typename T>

@@ -281,7 +281,7 @@ __device__ __forceinline__ void blockdiag_accumulate(const JParams<T>& jp, const
 }
 
 // (element e, local node a): its element's contribution added to the node's
-// block D[(r*NF+c)*nn + node] with atomics (batched engine).
+// packed block D[t*nn + node] with atomics (batched engine).
 template <typename T>
 __device__ __forceinline__ void blockdiag_elem_node(const Grid& g, const JParams<T>& jp, const T* __restrict__ H,
                                                     T* __restrict__ D, int64_t e, int a) {
@@ -291,18 +291,14 @@ __device__ __forceinline__ void blockdiag_elem_node(const Grid& g, const JParams
 #pragma unroll
   for (int i = 0; i < NBD; ++i) Db[i] = T(0);
   blockdiag_accumulate<T>(jp, H, e >> 2, int(e & 3) * 8, a, Db);
-  int idx = 0;
-  for (int r = 0; r < NF; ++r)
-    for (int c = r; c < NF; ++c) {
-      atomicAdd(&D[(r * NF + c) * nn + node], Db[idx]);
-      if (c != r) atomicAdd(&D[(c * NF + r) * nn + node], Db[idx]);
-      ++idx;
-    }
+#pragma unroll
+  for (int t = 0; t < NBD; ++t) atomicAdd(&D[t * nn + node], Db[t]);
 }
 
 // In-place inverse of one node's NF x NF block (Dirichlet rows/columns replaced
 // by identity first) by Gauss-Jordan elimination with partial pivoting; a
-// singular block sets *singular and is replaced by the identity.
+// singular block sets *singular and is replaced by the identity. Form for FP64:
+// one thread per node, bound by the FP64 pipe.
 template <typename T>
 __device__ __forceinline__ void block_invert_node(int64_t nn, const dmask_t* __restrict__ mask, T* __restrict__ D,
                                                   int* singular, int64_t node) {
@@ -310,7 +306,7 @@ __device__ __forceinline__ void block_invert_node(int64_t nn, const dmask_t* __r
   T a[NF][NF], x[NF][NF];
   for (int r = 0; r < NF; ++r)
     for (int c = 0; c < NF; ++c) {
-      T v = D[(r * NF + c) * nn + node];
+      T v = D[bidx(r, c) * nn + node];
       if (((dm >> r) & 1) || ((dm >> c) & 1)) v = (r == c) ? T(1) : T(0);
       a[r][c] = v;
       x[r][c] = (r == c) ? T(1) : T(0);
@@ -342,7 +338,86 @@ __device__ __forceinline__ void block_invert_node(int64_t nn, const dmask_t* __r
       for (int c = 0; c < NF; ++c) x[r][c] = (r == c) ? T(1) : T(0);
   }
   for (int r = 0; r < NF; ++r)
-    for (int c = 0; c < NF; ++c) D[(r * NF + c) * nn + node] = x[r][c];
+    for (int c = r; c < NF; ++c) D[bidx(r, c) * nn + node] = x[r][c];
+}
+
+// The same in FP32 by 16 lanes per node, lane r holding row r in registers: the
+// rows of one thread's matrix were indexed by the pivot and lay in local memory,
+// which bounded that form. In-place elimination with the row permutation kept
+// implicit (row p_k expresses x_k afterwards: Ainv[k][p_j] = M[p_k][j]); the
+// pivot row travels by shuffles. A CTA takes BI_NODES consecutive nodes, whose
+// blocks pass through shared memory so that global accesses are contiguous.
+constexpr int BI_NODES = 32;
+struct BlockInvertSmem {
+  float S[NBD][BI_NODES + 1];
+};
+__device__ __forceinline__ void block_invert_lanes(int64_t nn, const dmask_t* __restrict__ mask, float* __restrict__ D,
+                                                   int* singular, int64_t n0, BlockInvertSmem& sm) {
+  static_assert(NF <= 16, "one lane per row");
+  const int tid = int(threadIdx.x);
+  for (int i = tid; i < NBD * BI_NODES; i += int(blockDim.x)) {
+    const int t = i / BI_NODES, m = i % BI_NODES;
+    sm.S[t][m] = n0 + m < nn ? D[t * nn + n0 + m] : 0.f;
+  }
+  __syncthreads();
+  const int m = tid >> 4, r = tid & 15;
+  const bool valid = n0 + m < nn;
+  const dmask_t dm = valid ? mask[n0 + m] : MASK_ALL;  // padding nodes invert the identity
+  float a[NF];
+#pragma unroll
+  for (int c = 0; c < NF; ++c) {
+    float v = r < NF ? sm.S[bidx(r < NF ? r : 0, c)][m] : 0.f;
+    if (((dm >> r) & 1) || ((dm >> c) & 1)) v = r == c ? 1.f : 0.f;
+    a[c] = v;
+  }
+  int own = -1;   // the column this lane's row was the pivot of
+  bool bad = false;
+  int pc[NF];     // pivot row of every column
+#pragma unroll
+  for (int k = 0; k < NF; ++k) {
+    // largest |a_k| over the unused rows (bits of a non-negative float order as
+    // the float; a NaN counts as the largest), ties: the lowest row
+    unsigned key = r < NF && own < 0 ? (__float_as_uint(a[k]) & 0x7fffffffu) + 1u : 0u;
+    int p = r;
+#pragma unroll
+    for (int w = 8; w > 0; w >>= 1) {
+      const unsigned ok = __shfl_xor_sync(0xffffffffu, key, w, 16);
+      const int op = __shfl_xor_sync(0xffffffffu, p, w, 16);
+      if (ok > key || (ok == key && op < p)) {
+        key = ok;
+        p = op;
+      }
+    }
+    pc[k] = p;
+    const float pv = __shfl_sync(0xffffffffu, a[k], p, 16);
+    if (!(fabsf(pv) > 0.f)) bad = true;
+    const float ip = 1.f / pv;
+    const bool mine = r == p;
+    if (mine) own = k;
+    const float f = mine ? ip : -(a[k] * ip);  // this row's coefficient of the pivot row
+#pragma unroll
+    for (int c = 0; c < NF; ++c) {
+      const float pr = __shfl_sync(0xffffffffu, a[c], p, 16);
+      if (c != k) a[c] = mine ? pr * ip : fmaf(f, pr, a[c]);
+    }
+    a[k] = f;
+  }
+  __syncthreads();
+  if (bad) {
+    if (r == 0) atomicExch(singular, 1);
+#pragma unroll
+    for (int c = 0; c < NF; ++c)
+      if (r < NF && r <= c) sm.S[bidx(r, c)][m] = r == c ? 1.f : 0.f;
+  } else if (r < NF) {
+#pragma unroll
+    for (int j = 0; j < NF; ++j)
+      if (own <= pc[j]) sm.S[bidx(own, pc[j])][m] = a[j];
+  }
+  __syncthreads();
+  for (int i = tid; i < NBD * BI_NODES; i += int(blockDim.x)) {
+    const int t = i / BI_NODES, q = i % BI_NODES;
+    if (n0 + q < nn) D[t * nn + n0 + q] = sm.S[t][q];
+  }
 }
 
 // Element constants of a level: gradient-energy matrix, quadrature weight and
@@ -690,6 +765,13 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, unsigned parity, u
       if (dt > limit_ns) return false;
     }
   }
+}
+
+// Bulk prefetch of a contiguous global range into L2 by the bulk-copy engine
+// (no registers or shared memory involved); address 16-byte aligned, size a
+// multiple of 16 bytes.
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
 // Element constants of the staged tangent application. The Hessian part is

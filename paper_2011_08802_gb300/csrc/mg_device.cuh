@@ -352,49 +352,69 @@ inline __host__ __device__ bool nested(const Grid& f, const Grid& c) {
   return f.nx == 2 * c.nx && f.ny == 2 * c.ny && f.nz == 2 * c.nz;
 }
 
-// Chebyshev-accelerated point-block Jacobi at one node (Saad, Iterative
-// Methods, Alg. 12.1 applied to D^-1 J). First step: d = c D^-1 r0 with
-// r0 = src (also stored in r when copy_r), x = d (zero_x) or x += d.
+// z = D^-1 r at one node, D^-1 packed symmetric.
 template <typename T>
-__device__ __forceinline__ void cheb_first_node(int64_t nn, const T* __restrict__ D, const T* src, T c, bool copy_r,
-                                                bool zero_x, T* r, T* __restrict__ d, T* __restrict__ x,
+__device__ __forceinline__ void dinv_node(int64_t nn, const T* __restrict__ D, const T r[NF], T z[NF], int64_t node) {
+#pragma unroll
+  for (int f = 0; f < NF; ++f) z[f] = T(0);
+#pragma unroll
+  for (int f = 0; f < NF; ++f)
+#pragma unroll
+    for (int c = f; c < NF; ++c) {
+      const T v = D[bidx(f, c) * nn + node];
+      z[f] += v * r[c];
+      if (c != f) z[c] += v * r[f];
+    }
+}
+
+// Chebyshev-accelerated point-block Jacobi at one node (Saad, Iterative
+// Methods, Alg. 12.1 applied to D^-1 J), bound by reading D^-1 (NBD entries per
+// node) and the vectors. First step: r = b - y (y null: r = b), d = c D^-1 r,
+// x = d (zero_x) or x += d. yn (optional): d at prescribed DOFs and 0 elsewhere,
+// where the application of J to d starts from; it may be y, whose entries of
+// this node have been read by then.
+template <typename T>
+__device__ __forceinline__ void cheb_first_node(int64_t nn, const T* __restrict__ D, const T* __restrict__ b,
+                                                const T* y, T c, bool zero_x, T* __restrict__ r, T* __restrict__ d,
+                                                T* __restrict__ x, const dmask_t* __restrict__ mask, T* yn,
                                                 int64_t node) {
-  T rv[NF];
+  T rv[NF], z[NF];
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
-    rv[f] = src[f * nn + node];
-    if (copy_r) r[f * nn + node] = rv[f];
+    rv[f] = b[f * nn + node];
+    if (y) rv[f] -= y[f * nn + node];
+    r[f * nn + node] = rv[f];
   }
+  dinv_node<T>(nn, D, rv, z, node);
+  const dmask_t dm = yn ? mask[node] : dmask_t(0);
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
-    T s = T(0);
-#pragma unroll
-    for (int cc = 0; cc < NF; ++cc) s += D[(f * NF + cc) * nn + node] * rv[cc];
-    const T dv = c * s;
+    const T dv = c * z[f];
     d[f * nn + node] = dv;
     x[f * nn + node] = zero_x ? dv : x[f * nn + node] + dv;
+    if (yn) yn[f * nn + node] = ((dm >> f) & 1) ? dv : T(0);
   }
 }
 
-// Later steps: r -= y; d = a d + c D^-1 r; x += d.
+// Later steps: r -= y; d = a d + c D^-1 r; x += d; yn as above.
 template <typename T>
-__device__ __forceinline__ void cheb_step_node(int64_t nn, const T* __restrict__ D, const T* __restrict__ y, T a,
-                                               T c, T* __restrict__ r, T* __restrict__ d, T* __restrict__ x,
-                                               int64_t node) {
-  T rv[NF];
+__device__ __forceinline__ void cheb_step_node(int64_t nn, const T* __restrict__ D, const T* y, T a, T c,
+                                               T* __restrict__ r, T* __restrict__ d, T* __restrict__ x,
+                                               const dmask_t* __restrict__ mask, T* yn, int64_t node) {
+  T rv[NF], z[NF];
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     rv[f] = r[f * nn + node] - y[f * nn + node];
     r[f * nn + node] = rv[f];
   }
+  dinv_node<T>(nn, D, rv, z, node);
+  const dmask_t dm = yn ? mask[node] : dmask_t(0);
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
-    T s = T(0);
-#pragma unroll
-    for (int cc = 0; cc < NF; ++cc) s += D[(f * NF + cc) * nn + node] * rv[cc];
-    const T dv = a * d[f * nn + node] + c * s;
+    const T dv = a * d[f * nn + node] + c * z[f];
     d[f * nn + node] = dv;
     x[f * nn + node] += dv;
+    if (yn) yn[f * nn + node] = ((dm >> f) & 1) ? dv : T(0);
   }
 }
 

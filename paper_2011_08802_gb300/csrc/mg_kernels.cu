@@ -101,16 +101,26 @@ __global__ void k_smooth(int64_t nn, const T* __restrict__ D, const T* __restric
                          const T* __restrict__ y, T omega, T* __restrict__ x) {
   for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn;
        node += int64_t(gridDim.x) * blockDim.x) {
-    T r[NF];
+    T r[NF], z[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) r[f] = b[f * nn + node] - (y ? y[f * nn + node] : T(0));
+    dinv_node<T>(nn, D, r, z, node);
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      T s = T(0);
+    for (int f = 0; f < NF; ++f) x[f * nn + node] += omega * z[f];
+  }
+}
+
+// dst = D^-1 src per node.
+template <typename T>
+__global__ void k_dinv(int64_t nn, const T* __restrict__ D, const T* __restrict__ src, T* __restrict__ dst) {
+  for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn;
+       node += int64_t(gridDim.x) * blockDim.x) {
+    T r[NF], z[NF];
 #pragma unroll
-      for (int c = 0; c < NF; ++c) s += D[(f * NF + c) * nn + node] * r[c];
-      x[f * nn + node] += omega * s;
-    }
+    for (int f = 0; f < NF; ++f) r[f] = src[f * nn + node];
+    dinv_node<T>(nn, D, r, z, node);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) dst[f * nn + node] = z[f];
   }
 }
 
@@ -244,24 +254,25 @@ __global__ void k_coarse_solve(int n, const double* __restrict__ Ainv, const T* 
   if (lane == 0) x[warp] = T(s);
 }
 
-// Chebyshev-accelerated point-block Jacobi (Saad, Iterative Methods, Alg. 12.1
-// applied to D^-1 J): first step d = c D^-1 r0 with r0 = src (also stored in r
-// when copy_r), x = d (zero_x) or x += d.
+// Chebyshev-accelerated point-block Jacobi, first and later steps (mg_device.cuh).
+// 64 registers (4 CTAs of 256 threads per SM) let a node's 45 + 36 loads be in
+// flight together; with the compiler's own choice (32 registers) a step on
+// 129^3 nodes took about 0.27 ms for 1.0 GB.
 template <typename T>
-__global__ void k_cheb_first(int64_t nn, const T* __restrict__ D, const T* src, T c, bool copy_r,
-                             bool zero_x, T* r, T* __restrict__ d, T* __restrict__ x) {
+__global__ void __launch_bounds__(256, 4) k_cheb_first(int64_t nn, const T* __restrict__ D, const T* __restrict__ b, const T* y, T c, bool zero_x,
+                             T* __restrict__ r, T* __restrict__ d, T* __restrict__ x, const dmask_t* __restrict__ mask,
+                             T* yn) {
   for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn;
        node += int64_t(gridDim.x) * blockDim.x)
-    cheb_first_node<T>(nn, D, src, c, copy_r, zero_x, r, d, x, node);
+    cheb_first_node<T>(nn, D, b, y, c, zero_x, r, d, x, mask, yn, node);
 }
 
-// r -= y; d = a d + c D^-1 r; x += d.
 template <typename T>
-__global__ void k_cheb_step(int64_t nn, const T* __restrict__ D, const T* __restrict__ y, T a, T c,
-                            T* __restrict__ r, T* __restrict__ d, T* __restrict__ x) {
+__global__ void __launch_bounds__(256, 4) k_cheb_step(int64_t nn, const T* __restrict__ D, const T* y, T a, T c, T* __restrict__ r,
+                            T* __restrict__ d, T* __restrict__ x, const dmask_t* __restrict__ mask, T* yn) {
   for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn;
        node += int64_t(gridDim.x) * blockDim.x)
-    cheb_step_node<T>(nn, D, y, a, c, r, d, x, node);
+    cheb_step_node<T>(nn, D, y, a, c, r, d, x, mask, yn, node);
 }
 
 // Deterministic start vector of the power iteration (power_init_value).
@@ -285,8 +296,13 @@ __global__ void k_scale_inv_sqrt(int64_t n, const T* __restrict__ y, const doubl
 template <typename T>
 __global__ void k_lanczos_orth(int64_t n, T* __restrict__ u, const T* __restrict__ q, const T* __restrict__ qp,
                                const double* __restrict__ alpha, const double* __restrict__ beta2prev) {
-  const T a = T(*alpha);
-  const T b = beta2prev ? T(sqrt(*beta2prev)) : T(0);
+  __shared__ T ab[2];  // one FP64 square root per block, not per thread
+  if (threadIdx.x == 0) {
+    ab[0] = T(*alpha);
+    ab[1] = beta2prev ? T(sqrt(*beta2prev)) : T(0);
+  }
+  __syncthreads();
+  const T a = ab[0], b = ab[1];
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
     u[i] -= a * q[i] + (beta2prev ? b * qp[i] : T(0));
 }
@@ -301,15 +317,22 @@ void launch_lanczos_orth(int64_t n, T* u, const T* q, const T* qp, const double*
 }
 
 template <typename T>
-void launch_cheb_first(int64_t nn, const T* D, const T* src, T c, bool copy_r, bool zero_x, T* r, T* d, T* x,
-                       cudaStream_t s) {
-  k_cheb_first<T><<<grid_for(nn, 256), 256, 0, s>>>(nn, D, src, c, copy_r, zero_x, r, d, x);
+void launch_cheb_first(int64_t nn, const T* D, const T* b, const T* y, T c, bool zero_x, T* r, T* d, T* x,
+                       const dmask_t* mask, T* yn, cudaStream_t s) {
+  k_cheb_first<T><<<grid_for(nn, 256), 256, 0, s>>>(nn, D, b, y, c, zero_x, r, d, x, mask, yn);
   count_launches(1);
 }
 
 template <typename T>
-void launch_cheb_step(int64_t nn, const T* D, const T* y, T a, T c, T* r, T* d, T* x, cudaStream_t s) {
-  k_cheb_step<T><<<grid_for(nn, 256), 256, 0, s>>>(nn, D, y, a, c, r, d, x);
+void launch_cheb_step(int64_t nn, const T* D, const T* y, T a, T c, T* r, T* d, T* x, const dmask_t* mask, T* yn,
+                      cudaStream_t s) {
+  k_cheb_step<T><<<grid_for(nn, 256), 256, 0, s>>>(nn, D, y, a, c, r, d, x, mask, yn);
+  count_launches(1);
+}
+
+template <typename T>
+void launch_dinv(int64_t nn, const T* D, const T* src, T* dst, cudaStream_t s) {
+  k_dinv<T><<<grid_for(nn, 256), 256, 0, s>>>(nn, D, src, dst);
   count_launches(1);
 }
 
@@ -444,9 +467,11 @@ void launch_coarse_solve(int n, const double* Ainv, const T* b, T* x, cudaStream
   template void launch_coarse_assemble<T>(const Grid&, const DevParams&, const T*, const dmask_t*, \
                                           double*, int, cudaStream_t, bool);                    \
   template void launch_coarse_solve<T>(int, const double*, const T*, T*, cudaStream_t);         \
-  template void launch_cheb_first<T>(int64_t, const T*, const T*, T, bool, bool, T*, T*, T*,       \
-                                     cudaStream_t);                                             \
-  template void launch_cheb_step<T>(int64_t, const T*, const T*, T, T, T*, T*, T*, cudaStream_t); \
+  template void launch_cheb_first<T>(int64_t, const T*, const T*, const T*, T, bool, T*, T*, T*,   \
+                                     const dmask_t*, T*, cudaStream_t);                         \
+  template void launch_cheb_step<T>(int64_t, const T*, const T*, T, T, T*, T*, T*, const dmask_t*, T*, \
+                                    cudaStream_t);                                              \
+  template void launch_dinv<T>(int64_t, const T*, const T*, T*, cudaStream_t);                  \
   template void launch_power_init<T>(int64_t, const dmask_t*, T*, cudaStream_t);                  \
   template void launch_scale_inv_sqrt<T>(int64_t, const T*, const double*, T*, cudaStream_t);     \
   template void launch_lanczos_orth<T>(int64_t, T*, const T*, const T*, const double*, const double*, \
