@@ -137,6 +137,8 @@ struct BOut {
   const float* Hlo;
   const double* H64;
   const dmask_t* mask;
+  const DevParams* P;
+  const double* Un;
   double* V;     // (m+1) basis vectors
   float* Z;      // m preconditioned vectors
   double* w;     // work vector (J z, then the orthogonalised vector)
@@ -340,6 +342,33 @@ __global__ void __launch_bounds__(128) k_b_linearize(const BLin* __restrict__ S,
   const BLin& L = S[find_entry(S, ns, blk)];
   if (!on(L.problem)) return;
   linearize_lane<TC>(L.g, *L.P, L.U, L.Un, L.H64, L.H32, L.H32lo, blk - L.blk0, int(tid & 31));
+}
+
+// Residual of every active problem: first pass (displacement rows 0, nodal
+// gradient energy), then the elements of all problems in one launch (one launch
+// per problem left most SMs idle: a problem has 130 to 3456 warps, and each
+// takes about 0.1 ms of dependent FP64 work).
+__global__ void __launch_bounds__(GE_COLS * NV) k_b_residual_first(const BOut* __restrict__ O, const int* __restrict__ act) {
+  const int p = blockIdx.y;
+  if (!act[p]) return;
+  const BOut& o = O[p];
+  const int64_t ncol = grad_energy_columns(o.g);
+  __shared__ GradESmem<double> sm;
+  for (int64_t t = int64_t(blockIdx.x) * GE_COLS; t < ncol; t += int64_t(gridDim.x) * GE_COLS) {
+    grad_energy_block<double, GE_RES>(o.g, o.ge64, o.mask, o.U, o.b, t, ncol, sm, false);
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(128, 2) k_b_residual(const BOut* __restrict__ O, int np, int64_t nblk,
+                                                       const int* __restrict__ act) {
+  const int64_t tid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t blk = tid >> 5;
+  if (blk >= nblk) return;
+  const int p = find_entry(O, np, blk);
+  if (!act[p]) return;
+  const BOut& o = O[p];
+  residual_lane<double, false>(o.g, *o.P, o.U, o.Un, o.mask, o.b, nullptr, nullptr, 0, blk - o.blk0, int(tid & 31));
 }
 
 __global__ void k_b_zero_D(const BBd* __restrict__ S, Gate on) {
@@ -1170,6 +1199,8 @@ pfm_status engine_build(pfm_batch* b, const pfm_solve_opts& o, BatchEngine** out
     ob.Hlo = f.H32lo;
     ob.H64 = f.H64;
     ob.mask = f.mask;
+    ob.P = E->dP + p;
+    ob.Un = f.Un;
     ob.V = h->V;
     ob.Z = static_cast<float*>(h->Z);
     ob.w = h->wv;
@@ -1579,15 +1610,11 @@ pfm_status eng_fgmres(pfm_batch* b, BatchEngine* E) {
 
 pfm_status eng_residual_norms(pfm_batch* b, BatchEngine* E) {
   cudaStream_t s = E->s;
-  for (int p = 0; p < E->np; ++p) {
-    if (!E->hact[p]) continue;
-    pfm_handle* h = b->hs[p];
-    Level& f = h->L[0];
-    launch_residual(f.g, h->dp, f.U, f.Un, f.mask, h->R, nullptr, s);
-  }
+  k_b_residual_first<<<dim3(gdiv(E->maxcolO, GE_COLS), unsigned(E->np)), dim3(GE_COLS, NV), 0, s>>>(E->dO, E->dact);
+  k_b_residual<<<gdiv(E->nblkO * 32, 128), 128, 0, s>>>(E->dO, E->np, E->nblkO, E->dact);
   k_b_res_norm2<<<dim3(BCH, unsigned(E->np)), BT, 0, s>>>(E->dO, E->dact, E->partial);
   k_b_reduce_chunks<<<gdiv(E->np, 128), 128, 0, s>>>(E->np, BCH, E->partial, E->dots);
-  count_launches(2);
+  count_launches(4);
   BCK(cudaMemcpyAsync(E->hres, E->dots, sizeof(double) * E->np, cudaMemcpyDeviceToHost, s));
   BCK(cudaGetLastError());
   BCK(cudaStreamSynchronize(s));

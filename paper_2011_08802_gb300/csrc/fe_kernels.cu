@@ -35,40 +35,6 @@ namespace {
 #ifndef PFM_RES_MINB
 #define PFM_RES_MINB 2
 #endif
-// Residual rows and energy of one Gauss point (lane = 8 e + q of block blk)
-// from its energy gradient gr and energy density Wd: the nodal rows scattered
-// (DET: to the scratch W) with Dirichlet rows left out, the energy summed per
-// warp. The gradient energy is the nodal operator of grad_energy.cuh.
-template <typename TC, bool DET>
-__device__ __forceinline__ void residual_tail(const Grid& g, const TC* gr, TC Wd, int64_t node, bool valid, int l8,
-                                              int64_t blk, int lane, const dmask_t* __restrict__ mask,
-                                              double* __restrict__ R, double* energy, double* __restrict__ W,
-                                              int64_t ws) {
-  const int64_t nn = g.nn();
-  const TC ihx = TC(1.0 / g.hx), ihy = TC(1.0 / g.hy), ihz = TC(1.0 / g.hz);
-  const TC w = TC(g.w());
-  const dmask_t dm = valid ? mask[node] : dmask_t(0);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    TC r = w * q1_scatter_grad(gr[3 * i], gr[3 * i + 1], gr[3 * i + 2], l8, ihx, ihy, ihz);
-    scatter_row<DET>(R, W, ws, i, blk, lane, i * nn + node, double(r), valid && !((dm >> i) & 1));
-  }
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    TC r = w * q1_value(gr[9 + k]);
-    scatter_row<DET>(R, W, ws, 3 + k, blk, lane, (3 + k) * nn + node, double(r),
-                     valid && !((dm >> (3 + k)) & 1));
-  }
-  if (energy) {
-    double en = warp_sum(valid ? double(w * Wd) : 0.0);
-    if constexpr (DET) {
-      if (lane == 0) W[NF * ws + blk] = en;
-    } else {
-      if (lane == 0) atomicAdd(energy, en);
-    }
-  }
-}
-
 // Out-of-line copy for the linearisation pass, so that the register
 // allocation of its point physics does not see the residual's scatter.
 template <typename TC, bool DET>
@@ -86,22 +52,9 @@ __global__ void __launch_bounds__(128, PFM_RES_MINB) k_residual(Grid g, DevParam
                                                   double* __restrict__ R, double* energy, double* __restrict__ W,
                                                   int64_t ws) {
   const int64_t tid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t e = tid >> 3;
-  const int l8 = int(tid & 7);
   const int64_t blk = tid >> 5;
   if (blk >= g.nblk()) return;  // padding warps of the last block own no part of W
-  const int lane = int(tid & 31);
-  const bool valid = e < g.ne();
-  const int64_t nn = g.nn();
-  const int64_t node = valid ? elem_node(g, e, l8) : 0;
-  const TC ihx = TC(1.0 / g.hx), ihy = TC(1.0 / g.hy), ihz = TC(1.0 / g.hz);
-  TC F[9], eh[NV], ehn[NV];
-  gather_state<TC>(U, nn, node, valid, l8, ihx, ihy, ihz, F, eh);
-#pragma unroll
-  for (int k = 0; k < NV; ++k) ehn[k] = q1_value(valid ? TC(Un[(3 + k) * nn + node]) : TC(0.0));
-  TC Wd, gr[NZ];
-  qp_local<TC, false>(P, F, eh, ehn, &Wd, gr, nullptr);
-  residual_tail<TC, DET>(g, gr, Wd, node, valid, l8, blk, lane, mask, R, energy, W, ws);
+  residual_lane<TC, DET>(g, P, U, Un, mask, R, energy, W, ws, blk, int(tid & 31));
 }
 
 // Node pass of the atomic-free scatter (node_gather) over all nodes.
