@@ -31,17 +31,20 @@ __device__ __forceinline__ T shx(T v, int m) {
 template <typename T>
 __device__ __forceinline__ void q1_gather(T v, int l8, T ihx, T ihy, T ihz, T& val, T& gx, T& gy,
                                           T& gz) {
-  const T ga = T(GA), gb = T(GB);
-  T s = shx(v, 1);
-  T vx = gb * v + ga * s;
-  T dx = ((l8 & 1) ? (v - s) : (s - v)) * ihx;
+  const T ga = T(GA), gb = T(GB);  // ga + gb = 1: gb v + ga s = v + ga (s - v)
+  const T sx = (l8 & 1) ? -ihx : ihx, sy = (l8 & 2) ? -ihy : ihy, sz = (l8 & 4) ? -ihz : ihz;
+  const T d0 = shx(v, 1) - v;
+  T vx = v + ga * d0;
+  T dx = d0 * sx;
   T s1 = shx(vx, 2), s2 = shx(dx, 2);
-  T vxy = gb * vx + ga * s1;
-  T vdy = ((l8 & 2) ? (vx - s1) : (s1 - vx)) * ihy;
+  const T d1 = s1 - vx;
+  T vxy = vx + ga * d1;
+  T vdy = d1 * sy;
   T dxy = gb * dx + ga * s2;
   T t1 = shx(vxy, 4), t2 = shx(vdy, 4), t3 = shx(dxy, 4);
-  val = gb * vxy + ga * t1;
-  gz = ((l8 & 4) ? (vxy - t1) : (t1 - vxy)) * ihz;
+  const T d2 = t1 - vxy;
+  val = vxy + ga * d2;
+  gz = d2 * sz;
   gy = gb * vdy + ga * t2;
   gx = gb * dxy + ga * t3;
 }
@@ -174,6 +177,29 @@ struct NoLinTail {
   __device__ void operator()(const TC*, TC, int64_t, bool, int) const {}
 };
 
+// h = hi + lo as two FP32 numbers: hi = h rounded to nearest, lo = the rest
+// rounded. The conversions between FP64 and FP32 run on the FP64 pipe (4 of its
+// instructions per entry with the subtraction, a tenth of a linearisation), so
+// the rounding is done on the bits in the integer pipe: adding half a unit of
+// the 24-bit mantissa and cutting 29 bits rounds to nearest, and those 29 bits
+// read as a signed number are the rest. Numbers outside [2^-74, 2^127) and
+// non-finite ones take the conversions.
+__device__ __forceinline__ void split_f64(double h, float& hi, float& lo) {
+  const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(h));
+  const unsigned top = unsigned(u >> 32);
+  const unsigned e = (top >> 20) & 0x7ffu;
+  const unsigned sign = top & 0x80000000u;
+  if (e - 949u <= 200u) {
+    const unsigned m = unsigned(((u & 0x7fffffffffffffffull) + (1ull << 28)) >> 29) - (896u << 23);
+    const int rest = int(unsigned(u) << 3) >> 3;
+    hi = __uint_as_float(m | sign);
+    lo = __int2float_rn(rest) * __uint_as_float(((e - 948u) << 23) | sign);
+  } else {
+    hi = float(h);
+    lo = float(h - double(hi));
+  }
+}
+
 // Receives the Hessian entries of one Gauss point as they become final and
 // writes them to the requested stores (null stores are skipped; lanes without
 // an element write zeros).
@@ -195,8 +221,12 @@ struct HessStore {
     } else {
       const double h = valid ? double(v) : 0.0;
       if (H64) H64[hstore_offset<double>(blk, j, lane)] = h;
-      if (H32) H32[hstore_offset<float>(blk, j, lane)] = float(h);
-      if (H32lo) H32lo[hstore_offset<float>(blk, j, lane)] = float(h - double(float(h)));
+      if (H32) {
+        float hi, lo;
+        split_f64(h, hi, lo);
+        H32[hstore_offset<float>(blk, j, lane)] = hi;
+        if (H32lo) H32lo[hstore_offset<float>(blk, j, lane)] = lo;
+      }
     }
   }
 };
@@ -239,6 +269,10 @@ __device__ __forceinline__ void blockdiag_accumulate(const JParams<T>& jp, const
   constexpr int V = 16 / sizeof(T);
   using VT = typename Vec16<T>::type;
   const T ih[3] = {jp.ihx, jp.ihy, jp.ihz};
+  T D[NBD];
+#pragma unroll
+  for (int t = 0; t < NBD; ++t) D[t] = T(0);
+  T g2 = T(0);  // sum over the points of |grad N|^2
   for (int q = 0; q < 8; ++q) {
     T phi[3], dphi[3];
 #pragma unroll
@@ -249,35 +283,52 @@ __device__ __forceinline__ void blockdiag_accumulate(const JParams<T>& jp, const
     }
     const T N = phi[0] * phi[1] * phi[2];
     const T dN[3] = {dphi[0] * phi[1] * phi[2], phi[0] * dphi[1] * phi[2], phi[0] * phi[1] * dphi[2]};
+    // products of the shape functions, shared by all rows
+    T dd[3][3], dn[3];
+#pragma unroll
+    for (int J = 0; J < 3; ++J) {
+      dn[J] = dN[J] * N;
+#pragma unroll
+      for (int L = J; L < 3; ++L) dd[J][L] = dd[L][J] = dN[J] * dN[L];
+    }
+    const T n2 = N * N;
+    g2 += dd[0][0] + dd[1][1] + dd[2][2];
     // column map: DOF u_i -> z rows 3i+J (coef dN_J); eta_k -> z row 9+k (coef N)
     T Hq[NHP];
     const VT* Hv = reinterpret_cast<const VT*>(H) + blk * (NHP / V) * 32 + lane0 + q;
 #pragma unroll
     for (int jj = 0; jj < NHP / V; ++jj) Vec16<T>::unpack(Hv[jj * 32], Hq + jj * V);
-    const T g2 = dN[0] * dN[0] + dN[1] * dN[1] + dN[2] * dN[2];
     int idx = 0;
 #pragma unroll
     for (int r = 0; r < NF; ++r)
 #pragma unroll
       for (int c = r; c < NF; ++c) {
-        T s = T(0);
         if (r < 3 && c < 3) {
 #pragma unroll
           for (int J = 0; J < 3; ++J)
 #pragma unroll
             for (int L = 0; L < 3; ++L) {
               const int rr = 3 * r + J, cc = 3 * c + L;
-              s += dN[J] * dN[L] * Hq[rr <= cc ? hidx(rr, cc) : hidx(cc, rr)];
+              D[idx] += dd[J][L] * Hq[rr <= cc ? hidx(rr, cc) : hidx(cc, rr)];
             }
         } else if (r < 3) {
 #pragma unroll
-          for (int J = 0; J < 3; ++J) s += dN[J] * N * Hq[hidx(3 * r + J, 9 + (c - 3))];
+          for (int J = 0; J < 3; ++J) D[idx] += dn[J] * Hq[hidx(3 * r + J, 9 + (c - 3))];
         } else {
-          s = N * N * Hq[hidx(9 + (r - 3), 9 + (c - 3))] + g2 * jp.G[r - 3][c - 3];
+          D[idx] += n2 * Hq[hidx(9 + (r - 3), 9 + (c - 3))];
         }
-        Db[idx++] += jp.w * s;
+        ++idx;
       }
   }
+  int idx = 0;
+#pragma unroll
+  for (int r = 0; r < NF; ++r)
+#pragma unroll
+    for (int c = r; c < NF; ++c) {
+      if (r >= 3) D[idx] += g2 * jp.G[r - 3][c - 3];
+      Db[idx] += jp.w * D[idx];
+      ++idx;
+    }
 }
 
 // (element e, local node a): its element's contribution added to the node's

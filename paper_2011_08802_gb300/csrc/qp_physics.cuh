@@ -866,7 +866,7 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
     // sum over a, b, c of f2(a,b,c) T~_ab into the slots (a,c), (b,c)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      Mb[hm6(a, a)] += T(4) * f2d[a] * TJ[a];
+      Mb[hm6(a, a)] += f2d[a] * (T(4) * TJ[a]);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         if (c == a) continue;
@@ -937,7 +937,12 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
           Zf[p][b] = Mq[p][0] * R[0][b] + Mq[p][1] * R[1][b] + Mq[p][2] * R[2][b];
           Zu[p][b] = Uq[p][0] * R[0][b] + Uq[p][1] * R[1][b] + Uq[p][2] * R[2][b];
         }
-      auto dot = [](const T* x, const T* y) { return x[0] * y[0] + x[1] * y[1] + x[2] * y[2]; };
+      // acc += x . y, as three multiply-adds into acc
+      auto dot_to = [](T& acc, const T* x, const T* y) {
+        acc += x[0] * y[0];
+        acc += x[1] * y[1];
+        acc += x[2] * y[2];
+      };
 #pragma unroll
       for (int p = 0; p < 3; ++p)
 #pragma unroll
@@ -945,21 +950,24 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
           // F_pc with F_rc2 (final)
           if (c < c2 || p <= r) {
             const int i = 3 * p + c, j = 3 * r + c2;
-            emit(i <= j ? hidx(i, j) : hidx(j, i), dot(Zf[p], Mq[r]));
+            emit(i <= j ? hidx(i, j) : hidx(j, i), Zf[p][0] * Mq[r][0] + Zf[p][1] * Mq[r][1] + Zf[p][2] * Mq[r][2]);
           }
           // F_pc with F^t_(r, c2), and F_pc2 with F^t_(r, c)
-          FU[3 * p + c][voigt_slot(r, c2)] += dot(Zf[p], Uq[r]);
-          if (c < c2) FU[3 * p + c2][voigt_slot(r, c)] += dot(Zu[r], Mq[p]);
-          // F^t_(p, c) with F^t_(r, c2)
+          dot_to(FU[3 * p + c][voigt_slot(r, c2)], Zf[p], Uq[r]);
+          if (c < c2) dot_to(FU[3 * p + c2][voigt_slot(r, c)], Zu[r], Mq[p]);
+          // F^t_(p, c) with F^t_(r, c2); a pair within one slot counts twice
           if (c < c2 || p <= r) {
-            const T u = dot(Zu[p], Uq[r]);
             const int v = voigt_slot(p, c), x = voigt_slot(r, c2);
-            K[hm6(v, x)] += (v == x && !(p == r && c == c2)) ? u + u : u;
+            dot_to(K[hm6(v, x)], Zu[p], Uq[r]);
+            if (v == x && !(p == r && c == c2)) dot_to(K[hm6(v, x)], Zu[p], Uq[r]);
           }
         }
     }
   }
-  // second derivatives of F^e along F and F^t, and of J_t
+  // second derivatives of F^e along F and F^t, and of J_t: tr(A dU) P - A dU P^T
+  T At[6];
+#pragma unroll
+  for (int v = 0; v < 6; ++v) At[v] = v < 3 ? A[v] : A[v] + A[v];
 #pragma unroll
   for (int p = 0; p < 3; ++p)
 #pragma unroll
@@ -967,34 +975,34 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
 #pragma unroll
       for (int v = 0; v < 6; ++v) {
         const int i = sym_i(v), j = sym_j(v);
-        T s = A[v] * Pf[p][c];
-        if (v >= 3) s += s;
-        s -= symget(A, c, i) * Pf[p][j];
-        if (v >= 3) s -= symget(A, c, j) * Pf[p][i];
-        FU[3 * p + c][v] += s;
+        T& fu = FU[3 * p + c][v];
+        fu += At[v] * Pf[p][c];
+        fu -= symget(A, c, i) * Pf[p][j];
+        if (v >= 3) fu -= symget(A, c, j) * Pf[p][i];
       }
   // K += 2 tr(Z' dU A dU') - tr(A dU) tr(Z' dU') - tr(Z' dU) tr(A dU'), Z' = Zs - cW/2 A
   {
-    T Z[6], At[6], Zt[6];
+    T Z[6], Z2[6];
 #pragma unroll
     for (int v = 0; v < 6; ++v) {
       Z[v] = Zs[v] - T(0.5) * cW * A[v];
-      At[v] = v < 3 ? A[v] : A[v] + A[v];
-      Zt[v] = v < 3 ? Z[v] : Z[v] + Z[v];
+      Z2[v] = Z[v] + Z[v];
     }
 #pragma unroll
     for (int v = 0; v < 6; ++v)
 #pragma unroll
       for (int x = v; x < 6; ++x) {
         const int i = sym_i(v), j = sym_j(v), k = sym_i(x), l = sym_j(x);
-        // tr(Z E A E') over the entries (i,j), (j,i) of E and (k,l), (l,k) of E'
-        T s = symget(Z, l, i) * symget(A, j, k);
-        if (x >= 3) s += symget(Z, k, i) * symget(A, j, l);
+        T& kk = K[hm6(v, x)];
+        // tr(2 Z E A E') over the entries (i,j), (j,i) of E and (k,l), (l,k) of E'
+        kk += symget(Z2, l, i) * symget(A, j, k);
+        if (x >= 3) kk += symget(Z2, k, i) * symget(A, j, l);
         if (v >= 3) {
-          s += symget(Z, l, j) * symget(A, i, k);
-          if (x >= 3) s += symget(Z, k, j) * symget(A, i, l);
+          kk += symget(Z2, l, j) * symget(A, i, k);
+          if (x >= 3) kk += symget(Z2, k, j) * symget(A, i, l);
         }
-        K[hm6(v, x)] += s + s - (At[v] * Zt[x] + Zt[v] * At[x]);
+        kk -= At[v] * (x < 3 ? Z[x] : Z2[x]);
+        kk -= (v < 3 ? Z[v] : Z2[v]) * At[x];
       }
   }
   // per-phase stiffness: (dL_k h) along the directions, LX[k][v] for F^t
@@ -1059,9 +1067,8 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
       if (!P.same_L) {
         T ap = T(0), aq = T(0);  // tr(A dU_p), tr(A dU_q)
         for (int v = 0; v < 6; ++v) {
-          const T a2 = v < 3 ? A[v] : A[v] + A[v];
-          ap += a2 * T(P.dU[p][v]);
-          aq += a2 * T(P.dU[q][v]);
+          ap += At[v] * T(P.dU[p][v]);
+          aq += At[v] * T(P.dU[q][v]);
           s += LX[p][v] * T(P.dU[q][v]) + LX[q][v] * T(P.dU[p][v]);
         }
         s += T(0.5) * Jt * (ap * (hLh[q + 1] - hLh[0]) + aq * (hLh[p + 1] - hLh[0]));
