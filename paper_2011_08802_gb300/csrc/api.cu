@@ -1569,6 +1569,25 @@ pfm_status pfm_param_grad(pfm_handle* h, const double* w_dev, double* dPi, doubl
   Level& f = h->L[0];
   cudaStream_t s = h->stream;
   const int64_t n = ndof(f);
+  if (!dR_dev && !h->det) {
+    // sums only: one pass over the elements and one over the nodes
+    pfm_params q = p;
+    for (int ph = 0; ph < NPH; ++ph) q.F0[ph] = 0.0;
+    q.gamma_scale = 1.0;
+    DevParams d1;
+    make_dev_params(q, d1);
+    CK(cudaMemsetAsync(h->hdev, 0, sizeof(double) * 8, s));
+    launch_param_parts(f.g, h->dp, d1, f.U, f.mask, w_dev, h->hdev, s);
+    CKL();
+    double out[8];
+    CK(cudaMemcpyAsync(out, h->hdev, sizeof(out), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    for (int k = 0; k < 4; ++k) {
+      if (dPi) dPi[k] = out[k];
+      if (w_dev && wdR) wdR[k] = out[4 + k];
+    }
+    return PFM_OK;
+  }
   double* Rk = h->wv;  // work vector
   for (int k = 0; k < 4; ++k) {
     // the theta_k-part of the potential: unit C11 / C12 / C44 stiffness with

@@ -140,6 +140,11 @@ void count_launches(int n);
 void launch_residual(const Grid& g, const DevParams& P, const double* U, const double* Un,
                      const dmask_t* mask, double* R, double* energy, cudaStream_t s, double* W = nullptr,
                      bool df = false);
+// out[0..3] += dPi/dtheta_k and, with w, out[4..7] += w . dR/dtheta_k for theta =
+// (C11, C12, C44, gamma_scale) of a cubic stiffness shared by all phases; P1: the
+// parameters with only the interface terms, at gamma_scale = 1
+void launch_param_parts(const Grid& g, const DevParams& P, const DevParams& P1, const double* U, const dmask_t* mask,
+                        const double* w, double* out, cudaStream_t s);
 // arithmetic of the point physics in the linearisation
 enum { LIN_F64 = 0, LIN_F32 = 1, LIN_DF = 2 };
 // optional residual of the same state formed in the linearisation pass

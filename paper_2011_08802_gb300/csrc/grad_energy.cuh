@@ -111,6 +111,54 @@ struct GradESmem {
   TA L[NV][GE_Z][GE_COLS];
 };
 
+// The operator's values L and, up to the factor hx hy hz / 216, the mass matrix's
+// values M of one field x (at the column's first node) on the GE_Z nodes of the
+// column (i, j, k0).
+template <typename TA, typename TV>
+__device__ __forceinline__ void grad_energy_operator(const Grid& g, const typename GeArith<TA>::C& c, const TV* x, int i,
+                                                     int j, int k0, TA L[GE_Z], TA M[GE_Z]) {
+  using Ar = GeArith<TA>;
+  const int nxp = g.nx + 1;
+  const int64_t plane = int64_t(nxp) * (g.ny + 1);
+  const TA zero = TA(0.f);
+  const bool xm = i > 0, xp = i < g.nx, ym = j > 0, yp = j < g.ny;
+  const float ni = (xm ? 1.f : 0.f) + (xp ? 1.f : 0.f), nj = (ym ? 1.f : 0.f) + (yp ? 1.f : 0.f);
+  const TA cx = Ar::constant(c.cx), cy = Ar::constant(c.cy), cz = Ar::constant(c.cz);
+  TA mm0 = zero, q0 = zero, mm1 = zero, q1 = zero;  // planes k - 1 and k
+#pragma unroll
+  for (int p = -1; p <= GE_Z; ++p) {
+    TA mm2 = zero, q2 = zero;
+    const int k = k0 + p;
+    if (k >= 0 && k <= g.nz) {
+      // row: Mx = 2 n x + s, Kx = n x - s
+      const TV* xr = x + p * plane;
+      auto row = [&](const TV* a, TA& M, TA& K) {
+        const TA s = (xm ? Ar::load(a[-1]) : zero) + (xp ? Ar::load(a[1]) : zero);
+        const TA b = Ar::load(a[0]);
+        M = Ar::scaled(2.f * ni, b, s);
+        K = Ar::scaled(ni, b, -s);
+      };
+      TA M0, K0, Ma = zero, Ka = zero, Mb = zero, Kb = zero;
+      row(xr, M0, K0);
+      if (ym) row(xr - nxp, Ma, Ka);
+      if (yp) row(xr + nxp, Mb, Kb);
+      const TA sM = Ma + Mb, sK = Ka + Kb;
+      mm2 = Ar::scaled(2.f * nj, M0, sM);
+      q2 = cx * Ar::scaled(2.f * nj, K0, sK) + cy * Ar::scaled(nj, M0, -sM);
+    }
+    if (p >= 1) {
+      const int kz = k0 + p - 1;
+      const float n = (kz > 0 ? 1.f : 0.f) + (kz < g.nz ? 1.f : 0.f);
+      L[p - 1] = Ar::scaled(2.f * n, q1, q0 + q2) + cz * Ar::scaled(n, mm1, -(mm0 + mm2));
+      M[p - 1] = Ar::scaled(2.f * n, mm1, mm0 + mm2);
+    }
+    mm0 = mm1;
+    q0 = q1;
+    mm1 = mm2;
+    q1 = q2;
+  }
+}
+
 // Columns t0 .. t0 + 31 of grid g by one block (GE_COLS, NV); every thread of the
 // block calls it. Returns this thread's part of x . (operator x) / 2 (the gradient
 // energy) when `energy` is set.
@@ -132,44 +180,11 @@ __device__ __forceinline__ double grad_energy_block(const Grid& g, const typenam
   const int64_t nn = g.nn(), plane = int64_t(nxp) * nyp;
   const int64_t node0 = i + int64_t(nxp) * (j + int64_t(nyp) * k0);
   const int nk = !on ? 0 : (g.nz + 1 - k0 < GE_Z ? g.nz + 1 - k0 : GE_Z);
-  const TA zero = TA(0.f);
   if (on) {
-    const bool xm = i > 0, xp = i < g.nx, ym = j > 0, yp = j < g.ny;
-    const float ni = (xm ? 1.f : 0.f) + (xp ? 1.f : 0.f), nj = (ym ? 1.f : 0.f) + (yp ? 1.f : 0.f);
-    const TA cx = Ar::constant(c.cx), cy = Ar::constant(c.cy), cz = Ar::constant(c.cz);
-    const TV* x = v + (3 + l) * nn + node0;
-    TA mm0 = zero, q0 = zero, mm1 = zero, q1 = zero;  // planes k - 1 and k
+    TA L[GE_Z], M[GE_Z];
+    grad_energy_operator<TA>(g, c, v + (3 + l) * nn + node0, i, j, k0, L, M);
 #pragma unroll
-    for (int p = -1; p <= GE_Z; ++p) {
-      TA mm2 = zero, q2 = zero;
-      const int k = k0 + p;
-      if (k >= 0 && k <= g.nz) {
-        // row: Mx = 2 n x + s, Kx = n x - s
-        const TV* xr = x + p * plane;
-        auto row = [&](const TV* a, TA& M, TA& K) {
-          const TA s = (xm ? Ar::load(a[-1]) : zero) + (xp ? Ar::load(a[1]) : zero);
-          const TA b = Ar::load(a[0]);
-          M = Ar::scaled(2.f * ni, b, s);
-          K = Ar::scaled(ni, b, -s);
-        };
-        TA M0, K0, Ma = zero, Ka = zero, Mb = zero, Kb = zero;
-        row(xr, M0, K0);
-        if (ym) row(xr - nxp, Ma, Ka);
-        if (yp) row(xr + nxp, Mb, Kb);
-        const TA sM = Ma + Mb, sK = Ka + Kb;
-        mm2 = Ar::scaled(2.f * nj, M0, sM);
-        q2 = cx * Ar::scaled(2.f * nj, K0, sK) + cy * Ar::scaled(nj, M0, -sM);
-      }
-      if (p >= 1) {
-        const int kz = k0 + p - 1;
-        const float n = (kz > 0 ? 1.f : 0.f) + (kz < g.nz ? 1.f : 0.f);
-        sm.L[l][p - 1][col] = Ar::scaled(2.f * n, q1, q0 + q2) + cz * Ar::scaled(n, mm1, -(mm0 + mm2));
-      }
-      mm0 = mm1;
-      q0 = q1;
-      mm1 = mm2;
-      q1 = q2;
-    }
+    for (int z = 0; z < GE_Z; ++z) sm.L[l][z][col] = L[z];
   }
   __syncthreads();
   double en = 0.0;

@@ -557,6 +557,110 @@ PFM_HD T dd2_log(const T x[3], T f12, T f02, T f01) {
   return (f01 - f02) / (x[1] - x[2]);
 }
 
+// Kinematics of one Gauss point: A = (F^t)^-1 and J_t, M = F^e = F A, the
+// eigen-decomposition of C^e = M^T M (lam = 1 + x), the Hencky strain h at the
+// eigenvalues (halved log, or the Pade approximant) and the divided differences
+// of the function: f1 in the Voigt slots and, with F2, f2d[a] = f2(a,a,a),
+// f2p[n] = {f2(p,p,r), f2(p,r,r)} for the pair (p, r), p < r, without n, and
+// f2t = f2(0,1,2).
+template <typename T>
+struct Kinematics {
+  T A[6], Jt, M[3][3], x[3], lam[3], Q[3][3], h[3], f1[6];
+  T f2d[3], f2p[3][2], f2t;
+};
+template <bool F2, typename T>
+PFM_HD void kinematics(const DevParams& P, const T Fin[9], const T eh[NV], Kinematics<T>& kin) {
+  // transformation stretch F^t = U_0 + sum eta_hat_k dU_k, its inverse and determinant
+  {
+    T Ft[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      T s = eh[0] * T(P.dU[0][v]);
+#pragma unroll
+      for (int k = 1; k < NV; ++k) s += eh[k] * T(P.dU[k][v]);
+      Ft[v] = T(P.U0[v]) + s;  // one rounding near 1
+    }
+    kin.Jt = inv_sym6(Ft, kin.A);
+  }
+  T (&M)[3][3] = kin.M;
+  const T* A = kin.A;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      M[i][j] = Fin[3 * i] * symget(A, 0, j) + Fin[3 * i + 1] * symget(A, 1, j) + Fin[3 * i + 2] * symget(A, 2, j);
+  T (&x)[3] = kin.x;
+  T (&lam)[3] = kin.lam;
+  {
+    T E[6];  // C^e = M^T M
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      const int i = sym_i(v), j = sym_j(v);
+      E[v] = M[0][i] * M[0][j] + M[1][i] * M[1][j] + M[2][i] * M[2][j];
+    }
+    eig_sym6(E, x, kin.Q);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) lam[a] = T(1) + x[a];
+  }
+  T (&h)[3] = kin.h;
+  T (&f1)[6] = kin.f1;
+  T (&f2d)[3] = kin.f2d;
+  T (&f2p)[3][2] = kin.f2p;
+  T& f2t = kin.f2t;
+  f2t = T(0);
+  if (P.hencky == 0) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) f1[a] = T(1) / lam[a];
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+      const int p = n == 0 ? 1 : 0, r = n == 2 ? 1 : 2;
+      f1[3 + n] = dd_log<F2>(lam[p], lam[r], x[p] - x[r], f1[p], f1[r], &f2p[n][0], &f2p[n][1]);
+    }
+    // log at one eigenvalue, the others through the divided differences
+    const T l0 = x[0] * dd_log<false>(lam[0], T(1), x[0], T(0), T(0), (T*)nullptr, (T*)nullptr);
+    h[0] = T(0.5) * l0;
+    h[1] = T(0.5) * (l0 + (x[1] - x[0]) * f1[5]);
+    h[2] = T(0.5) * (l0 + (x[2] - x[0]) * f1[4]);
+    if (F2) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) f2d[a] = T(-0.5) * f1[a] * f1[a];
+      f2t = dd2_log(x, f1[3], f1[4], f1[5]);
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) h[a] = f2d[a] = f2p[a][0] = f2p[a][1] = T(0);
+#pragma unroll
+    for (int v = 0; v < 6; ++v) f1[v] = T(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (k < P.hencky) {
+        const T sk = T(P.pade_s[k]), wk = T(P.pade_w[k]);
+        T rp[3];  // 1 / p_k(lam_a)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          rp[a] = T(1) / (T(1) + sk * x[a]);
+          h[a] += T(0.5) * wk * x[a] * rp[a];
+        }
+#pragma unroll
+        for (int v = 0; v < 6; ++v) f1[v] += wk * rp[sym_i(v)] * rp[sym_j(v)];
+        if (F2) {
+          const T ws = wk * sk;
+#pragma unroll
+          for (int a = 0; a < 3; ++a) f2d[a] -= ws * rp[a] * rp[a] * rp[a];
+#pragma unroll
+          for (int n = 0; n < 3; ++n) {
+            const int p = n == 0 ? 1 : 0, r = n == 2 ? 1 : 2;
+            const T wpr = ws * rp[p] * rp[r];
+            f2p[n][0] -= wpr * rp[p];
+            f2p[n][1] -= wpr * rp[r];
+          }
+          f2t -= ws * rp[0] * rp[1] * rp[2];
+        }
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Local energy density with gradient and (optionally) packed Hessian.
 //
@@ -579,94 +683,18 @@ struct HessArray {
 template <typename T, typename Emit>
 PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T ehn[NV], T* W, T g[NZ],
                      const Emit& emit) {
-  // transformation stretch F^t = U_0 + sum eta_hat_k dU_k, its inverse and determinant
-  T A[6];
-  T Jt;
-  {
-    T Ft[6];
-#pragma unroll
-    for (int v = 0; v < 6; ++v) {
-      T s = eh[0] * T(P.dU[0][v]);
-#pragma unroll
-      for (int k = 1; k < NV; ++k) s += eh[k] * T(P.dU[k][v]);
-      Ft[v] = T(P.U0[v]) + s;  // one rounding near 1
-    }
-    Jt = inv_sym6(Ft, A);
-  }
-  T M[3][3];  // F^e = F A
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-      M[i][j] = Fin[3 * i] * symget(A, 0, j) + Fin[3 * i + 1] * symget(A, 1, j) + Fin[3 * i + 2] * symget(A, 2, j);
-  T x[3], lam[3], Q[3][3];  // eigenvalues lam = 1 + x
-  {
-    T E[6];  // C^e = M^T M
-#pragma unroll
-    for (int v = 0; v < 6; ++v) {
-      const int i = sym_i(v), j = sym_j(v);
-      E[v] = M[0][i] * M[0][j] + M[1][i] * M[1][j] + M[2][i] * M[2][j];
-    }
-    eig_sym6(E, x, Q);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) lam[a] = T(1) + x[a];
-  }
-  // h = log (exact mode) or the Pade approximant r_m at the eigenvalues (halved:
-  // the Hencky strain), and its divided differences: f1 in the Voigt slots,
-  // f2d[a] = f2(a,a,a), f2p[n] = {f2(p,p,r), f2(p,r,r)} for the pair (p, r), p < r,
-  // without n, and f2t = f2(0,1,2)
-  T h[3], f1[6], f2d[3], f2p[3][2], f2t = T(0);
-  if (P.hencky == 0) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) f1[a] = T(1) / lam[a];
-#pragma unroll
-    for (int n = 0; n < 3; ++n) {
-      const int p = n == 0 ? 1 : 0, r = n == 2 ? 1 : 2;
-      f1[3 + n] = dd_log<Emit::want>(lam[p], lam[r], x[p] - x[r], f1[p], f1[r], &f2p[n][0], &f2p[n][1]);
-    }
-    // log at one eigenvalue, the others through the divided differences
-    const T l0 = x[0] * dd_log<false>(lam[0], T(1), x[0], T(0), T(0), (T*)nullptr, (T*)nullptr);
-    h[0] = T(0.5) * l0;
-    h[1] = T(0.5) * (l0 + (x[1] - x[0]) * f1[5]);
-    h[2] = T(0.5) * (l0 + (x[2] - x[0]) * f1[4]);
-    if (Emit::want) {
-#pragma unroll
-      for (int a = 0; a < 3; ++a) f2d[a] = T(-0.5) * f1[a] * f1[a];
-      f2t = dd2_log(x, f1[3], f1[4], f1[5]);
-    }
-  } else {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) h[a] = f2d[a] = f2p[a][0] = f2p[a][1] = T(0);
-#pragma unroll
-    for (int v = 0; v < 6; ++v) f1[v] = T(0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      if (k < P.hencky) {
-        const T sk = T(P.pade_s[k]), wk = T(P.pade_w[k]);
-        T rp[3];  // 1 / p_k(lam_a)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          rp[a] = T(1) / (T(1) + sk * x[a]);
-          h[a] += T(0.5) * wk * x[a] * rp[a];
-        }
-#pragma unroll
-        for (int v = 0; v < 6; ++v) f1[v] += wk * rp[sym_i(v)] * rp[sym_j(v)];
-        if (Emit::want) {
-          const T ws = wk * sk;
-#pragma unroll
-          for (int a = 0; a < 3; ++a) f2d[a] -= ws * rp[a] * rp[a] * rp[a];
-#pragma unroll
-          for (int n = 0; n < 3; ++n) {
-            const int p = n == 0 ? 1 : 0, r = n == 2 ? 1 : 2;
-            const T wpr = ws * rp[p] * rp[r];
-            f2p[n][0] -= wpr * rp[p];
-            f2p[n][1] -= wpr * rp[r];
-          }
-          f2t -= ws * rp[0] * rp[1] * rp[2];
-        }
-      }
-    }
-  }
+  Kinematics<T> kin;
+  kinematics<Emit::want>(P, Fin, eh, kin);
+  const T (&A)[6] = kin.A;
+  const T Jt = kin.Jt;
+  const T (&M)[3][3] = kin.M;
+  const T (&lam)[3] = kin.lam;
+  const T (&Q)[3][3] = kin.Q;
+  const T (&h)[3] = kin.h;
+  const T (&f1)[6] = kin.f1;
+  const T (&f2d)[3] = kin.f2d;
+  const T (&f2p)[3][2] = kin.f2p;
+  const T f2t = kin.f2t;
 
   // products of the rows of Q: w[n][v] = Q_na Q_nb for the slot v = (a, b)
   T w[3][6];
@@ -1075,6 +1103,87 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
       }
       emit(hidx(9 + p, 9 + q), s + loc);
     }
+  }
+}
+
+// Parts of the elastic energy that belong to the cubic constants
+// theta = (C11, C12, C44) of a stiffness shared by all phases (the energy is
+// linear in them): E[k] = the energy density at unit theta_k with the others 0,
+// and D[k] = its derivative along a direction of the unknowns with the gradient
+// dF (row-major) of the displacements and the change dUt (Voigt entries) of F^t.
+// One set of kinematics serves the three parts. In the eigenbasis the unit
+// stiffnesses give the stresses sum_n c_n w_n w_n^T-wise for C11 (c = w h), the
+// trace minus that for C12, and 2 h minus twice that for C44.
+template <typename T>
+PFM_HD void qp_cubic_parts(const DevParams& P, const T Fin[9], const T eh[NV], const T dF[9], const T dUt[6], T E[3],
+                           T D[3]) {
+  Kinematics<T> kin;
+  kinematics<false>(P, Fin, eh, kin);
+  const T (&Q)[3][3] = kin.Q;
+  const T (&h)[3] = kin.h;
+  T cu[6];  // Voigt slots of sum_n (w_n . h) w_n
+#pragma unroll
+  for (int v = 0; v < 6; ++v) cu[v] = T(0);
+#pragma unroll
+  for (int n = 0; n < 3; ++n) {
+    T w[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) w[v] = Q[n][sym_i(v)] * Q[n][sym_j(v)];
+    const T c = w[0] * h[0] + w[1] * h[1] + w[2] * h[2];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) cu[v] += c * w[v];
+  }
+  const T tr = h[0] + h[1] + h[2];
+  T Aq[3][3], Mq[3][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      Aq[c][a] = symget(kin.A, c, 0) * Q[0][a] + symget(kin.A, c, 1) * Q[1][a] + symget(kin.A, c, 2) * Q[2][a];
+      Mq[c][a] = kin.M[c][0] * Q[0][a] + kin.M[c][1] * Q[1][a] + kin.M[c][2] * Q[2][a];
+    }
+  T trAdU = T(0);  // tr(A dF^t)
+#pragma unroll
+  for (int v = 0; v < 6; ++v) trAdU += (v < 3 ? kin.A[v] : kin.A[v] + kin.A[v]) * dUt[v];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    T TJ[6], S2[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      T t = k == 0 ? cu[v] : (k == 1 ? -cu[v] : T(-2) * cu[v]);
+      if (v < 3) {
+        if (k == 1) t += tr;
+        if (k == 2) t += T(2) * h[v];
+      }
+      TJ[v] = kin.Jt * t;
+      S2[v] = kin.f1[v] * TJ[v];
+    }
+    const T cW = T(0.5) * (h[0] * TJ[0] + h[1] * TJ[1] + h[2] * TJ[2]);
+    T Pf[3][3];
+    T d = T(0);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      T n[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        n[a] = Mq[p][0] * symget(S2, 0, a) + Mq[p][1] * symget(S2, 1, a) + Mq[p][2] * symget(S2, 2, a);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        Pf[p][c] = n[0] * Aq[c][0] + n[1] * Aq[c][1] + n[2] * Aq[c][2];
+        d += Pf[p][c] * dF[3 * p + c];
+      }
+    }
+    // along F^t: cW A - sym(M^T Pf)
+    d += cW * trAdU;
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      const int i = sym_i(v), j = sym_j(v);
+      T z = kin.M[0][i] * Pf[0][j] + kin.M[1][i] * Pf[1][j] + kin.M[2][i] * Pf[2][j];
+      if (v >= 3) z += kin.M[0][j] * Pf[0][i] + kin.M[1][j] * Pf[1][i] + kin.M[2][j] * Pf[2][i];
+      d -= z * dUt[v];
+    }
+    E[k] = cW;
+    D[k] = d;
   }
 }
 
