@@ -322,6 +322,9 @@ pfm_status estimate_lambda(pfm_handle* h, size_t l) {
   return PFM_OK;
 }
 
+template <typename T>
+pfm_status run_vcycle(pfm_handle* h, const SmoothCfg& sc);
+
 // z = M r with r, z in the preconditioner's precision (device arrays of the finest level).
 template <typename T>
 pfm_status apply_vcycle(pfm_handle* h, const T* r, T* z, const SmoothCfg& c) {
@@ -329,7 +332,7 @@ pfm_status apply_vcycle(pfm_handle* h, const T* r, T* z, const SmoothCfg& c) {
   TRY(ensure_level_vectors<T>(h));
   Level& f = h->L[0];
   CK(cudaMemcpyAsync(LvVec<T>::b(f), r, sizeof(T) * ndof(f), cudaMemcpyDeviceToDevice, h->stream));
-  TRY(vcycle_level<T>(h, 0, c));
+  TRY(run_vcycle<T>(h, c));
   CK(cudaMemcpyAsync(z, LvVec<T>::x(f), sizeof(T) * ndof(f), cudaMemcpyDeviceToDevice, h->stream));
   return PFM_OK;
 }
@@ -392,10 +395,8 @@ bool residual_fusable(const pfm_handle* h) { return !h->res_df && !h->lin_df; }
 // energy_dev), as residual_impl would.
 pfm_status linearize_impl(pfm_handle* h, pfm_precision prec, double* R_fused = nullptr) {
   cudaStream_t s = h->stream;
-  if (h->vgraph) {  // smoother coefficients change with the eigenvalue estimates
-    cudaGraphExecDestroy(h->vgraph);
-    h->vgraph = nullptr;
-  }
+  h->vgraph_stale = true;  // smoother coefficients change with the eigenvalue estimates
+  h->vcycles = 0;
   TRY(det_ready(h));
   const size_t nl = h->L.size();
   for (size_t l = 1; l < nl; ++l) {
@@ -624,7 +625,7 @@ pfm_status fgm_begin_finish(pfm_handle* h, Fgm& F) {
 }
 
 template <typename T>
-pfm_status capture_vcycle(pfm_handle* h, const SmoothCfg& sc);
+pfm_status run_vcycle(pfm_handle* h, const SmoothCfg& sc);
 pfm_status true_residual(pfm_handle* h, const double* b, const double* x, double* r);
 
 // z_j = M v_j, w = J z_j, two Gram-Schmidt passes and ||w||^2, with the
@@ -638,12 +639,7 @@ pfm_status fgm_enqueue(pfm_handle* h, Fgm& F) {
   if (F.mixed) {
     float* zj = static_cast<float*>(h->Z) + size_t(j) * n;
     launch_cast_d2f(n, vj, fl.b32, s);
-    if (h->use_graphs) {
-      TRY(capture_vcycle<float>(h, F.sc));
-      CK(cudaGraphLaunch(h->vgraph, s));
-    } else {
-      TRY(vcycle_level<float>(h, 0, F.sc));
-    }
+    TRY(run_vcycle<float>(h, F.sc));
     CK(cudaMemcpyAsync(zj, fl.x32, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
     // w = J z_j with the FP64-accurate operator: either the FP64 kernel or,
     // since z_j is exactly FP32, the double-float kernel on the FP32 pipes;
@@ -668,12 +664,7 @@ pfm_status fgm_enqueue(pfm_handle* h, Fgm& F) {
   } else {
     double* zj = static_cast<double*>(h->Z) + size_t(j) * n;
     CK(cudaMemcpyAsync(fl.b64, vj, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-    if (h->use_graphs) {
-      TRY(capture_vcycle<double>(h, F.sc));
-      CK(cudaGraphLaunch(h->vgraph, s));
-    } else {
-      TRY(vcycle_level<double>(h, 0, F.sc));
-    }
+    TRY(run_vcycle<double>(h, F.sc));
     CK(cudaMemcpyAsync(zj, fl.x64, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(h->zd, zj, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
   }
@@ -917,41 +908,82 @@ pfm_status linear_solve(pfm_handle* h, const pfm_solve_opts& o, const double* b,
   return fgmres_impl(h, o, b, x, its_out, relres_out, outer_out);
 }
 
-// Capture the V-cycle on the handle's stream into a CUDA graph (once per
-// linearisation and smoother configuration) so that a batch replays it with
-// one launch per problem and iteration.
+// Capture the V-cycle into a CUDA graph (once per linearisation and smoother
+// configuration; a graph of the same shape takes the new coefficients by an
+// update). A V-cycle is 200 to 300 launches of a few microseconds on its coarse
+// levels, so issuing them one by one left the GPU idle for up to a tenth of a
+// solve at 32^3.
 template <typename T>
 pfm_status capture_vcycle(pfm_handle* h, const SmoothCfg& sc) {
   const int key_prec = sizeof(T) == 4 ? 0 : 1;
-  if (h->vgraph && h->vgraph_prec == key_prec && h->vgraph_cfg.nu_pre == sc.nu_pre &&
+  if (h->vgraph && !h->vgraph_stale && h->vgraph_prec == key_prec && h->vgraph_cfg.nu_pre == sc.nu_pre &&
       h->vgraph_cfg.nu_post == sc.nu_post && h->vgraph_cfg.type == sc.type && h->vgraph_cfg.omega == sc.omega &&
       h->vgraph_cfg.lo == sc.lo && h->vgraph_cfg.hi == sc.hi && h->vgraph_cfg.gamma == sc.gamma &&
       h->vgraph_cfg.growth == sc.growth && h->vgraph_cfg.det == h->det)
     return PFM_OK;
-  if (h->vgraph) {
-    cudaGraphExecDestroy(h->vgraph);
-    h->vgraph = nullptr;
-  }
+  if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   const bool prof = h->prof;
+  const cudaStream_t stream = h->stream;
   h->prof = false;
-  CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-  pfm_status st = vcycle_level<T>(h, 0, sc);
+  h->stream = h->cap_stream;
+  cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
+  pfm_status st = PFM_OK;
   cudaGraph_t graph = nullptr;
-  cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
+  const int64_t c0 = g_launches.load(std::memory_order_relaxed);
+  int64_t count = 0;
+  if (e == cudaSuccess) {
+    st = vcycle_level<T>(h, 0, sc);
+    count = g_launches.load(std::memory_order_relaxed) - c0;
+    g_launches.fetch_sub(count, std::memory_order_relaxed);  // counted at every replay
+    e = cudaStreamEndCapture(h->stream, &graph);
+  }
   h->prof = prof;
+  h->stream = stream;
   if (st != PFM_OK) {
     if (graph) cudaGraphDestroy(graph);
     return st;
   }
   if (e != cudaSuccess) return h->fail(PFM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-  e = cudaGraphInstantiate(&h->vgraph, graph, 0);
+  if (h->vgraph) {
+    cudaGraphExecUpdateResultInfo info{};
+    if (cudaGraphExecUpdate(h->vgraph, graph, &info) != cudaSuccess) {  // another shape: a new executable
+      cudaGetLastError();
+      cudaGraphExecDestroy(h->vgraph);
+      h->vgraph = nullptr;
+    }
+  }
+  if (!h->vgraph) e = cudaGraphInstantiate(&h->vgraph, graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) {
     h->vgraph = nullptr;
     return h->fail(PFM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
   }
+  h->vgraph_stale = false;
+  h->vgraph_launches = count;
   h->vgraph_prec = key_prec;
   h->vgraph_cfg = {sc.nu_pre, sc.nu_post, sc.type, sc.omega, sc.lo, sc.hi, sc.gamma, sc.growth, h->det};
+  return PFM_OK;
+}
+
+// One V-cycle on the finest level's vectors b -> x: the first one after a
+// linearisation is issued launch by launch (it may tune launch shapes, and a
+// single V-cycle would not repay a capture), the later ones replay the graph.
+// Not while the caller captures the stream or the phases are being timed.
+template <typename T>
+pfm_status run_vcycle(pfm_handle* h, const SmoothCfg& sc) {
+  bool graph = h->use_graphs || (h->vcycles > 0 && !h->prof);
+  if (graph && !h->use_graphs) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      graph = false;
+    }
+  }
+  ++h->vcycles;
+  if (!graph) return vcycle_level<T>(h, 0, sc);
+  TRY(capture_vcycle<T>(h, sc));
+  CK(cudaGraphLaunch(h->vgraph, h->stream));
+  count_launches(int(h->vgraph_launches));
   return PFM_OK;
 }
 
@@ -1155,6 +1187,7 @@ void pfm_destroy(pfm_handle* h) {
   dfree(h->gj_used); dfree(h->gj_piv); dfree(h->amax_dev);
   if (h->Z) cudaFree(h->Z);
   if (h->vgraph) cudaGraphExecDestroy(h->vgraph);
+  if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   if (h->hpin) cudaFreeHost(h->hpin);
   if (h->pipe_in) {
     cudaStreamDestroy(h->pipe_in);

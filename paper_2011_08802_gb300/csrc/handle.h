@@ -128,9 +128,14 @@ struct pfm_handle {
   unsigned* amax_dev = nullptr;  // one word for the store's max |entry|
   // pinned host slots for Hessenberg columns and scalars
   double* hpin = nullptr;
-  // captured V-cycle (valid until the next linearisation)
-  bool use_graphs = false;
+  // captured V-cycle: replayed while the linearisation and the options stay the
+  // same; after a linearisation (vgraph_stale) its node parameters are updated
+  bool use_graphs = false;           // replay from the first V-cycle on
   cudaGraphExec_t vgraph = nullptr;
+  bool vgraph_stale = false;
+  int64_t vgraph_launches = 0;       // kernels per replay
+  int vcycles = 0;                   // V-cycles issued since the linearisation
+  cudaStream_t cap_stream = nullptr; // capture runs here (the legacy default stream cannot be captured)
   int vgraph_prec = -1;
   struct { int nu_pre, nu_post, type; double omega, lo, hi; int gamma; double growth; bool det; } vgraph_cfg{};
   // device timing of hot phases (pairs of events per timed launch)
