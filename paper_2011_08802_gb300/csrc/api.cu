@@ -295,21 +295,17 @@ pfm_status estimate_lambda(pfm_handle* h, size_t l) {
   launch_power_init<T>(lv.nn, lv.mask, q, s);
   launch_dinv<T>(lv.nn, D, q, z, s);
   launch_dot<T>(n, q, z, h->partial, nrm, s);
-  launch_scale_inv_sqrt<T>(n, q, nrm, q, s);
-  launch_scale_inv_sqrt<T>(n, z, nrm, z, s);
+  launch_scale2_inv_sqrt<T>(n, q, z, nrm, q, z, s);
   CK(cudaMemsetAsync(qp, 0, sizeof(T) * n, s));
   CKL_AT("eigenvalue estimate start");
   for (int j = 0; j < K; ++j) {
     precond_apply<T>(h, l, z, u, false);
     CKL_AT("eigenvalue estimate: tangent application");
     launch_dot<T>(n, z, u, h->partial, al + j, s);
-    launch_lanczos_orth<T>(n, u, q, qp, al + j, j > 0 ? be + j - 1 : nullptr, s);
-    launch_dinv<T>(lv.nn, D, u, w, s);
-    launch_dot<T>(n, u, w, h->partial, be + j, s);
+    launch_lanczos_step<T>(lv.nn, D, u, q, qp, al + j, j > 0 ? be + j - 1 : nullptr, w, h->partial, be + j, s);
     if (j + 1 < K) {
       std::swap(q, qp);
-      launch_scale_inv_sqrt<T>(n, u, be + j, q, s);
-      launch_scale_inv_sqrt<T>(n, w, be + j, z, s);
+      launch_scale2_inv_sqrt<T>(n, u, w, be + j, q, z, s);
     }
     CKL_AT("eigenvalue estimate");
   }

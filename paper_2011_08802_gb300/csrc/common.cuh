@@ -226,12 +226,13 @@ void launch_dinv(int64_t nn, const T* D, const T* src, T* dst, cudaStream_t s); 
 template <typename T>
 void launch_power_init(int64_t nn, const dmask_t* mask, T* x, cudaStream_t s);
 template <typename T>
-void launch_scale_inv_sqrt(int64_t n, const T* y, const double* dot, T* x, cudaStream_t s);
+void launch_scale2_inv_sqrt(int64_t n, const T* a, const T* b, const double* dot, T* xa, T* xb, cudaStream_t s);
 // Lanczos step: u -= alpha q + sqrt(beta2prev) qp (alpha, beta2prev: device
-// scalars; beta2prev null for the first step)
+// scalars; beta2prev null for the first step), w = D^-1 u, *out = u . w
+// (partial: min(ceil(nn / 256), 1024) doubles of work)
 template <typename T>
-void launch_lanczos_orth(int64_t n, T* u, const T* q, const T* qp, const double* alpha, const double* beta2prev,
-                         cudaStream_t s);
+void launch_lanczos_step(int64_t nn, const T* D, T* u, const T* q, const T* qp, const double* alpha,
+                         const double* beta2prev, T* w, double* partial, double* out, cudaStream_t s);
 void launch_coarse_inverse(double* M, int n, double* Ainv, int* used, int* piv, int* singular, cudaStream_t s);
 template <typename T>
 void launch_coarse_solve(int n, const double* Ainv, const T* b, T* x, cudaStream_t s);
@@ -270,6 +271,7 @@ void launch_mdot(int64_t n, int k, const double* V, int64_t ldv, const double* w
                  double* out, cudaStream_t s);
 template <typename T>
 void launch_dot(int64_t n, const T* a, const T* b, double* partial, double* out, cudaStream_t s);
+void launch_sum_partials(int nb, const double* partial, double* out, cudaStream_t s);
 void launch_maxpy(int64_t n, int k, const double* V, int64_t ldv, const double* h, double* w,
                   cudaStream_t s);
 void launch_scale_copy(int64_t n, const double* a, const double* alpha_dev, double* b,

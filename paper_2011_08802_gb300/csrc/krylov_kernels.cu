@@ -247,6 +247,11 @@ void launch_dot(int64_t n, const T* a, const T* b, double* partial, double* out,
   k_mdot_final<<<1, RED_THREADS, 0, s>>>(nb, 1, partial, 1, out);
   count_launches(1);
 }
+// *out = sum of nb block partials in a fixed order
+void launch_sum_partials(int nb, const double* partial, double* out, cudaStream_t s) {
+  k_mdot_final<<<1, RED_THREADS, 0, s>>>(nb, 1, partial, 1, out);
+  count_launches(1);
+}
 template void launch_dot<float>(int64_t, const float*, const float*, double*, double*, cudaStream_t);
 template void launch_dot<double>(int64_t, const double*, const double*, double*, double*, cudaStream_t);
 

@@ -8,6 +8,7 @@
 // i*nc = I0*nf + rem, its interpolation weights are (1 - rem/nf) on coarse
 // node I0 and rem/nf on I0+1. All index arithmetic is integer, so P and
 // R = P^T use identical weights on nested (nf = 2 nc) and non-nested grids.
+#include <algorithm>
 #include <type_traits>
 
 #include "coarse_inverse.cuh"
@@ -282,20 +283,28 @@ __global__ void k_power_init(int64_t nn, const dmask_t* __restrict__ mask, T* __
     x[i] = T(power_init_value(i, nn, mask));
 }
 
-// x = y / sqrt(*dot)
+// xa = a / sqrt(*dot), xb = b / sqrt(*dot)
 template <typename T>
-__global__ void k_scale_inv_sqrt(int64_t n, const T* __restrict__ y, const double* __restrict__ dot, T* __restrict__ x) {
+__global__ void k_scale2_inv_sqrt(int64_t n, const T* a, const T* b, const double* __restrict__ dot, T* xa, T* xb) {
   __shared__ T s;  // one FP64 square root and division per block, not per thread
   if (threadIdx.x == 0) s = T(1.0 / sqrt(*dot));
   __syncthreads();
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    x[i] = y[i] * s;
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+    xa[i] = a[i] * s;
+    xb[i] = b[i] * s;
+  }
 }
 
-// u -= alpha q + sqrt(beta2prev) qp (one Lanczos three-term step)
+// One Lanczos three-term step with the smoother's blocks: u -= alpha q +
+// sqrt(beta2prev) qp, w = D^-1 u, and the block's part of u . w (FP64). One pass
+// over the nodes and one launch for what took three (the vectors of a coarse
+// level take a few microseconds each, so the launches count).
 template <typename T>
-__global__ void k_lanczos_orth(int64_t n, T* __restrict__ u, const T* __restrict__ q, const T* __restrict__ qp,
-                               const double* __restrict__ alpha, const double* __restrict__ beta2prev) {
+__global__ void __launch_bounds__(256) k_lanczos_step(int64_t nn, const T* __restrict__ D, T* __restrict__ u,
+                                                      const T* __restrict__ q, const T* __restrict__ qp,
+                                                      const double* __restrict__ alpha,
+                                                      const double* __restrict__ beta2prev, T* __restrict__ w,
+                                                      double* __restrict__ partial) {
   __shared__ T ab[2];  // one FP64 square root per block, not per thread
   if (threadIdx.x == 0) {
     ab[0] = T(*alpha);
@@ -303,17 +312,45 @@ __global__ void k_lanczos_orth(int64_t n, T* __restrict__ u, const T* __restrict
   }
   __syncthreads();
   const T a = ab[0], b = ab[1];
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    u[i] -= a * q[i] + (beta2prev ? b * qp[i] : T(0));
+  double acc = 0.0;
+  for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn;
+       node += int64_t(gridDim.x) * blockDim.x) {
+    T r[NF], z[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const int64_t i = f * nn + node;
+      r[f] = u[i] - (a * q[i] + (beta2prev ? b * qp[i] : T(0)));
+      u[i] = r[f];
+    }
+    dinv_node<T>(nn, D, r, z, node);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      w[f * nn + node] = z[f];
+      acc += double(r[f]) * double(z[f]);
+    }
+  }
+  __shared__ double red[8];
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int m = 0; m < 8; ++m) t += red[m];
+    partial[blockIdx.x] = t;
+  }
 }
 
 }  // namespace
 
 template <typename T>
-void launch_lanczos_orth(int64_t n, T* u, const T* q, const T* qp, const double* alpha, const double* beta2prev,
-                         cudaStream_t s) {
-  k_lanczos_orth<T><<<grid_for(n, 256), 256, 0, s>>>(n, u, q, qp, alpha, beta2prev);
+void launch_lanczos_step(int64_t nn, const T* D, T* u, const T* q, const T* qp, const double* alpha,
+                         const double* beta2prev, T* w, double* partial, double* out, cudaStream_t s) {
+  // at most 1024 partials, as many as fit the dot products' work array
+  const int nb = int(std::min<int64_t>((nn + 255) / 256, 1024));
+  k_lanczos_step<T><<<nb, 256, 0, s>>>(nn, D, u, q, qp, alpha, beta2prev, w, partial);
   count_launches(1);
+  launch_sum_partials(nb, partial, out, s);
 }
 
 template <typename T>
@@ -343,8 +380,8 @@ void launch_power_init(int64_t nn, const dmask_t* mask, T* x, cudaStream_t s) {
 }
 
 template <typename T>
-void launch_scale_inv_sqrt(int64_t n, const T* y, const double* dot, T* x, cudaStream_t s) {
-  k_scale_inv_sqrt<T><<<grid_for(n, 256), 256, 0, s>>>(n, y, dot, x);
+void launch_scale2_inv_sqrt(int64_t n, const T* a, const T* b, const double* dot, T* xa, T* xb, cudaStream_t s) {
+  k_scale2_inv_sqrt<T><<<grid_for(n, 256), 256, 0, s>>>(n, a, b, dot, xa, xb);
   count_launches(1);
 }
 
@@ -473,9 +510,9 @@ void launch_coarse_solve(int n, const double* Ainv, const T* b, T* x, cudaStream
                                     cudaStream_t);                                              \
   template void launch_dinv<T>(int64_t, const T*, const T*, T*, cudaStream_t);                  \
   template void launch_power_init<T>(int64_t, const dmask_t*, T*, cudaStream_t);                  \
-  template void launch_scale_inv_sqrt<T>(int64_t, const T*, const double*, T*, cudaStream_t);     \
-  template void launch_lanczos_orth<T>(int64_t, T*, const T*, const T*, const double*, const double*, \
-                                       cudaStream_t);
+  template void launch_scale2_inv_sqrt<T>(int64_t, const T*, const T*, const double*, T*, T*, cudaStream_t); \
+  template void launch_lanczos_step<T>(int64_t, const T*, T*, const T*, const T*, const double*,  \
+                                       const double*, T*, double*, double*, cudaStream_t);
 PFM_INST(float)
 PFM_INST(double)
 #undef PFM_INST
