@@ -155,9 +155,11 @@ SmoothCfg smooth_cfg(const pfm_solve_opts* o) {
 }
 
 // nu steps on level l from x = 0 (zero_x) or from the current x; with
-// want_res the final residual b - J x is left in the level's r vector.
+// want_res the final residual b - J x is left as the difference r - y of two of
+// the level's vectors (y null in *res_y: r alone), which the restriction takes.
 template <typename T>
-pfm_status smooth(pfm_handle* h, size_t l, bool zero_x, int nu, bool want_res, const SmoothCfg& c) {
+pfm_status smooth(pfm_handle* h, size_t l, bool zero_x, int nu, bool want_res, const SmoothCfg& c,
+                  const T** res_y = nullptr) {
   Level& lv = h->L[l];
   cudaStream_t s = h->stream;
   T* x = LvVec<T>::x(lv);
@@ -182,6 +184,7 @@ pfm_status smooth(pfm_handle* h, size_t l, bool zero_x, int nu, bool want_res, c
     if (want_res) {
       precond_apply<T>(h, l, x, y);
       launch_sub<T>(n, b, y, r, s);
+      *res_y = nullptr;
     }
     CKL();
     return PFM_OK;
@@ -208,7 +211,7 @@ pfm_status smooth(pfm_handle* h, size_t l, bool zero_x, int nu, bool want_res, c
   }
   if (want_res) {
     precond_apply<T>(h, l, d, y, true, rows);
-    launch_sub<T>(n, r, y, r, s);
+    *res_y = y;
   }
   CKL();
   return PFM_OK;
@@ -231,15 +234,17 @@ pfm_status vcycle_level(pfm_handle* h, size_t l, const SmoothCfg& c) {
   const double gl = std::pow(c.growth, double(l));
   const int nu_pre = std::max(1, int(std::lround(c.nu_pre * gl)));
   const int nu_post = c.nu_post > 0 ? std::max(1, int(std::lround(c.nu_post * gl))) : 0;
-  TRY(smooth<T>(h, l, true, nu_pre, true, c));
+  const T* res_y = nullptr;
+  TRY(smooth<T>(h, l, true, nu_pre, true, c, &res_y));
   Level& cv = h->L[l + 1];
   for (int g = 0; g < c.gamma; ++g) {
     // coarse correction of the current residual r (recomputed after the first one)
     if (g > 0) {
       precond_apply<T>(h, l, x, LvVec<T>::y(lv));
       launch_sub<T>(ndof(lv), b, LvVec<T>::y(lv), LvVec<T>::r(lv), s);
+      res_y = nullptr;
     }
-    launch_restrict<T>(lv.g, cv.g, LvVec<T>::r(lv), cv.mask, LvVec<T>::b(cv), s);
+    launch_restrict<T>(lv.g, cv.g, LvVec<T>::r(lv), res_y, cv.mask, LvVec<T>::b(cv), s);
     CKL();
     TRY(vcycle_level<T>(h, l + 1, c));
     launch_prolong_add<T>(lv.g, cv.g, LvVec<T>::x(cv), lv.mask, x, s);

@@ -201,8 +201,9 @@ void launch_coarse_mask(const Grid& fine, const Grid& coarse, const dmask_t* mf,
 template <typename T>
 void launch_prolong_add(const Grid& fine, const Grid& coarse, const T* xc, const dmask_t* mf, T* xf,
                         cudaStream_t s);
+// rc = P^T (rf - y), y optional
 template <typename T>
-void launch_restrict(const Grid& fine, const Grid& coarse, const T* rf, const dmask_t* mc, T* rc,
+void launch_restrict(const Grid& fine, const Grid& coarse, const T* rf, const T* y, const dmask_t* mc, T* rc,
                      cudaStream_t s);
 template <typename T>
 void launch_smooth(int64_t nn, const T* D, const T* b, const T* y, T omega, T* x, cudaStream_t s);

@@ -96,12 +96,14 @@ __host__ __device__ __forceinline__ void prolong_node(const Grid& f, const Grid&
   }
 }
 
-// Coarse node idx: rc = (P^T rf) there, zero at its Dirichlet DOFs. Coarse
+// Coarse node idx: rc = (P^T (rf - y)) there (y null: P^T rf), zero at its
+// Dirichlet DOFs. Coarse
 // node I collects fine nodes i with |i*nc - I*nf| < nf, weight
 // 1 - |i*nc - I*nf|/nf (per axis).
 template <typename T>
 __host__ __device__ __forceinline__ void restrict_node(const Grid& f, const Grid& c, const T* __restrict__ rf,
-                                              const dmask_t* __restrict__ mc, T* __restrict__ rc, int64_t idx) {
+                                              const dmask_t* __restrict__ mc, T* __restrict__ rc, int64_t idx,
+                                              const T* __restrict__ y = nullptr) {
   const int64_t nnf = f.nn();
   const int64_t nnc = c.nn();
   const int Ic[3] = {int(idx % (c.nx + 1)), int((idx / (c.nx + 1)) % (c.ny + 1)),
@@ -141,7 +143,7 @@ __host__ __device__ __forceinline__ void restrict_node(const Grid& f, const Grid
         const int m = i - lo[0];
         const double w = (m < WX ? wxa[m & (WX - 1)] : weight(0, i)) * wyz;
         const int64_t fn = i + int64_t(f.nx + 1) * (j + int64_t(f.ny + 1) * k);
-        for (int fld = 0; fld < NF; ++fld) acc[fld] += w * double(rf[fld * nnf + fn]);
+        for (int fld = 0; fld < NF; ++fld) acc[fld] += w * double(y ? rf[fld * nnf + fn] - y[fld * nnf + fn] : rf[fld * nnf + fn]);
       }
     }
   }
@@ -224,9 +226,9 @@ __host__ __device__ __forceinline__ float prolong_value_int(const Grid& f, const
   return a.over(float(transfer_denominator(f)));
 }
 
-// (P^T r)(I, J, K) of the fine field r.
+// (P^T (r - y))(I, J, K) of the fine fields r and y (y null: P^T r).
 __host__ __device__ __forceinline__ float restrict_value_int(const Grid& f, const Grid& c, const float* __restrict__ r,
-                                                             int I, int J, int K) {
+                                                             const float* __restrict__ y, int I, int J, int K) {
   const int Ic[3] = {I, J, K}, nf[3] = {f.nx, f.ny, f.nz}, nc[3] = {c.nx, c.ny, c.nz};
   int lo[3], hi[3];
 #pragma unroll
@@ -247,9 +249,10 @@ __host__ __device__ __forceinline__ float restrict_value_int(const Grid& f, cons
     const int wz = weight(2, k);
     for (int j = lo[1]; j <= hi[1]; ++j) {
       const int wyz = weight(1, j) * wz;
-      const float* row = r + j * sy + k * sz;
+      const int64_t row = j * sy + k * sz;
 #pragma unroll 4
-      for (int i = lo[0]; i <= hi[0]; ++i) a.add(float(weight(0, i) * wyz), row[i]);
+      for (int i = lo[0]; i <= hi[0]; ++i)
+        a.add(float(weight(0, i) * wyz), y ? r[row + i] - y[row + i] : r[row + i]);
     }
   }
   return a.over(float(transfer_denominator(f)));
@@ -269,7 +272,7 @@ __host__ __device__ __forceinline__ void prolong_entry_int(const Grid& f, const 
 }
 __host__ __device__ __forceinline__ void restrict_entry_int(const Grid& f, const Grid& c, const float* __restrict__ rf,
                                                             const dmask_t* __restrict__ mc, float* __restrict__ rc,
-                                                            int64_t idx) {
+                                                            int64_t idx, const float* __restrict__ y = nullptr) {
   const int64_t nnc = c.nn();
   const int fld = int(idx / nnc);
   const int64_t node = idx - fld * nnc;
@@ -277,7 +280,8 @@ __host__ __device__ __forceinline__ void restrict_entry_int(const Grid& f, const
   const int64_t r = node / nxp;
   rc[idx] = ((mc[node] >> fld) & 1)
                 ? 0.f
-                : restrict_value_int(f, c, rf + fld * f.nn(), int(node - r * nxp), int(r % nyp), int(r / nyp));
+                : restrict_value_int(f, c, rf + fld * f.nn(), y ? y + fld * f.nn() : nullptr, int(node - r * nxp),
+                                     int(r % nyp), int(r / nyp));
 }
 
 // Nested grids (nf = 2 nc on every axis), the case of every level of a
@@ -346,6 +350,46 @@ __host__ __device__ __forceinline__ void restrict_node_nested(const Grid& f, con
     }
     rc[fld * nnc + idx] = acc;
   }
+}
+
+// One (node, field) of the nested transfers, for one thread each. Prolongation
+// averages the coarse values at floor and ceil of half the index on every axis
+// (the same one twice at an even index: (a + a) / 2 = a exactly), so lanes at
+// odd and even nodes run the same instructions.
+template <typename T>
+__host__ __device__ __forceinline__ T prolong_value_nested(const T* __restrict__ X, int64_t sy, int64_t sz, int i, int j,
+                                                           int k) {
+  const int i0 = i >> 1, i1 = (i + 1) >> 1;
+  const int64_t r0 = (j >> 1) * sy, r1 = ((j + 1) >> 1) * sy, p0 = (k >> 1) * sz, p1 = ((k + 1) >> 1) * sz;
+  const T a = (X[p0 + r0 + i0] + X[p0 + r0 + i1]) + (X[p0 + r1 + i0] + X[p0 + r1 + i1]);
+  const T b = (X[p1 + r0 + i0] + X[p1 + r0 + i1]) + (X[p1 + r1 + i0] + X[p1 + r1 + i1]);
+  return T(0.125) * (a + b);
+}
+// P^T (r - y) at coarse node (I, J, K) of one field (y null: P^T r).
+template <typename T>
+__host__ __device__ __forceinline__ T restrict_value_nested(const Grid& f, const T* __restrict__ r,
+                                                            const T* __restrict__ y, int I, int J, int K) {
+  const int64_t sy = f.nx + 1, sz = int64_t(f.nx + 1) * (f.ny + 1);
+  T acc = T(0);
+#pragma unroll
+  for (int dk = -1; dk <= 1; ++dk) {
+    const int k = 2 * K + dk;
+    if (k < 0 || k > f.nz) continue;
+    T sj = T(0);
+#pragma unroll
+    for (int dj = -1; dj <= 1; ++dj) {
+      const int j = 2 * J + dj;
+      if (j < 0 || j > f.ny) continue;
+      const int64_t o = j * sy + k * sz + 2 * I;
+      auto at = [&](int64_t m) { return y ? r[m] - y[m] : r[m]; };
+      T si = at(o);
+      if (I > 0) si += T(0.5) * at(o - 1);
+      if (2 * I + 1 <= f.nx) si += T(0.5) * at(o + 1);
+      sj += (dj ? T(0.5) : T(1)) * si;
+    }
+    acc += (dk ? T(0.5) : T(1)) * sj;
+  }
+  return acc;
 }
 
 inline __host__ __device__ bool nested(const Grid& f, const Grid& c) {
