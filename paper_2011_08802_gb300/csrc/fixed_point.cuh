@@ -1,0 +1,115 @@
+// Fixed-point contraction of FP64 numbers with integer multiply-adds.
+//
+// The FP64 pipe does 1.8 multiply-adds per clock and SM, the integer pipe tens of
+// 32 x 32 -> 64 bit ones, and a symmetric contraction sigma = H x over the
+// unknowns of a Gauss point needs no exponents of its own once every number is
+// taken relative to a power of two:
+//   H_rc = 2^(a_r + a_c) h_rc,  x_c = 2^(Z - a_c) y_c,  |h|, |y| < 1,
+//   sigma_r = 2^(a_r + Z) sum_c h_rc y_c,
+// with one exponent a for the unknowns of F and one for the order parameters
+// (per point, from the largest entries of the three parts of H) and one Z per
+// point. h and y are 58-bit integers in two limbs of 29 bits with their sign; the
+// three leading limb products are summed exactly (sums below 2^62), the fourth is
+// below 2^-58 of the largest product. Truncation leaves about 2^-57 of 2^(a_r + Z)
+// per row, against 2^-53 of the partial sums per multiply-add in FP64.
+// Compiles for the host too (test of the arithmetic).
+#pragma once
+
+#include <cstdint>
+#include <cstring>
+
+namespace pfm {
+
+#ifdef __CUDACC__
+#define PFM_FX __host__ __device__ __forceinline__
+#else
+#define PFM_FX inline
+#endif
+
+PFM_FX uint64_t fx_bits(double v) {
+#ifdef __CUDA_ARCH__
+  return static_cast<uint64_t>(__double_as_longlong(v));
+#else
+  uint64_t u;
+  std::memcpy(&u, &v, sizeof u);
+  return u;
+#endif
+}
+PFM_FX double fx_from_bits(uint64_t u) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double(static_cast<long long>(u));
+#else
+  double v;
+  std::memcpy(&v, &u, sizeof v);
+  return v;
+#endif
+}
+PFM_FX int fx_clz(uint64_t a) {
+#ifdef __CUDA_ARCH__
+  return __clzll(static_cast<long long>(a));
+#else
+  return a ? __builtin_clzll(a) : 64;
+#endif
+}
+
+// high word of |v|: orders as |v| up to its low word; exponent e = top >> 20 with
+// |v| < 2^(e - 1022) (e = 0: zero or below the normal numbers, read as zero)
+PFM_FX unsigned fx_top(double v) { return unsigned(fx_bits(v) >> 32) & 0x7fffffffu; }
+
+// Scales of a point's Hessian, a_F in the high and a_e in the low 16 bits, from
+// the largest fx_top of its parts (F, F), (F, eta), (eta, eta); FX_NONE when an
+// entry is not finite or a scale is outside +-FX_RANGE.
+constexpr int FX_NONE = -2147483647 - 1;
+constexpr int FX_RANGE = 400;
+PFM_FX int fx_hess_scales(const unsigned top[3]) {
+  const int e0 = int(top[0] >> 20), e1 = int(top[1] >> 20), e2 = int(top[2] >> 20);
+  if (e0 == 0x7ff || e1 == 0x7ff || e2 == 0x7ff) return FX_NONE;
+  if (e0 == 0 && e1 == 0 && e2 == 0) return 0;
+  const int aF = e0 ? (e0 - 1021) >> 1 : -FX_RANGE;
+  int ae = e2 ? (e2 - 1021) >> 1 : -FX_RANGE;
+  if (e1 && e1 - 1022 - aF > ae) ae = e1 - 1022 - aF;
+  if (aF < -FX_RANGE || aF > FX_RANGE || ae < -FX_RANGE || ae > FX_RANGE) return FX_NONE;
+  return int((unsigned(aF) << 16) | (unsigned(ae) & 0xffffu));
+}
+PFM_FX int fx_scale_F(int hx) { return hx >> 16; }
+PFM_FX int fx_scale_eta(int hx) { return int(int16_t(uint16_t(unsigned(hx) & 0xffffu))); }
+
+// Z of the input from the largest fx_top of its two parts; false when the
+// contraction does not take the point (then it goes through FP64).
+PFM_FX bool fx_input_scale(int hx, unsigned topF, unsigned tope, int& Z) {
+  const int eF = int(topF >> 20), ee = int(tope >> 20);
+  const int zF = eF ? eF - 1022 + fx_scale_F(hx) : -3 * FX_RANGE;
+  const int ze = ee ? ee - 1022 + fx_scale_eta(hx) : -3 * FX_RANGE;
+  Z = eF == 0 && ee == 0 ? 0 : (zF > ze ? zF : ze);
+  return hx != FX_NONE && eF != 0x7ff && ee != 0x7ff && Z >= -FX_RANGE && Z <= FX_RANGE;
+}
+
+// Limbs of v 2^-E as a 58-bit fraction, k = 1027 + E (truncated towards zero).
+PFM_FX void fx_limbs(double v, int k, int& x1, int& x0) {
+  const uint64_t u = fx_bits(v);
+  const unsigned hi = unsigned(u >> 32), lo = unsigned(u);
+  int r = k - int((hi >> 20) & 0x7ffu);  // >= 5: the mantissa's leading bit moves from bit 62 below bit 58
+  r = r < 63 ? r : 63;
+  const uint64_t w = ((uint64_t((hi & 0xfffffu) | 0x100000u) << 42) | (uint64_t(lo) << 10)) >> r;
+  const int sg = (int(hi) >> 31) | 1;
+  x1 = int(unsigned(w >> 29)) * sg;
+  x0 = int(unsigned(w) & 0x1fffffffu) * sg;
+}
+// s1 + s0 2^-29 += h x
+PFM_FX void fx_mad(int64_t& s1, int64_t& s0, int h1, int h0, int x1, int x0) {
+  s1 += int64_t(h1) * x1;
+  s0 += int64_t(h1) * x0;
+  s0 += int64_t(h0) * x1;
+}
+// (s1 + s0 2^-29) 2^-58 2^E rounded to nearest, k = 1027 + E
+PFM_FX double fx_value(int64_t s1, int64_t s0, int k) {
+  const int64_t t = 2 * s1 + (s0 >> 28);  // units of 2^-59
+  const int64_t sg = t >> 63;
+  const uint64_t a = uint64_t((t ^ sg) - sg);
+  const int lz = fx_clz(a);
+  const uint64_t q = (((a << (lz & 63)) >> 10) + 1) >> 1;  // 53 bits; the leading one counts in the exponent
+  const uint64_t u = (uint64_t(unsigned(k - 1 - lz)) << 52) + q;
+  return t == 0 ? 0.0 : fx_from_bits(u | (uint64_t(sg) << 63));
+}
+
+}  // namespace pfm
