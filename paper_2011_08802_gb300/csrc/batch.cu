@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(GJ_MAX_THREADS) k_b_gj_panel(const BGj* __rest
            blockIdx.x, gridDim.x);
 }
 
-__global__ void __launch_bounds__(64) k_b_gj_update(const BGj* __restrict__ G, int k0, Gate on) {
+__global__ void __launch_bounds__(GJ_UPD) k_b_gj_update(const BGj* __restrict__ G, int k0, Gate on) {
   const BGj& q = G[blockIdx.z];
   const int r0 = int(blockIdx.y) * GJ_TILE, c0 = int(blockIdx.x) * GJ_TILE;
   if (k0 >= q.n || r0 >= q.n || c0 >= q.n || !on(q.problem)) return;
@@ -1454,7 +1454,7 @@ pfm_status eng_linearize(pfm_batch* b, BatchEngine* E, int power_its) {
     cudaLaunchAttribute at = {};
     gj_panel_config(sh, nG, s, &cfg, &at);
     BCK(cudaLaunchKernelEx(&cfg, k_b_gj_panel, static_cast<const BGj*>(E->dG), k0, E->singular, g));
-    k_b_gj_update<<<dim3(tiles, tiles, unsigned(nG)), 64, 0, s>>>(E->dG, k0, g);
+    k_b_gj_update<<<dim3(tiles, tiles, unsigned(nG)), GJ_UPD, 0, s>>>(E->dG, k0, g);
     count_launches(2);
   }
   k_b_gj_extract<<<dim3(unsigned(E->maxnG), unsigned(nG)), 256, 0, s>>>(E->dG, g);

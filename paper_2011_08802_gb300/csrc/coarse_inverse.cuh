@@ -16,9 +16,9 @@
 //  * update of the other columns J: M[i, J] = (i a pivot row of this panel ? 0
 //    : M[i, J]) + sum_j T[i][j] W[j, J].
 //
-// What bounds it: n^3 FP64 multiply-adds in the updates (0.53e12 per second on
-// this chip: 2.7 ms at n = 1125) and, in the panel, one exchange of pivot
-// candidates per column. The panel runs on one cluster of up to 8 CTAs with
+// What bounds it: n^3 multiply-adds in the updates (in fixed point on the integer
+// pipe; 0.53e12 per second on the FP64 pipe, 2.7 ms at n = 1125) and, in the panel,
+// one exchange of pivot candidates per column. The panel runs on one cluster of up to 8 CTAs with
 // one row per thread, the row's nb entries in registers; per column every CTA
 // sends its best candidate (value, row and the row scaled by the pivot) to all
 // CTAs through distributed shared memory and one cluster barrier follows, so a
@@ -31,13 +31,15 @@
 #include <cstdint>
 
 #include "common.cuh"
+#include "fixed_point.cuh"
 
 namespace pfm {
 
 constexpr int GJ_NB = 16;        // columns per panel
 constexpr int GJ_MAX_CLUSTER = 8;  // CTAs per panel (the portable cluster size)
 constexpr int GJ_MAX_THREADS = 640;  // rows per CTA: 8 x 640 covers MAX_COARSE_DOFS
-constexpr int GJ_TILE = 32;      // update: 32 x 32 entries per CTA of 64 threads
+constexpr int GJ_TILE = 32;      // update: 32 x 32 entries per CTA of GJ_UPD threads
+constexpr int GJ_UPD = 128;
 
 // A CTA's pivot candidate: row (scaled by the pivot, with 1 / pivot in the
 // pivot's own column), pivot value, search key and row index (-1: no row left).
@@ -168,55 +170,134 @@ __device__ __forceinline__ void gj_panel(double* __restrict__ M, int n, int k0, 
   }
 }
 
-// Update of one 32 x 32 tile (rows r0.., columns c0..) by 64 threads, 4 x 4
-// entries each.
+// Update of one 32 x 32 tile (rows r0.., columns c0..) by 128 threads, 4 x 2
+// entries each. The FP64 form is bound by the FP64 pipe (16 multiply-adds per
+// entry, 42.6 us per step at n = 1125), so the sum over the nb pivot rows is formed
+// in fixed point (fixed_point.cuh): with g_k the exponent of W's row k in the tile,
+// T[i][k] 2^(g_k) relative to its largest in row i and W[k][j] 2^(-g_k) relative to
+// its largest in column j, 48 integer multiply-adds and one FP64 add per entry
+// (26.8 us). Tiles with a non-finite entry or an exponent out of range take
+// the FP64 sums.
 __device__ __forceinline__ void gj_update_tile(double* __restrict__ M, int n, int k0, const int* __restrict__ used,
                                                const double* __restrict__ W, int r0, int c0) {
-  __shared__ double Ts[GJ_TILE][GJ_NB + 1];
-  __shared__ double Ws[GJ_NB][GJ_TILE];
+  __shared__ uint64_t Ts[GJ_TILE][GJ_NB + 1];  // bits of the numbers, then their limbs
+  __shared__ uint64_t Ws[GJ_NB][GJ_TILE];
+  __shared__ int gam[GJ_NB], al[GJ_TILE], be[GJ_TILE];
   const int tid = int(threadIdx.x);
   const int nb = n - k0 < GJ_NB ? n - k0 : GJ_NB;
-  for (int i = tid; i < GJ_TILE * GJ_NB; i += 64) {
+  for (int i = tid; i < GJ_TILE * GJ_NB; i += GJ_UPD) {
     const int r = i / GJ_NB, k = i % GJ_NB;
-    Ts[r][k] = r0 + r < n && k < nb ? M[int64_t(r0 + r) * n + k0 + k] : 0.0;
+    Ts[r][k] = fx_bits(r0 + r < n && k < nb ? M[int64_t(r0 + r) * n + k0 + k] : 0.0);
     const int kw = i / GJ_TILE, c = i % GJ_TILE;
     const int col = c0 + c;
-    Ws[kw][c] = col < n && kw < nb && (col < k0 || col >= k0 + nb) ? W[int64_t(kw) * n + col] : 0.0;
+    Ws[kw][c] = fx_bits(col < n && kw < nb && (col < k0 || col >= k0 + nb) ? W[int64_t(kw) * n + col] : 0.0);
   }
-  const int tx = tid & 7, ty = tid >> 3;
-  double acc[4][4];
+  const int tx = tid & 15, ty = tid >> 4;
+  double acc[4][2];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = r0 + ty + 8 * i;
     const int u = r < n ? used[r] - 1 : -1;
     const bool keep = r < n && !(u >= k0 && u < k0 + nb);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = c0 + tx + 8 * q;
+    for (int q = 0; q < 2; ++q) {
+      const int c = c0 + tx + 16 * q;
       acc[i][q] = keep && c < n ? M[int64_t(r) * n + c] : 0.0;
     }
   }
   __syncthreads();
+  bool bad = false;
+  {  // exponents of the rows of W: eight threads per row
+    const int k = tid >> 3;
+    unsigned top = 0;
 #pragma unroll
-  for (int k = 0; k < GJ_NB; ++k) {
-    double t[4], w[4];
+    for (int c = 0; c < GJ_TILE / 8; ++c) {
+      const unsigned t = fx_top(fx_from_bits(Ws[k][(tid & 7) + 8 * c]));
+      top = t > top ? t : top;
+    }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      t[i] = Ts[ty + 8 * i][k];
-      w[i] = Ws[k][tx + 8 * i];
+    for (int m = 1; m <= 4; m <<= 1) {
+      const unsigned o = __shfl_xor_sync(0xffffffffu, top, m);
+      top = o > top ? o : top;
+    }
+    const int e = int(top >> 20);
+    const int g = e ? e - 1022 : 0;
+    bad = e == 0x7ff || g < -FX_RANGE || g > FX_RANGE;
+    if ((tid & 7) == 0) gam[k] = g;
+  }
+  __syncthreads();
+  {  // of the rows of T (t < 32) and the columns of W: two threads each
+    const int t = tid >> 1;
+    const bool row = t < GJ_TILE;
+    int x = -4 * FX_RANGE;
+#pragma unroll
+    for (int h = 0; h < GJ_NB / 2; ++h) {
+      const int k = 2 * h + (tid & 1);
+      const int e = int(fx_top(fx_from_bits(row ? Ts[t & 31][k] : Ws[k][t & 31])) >> 20);
+      const int v = e - 1022 + (row ? gam[k] : -gam[k]);
+      if (e && v > x) x = v;
+      bad |= e == 0x7ff;
+    }
+    const int o = __shfl_xor_sync(0xffffffffu, x, 1);
+    x = o > x ? o : x;
+    if (x == -4 * FX_RANGE)
+      x = 0;  // all zero
+    else
+      bad |= x < -FX_RANGE || x > FX_RANGE;
+    if ((tid & 1) == 0) (row ? al : be)[t & 31] = x;
+  }
+  if (__syncthreads_or(bad)) {
+#pragma unroll 1
+    for (int k = 0; k < GJ_NB; ++k)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          acc[i][q] += fx_from_bits(Ts[ty + 8 * i][k]) * fx_from_bits(Ws[k][tx + 16 * q]);
+  } else {
+    auto limbs = [](uint64_t& x, int k) {
+      int x1, x0;
+      fx_limbs(fx_from_bits(x), k, x1, x0);
+      x = (uint64_t(unsigned(x1)) << 32) | unsigned(x0);
+    };
+    for (int i = tid; i < GJ_TILE * GJ_NB; i += GJ_UPD) {
+      const int r = i / GJ_NB, k = i % GJ_NB;
+      limbs(Ts[r][k], 1027 + al[r] - gam[k]);
+      const int kw = i / GJ_TILE, c = i % GJ_TILE;
+      limbs(Ws[kw][c], 1027 + be[c] + gam[kw]);
+    }
+    __syncthreads();
+    int64_t s1[4][2], s0[4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) s1[i][q] = s0[i][q] = 0;
+#pragma unroll 4
+    for (int k = 0; k < GJ_NB; ++k) {
+      uint64_t t[4], w[2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) t[i] = Ts[ty + 8 * i][k];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) w[q] = Ws[k][tx + 16 * q];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          fx_mad(s1[i][q], s0[i][q], int(t[i] >> 32), int(unsigned(t[i])), int(w[q] >> 32), int(unsigned(w[q])));
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[i][q] += t[i] * w[q];
+      for (int q = 0; q < 2; ++q)
+        acc[i][q] += fx_value(s1[i][q], s0[i][q], 1027 + al[ty + 8 * i] + be[tx + 16 * q]);
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = r0 + ty + 8 * i;
     if (r >= n) continue;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = c0 + tx + 8 * q;
+    for (int q = 0; q < 2; ++q) {
+      const int c = c0 + tx + 16 * q;
       if (c < n && (c < k0 || c >= k0 + nb)) M[int64_t(r) * n + c] = acc[i][q];
     }
   }

@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(GJ_MAX_THREADS) k_gj_panel(double* __restrict_
   gj_panel(M, n, k0, R, used, piv, W, singular, blockIdx.x, gridDim.x);
 }
 
-__global__ void __launch_bounds__(64) k_gj_update(double* __restrict__ M, int n, int k0, const int* __restrict__ used,
+__global__ void __launch_bounds__(GJ_UPD) k_gj_update(double* __restrict__ M, int n, int k0, const int* __restrict__ used,
                                                   const double* __restrict__ W) {
   gj_update_tile(M, n, k0, used, W, int(blockIdx.y) * GJ_TILE, int(blockIdx.x) * GJ_TILE);
 }
@@ -482,7 +482,7 @@ void launch_coarse_assemble(const Grid& g, const DevParams& P, const T* H, const
 // Invert the dense coarse operator M (n x n, overwritten; followed by GJ_NB * n
 // doubles of work) into Ainv (n x n). used, piv: n integers of work each.
 // One panel and one update per GJ_NB columns. Measured at n = 1125 (the 4^3
-// coarsest level): 71 panels of 60 us and 71 updates of 42 us, 7.3 ms; one
+// coarsest level): 71 panels of 60 us and 71 updates of 27 us, 6.2 ms; one
 // launch per column over the augmented matrix took 15.2 ms.
 void launch_coarse_inverse(double* M, int n, double* Ainv, int* used, int* piv, int* singular, cudaStream_t s) {
   double* W = M + int64_t(n) * n;
@@ -495,7 +495,7 @@ void launch_coarse_inverse(double* M, int n, double* Ainv, int* used, int* piv, 
     cudaLaunchAttribute at = {};
     gj_panel_config(sh, 1, s, &cfg, &at);
     cudaLaunchKernelEx(&cfg, k_gj_panel, M, n, k0, sh.rows, used, piv, W, singular);
-    k_gj_update<<<dim3(tiles, tiles), 64, 0, s>>>(M, n, k0, used, W);
+    k_gj_update<<<dim3(tiles, tiles), GJ_UPD, 0, s>>>(M, n, k0, used, W);
     count_launches(2);
   }
   k_gj_extract<<<n, 256, 0, s>>>(M, n, piv, Ainv);
