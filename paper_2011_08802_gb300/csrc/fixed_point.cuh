@@ -112,4 +112,41 @@ PFM_FX double fx_value(int64_t s1, int64_t s0, int k) {
   return t == 0 ? 0.0 : fx_from_bits(u | (uint64_t(sg) << 63));
 }
 
+// Chains of such contractions: a block of numbers is kept as limbs x = h 2^29 + l
+// with one power of two, x 2^(E - 58). After each contraction the sums are shifted
+// to fill the 58 bits, so a stage loses about 2^-57 of its largest result.
+struct Fx {
+  int h, l;
+};
+// E with |v| < 2^E for the largest fx_top of a block (0: all zero); `ok` is cleared
+// when a number is not finite or E is outside +-range
+PFM_FX int fx_block_exponent(unsigned top, int range, bool& ok) {
+  const int e = int(top >> 20);
+  const int E = e ? e - 1022 : 0;
+  ok = ok && e != 0x7ff && E >= -range && E <= range;
+  return E;
+}
+PFM_FX Fx fx_of(double v, int E) {
+  Fx x;
+  fx_limbs(v, 1027 + E, x.h, x.l);
+  return x;
+}
+PFM_FX void fx_mad(int64_t& s1, int64_t& s0, Fx a, Fx b) { fx_mad(s1, s0, a.h, a.l, b.h, b.l); }
+PFM_FX int64_t fx_sum(int64_t s1, int64_t s0) { return 2 * s1 + (s0 >> 28); }  // units of 2^(E - 59)
+// limbs of the block t (|t| < 2^62, units of 2^(E - 59)); returns the change of E
+template <int N>
+PFM_FX int fx_normalise(const int64_t (&t)[N], Fx (&x)[N]) {
+  uint64_t m = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) m |= uint64_t(t[i] ^ (t[i] >> 63));
+  const int lz = fx_clz(m);  // >= 2
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int64_t y = int64_t(uint64_t(t[i]) << ((lz - 2) & 63));  // below 2^62
+    x[i].h = int(y >> 33);
+    x[i].l = int(unsigned(y >> 4) & 0x1fffffffu);
+  }
+  return 5 - lz;
+}
+
 }  // namespace pfm

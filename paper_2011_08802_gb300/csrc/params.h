@@ -1,6 +1,7 @@
 // Conversion of the public parameter block into the kernels' parameter block.
 #pragma once
 
+#include <algorithm>
 #include <cmath>
 
 #include "../../include/pfm.h"
@@ -22,6 +23,18 @@ inline void make_dev_params(const pfm_params& in, DevParams& out) {
   for (int v = 0; v < 6; ++v) out.U0[v] = in.Ut[0][3 * si[v] + sj[v]];
   for (int k = 0; k < NV; ++k)
     for (int v = 0; v < 6; ++v) out.dU[k][v] = in.Ut[k + 1][3 * si[v] + sj[v]] - out.U0[v];
+  unsigned top = 0;
+  for (int k = 0; k < NV; ++k)
+    for (int v = 0; v < 6; ++v) top = std::max(top, fx_top(out.dU[k][v]));
+  bool ok = true;
+  const int e = fx_block_exponent(top, 100, ok);
+  out.dUe = ok ? e : FX_NONE;
+  for (int k = 0; k < NV; ++k)
+    for (int v = 0; v < 6; ++v) {
+      const Fx x = ok ? fx_of(out.dU[k][v], e) : Fx{0, 0};
+      out.dU1[k][v] = x.h;
+      out.dU0[k][v] = x.l;
+    }
   for (int p = 0; p < NPH; ++p) {
     for (int I = 0; I < 6; ++I)
       for (int J = 0; J < 6; ++J) out.Lv[p][I][J] = in.Lvoigt[p][6 * I + J];

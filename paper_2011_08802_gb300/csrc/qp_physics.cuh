@@ -54,6 +54,10 @@
 // r_m[a,b,c] = -sum_k w_k s_k / (p_k(a) p_k(b) p_k(c)).
 #pragma once
 
+#include <type_traits>
+
+#include "fixed_point.cuh"
+
 #ifdef __CUDACC__
 #define PFM_HD __host__ __device__ __forceinline__
 #define PFM_HD_BIG __host__ __device__
@@ -159,6 +163,7 @@ constexpr int NHP = (NH + 7) / 8 * 8;
 struct DevParams {
   double U0[6];             // transformation stretch U_0 (Voigt slots 00, 11, 22, 12, 02, 01)
   double dU[NV][6];         // U_k - U_0, the derivative of F^t with respect to eta_hat_k
+  int dU1[NV][6], dU0[NV][6], dUe;  // and as limbs relative to 2^dUe (fixed_point.cuh; FX_NONE: not available)
   double Lv[NPH][6][6];     // stiffness L_i in Voigt form (engineering shear)
   double inv_mtau[NPH];     // 1 / (m_i tau)
   // chemical and obstacle energy in the condensed unknowns (eta_0 = 1 - sum eta_hat):
@@ -661,6 +666,85 @@ PFM_HD void kinematics(const DevParams& P, const T Fin[9], const T eh[NV], Kinem
   }
 }
 
+// The order-parameter columns of the Hessian (stiffness shared by all phases) from
+// FU and K in fixed point (fixed_point.cuh): FU dU_k and dU_p K dU_q were 666 of
+// about 4100 FP64 operations per point with six variants (1548 with twelve) in a
+// kernel bound by the FP64 pipe; as integer operations in rolled loops they run
+// beside the rest (linearisation call on 80x72x56 elements 28.8 -> 25.5 ms).
+// The loops stay rolled: with the whole chain from Mb unrolled in fixed point the
+// kernel was bound by instruction fetch. False (nothing done) when a number is not
+// finite or far from 1.
+template <typename Emit>
+PFM_HD bool eta_fx(const DevParams& P, const double (&FU)[9][6], const double (&K)[21], const double eh[NV], double eta0,
+                   const Emit& emit) {
+  auto hm6 = [](int I, int J) { return I <= J ? I * 6 - (I * (I - 1)) / 2 + (J - I) : J * 6 - (J * (J - 1)) / 2 + (I - J); };
+  unsigned tF = 0, tK = 0;
+  auto top = [](unsigned& t, double v) {
+    const unsigned x = fx_top(v);
+    t = x > t ? x : t;
+  };
+#pragma unroll
+  for (int r = 0; r < 9; ++r)
+#pragma unroll
+    for (int v = 0; v < 6; ++v) top(tF, FU[r][v]);
+#pragma unroll
+  for (int v = 0; v < 21; ++v) top(tK, K[v]);
+  bool ok = P.dUe != FX_NONE;
+  const int EF = fx_block_exponent(tF, 400, ok), EK = fx_block_exponent(tK, 400, ok);
+  if (!ok) return false;
+  const int Ed = P.dUe;
+  {
+    Fx F[9][6];
+#pragma unroll
+    for (int r = 0; r < 9; ++r)
+#pragma unroll
+      for (int v = 0; v < 6; ++v) F[r][v] = fx_of(FU[r][v], EF);
+#pragma unroll 1
+    for (int k = 0; k < NV; ++k) {
+      Fx d[6];
+#pragma unroll
+      for (int v = 0; v < 6; ++v) d[v] = Fx{P.dU1[k][v], P.dU0[k][v]};
+#pragma unroll
+      for (int r = 0; r < 9; ++r) {
+        int64_t s1 = 0, s0 = 0;
+#pragma unroll
+        for (int v = 0; v < 6; ++v) fx_mad(s1, s0, F[r][v], d[v]);
+        emit(hidx(r, 9 + k), fx_value(s1, s0, 1027 + EF + Ed), 1);
+      }
+    }
+  }
+  Fx Kx[21];
+#pragma unroll
+  for (int v = 0; v < 21; ++v) Kx[v] = fx_of(K[v], EK);
+  const double dd0 = P.inv_mtau[0] + (eta0 < 0.0 ? P.eps_eta : 0.0);
+#pragma unroll 1
+  for (int q = 0; q < NV; ++q) {
+    Fx t[6];
+    int Et = EK + Ed;
+    {
+      int64_t u[6];
+#pragma unroll
+      for (int v = 0; v < 6; ++v) {
+        int64_t s1 = 0, s0 = 0;
+#pragma unroll
+        for (int x = 0; x < 6; ++x) fx_mad(s1, s0, Kx[hm6(v, x)], Fx{P.dU1[q][x], P.dU0[q][x]});
+        u[v] = fx_sum(s1, s0);
+      }
+      Et += fx_normalise(u, t);
+    }
+#pragma unroll 1
+    for (int p = 0; p <= q; ++p) {
+      int64_t s1 = 0, s0 = 0;
+#pragma unroll
+      for (int v = 0; v < 6; ++v) fx_mad(s1, s0, t[v], Fx{P.dU1[p][v], P.dU0[p][v]});
+      double loc = dd0 + P.Cc[p][q];
+      if (p == q) loc += P.inv_mtau[p + 1] + (eh[p] < 0.0 ? P.eps_eta : 0.0);
+      emit(hidx(9 + p, 9 + q), fx_value(s1, s0, 1027 + Et + Ed) + loc, 2);
+    }
+  }
+  return true;
+}
+
 // ---------------------------------------------------------------------------
 // Local energy density with gradient and (optionally) packed Hessian.
 //
@@ -1061,6 +1145,9 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
       }
     }
   } else {
+    if constexpr (std::is_same<T, double>::value) {
+      if (eta_fx(P, FU, K, eh, eta0, emit)) return;
+    }
 #pragma unroll 1
     for (int k = 0; k < NV; ++k) {
       T d[6];
