@@ -34,7 +34,8 @@
 // close, which needs one reciprocal and no logarithm. Measured against the form
 // with one direction per unknown, a Jacobi eigensolve in FP64 and a 120-entry
 // array of the Hessian: linearisation with residual of 80x72x56 elements 37.8 ->
-// 23.6 ms (stack per thread 5.9 -> 1.6 KB), residual of 97x65x50 10.1 -> 7.0 ms.
+// 23.6 ms (stack per thread 5.9 -> 1.6 KB), residual of 97x65x50 10.1 -> 7.0 ms
+// (5.4 ms with the nodal gradient energy and shared differences in the gather).
 //
 // The matrix logarithm's derivatives are the Daleckii-Krein formulas: in the
 // eigenbasis Dlog[X]_ab = f1(l_a,l_b) X_ab and
