@@ -270,8 +270,10 @@ __global__ void k_coarse_solve(int n, const double* __restrict__ Ainv, const T* 
 
 // Chebyshev-accelerated point-block Jacobi, first and later steps (mg_device.cuh).
 // 64 registers (4 CTAs of 256 threads per SM) let a node's 45 + 36 loads be in
-// flight together; with the compiler's own choice (32 registers) a step on
-// 129^3 nodes took about 0.27 ms for 1.0 GB.
+// flight together. Against the compiler's own choice (32 registers): V-cycle from
+// the binary16 store on 75^3 elements 3.14 against 3.31 ms, FP64 Newton step on 32^3
+// 171 against 175 ms, but 38.2 against 35.1 us per step on average over the levels
+// of 128^3 elements (bound by HBM there, about 470 bytes per node).
 template <typename T>
 __global__ void __launch_bounds__(256, 4) k_cheb_first(int64_t nn, const T* __restrict__ D, const T* __restrict__ b, const T* y, T c, bool zero_x,
                              T* __restrict__ r, T* __restrict__ d, T* __restrict__ x, const dmask_t* __restrict__ mask,
