@@ -399,10 +399,17 @@ PFM_HD void rot_sym6(const T R[3][3], const T X[6], T b[6]) {
   }
 }
 
-// Nearly equal eigenvalues (a gap below about 1e-4 of the deviator): Jacobi
-// rotations with exact angles on the rotated matrix. Rare, and out of line so
-// that it takes no registers from the common path.
-PFM_HD_COLD void eig_finish_jacobi(const double b[6], double lam[3], double R[3][3]) {
+// Where FP32 angles are not good enough: Jacobi rotations with exact angles on
+// R^T A R (on A, R = I, where that is not finite), R <- the eigenvectors of A. Rare,
+// and out of line so that it takes no registers from the common path.
+PFM_HD_COLD void eig_finish_jacobi(const double A[6], double lam[3], double R[3][3]) {
+  double b[6];
+  rot_sym6(R, A, b);
+  if (!(fabs(b[0]) + fabs(b[1]) + fabs(b[2]) + fabs(b[3]) + fabs(b[4]) + fabs(b[5]) < HUGE_VAL)) {
+    for (int v = 0; v < 6; ++v) b[v] = A[v];
+    for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j) R[i][j] = i == j ? 1.0 : 0.0;
+  }
   double a[3][3] = {{b[0], b[5], b[4]}, {b[5], b[1], b[3]}, {b[4], b[3], b[2]}};
   double Q1[3][3], Q[3][3];
   jacobi_eig3(a, lam, Q1);
@@ -411,62 +418,80 @@ PFM_HD_COLD void eig_finish_jacobi(const double b[6], double lam[3], double R[3]
     for (int j = 0; j < 3; ++j) R[i][j] = Q[i][j];
 }
 
-// Eigen-decomposition E = Q diag(1 + x) Q^T of the packed symmetric matrix E. The
-// deviator is rotated and x = (mean - 1) + its eigenvalues, so that neither x
-// nor the differences of eigenvalues carry the rounding of numbers near 1.
-PFM_HD void eig_sym6(const float E[6], float x[3], float Q[3][3]) {
-  const float m = (E[0] + E[1] + E[2]) * (1.f / 3.f);
+// Eigen-decomposition E = Q diag(m + d) Q^T of the packed symmetric matrix E.
+// Usually m is the mean of E's diagonal and d belongs to the deviator, so that neither
+// the distances of the eigenvalues from 1, (m - 1) + d, nor their differences carry
+// the rounding of numbers near 1; the eigenvalues are m + d, not 1 + ((m - 1) + d), so
+// that small ones (strong compression) do not carry it either. Where the deviator is
+// large against the smallest eigenvalue (more than twice that: stretches apart by a
+// factor of about 2 or more) the small ones would carry the deviator's rounding: then
+// E itself is rotated and m is 0.
+PFM_HD bool eig_wide(const float a[3], float m) {
+  const float dev = 0.5f * (fabsf(a[0]) + fabsf(a[1]) + fabsf(a[2]));  // NaN and infinite numbers count as wide
+  return !(dev <= 2.f * fminf(m + fminf(a[0], fminf(a[1], a[2])), 1e37f));
+}
+PFM_HD void eig_sym6(const float E[6], float& m, float x[3], float Q[3][3]) {
+  m = (E[0] + E[1] + E[2]) * (1.f / 3.f);
   float a[6] = {E[0] - m, E[1] - m, E[2] - m, E[3], E[4], E[5]}, q[4];
   jacobi_quat(a, q);
+  if (eig_wide(a, m)) {
+    m = 0.f;
+#pragma unroll
+    for (int v = 0; v < 6; ++v) a[v] = E[v];
+    jacobi_quat(a, q);
+  }
   quat_rot(q, Q);
 #pragma unroll
-  for (int i = 0; i < 3; ++i) x[i] = (m - 1.f) + a[i];
+  for (int i = 0; i < 3; ++i) x[i] = a[i];
 }
 // FP64: eigenvectors from FP32 Jacobi, then twice b = R^T X R and the
 // simultaneous small rotation tan(phi/2) = b_pr / (2 (b_rr - b_pp)) in the three
 // planes, its angles in FP32 (the error left after the first correction is the
 // square of the angles, about 1e-13 of the deviator, and nothing after the
 // second). Angles above 1e-3 in the first correction mean nearly equal
-// eigenvalues, where Jacobi with exact angles takes over.
-PFM_HD void eig_sym6(const double E[6], double x[3], double Q[3][3]) {
-  const double m = (E[0] + E[1] + E[2]) * (1.0 / 3.0);
+// eigenvalues, where Jacobi with exact angles takes over, as it does for wide ones.
+PFM_HD void eig_sym6(const double E[6], double& m, double x[3], double Q[3][3]) {
+  m = (E[0] + E[1] + E[2]) * (1.0 / 3.0);
   const double X[6] = {E[0] - m, E[1] - m, E[2] - m, E[3], E[4], E[5]};
   float a[6], qf[4];
 #pragma unroll
   for (int v = 0; v < 6; ++v) a[v] = float(X[v]);
   jacobi_quat(a, qf);
+  const bool wide = eig_wide(a, float(m));
   double q[4] = {double(qf[0]), double(qf[1]), double(qf[2]), double(qf[3])};
   double b[6];
 #pragma unroll
   for (int pass = 0; pass < 2; ++pass) {
     quat_rot(q, Q);
     rot_sym6(Q, X, b);
-    float tau[3], big = 0.f;  // tau[n]: the plane that keeps axis n
+    float tau[3];  // tau[n]: the plane that keeps axis n
     const float num[3] = {float(b[3]), float(b[4]), float(b[5])};
     const float den[3] = {float(b[2] - b[1]), float(b[2] - b[0]), float(b[1] - b[0])};
+    bool rough = wide;
 #pragma unroll
     for (int n = 0; n < 3; ++n) {
       tau[n] = num[n] == 0.f ? 0.f : 0.5f * num[n] / den[n];
-      const float t = fabsf(tau[n]);
-      big = t <= big ? big : t;  // a NaN stays
+      rough = rough || !(fabsf(tau[n]) <= 1e-3f);
     }
-    if (pass == 0 && !(big <= 1e-3f)) {
-      eig_finish_jacobi(b, x, Q);
+    if (pass == 0 && rough) {
+      double A[6];
 #pragma unroll
-      for (int i = 0; i < 3; ++i) x[i] += m - 1.0;
+      for (int v = 0; v < 6; ++v) A[v] = wide ? E[v] : X[v];
+      if (wide) m = 0.0;
+      eig_finish_jacobi(A, x, Q);
       return;
     }
     quat_mul_unit(q, double(-tau[0]), double(tau[1]), double(-tau[2]));
   }
   quat_rot(q, Q);
 #pragma unroll
-  for (int i = 0; i < 3; ++i) x[i] = (m - 1.0) + b[i];
+  for (int i = 0; i < 3; ++i) x[i] = b[i];
 }
 
 #ifdef __CUDACC__
 // Double-float version of the FP64 eigen-decomposition: FP32 Jacobi seed,
 // re-orthonormalisation and the finishing sweeps in double-float.
-__device__ __forceinline__ void eig_sym6(const df64 E[6], df64 x[3], df64 Q[3][3]) {
+__device__ __forceinline__ void eig_sym6(const df64 E[6], df64& m, df64 x[3], df64 Q[3][3]) {
   df64 a[3][3] = {{E[0], E[5], E[4]}, {E[5], E[1], E[3]}, {E[4], E[3], E[2]}};
   float af[3][3], lf[3], Qf[3][3];
   for (int i = 0; i < 3; ++i)
@@ -484,9 +509,8 @@ __device__ __forceinline__ void eig_sym6(const df64 E[6], df64 x[3], df64 Q[3][3
     for (int i = 0; i < 3; ++i) Q0[i][c] *= inrm;
   }
   rot_in(Q0, a, b);
-  df64 lam[3];
-  jacobi_eig3(b, lam, Q1);
-  for (int i = 0; i < 3; ++i) x[i] = lam[i] - df64(1.0);
+  jacobi_eig3(b, x, Q1);
+  m = df64(0.0);  // the rotated matrix is E itself
   mm3(Q0, Q1, Q);
 }
 #endif
@@ -536,19 +560,19 @@ PFM_HD T dd_log(T a, T b, T d, T ia, T ib, T* faab, T* fabb) {
   return f1;
 }
 
-// Second divided difference of log at three values from their first ones
-// (f12 = f[l1,l2] and so on; x = l - 1). Narrow spread (the whole spread at most
+// Second divided difference of log at three values l = m0 + d from their first ones
+// (f12 = f[l1,l2] and so on). Narrow spread (the whole spread below
 // Tol::f2_gap of the mean m): f^(2+j)(m)/(2+j)! h_j(x - m) summed over j, for log
 // (1/m^2) sum_j (-1)^(j+1) h_j(u)/(j+2), u = (x - m)/m, with the complete
 // homogeneous symmetric polynomials h_j; the u sum to zero, so
 // h_j = -e2 h_(j-2) + e3 h_(j-3). Otherwise the quotient over the largest gap.
 template <typename T>
-PFM_HD T dd2_log(const T x[3], T f12, T f02, T f01) {
+PFM_HD T dd2_log(T m0, const T x[3], T f12, T f02, T f01) {
   const float g01 = fabsf(to_f32(x[0] - x[1])), g02 = fabsf(to_f32(x[0] - x[2])), g12 = fabsf(to_f32(x[1] - x[2]));
   const float gap = fmaxf(g01, fmaxf(g02, g12));
-  const T m = (x[0] + x[1] + x[2]) * T(1.0 / 3.0);
-  if (gap <= Tol<T>::f2_gap * fabsf(1.f + to_f32(m))) {
-    const T im = T(1) / (T(1) + m);
+  const T m = (x[0] + x[1] + x[2]) * T(1.0 / 3.0), ml = m0 + m;
+  if (gap < Tol<T>::f2_gap * fminf(fabsf(to_f32(ml)), 1e38f)) {  // beyond FP32: the quotient
+    const T im = T(1) / ml;
     const T u0 = (x[0] - m) * im, u1 = (x[1] - m) * im, u2 = (x[2] - m) * im;
     const T ne2 = u0 * u0 + u1 * (u0 + u1);  // -e2 = u0^2 + u0 u1 + u1^2
     const T e3 = u0 * u1 * u2;
@@ -564,14 +588,14 @@ PFM_HD T dd2_log(const T x[3], T f12, T f02, T f01) {
 }
 
 // Kinematics of one Gauss point: A = (F^t)^-1 and J_t, M = F^e = F A, the
-// eigen-decomposition of C^e = M^T M (lam = 1 + x), the Hencky strain h at the
+// eigen-decomposition of C^e = M^T M = Q diag(lam) Q^T, the Hencky strain h at the
 // eigenvalues (halved log, or the Pade approximant) and the divided differences
 // of the function: f1 in the Voigt slots and, with F2, f2d[a] = f2(a,a,a),
 // f2p[n] = {f2(p,p,r), f2(p,r,r)} for the pair (p, r), p < r, without n, and
 // f2t = f2(0,1,2).
 template <typename T>
 struct Kinematics {
-  T A[6], Jt, M[3][3], x[3], lam[3], Q[3][3], h[3], f1[6];
+  T A[6], Jt, M[3][3], lam[3], Q[3][3], h[3], f1[6];
   T f2d[3], f2p[3][2], f2t;
 };
 template <bool F2, typename T>
@@ -595,7 +619,7 @@ PFM_HD void kinematics(const DevParams& P, const T Fin[9], const T eh[NV], Kinem
 #pragma unroll
     for (int j = 0; j < 3; ++j)
       M[i][j] = Fin[3 * i] * symget(A, 0, j) + Fin[3 * i + 1] * symget(A, 1, j) + Fin[3 * i + 2] * symget(A, 2, j);
-  T (&x)[3] = kin.x;
+  T m, d[3];
   T (&lam)[3] = kin.lam;
   {
     T E[6];  // C^e = M^T M
@@ -604,9 +628,9 @@ PFM_HD void kinematics(const DevParams& P, const T Fin[9], const T eh[NV], Kinem
       const int i = sym_i(v), j = sym_j(v);
       E[v] = M[0][i] * M[0][j] + M[1][i] * M[1][j] + M[2][i] * M[2][j];
     }
-    eig_sym6(E, x, kin.Q);
+    eig_sym6(E, m, d, kin.Q);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) lam[a] = T(1) + x[a];
+    for (int a = 0; a < 3; ++a) lam[a] = m + d[a];
   }
   T (&h)[3] = kin.h;
   T (&f1)[6] = kin.f1;
@@ -620,21 +644,26 @@ PFM_HD void kinematics(const DevParams& P, const T Fin[9], const T eh[NV], Kinem
 #pragma unroll
     for (int n = 0; n < 3; ++n) {
       const int p = n == 0 ? 1 : 0, r = n == 2 ? 1 : 2;
-      f1[3 + n] = dd_log<F2>(lam[p], lam[r], x[p] - x[r], f1[p], f1[r], &f2p[n][0], &f2p[n][1]);
+      f1[3 + n] = dd_log<F2>(lam[p], lam[r], d[p] - d[r], f1[p], f1[r], &f2p[n][0], &f2p[n][1]);
     }
     // log at one eigenvalue, the others through the divided differences
-    const T l0 = x[0] * dd_log<false>(lam[0], T(1), x[0], T(0), T(0), (T*)nullptr, (T*)nullptr);
+    const T x0 = (m - T(1)) + d[0];
+    const T l0 = x0 * dd_log<false>(lam[0], T(1), x0, T(0), T(0), (T*)nullptr, (T*)nullptr);
     h[0] = T(0.5) * l0;
-    h[1] = T(0.5) * (l0 + (x[1] - x[0]) * f1[5]);
-    h[2] = T(0.5) * (l0 + (x[2] - x[0]) * f1[4]);
+    h[1] = T(0.5) * (l0 + (d[1] - d[0]) * f1[5]);
+    h[2] = T(0.5) * (l0 + (d[2] - d[0]) * f1[4]);
     if (F2) {
 #pragma unroll
       for (int a = 0; a < 3; ++a) f2d[a] = T(-0.5) * f1[a] * f1[a];
-      f2t = dd2_log(x, f1[3], f1[4], f1[5]);
+      f2t = dd2_log(m, d, f1[3], f1[4], f1[5]);
     }
   } else {
+    T x[3];  // lam - 1
 #pragma unroll
-    for (int a = 0; a < 3; ++a) h[a] = f2d[a] = f2p[a][0] = f2p[a][1] = T(0);
+    for (int a = 0; a < 3; ++a) {
+      x[a] = (m - T(1)) + d[a];
+      h[a] = f2d[a] = f2p[a][0] = f2p[a][1] = T(0);
+    }
 #pragma unroll
     for (int v = 0; v < 6; ++v) f1[v] = T(0);
 #pragma unroll
