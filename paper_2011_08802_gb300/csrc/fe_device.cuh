@@ -29,25 +29,46 @@ __device__ __forceinline__ T shx(T v, int m) {
 }
 
 // Nodal value v of this lane's node -> value and gradient at this lane's point.
-template <typename T>
+// SHARED: the difference of the two values of an axis serves the interpolation too
+// (ga + gb = 1: gb v + ga s = v + ga (s - v)), which saves FP64 operations but makes
+// the chain of dependent ones longer. Register-fed FP32 applications, which have
+// operations to spare and wait for their shuffles, take the separate form: the slab
+// kernel of the host-buffer application on 128^3 elements 1790 us per call with the
+// shared form, 1560 with this one, a batch of 64 Newton corrections 131.1 and 129.1 ms.
+template <typename T, bool SHARED = true>
 __device__ __forceinline__ void q1_gather(T v, int l8, T ihx, T ihy, T ihz, T& val, T& gx, T& gy,
                                           T& gz) {
-  const T ga = T(GA), gb = T(GB);  // ga + gb = 1: gb v + ga s = v + ga (s - v)
-  const T sx = (l8 & 1) ? -ihx : ihx, sy = (l8 & 2) ? -ihy : ihy, sz = (l8 & 4) ? -ihz : ihz;
-  const T d0 = shx(v, 1) - v;
-  T vx = v + ga * d0;
-  T dx = d0 * sx;
-  T s1 = shx(vx, 2), s2 = shx(dx, 2);
-  const T d1 = s1 - vx;
-  T vxy = vx + ga * d1;
-  T vdy = d1 * sy;
-  T dxy = gb * dx + ga * s2;
-  T t1 = shx(vxy, 4), t2 = shx(vdy, 4), t3 = shx(dxy, 4);
-  const T d2 = t1 - vxy;
-  val = vxy + ga * d2;
-  gz = d2 * sz;
-  gy = gb * vdy + ga * t2;
-  gx = gb * dxy + ga * t3;
+  const T ga = T(GA), gb = T(GB);
+  if constexpr (SHARED) {
+    const T sx = (l8 & 1) ? -ihx : ihx, sy = (l8 & 2) ? -ihy : ihy, sz = (l8 & 4) ? -ihz : ihz;
+    const T d0 = shx(v, 1) - v;
+    T vx = v + ga * d0;
+    T dx = d0 * sx;
+    T s1 = shx(vx, 2), s2 = shx(dx, 2);
+    const T d1 = s1 - vx;
+    T vxy = vx + ga * d1;
+    T vdy = d1 * sy;
+    T dxy = gb * dx + ga * s2;
+    T t1 = shx(vxy, 4), t2 = shx(vdy, 4), t3 = shx(dxy, 4);
+    const T d2 = t1 - vxy;
+    val = vxy + ga * d2;
+    gz = d2 * sz;
+    gy = gb * vdy + ga * t2;
+    gx = gb * dxy + ga * t3;
+  } else {
+    T s = shx(v, 1);
+    T vx = gb * v + ga * s;
+    T dx = ((l8 & 1) ? (v - s) : (s - v)) * ihx;
+    T s1 = shx(vx, 2), s2 = shx(dx, 2);
+    T vxy = gb * vx + ga * s1;
+    T vdy = ((l8 & 2) ? (vx - s1) : (s1 - vx)) * ihy;
+    T dxy = gb * dx + ga * s2;
+    T t1 = shx(vxy, 4), t2 = shx(vdy, 4), t3 = shx(dxy, 4);
+    val = gb * vxy + ga * t1;
+    gz = ((l8 & 4) ? (vxy - t1) : (t1 - vxy)) * ihz;
+    gy = gb * vdy + ga * t2;
+    gx = gb * dxy + ga * t3;
+  }
 }
 
 // Nodal value -> value at this lane's point; also its transpose (point weights
@@ -588,13 +609,13 @@ __device__ __forceinline__ void japply_block(const Grid& g, const JParams<T>& jp
   for (int i = 0; i < 3; ++i) {
     T x = ((dm >> i) & 1) ? T(0) : v[i * nn + node];
     T val;
-    q1_gather(x, l8, jp.ihx, jp.ihy, jp.ihz, val, dz[3 * i], dz[3 * i + 1], dz[3 * i + 2]);
+    q1_gather<T, sizeof(T) == 8>(x, l8, jp.ihx, jp.ihy, jp.ihz, val, dz[3 * i], dz[3 * i + 1], dz[3 * i + 2]);
   }
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     T x = ((dm >> (3 + k)) & 1) ? T(0) : v[(3 + k) * nn + node];
     if constexpr (GE)
-      q1_gather(x, l8, jp.ihx, jp.ihy, jp.ihz, dz[9 + k], ge[3 * k], ge[3 * k + 1], ge[3 * k + 2]);
+      q1_gather<T, sizeof(T) == 8>(x, l8, jp.ihx, jp.ihy, jp.ihz, dz[9 + k], ge[3 * k], ge[3 * k + 1], ge[3 * k + 2]);
     else
       dz[9 + k] = q1_value(x);
   }
