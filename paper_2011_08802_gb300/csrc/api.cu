@@ -114,7 +114,7 @@ void precond_apply(pfm_handle* h, size_t l, const T* x, T* y, bool timed = true,
     }
   }
   ProfScope ps(h, sizeof(T) == 4 ? PFM_PROF_JAPPLY_F32 : PFM_PROF_JAPPLY_F64, on);
-  launch_japply<T>(lv.g, h->dp, LvVec<T>::H(lv), lv.mask, x, y, h->stream, det_W<T>(h), y_ready, lv.HX);
+  launch_japply<T>(lv.g, h->dp, LvVec<T>::H(lv), lv.mask, x, y, h->stream, det_W<T>(h), y_ready);
   if (h->contact_on) launch_contact_apply<T, T, T>(lv.g, LvVec<T>::Kc(lv), lv.mask, x, y, h->stream);
 }
 
@@ -416,7 +416,6 @@ pfm_status linearize_impl(pfm_handle* h, pfm_precision prec, double* R_fused = n
     // double-float outer operator reads it), also when it is the only level
     const bool need32 = prec == PFM_F32 && (fine || !coarsest);
     if (need64) TRY(dalloc(h, &lv.H64, hsz));
-    if (need64 && NV == 6) TRY(dalloc(h, &lv.HX, size_t(lv.nblk) * 32));
     if (need32) TRY(dalloc(h, &lv.H32, hsz));
     const bool needlo = fine && need32;
     if (needlo) TRY(dalloc(h, &lv.H32lo, hsz));
@@ -430,11 +429,11 @@ pfm_status linearize_impl(pfm_handle* h, pfm_precision prec, double* R_fused = n
         CK(cudaMemsetAsync(h->energy_dev, 0, sizeof(double), s));
         const LinResidual res{lv.mask, R_fused, h->energy_dev, det_W<double>(h)};
         launch_linearize(lv.g, h->dp, lv.U, lv.Un, need64 ? lv.H64 : nullptr, need32 ? lv.H32 : nullptr,
-                         needlo ? lv.H32lo : nullptr, need64 ? lv.HX : nullptr, arith, s, &res);
+                         needlo ? lv.H32lo : nullptr, arith, s, &res);
         if (h->contact_on) launch_contact_residual(lv.g, h->contact, lv.U, lv.mask, R_fused, h->energy_dev, nullptr, s);
       } else {
         launch_linearize(lv.g, h->dp, lv.U, lv.Un, need64 ? lv.H64 : nullptr, need32 ? lv.H32 : nullptr,
-                         needlo ? lv.H32lo : nullptr, need64 ? lv.HX : nullptr, arith, s);
+                         needlo ? lv.H32lo : nullptr, arith, s);
       }
     }
     CKL_AT("Gauss-point Hessians");
@@ -1178,7 +1177,7 @@ void pfm_destroy(pfm_handle* h) {
   for (int id = 0; id < PFM_PROF_COUNT; ++id)
     for (auto& e : h->prof_ev[id]) { cudaEventDestroy(e.first); cudaEventDestroy(e.second); }
   for (auto& lv : h->L) {
-    dfree(lv.U); dfree(lv.Un); dfree(lv.mask); dfree(lv.H64); dfree(lv.HX); dfree(lv.H32); dfree(lv.H32lo); dfree(lv.H16); dfree(lv.D64);
+    dfree(lv.U); dfree(lv.Un); dfree(lv.mask); dfree(lv.H64); dfree(lv.H32); dfree(lv.H32lo); dfree(lv.H16); dfree(lv.D64);
     dfree(lv.D32);
     dfree(lv.x32); dfree(lv.b32); dfree(lv.y32); dfree(lv.x64); dfree(lv.b64); dfree(lv.y64);
     dfree(lv.r32); dfree(lv.d32); dfree(lv.r64); dfree(lv.d64); dfree(lv.Kc64); dfree(lv.Kc32);

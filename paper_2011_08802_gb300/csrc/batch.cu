@@ -91,7 +91,6 @@ struct BLin {
   double* H64;
   float* H32;
   float* H32lo;
-  int* HX;
   int64_t blk0;
 };
 
@@ -342,7 +341,7 @@ __global__ void __launch_bounds__(128) k_b_linearize(const BLin* __restrict__ S,
   if (blk >= nblk) return;
   const BLin& L = S[find_entry(S, ns, blk)];
   if (!on(L.problem)) return;
-  linearize_lane<TC>(L.g, *L.P, L.U, L.Un, L.H64, L.H32, L.H32lo, L.HX, blk - L.blk0, int(tid & 31));
+  linearize_lane<TC>(L.g, *L.P, L.U, L.Un, L.H64, L.H32, L.H32lo, blk - L.blk0, int(tid & 31));
 }
 
 // Residual of every active problem: first pass (displacement rows 0, nodal
@@ -1046,7 +1045,6 @@ pfm_status engine_buffers(pfm_handle* h, int m) {
     const size_t hsz = size_t(lv.nblk) * HBLK;
     const bool fine = l == 0, coarsest = l + 1 == nl;
     if (fine || coarsest) TRY(dalloc(h, &lv.H64, hsz));
-    if ((fine || coarsest) && NV == 6) TRY(dalloc(h, &lv.HX, size_t(lv.nblk) * 32));
     if (fine || !coarsest) TRY(dalloc(h, &lv.H32, hsz));
     if (fine) TRY(dalloc(h, &lv.H32lo, hsz));
     if (h->pre_h16 && !coarsest) TRY(dalloc(h, &lv.H16, hsz));
@@ -1121,12 +1119,10 @@ pfm_status engine_build(pfm_batch* b, const pfm_solve_opts& o, BatchEngine** out
       li.Un = lv.Un;
       if (l == 0) {
         li.H64 = lv.H64;
-        li.HX = lv.HX;
         li.H32 = lv.H32;
         li.H32lo = lv.H32lo;
       } else if (coarsest) {
         li.H64 = lv.H64;
-        li.HX = lv.HX;
       } else {
         li.H32 = lv.H32;
       }
@@ -1632,7 +1628,7 @@ std::vector<uint64_t> engine_signature(const pfm_batch* b) {
   auto add = [&](const void* q) { sig.push_back(uint64_t(reinterpret_cast<uintptr_t>(q))); };
   for (const pfm_handle* h : b->hs) {
     for (const Level& lv : h->L) {
-      add(lv.U); add(lv.Un); add(lv.mask); add(lv.H64); add(lv.HX); add(lv.H32); add(lv.H32lo); add(lv.D32);
+      add(lv.U); add(lv.Un); add(lv.mask); add(lv.H64); add(lv.H32); add(lv.H32lo); add(lv.D32);
       add(h->pre_h16 ? lv.H16 : nullptr);
       add(lv.x32); add(lv.b32); add(lv.y32); add(lv.r32); add(lv.d32);
     }

@@ -157,15 +157,14 @@ struct LinResidual {
   double* W;
 };
 void launch_linearize(const Grid& g, const DevParams& P, const double* U, const double* Un,
-                      double* H64, float* H32, float* H32lo, int* HX, int arith, cudaStream_t s,
+                      double* H64, float* H32, float* H32lo, int arith, cudaStream_t s,
                       const LinResidual* res = nullptr);
 void launch_japply_df(const Grid& g, const DevParams& P, const float* Hhi, const float* Hlo, const dmask_t* mask,
                       const float* v, double* y, cudaStream_t s, double* W = nullptr);
-// y_ready (FP32 without W): y already holds v at prescribed DOFs and 0 elsewhere;
-// HX (FP64 with six variants): the scales written with the store
+// y_ready (FP32 without W): y already holds v at prescribed DOFs and 0 elsewhere
 template <typename T>
 void launch_japply(const Grid& g, const DevParams& P, const T* H, const dmask_t* mask, const T* v,
-                   T* y, cudaStream_t s, T* W = nullptr, bool y_ready = false, const int* HX = nullptr);
+                   T* y, cudaStream_t s, T* W = nullptr, bool y_ready = false);
 // y = J v from a binary16 copy of the FP32 store holding s H (FP32 arithmetic;
 // inv_scale = 1/s), and the conversion that makes that copy: returns s, a
 // power of two putting max |H| in [2^14, 2^15), or 0 on failure (scratch: one

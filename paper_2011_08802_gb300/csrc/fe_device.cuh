@@ -18,7 +18,6 @@
 #include <cstdint>
 #include <type_traits>
 
-#include "fixed_point.cuh"
 #include "common.cuh"
 
 namespace pfm {
@@ -234,8 +233,7 @@ struct HessStore {
   int64_t blk;
   int lane;
   bool valid;
-  unsigned* top;  // largest high word of |entry| in each part (fx_hess_scales)
-  __device__ __forceinline__ void operator()(int j, TC v, int part) const {
+  __device__ __forceinline__ void operator()(int j, TC v) const {
     if constexpr (std::is_same<TC, float>::value) {
       const float h = valid ? v : 0.f;
       if (H64) H64[hstore_offset<double>(blk, j, lane)] = double(h);
@@ -244,8 +242,6 @@ struct HessStore {
     } else {
       const double h = valid ? double(v) : 0.0;
       if (H64) H64[hstore_offset<double>(blk, j, lane)] = h;
-      const unsigned t = fx_top(h);
-      top[part] = t > top[part] ? t : top[part];
       if (H32) {
         float hi, lo;
         split_f64(h, hi, lo);
@@ -266,8 +262,7 @@ template <typename TC, typename Tail = NoLinTail>
 __device__ __forceinline__ void linearize_lane(const Grid& g, const DevParams& P, const double* __restrict__ U,
                                                const double* __restrict__ Un, double* __restrict__ H64,
                                                float* __restrict__ H32, float* __restrict__ H32lo,
-                                               int* __restrict__ HX, int64_t blk, int lane,
-                                               const Tail& tail = Tail{}) {
+                                               int64_t blk, int lane, const Tail& tail = Tail{}) {
   const int64_t e = blk * 4 + (lane >> 3);
   const int l8 = lane & 7;
   const bool valid = e < g.ne();
@@ -279,13 +274,9 @@ __device__ __forceinline__ void linearize_lane(const Grid& g, const DevParams& P
 #pragma unroll
   for (int k = 0; k < NV; ++k) ehn[k] = q1_value(valid ? TC(Un[(3 + k) * nn + node]) : TC(0));
   TC W, gr[NZ];
-  unsigned top[3] = {0, 0, 0};
-  const HessStore<TC> store{H64, H32, H32lo, blk, lane, valid, top};
+  const HessStore<TC> store{H64, H32, H32lo, blk, lane, valid};
   qp_point<TC>(P, F, eh, ehn, &W, gr, store);
-  for (int j = NH; j < NHP; ++j) store(j, TC(0), 2);  // padding entries are stored as zeros
-  if constexpr (!std::is_same<TC, float>::value) {
-    if (HX) HX[blk * 32 + lane] = fx_hess_scales(top);
-  }
+  for (int j = NH; j < NHP; ++j) store(j, TC(0));  // padding entries are stored as zeros
   tail(gr, W, node, valid, l8);
 }
 
@@ -664,96 +655,6 @@ __device__ __forceinline__ void japply_block(const Grid& g, const JParams<T>& jp
     if (valid && !((dm >> (3 + k)) & 1)) atomicAdd(&y[(3 + k) * nn + node], r);
   }
 }
-#if PFM_NV == 6
-// FP64 application with the contraction sigma = H dz in fixed point
-// (fixed_point.cuh): it was 225 of the about 380 FP64 operations per point of an
-// application bound by the FP64 pipe; as integer multiply-adds it runs beside
-// the Q1 gather and scatter, which stay in FP64. A point with a non-finite entry
-// or an exponent out of range makes its warp take the FP64 form.
-// Measured: 61x45x33 elements 580 -> 426 us with the first pass (nodal gradient
-// energy) included; error against 64 bits 4.2e-16 -> 3.8e-16 of the largest value.
-// the FP64 form of one block, out of line
-inline __device__ __noinline__ void japply_block_f64(const Grid& g, const JParams<double>& jp, const double* __restrict__ H,
-                                              const dmask_t* __restrict__ mask, const double* __restrict__ v,
-                                              double* __restrict__ y, int64_t blk, int lane) {
-  japply_block<double, false>(g, jp, H, mask, v, y, blk, lane);
-}
-
-__device__ __forceinline__ void japply_block_fx(const Grid& g, const JParams<double>& jp, const double* __restrict__ H,
-                                                const int* __restrict__ HX, const dmask_t* __restrict__ mask,
-                                                const double* __restrict__ v, double* __restrict__ y, int64_t blk,
-                                                int lane) {
-  const int l8 = lane & 7;
-  const int64_t nn = g.nn();
-  const int64_t e = blk * 4 + (lane >> 3);
-  const bool valid = e < g.ne();
-  const int64_t node = valid ? elem_node(g, e, l8) : 0;
-  const dmask_t dm = valid ? mask[node] : MASK_ALL;
-  const int hx = HX[blk * 32 + lane];
-  const int aF = fx_scale_F(hx), ae = fx_scale_eta(hx);
-  int X1[NZ], X0[NZ], Z;
-  {
-    double dz[NZ];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const double x = ((dm >> i) & 1) ? 0.0 : v[i * nn + node];
-      double val;
-      q1_gather(x, l8, jp.ihx, jp.ihy, jp.ihz, val, dz[3 * i], dz[3 * i + 1], dz[3 * i + 2]);
-    }
-#pragma unroll
-    for (int k = 0; k < NV; ++k) dz[9 + k] = q1_value(((dm >> (3 + k)) & 1) ? 0.0 : v[(3 + k) * nn + node]);
-    unsigned tF = 0, te = 0;
-#pragma unroll
-    for (int c = 0; c < NZ; ++c) {
-      const unsigned t = fx_top(dz[c]);
-      if (c < 9)
-        tF = t > tF ? t : tF;
-      else
-        te = t > te ? t : te;
-    }
-    const bool ok = fx_input_scale(hx, tF, te, Z);
-    if (!__all_sync(0xffffffffu, ok)) {
-      japply_block_f64(g, jp, H, mask, v, y, blk, lane);
-      return;
-    }
-#pragma unroll
-    for (int c = 0; c < NZ; ++c) fx_limbs(dz[c], 1027 + Z - (c < 9 ? aF : ae), X1[c], X0[c]);
-  }
-  int64_t S1[NZ], S0[NZ];
-#pragma unroll
-  for (int r = 0; r < NZ; ++r) S1[r] = S0[r] = 0;
-  const int cF = 1027 + 2 * aF, cX = 1027 + aF + ae, ce = 1027 + 2 * ae;
-  const double2* Hv = reinterpret_cast<const double2*>(H) + blk * (NHP / 2) * 32 + lane;
-#pragma unroll
-  for (int j = 0; j < NHP / 2; ++j) {
-    const double2 hv = __ldcs(Hv + j * 32);
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int idx = 2 * j + t;
-      if (idx >= NH) continue;
-      const int r = packed_row(idx);
-      const int c = r + (idx - packed_row_start(r));
-      int h1, h0;
-      fx_limbs(t ? hv.y : hv.x, c < 9 ? cF : (r < 9 ? cX : ce), h1, h0);
-      fx_mad(S1[r], S0[r], h1, h0, X1[c], X0[c]);
-      if (c != r) fx_mad(S1[c], S0[c], h1, h0, X1[r], X0[r]);
-    }
-  }
-  const int kF = 1027 + aF + Z, ke = 1027 + ae + Z;
-  const double w = jp.w, wx = w * jp.ihx, wy = w * jp.ihy, wz = w * jp.ihz;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const double r = q1_scatter_grad(fx_value(S1[3 * i], S0[3 * i], kF), fx_value(S1[3 * i + 1], S0[3 * i + 1], kF),
-                                     fx_value(S1[3 * i + 2], S0[3 * i + 2], kF), l8, wx, wy, wz);
-    if (valid && !((dm >> i) & 1)) atomicAdd(&y[i * nn + node], r);
-  }
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const double r = w * q1_value(fx_value(S1[9 + k], S0[9 + k], ke));
-    if (valid && !((dm >> (3 + k)) & 1)) atomicAdd(&y[(3 + k) * nn + node], r);
-  }
-}
-#endif
 // ---- END tangent application kernel
 
 // The same body in the atomic-free form (deterministic mode): the lane's

@@ -150,8 +150,7 @@ template <typename TC, bool RES = false>
 __global__ void __launch_bounds__(128) k_linearize(Grid g, DevParams P, const double* __restrict__ U,
                                                    const double* __restrict__ Un,
                                                    double* __restrict__ H64, float* __restrict__ H32,
-                                                   float* __restrict__ H32lo, int* __restrict__ HX,
-                                                   const dmask_t* __restrict__ mask,
+                                                   float* __restrict__ H32lo, const dmask_t* __restrict__ mask,
                                                    double* __restrict__ R, double* energy,
                                                    double* __restrict__ RW) {
   const int64_t w0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -161,7 +160,7 @@ __global__ void __launch_bounds__(128) k_linearize(Grid g, DevParams P, const do
     if constexpr (RES) {
       static_assert(std::is_same<TC, double>::value, "residual pass in FP64 only");
       const int64_t ws = g.nblk() * 32;
-      linearize_lane<TC>(g, P, U, Un, H64, H32, H32lo, HX, blk, lane,
+      linearize_lane<TC>(g, P, U, Un, H64, H32, H32lo, blk, lane,
                          [&](const TC* gr, TC Wd, int64_t node, bool valid, int l8) {
                            if (RW)
                              residual_tail_call<TC, true>(g, gr, Wd, node, valid, l8, blk, lane, mask, R, energy, RW,
@@ -171,7 +170,7 @@ __global__ void __launch_bounds__(128) k_linearize(Grid g, DevParams P, const do
                                                            nullptr, 0);
                          });
     } else {
-      linearize_lane<TC>(g, P, U, Un, H64, H32, H32lo, HX, blk, lane);
+      linearize_lane<TC>(g, P, U, Un, H64, H32, H32lo, blk, lane);
     }
   }
 }
@@ -208,30 +207,6 @@ __global__ void __launch_bounds__(256, PFM_JAPPLY_MINB) k_japply(Grid g, JParams
     japply_block<T, sizeof(T) == 4>(g, jp, H, mask, v, y, blk, lane);
   }
 }
-
-#if PFM_NV == 6
-// FP64 with the fixed-point contraction (japply_block_fx), for stores whose
-// scales HX the linearisation wrote.
-#ifndef PFM_JAPPLY_FX_MINB
-#define PFM_JAPPLY_FX_MINB 2
-#endif
-__global__ void __launch_bounds__(256, PFM_JAPPLY_FX_MINB) k_japply_fx(Grid g, JParams<double> jp,
-                                                                       const double* __restrict__ H,
-                                                                       const int* __restrict__ HX,
-                                                                       const dmask_t* __restrict__ mask,
-                                                                       const double* __restrict__ v,
-                                                                       double* __restrict__ y) {
-  const int64_t nblk = g.nblk();
-  const int64_t wg = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
-  const int lane = int(threadIdx.x & 31);
-  constexpr unsigned BLK_BYTES = unsigned(HBLK * sizeof(double));
-  for (int64_t blk = wg; blk < nblk; blk += nw) {
-    if (lane == 0) prefetch_l2(H + blk * HBLK, BLK_BYTES);
-    japply_block_fx(g, jp, H, HX, mask, v, y, blk, lane);
-  }
-}
-#endif
 
 // The atomic-free form (deterministic mode): the same walk, element results
 // to the scratch W (9 x 32 x nblk entries) for the node pass.
@@ -714,8 +689,7 @@ void launch_param_parts(const Grid& g, const DevParams& P, const DevParams& P1, 
 }
 
 void launch_linearize(const Grid& g, const DevParams& P, const double* U, const double* Un,
-                      double* H64, float* H32, float* H32lo, int* HX, int arith, cudaStream_t s,
-                      const LinResidual* res) {
+                      double* H64, float* H32, float* H32lo, int arith, cudaStream_t s, const LinResidual* res) {
   const int64_t threads = g.nblk() * 32;
   unsigned blocks = grid_for(threads, 128);
   if (arith != LIN_F32 && PFM_LIN_CTAS_PER_SM > 0) {
@@ -730,13 +704,13 @@ void launch_linearize(const Grid& g, const DevParams& P, const double* U, const 
   double* RW = with_res ? res->W : nullptr;
   if (with_res && !RW) launch_grad_energy<double, GE_RES>(g, P, mask, U, R, s, energy);
   if (arith == LIN_F32)
-    k_linearize<float><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, HX, nullptr, nullptr, nullptr, nullptr);
+    k_linearize<float><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, nullptr, nullptr, nullptr, nullptr);
   else if (arith == LIN_DF)
-    k_linearize<df64><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, HX, nullptr, nullptr, nullptr, nullptr);
+    k_linearize<df64><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, nullptr, nullptr, nullptr, nullptr);
   else if (with_res)
-    k_linearize<double, true><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, HX, mask, R, energy, RW);
+    k_linearize<double, true><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, mask, R, energy, RW);
   else
-    k_linearize<double><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, HX, nullptr, nullptr, nullptr, nullptr);
+    k_linearize<double><<<blocks, 128, 0, s>>>(g, P, U, Un, H64, H32, H32lo, nullptr, nullptr, nullptr, nullptr);
   count_launches(1);
   if (RW) residual_det_tail(g, P, U, mask, R, energy, RW, s);
 }
@@ -908,22 +882,15 @@ void staged_launch(const Grid& g, const JStaged& jp, const S* H, const dmask_t* 
 // element kernel of the tangent application for a store of type S (wh: weight
 // of the Hessian part, used by the scaled binary16 store only)
 template <typename T>
-void japply_elem(const Grid& g, const JParams<T>& jp, float, const T* H, const int* HX, const dmask_t* mask,
-                 const T* v, T* y, T* W, unsigned blocks, int threads, cudaStream_t s) {
-  if (W) {
+void japply_elem(const Grid& g, const JParams<T>& jp, float, const T* H, const dmask_t* mask, const T* v, T* y,
+                 T* W, unsigned blocks, int threads, cudaStream_t s) {
+  if (W)
     k_japply_det<T><<<blocks, threads, 0, s>>>(g, jp, H, mask, v, W, g.nblk() * 32);
-    return;
-  }
-#if PFM_NV == 6
-  if constexpr (std::is_same<T, double>::value)
-    k_japply_fx<<<blocks, threads, 0, s>>>(g, jp, H, HX, mask, v, y);
   else
-#endif
     k_japply<T><<<blocks, threads, 0, s>>>(g, jp, H, mask, v, y);
 }
-inline void japply_elem(const Grid& g, const JParams<float>& jp, float wh, const __half* H, const int*,
-                        const dmask_t* mask, const float* v, float* y, float* W, unsigned blocks, int threads,
-                        cudaStream_t s) {
+inline void japply_elem(const Grid& g, const JParams<float>& jp, float wh, const __half* H, const dmask_t* mask,
+                        const float* v, float* y, float* W, unsigned blocks, int threads, cudaStream_t s) {
   if (W)
     k_japply_h16<true><<<blocks, threads, 0, s>>>(g, jp, wh, H, mask, v, y, W, g.nblk() * 32);
   else
@@ -933,9 +900,6 @@ template <typename T>
 const void* japply_elem_fn(const T*) {
   return reinterpret_cast<const void*>(k_japply<T>);
 }
-#if PFM_NV == 6
-inline const void* japply_elem_fn(const double*) { return reinterpret_cast<const void*>(k_japply_fx); }
-#endif
 inline const void* japply_elem_fn(const __half*) { return reinterpret_cast<const void*>(k_japply_h16<false>); }
 
 // One tangent application with launch shape js; with a scratch W (9 * 32 *
@@ -947,7 +911,7 @@ inline const void* japply_elem_fn(const __half*) { return reinterpret_cast<const
 template <typename T, typename S = T>
 void japply_launch_shape(const Grid& g, const DevParams& P, const JParams<T>& jp, float wh, const S* H, const dmask_t* mask, const T* v,
                          T* y, const JShape& js, cudaStream_t s, T* W = nullptr, const JStaged* jst = nullptr,
-                         bool y_ready = false, const int* HX = nullptr) {
+                         bool y_ready = false) {
   const int64_t nn = g.nn();
   // FP32 arithmetic keeps the gradient energy in its element kernel (bound by
   // reading the store, or, with the binary16 store, faster than another pass);
@@ -974,7 +938,7 @@ void japply_launch_shape(const Grid& g, const DevParams& P, const JParams<T>& jp
   const int64_t need = (g.nblk() * 32 + cs.threads - 1) / cs.threads;
   const int64_t full = int64_t(sm_count()) * cs.per_sm;
   const unsigned blocks = unsigned(need < full ? need : full);
-  japply_elem(g, jp, wh, H, HX, mask, v, y, W, blocks, cs.threads, s);
+  japply_elem(g, jp, wh, H, mask, v, y, W, blocks, cs.threads, s);
   count_launches(1);
   if (W) {
     k_node_gather<T, T, T><<<grid_for(nn, 128), 128, 0, s>>>(g, W, g.nblk() * 32, mask, v, y);
@@ -985,7 +949,7 @@ void japply_launch_shape(const Grid& g, const DevParams& P, const JParams<T>& jp
 
 template <typename T, typename S = T>
 JShape japply_tune(const Grid& g, const DevParams& P, const JParams<T>& jp, float wh, const S* H, const dmask_t* mask, const T* v, T* y,
-                   cudaStream_t s, const JStaged* jst = nullptr, bool* timed = nullptr, const int* HX = nullptr) {
+                   cudaStream_t s, const JStaged* jst = nullptr, bool* timed = nullptr) {
   const int pr = sizeof(S) == 2 ? 2 : (sizeof(T) == 4 ? 0 : 1);
   int cl = 0;
   for (int64_t b = g.nblk(); b > 1; b >>= 1) ++cl;
@@ -1016,13 +980,13 @@ JShape japply_tune(const Grid& g, const DevParams& P, const JParams<T>& jp, floa
       }
   }
   for (const JShape& js : cand) {
-    japply_launch_shape<T, S>(g, P, jp, wh, H, mask, v, y, js, s, nullptr, jst, false, HX);  // warm
+    japply_launch_shape<T, S>(g, P, jp, wh, H, mask, v, y, js, s, nullptr, jst);  // warm
     // best of three timings of three applications each (the shapes differ
     // by a few per cent, about the run-to-run spread of one timing)
     float ms = 1e30f;
     for (int t = 0; t < 3; ++t) {
       cudaEventRecord(a, s);
-      for (int r = 0; r < 3; ++r) japply_launch_shape<T, S>(g, P, jp, wh, H, mask, v, y, js, s, nullptr, jst, false, HX);
+      for (int r = 0; r < 3; ++r) japply_launch_shape<T, S>(g, P, jp, wh, H, mask, v, y, js, s, nullptr, jst);
       cudaEventRecord(b, s);
       cudaEventSynchronize(b);
       float m = 0.f;
@@ -1044,7 +1008,7 @@ JShape japply_tune(const Grid& g, const DevParams& P, const JParams<T>& jp, floa
 
 template <typename T>
 void launch_japply(const Grid& g, const DevParams& P, const T* H, const dmask_t* mask, const T* v,
-                   T* y, cudaStream_t s, T* W, bool y_ready, const int* HX) {
+                   T* y, cudaStream_t s, T* W, bool y_ready) {
   const JParams<T> jp = make_jparams<T>(g, P);
   if constexpr (std::is_same<T, float>::value) {
     const JStaged jst = make_jstaged(g, P, g.w());
@@ -1052,8 +1016,8 @@ void launch_japply(const Grid& g, const DevParams& P, const T* H, const dmask_t*
     const JShape js = japply_tune<T>(g, P, jp, 0.f, H, mask, v, y, s, &jst, &timed);
     japply_launch_shape<T>(g, P, jp, 0.f, H, mask, v, y, js, s, W, &jst, y_ready && !timed);
   } else {
-    const JShape js = japply_tune<T>(g, P, jp, 0.f, H, mask, v, y, s, nullptr, nullptr, HX);
-    japply_launch_shape<T>(g, P, jp, 0.f, H, mask, v, y, js, s, W, nullptr, false, HX);
+    const JShape js = japply_tune<T>(g, P, jp, 0.f, H, mask, v, y, s);
+    japply_launch_shape<T>(g, P, jp, 0.f, H, mask, v, y, js, s, W);
   }
 }
 
@@ -1198,9 +1162,9 @@ template void launch_identity_rows<double>(int64_t, const dmask_t*, const double
                                            cudaStream_t);
 
 template void launch_japply<float>(const Grid&, const DevParams&, const float*, const dmask_t*,
-                                   const float*, float*, cudaStream_t, float*, bool, const int*);
+                                   const float*, float*, cudaStream_t, float*, bool);
 template void launch_japply<double>(const Grid&, const DevParams&, const double*, const dmask_t*,
-                                     const double*, double*, cudaStream_t, double*, bool, const int*);
+                                     const double*, double*, cudaStream_t, double*, bool);
 template void launch_blockdiag<float>(const Grid&, const DevParams&, const float*, const dmask_t*, float*,
                                       float*, cudaStream_t);
 template void launch_blockdiag<double>(const Grid&, const DevParams&, const double*, const dmask_t*, double*,

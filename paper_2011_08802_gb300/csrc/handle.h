@@ -21,7 +21,6 @@ struct Level {
   double* Un = nullptr;
   dmask_t* mask = nullptr;
   double* H64 = nullptr;
-  int* HX = nullptr;       // scales of each point's H64 for the fixed-point contraction (six variants)
   float* H32 = nullptr;
   float* H32lo = nullptr;  // finest level, mixed mode: H64 - H32 rounded to FP32
   __half* H16 = nullptr;   // binary16 copy of s H32 for the preconditioner (optional)

@@ -739,7 +739,7 @@ PFM_HD bool eta_fx(const DevParams& P, const double (&FU)[9][6], const double (&
         int64_t s1 = 0, s0 = 0;
 #pragma unroll
         for (int v = 0; v < 6; ++v) fx_mad(s1, s0, F[r][v], d[v]);
-        emit(hidx(r, 9 + k), fx_value(s1, s0, 1027 + EF + Ed), 1);
+        emit(hidx(r, 9 + k), fx_value(s1, s0, 1027 + EF + Ed));
       }
     }
   }
@@ -769,7 +769,7 @@ PFM_HD bool eta_fx(const DevParams& P, const double (&FU)[9][6], const double (&
       for (int v = 0; v < 6; ++v) fx_mad(s1, s0, t[v], Fx{P.dU1[p][v], P.dU0[p][v]});
       double loc = dd0 + P.Cc[p][q];
       if (p == q) loc += P.inv_mtau[p + 1] + (eh[p] < 0.0 ? P.eps_eta : 0.0);
-      emit(hidx(9 + p, 9 + q), fx_value(s1, s0, 1027 + Et + Ed) + loc, 2);
+      emit(hidx(9 + p, 9 + q), fx_value(s1, s0, 1027 + Et + Ed) + loc);
     }
   }
   return true;
@@ -780,19 +780,18 @@ PFM_HD bool eta_fx(const DevParams& P, const double (&FU)[9][6], const double (&
 //
 // Fin: F row-major; eh, ehn: eta_1..eta_6 at t_{n+1} and t_n.
 // Outputs: *W, g[15] = dW/dz; with Emit::want every entry of the packed Hessian
-// d^2W/dz^2 is handed once to emit(index, value, part) when it is final (no order),
-// so no array of the whole Hessian is kept; part: 0 both unknowns in F, 1 one of
-// them, 2 neither.
+// d^2W/dz^2 is handed once to emit(index, value) when it is final (no order), so no
+// array of the whole Hessian is kept.
 template <typename T>
 struct NoHess {
   static constexpr bool want = false;
-  PFM_HD void operator()(int, T, int) const {}
+  PFM_HD void operator()(int, T) const {}
 };
 template <typename T>
 struct HessArray {
   static constexpr bool want = true;
   T* Hp;
-  PFM_HD void operator()(int i, T v, int) const { Hp[i] = v; }
+  PFM_HD void operator()(int i, T v) const { Hp[i] = v; }
 };
 
 template <typename T, typename Emit>
@@ -1093,8 +1092,7 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
           // F_pc with F_rc2 (final)
           if (c < c2 || p <= r) {
             const int i = 3 * p + c, j = 3 * r + c2;
-            emit(i <= j ? hidx(i, j) : hidx(j, i), Zf[p][0] * Mq[r][0] + Zf[p][1] * Mq[r][1] + Zf[p][2] * Mq[r][2],
-                 0);
+            emit(i <= j ? hidx(i, j) : hidx(j, i), Zf[p][0] * Mq[r][0] + Zf[p][1] * Mq[r][1] + Zf[p][2] * Mq[r][2]);
           }
           // F_pc with F^t_(r, c2), and F_pc2 with F^t_(r, c)
           dot_to(FU[3 * p + c][voigt_slot(r, c2)], Zf[p], Uq[r]);
@@ -1169,7 +1167,7 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
         for (int p = 0; p < 3; ++p) {
           T fk = t[0] * Mq[p][0] + t[1] * Mq[p][1] + t[2] * Mq[p][2];
           for (int v = 0; v < 6; ++v) fk += FU[3 * p + c][v] * T(P.dU[k][v]);
-          emit(hidx(3 * p + c, 9 + k), fk, 1);
+          emit(hidx(3 * p + c, 9 + k), fk);
           LX[k][voigt_slot(p, c)] += t[0] * Uq[p][0] + t[1] * Uq[p][1] + t[2] * Uq[p][2];
         }
       }
@@ -1188,7 +1186,7 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
         T s = FU[r][0] * d[0];
 #pragma unroll
         for (int v = 1; v < 6; ++v) s += FU[r][v] * d[v];
-        emit(hidx(r, 9 + k), s, 1);
+        emit(hidx(r, 9 + k), s);
       }
     }
   }
@@ -1220,7 +1218,7 @@ PFM_HD void qp_point(const DevParams& P, const T Fin[9], const T eh[NV], const T
         }
         s += T(0.5) * Jt * (ap * (hLh[q + 1] - hLh[0]) + aq * (hLh[p + 1] - hLh[0]));
       }
-      emit(hidx(9 + p, 9 + q), s + loc, 2);
+      emit(hidx(9 + p, 9 + q), s + loc);
     }
   }
 }
