@@ -36,6 +36,7 @@
 namespace pfm {
 
 constexpr int GJ_NB = 16;        // columns per panel
+static_assert(GJ_NB <= FX_TERMS, "the update sums GJ_NB fixed-point products");
 constexpr int GJ_MAX_CLUSTER = 8;  // CTAs per panel (the portable cluster size)
 constexpr int GJ_MAX_THREADS = 640;  // rows per CTA: 8 x 640 covers MAX_COARSE_DOFS
 constexpr int GJ_TILE = 32;      // update: 32 x 32 entries per CTA of GJ_UPD threads

@@ -7,10 +7,13 @@
 //   sigma_r = 2^(a_r + Z) sum_c h_rc y_c,
 // with one exponent a for the unknowns of F and one for the order parameters
 // (per point, from the largest entries of the three parts of H) and one Z per
-// point. h and y are 58-bit integers in two limbs of 29 bits with their sign; the
-// three leading limb products are summed exactly (sums below 2^62), the fourth is
-// below 2^-58 of the largest product. Truncation leaves about 2^-57 of 2^(a_r + Z)
-// per row, against 2^-53 of the partial sums per multiply-add in FP64.
+// point. h and y are 58-bit integers in two limbs of 29 bits with their sign, cut
+// towards zero. Of the four limb products the leading one (below 2^58) goes to s1 and
+// the two middle ones to s0; the last one, below 2^-58 of the product's scale, is left
+// out. A sum takes FX_TERMS = 16 products at most: then s1 < 2^62, s0 < 2^63 - 2^35 and
+// 2 s1 + s0 2^-28 < 2^63 - 2^7. Error of n products: two cut operands and the product
+// left out, 2^-58 of 2^(a_r + Z) each, and 2^-59 for the final shift: at most
+// (3 n + 1/2) 2^-58 of 2^(a_r + Z), whatever the size of the row's own terms.
 // Used where the numbers of a sum share their scale: the rank-16 updates of the coarse
 // inverse (one power of two per row and column of a tile) and the order-parameter
 // columns of the Hessian. Not in the FP64 tangent application: its error is relative to
@@ -65,6 +68,7 @@ PFM_FX unsigned fx_top(double v) { return unsigned(fx_bits(v) >> 32) & 0x7ffffff
 // Scales of a point's Hessian, a_F in the high and a_e in the low 16 bits, from
 // the largest fx_top of its parts (F, F), (F, eta), (eta, eta); FX_NONE when an
 // entry is not finite or a scale is outside +-FX_RANGE.
+constexpr int FX_TERMS = 16;
 constexpr int FX_NONE = -2147483647 - 1;
 constexpr int FX_RANGE = 400;
 PFM_FX int fx_hess_scales(const unsigned top[3]) {
@@ -101,7 +105,7 @@ PFM_FX void fx_limbs(double v, int k, int& x1, int& x0) {
   x1 = int(unsigned(w >> 29)) * sg;
   x0 = int(unsigned(w) & 0x1fffffffu) * sg;
 }
-// s1 + s0 2^-29 += h x
+// s1 + s0 2^-29 += h x, at most FX_TERMS times
 PFM_FX void fx_mad(int64_t& s1, int64_t& s0, int h1, int h0, int x1, int x0) {
   s1 += int64_t(h1) * x1;
   s0 += int64_t(h1) * x0;
