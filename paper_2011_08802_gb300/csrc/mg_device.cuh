@@ -292,66 +292,6 @@ __host__ __device__ __forceinline__ void restrict_entry_int(const Grid& f, const
 // binary arithmetic, so the node bodies below form their sums in T (FP32 in
 // the FP32 preconditioner) and take the node from its (i, j, k) position.
 
-// Fine node (i, j, k): xf += P xc at its free DOFs.
-template <typename T>
-__host__ __device__ __forceinline__ void prolong_node_nested(const Grid& f, const Grid& c, const T* __restrict__ xc,
-                                                    const dmask_t* __restrict__ mf, T* __restrict__ xf, int i,
-                                                    int j, int k) {
-  const int64_t nnf = f.nn(), nnc = c.nn();
-  const int64_t idx = i + int64_t(f.nx + 1) * (j + int64_t(f.ny + 1) * k);
-  const dmask_t dm = mf[idx];
-  if (dm == MASK_ALL) return;
-  const int ni = (i & 1) + 1, nj = (j & 1) + 1, nk = (k & 1) + 1;
-  const T w = ((i & 1) ? T(0.5) : T(1)) * ((j & 1) ? T(0.5) : T(1)) * ((k & 1) ? T(0.5) : T(1));
-  const int64_t c0 = (i >> 1) + int64_t(c.nx + 1) * ((j >> 1) + int64_t(c.ny + 1) * (k >> 1));
-  const int64_t sy = c.nx + 1, sz = int64_t(c.nx + 1) * (c.ny + 1);
-  for (int fld = 0; fld < NF; ++fld) {
-    if ((dm >> fld) & 1) continue;
-    const T* X = xc + fld * nnc + c0;
-    T s = T(0);
-    for (int a2 = 0; a2 < nk; ++a2)
-      for (int a1 = 0; a1 < nj; ++a1)
-        for (int a0 = 0; a0 < ni; ++a0) s += X[a0 + a1 * sy + a2 * sz];
-    xf[fld * nnf + idx] += w * s;
-  }
-}
-
-// Coarse node (I, J, K): rc = (P^T rf) there, zero at its Dirichlet DOFs;
-// it collects fine nodes 2I-1, 2I, 2I+1 per axis with weights 1/2, 1, 1/2.
-template <typename T>
-__host__ __device__ __forceinline__ void restrict_node_nested(const Grid& f, const Grid& c, const T* __restrict__ rf,
-                                                     const dmask_t* __restrict__ mc, T* __restrict__ rc, int I,
-                                                     int J, int K) {
-  const int64_t nnf = f.nn(), nnc = c.nn();
-  const int64_t idx = I + int64_t(c.nx + 1) * (J + int64_t(c.ny + 1) * K);
-  const dmask_t dm = mc[idx];
-  const int64_t sy = f.nx + 1, sz = int64_t(f.nx + 1) * (f.ny + 1);
-  for (int fld = 0; fld < NF; ++fld) {
-    if ((dm >> fld) & 1) {
-      rc[fld * nnc + idx] = T(0);
-      continue;
-    }
-    const T* X = rf + fld * nnf;
-    T acc = T(0);
-    for (int dk = -1; dk <= 1; ++dk) {
-      const int k = 2 * K + dk;
-      if (k < 0 || k > f.nz) continue;
-      T sj = T(0);
-      for (int dj = -1; dj <= 1; ++dj) {
-        const int j = 2 * J + dj;
-        if (j < 0 || j > f.ny) continue;
-        const T* row = X + j * sy + k * sz;
-        T si = row[2 * I];
-        if (I > 0) si += T(0.5) * row[2 * I - 1];
-        if (2 * I + 1 <= f.nx) si += T(0.5) * row[2 * I + 1];
-        sj += (dj ? T(0.5) : T(1)) * si;
-      }
-      acc += (dk ? T(0.5) : T(1)) * sj;
-    }
-    rc[fld * nnc + idx] = acc;
-  }
-}
-
 // One (node, field) of the nested transfers, for one thread each. Prolongation
 // averages the coarse values at floor and ceil of half the index on every axis
 // (the same one twice at an even index: (a + a) / 2 = a exactly), so lanes at
@@ -390,6 +330,39 @@ __host__ __device__ __forceinline__ T restrict_value_nested(const Grid& f, const
     acc += (dk ? T(0.5) : T(1)) * sj;
   }
   return acc;
+}
+
+// (node, field) fld of fine node (i, j, k): xf += P xc if it is free; of coarse node
+// (I, J, K): rc = P^T (rf - y), zero if prescribed.
+template <typename T>
+__host__ __device__ __forceinline__ void prolong_entry_nested(const Grid& f, const Grid& c, const T* __restrict__ xc,
+                                                              const dmask_t* __restrict__ mf, T* __restrict__ xf,
+                                                              int fld, int i, int j, int k) {
+  const int64_t node = i + int64_t(f.nx + 1) * (j + int64_t(f.ny + 1) * k);
+  if ((mf[node] >> fld) & 1) return;
+  xf[fld * f.nn() + node] +=
+      prolong_value_nested<T>(xc + fld * c.nn(), c.nx + 1, int64_t(c.nx + 1) * (c.ny + 1), i, j, k);
+}
+template <typename T>
+__host__ __device__ __forceinline__ void restrict_entry_nested(const Grid& f, const Grid& c, const T* __restrict__ rf,
+                                                               const T* __restrict__ y, const dmask_t* __restrict__ mc,
+                                                               T* __restrict__ rc, int fld, int I, int J, int K) {
+  const int64_t node = I + int64_t(c.nx + 1) * (J + int64_t(c.ny + 1) * K), off = fld * f.nn();
+  rc[fld * c.nn() + node] =
+      ((mc[node] >> fld) & 1) ? T(0) : restrict_value_nested<T>(f, rf + off, y ? y + off : nullptr, I, J, K);
+}
+// every field of one node
+template <typename T>
+__host__ __device__ __forceinline__ void prolong_node_nested(const Grid& f, const Grid& c, const T* __restrict__ xc,
+                                                    const dmask_t* __restrict__ mf, T* __restrict__ xf, int i,
+                                                    int j, int k) {
+  for (int fld = 0; fld < NF; ++fld) prolong_entry_nested<T>(f, c, xc, mf, xf, fld, i, j, k);
+}
+template <typename T>
+__host__ __device__ __forceinline__ void restrict_node_nested(const Grid& f, const Grid& c, const T* __restrict__ rf,
+                                                     const dmask_t* __restrict__ mc, T* __restrict__ rc, int I,
+                                                     int J, int K) {
+  for (int fld = 0; fld < NF; ++fld) restrict_entry_nested<T>(f, c, rf, nullptr, mc, rc, fld, I, J, K);
 }
 
 inline __host__ __device__ bool nested(const Grid& f, const Grid& c) {

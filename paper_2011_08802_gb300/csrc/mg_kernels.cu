@@ -79,11 +79,7 @@ __global__ void __launch_bounds__(128) k_prolong_add_nested(Grid f, Grid c, cons
                                                             const dmask_t* __restrict__ mf, T* __restrict__ xf) {
   const int i = int(blockIdx.x * 32 + threadIdx.x), j = int(blockIdx.y * 4 + threadIdx.y);
   if (i > f.nx || j > f.ny) return;
-  const int k = int(blockIdx.z) / NF, fld = int(blockIdx.z) % NF;
-  const int64_t node = i + int64_t(f.nx + 1) * (j + int64_t(f.ny + 1) * k);
-  if ((mf[node] >> fld) & 1) return;
-  xf[fld * f.nn() + node] +=
-      prolong_value_nested<T>(xc + fld * c.nn(), c.nx + 1, int64_t(c.nx + 1) * (c.ny + 1), i, j, k);
+  prolong_entry_nested<T>(f, c, xc, mf, xf, int(blockIdx.z) % NF, i, j, int(blockIdx.z) / NF);
 }
 
 template <typename T>
@@ -92,11 +88,7 @@ __global__ void __launch_bounds__(128) k_restrict_nested(Grid f, Grid c, const T
                                                          T* __restrict__ rc) {
   const int I = int(blockIdx.x * 32 + threadIdx.x), J = int(blockIdx.y * 4 + threadIdx.y);
   if (I > c.nx || J > c.ny) return;
-  const int K = int(blockIdx.z) / NF, fld = int(blockIdx.z) % NF;
-  const int64_t node = I + int64_t(c.nx + 1) * (J + int64_t(c.ny + 1) * K);
-  const int64_t off = fld * f.nn();
-  rc[fld * c.nn() + node] =
-      ((mc[node] >> fld) & 1) ? T(0) : restrict_value_nested<T>(f, rf + off, y ? y + off : nullptr, I, J, K);
+  restrict_entry_nested<T>(f, c, rf, y, mc, rc, int(blockIdx.z) % NF, I, J, int(blockIdx.z) / NF);
 }
 
 // rc = P^T (rf - y), zero at coarse Dirichlet DOFs.
