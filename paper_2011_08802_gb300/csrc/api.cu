@@ -19,6 +19,7 @@ using namespace pfm;
 
 namespace {
 std::atomic<int64_t> g_launches{0};
+thread_local int64_t* t_captured = nullptr;  // count of the capture this thread is in
 
 // Arithmetic peak probe: every thread runs 8 independent chains of fused
 // multiply-adds (x = x * a + b) for `iters` steps and stores their sum, so
@@ -39,7 +40,14 @@ __global__ void __launch_bounds__(256) k_fma_peak(int iters, T a, T b, T* __rest
 }
 }  // namespace
 
-void pfm::count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+void pfm::count_launches(int n) {
+  if (t_captured)
+    *t_captured += n;
+  else
+    g_launches.fetch_add(n, std::memory_order_relaxed);
+}
+pfm::CaptureCount::CaptureCount() : outer(t_captured) { t_captured = &kernels; }
+pfm::CaptureCount::~CaptureCount() { t_captured = outer; }
 
 namespace {
 std::string g_create_error;
@@ -930,12 +938,11 @@ pfm_status capture_vcycle(pfm_handle* h, const SmoothCfg& sc) {
   cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
   pfm_status st = PFM_OK;
   cudaGraph_t graph = nullptr;
-  const int64_t c0 = g_launches.load(std::memory_order_relaxed);
   int64_t count = 0;
   if (e == cudaSuccess) {
+    CaptureCount cc;
     st = vcycle_level<T>(h, 0, sc);
-    count = g_launches.load(std::memory_order_relaxed) - c0;
-    g_launches.fetch_sub(count, std::memory_order_relaxed);  // counted at every replay
+    count = cc.kernels;
     e = cudaStreamEndCapture(h->stream, &graph);
   }
   h->prof = prof;

@@ -1554,11 +1554,11 @@ void eng_cycle_start(BatchEngine* E, bool first) {
 pfm_status eng_capture(pfm_batch* b, BatchEngine* E, int j, cudaGraphExec_t* out) {
   cudaGraph_t graph = nullptr;
   BCK(cudaStreamBeginCapture(E->s, cudaStreamCaptureModeThreadLocal));
-  const int64_t c0 = pfm_launch_count();
-  eng_iteration(E, j);
-  const int64_t nk = pfm_launch_count() - c0;  // counted again at every replay
-  count_launches(int(-nk));
-  E->itg_launches[j] = nk;
+  {
+    CaptureCount cc;
+    eng_iteration(E, j);
+    E->itg_launches[j] = cc.kernels;
+  }
   cudaError_t e = cudaStreamEndCapture(E->s, &graph);
   if (e != cudaSuccess) return b->fail(PFM_ERR_CUDA, std::string("batch graph capture: ") + cudaGetErrorString(e));
   e = cudaGraphInstantiate(out, graph, 0);

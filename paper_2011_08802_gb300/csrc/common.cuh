@@ -128,6 +128,15 @@ namespace pfm {
 
 // Kernel launches issued by the library (incremented by every launcher).
 void count_launches(int n);
+// While one lives, the launches of its thread are counted in `kernels` instead: those
+// that a stream capture records (the graph's kernels count at every replay). Other
+// threads' launches are not seen.
+struct CaptureCount {
+  int64_t kernels = 0;
+  int64_t* outer;
+  CaptureCount();
+  ~CaptureCount();
+};
 
 // element kernels (fe_kernels.cu)
 // The element kernels below take an optional scratch W: null = element
