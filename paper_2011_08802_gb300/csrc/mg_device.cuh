@@ -11,6 +11,7 @@
 // R = P^T use identical weights on nested (nf = 2 nc) and non-nested grids.
 #pragma once
 
+#include <cfloat>
 #include <cstdint>
 
 #include "common.cuh"
@@ -196,6 +197,53 @@ struct CSum {
 inline __host__ __device__ int64_t transfer_denominator(const Grid& f) { return int64_t(f.nx) * f.ny * f.nz; }
 inline __host__ __device__ bool transfer_integer(const Grid& f) { return transfer_denominator(f) < (int64_t(1) << 24); }
 
+// Fine nodes lo..hi of an axis with a weight at coarse node I: |i nc - I nf| < nf.
+inline __host__ __device__ void transfer_support(int I, int nf, int nc, int& lo, int& hi) {
+  const int64_t center = int64_t(I) * nf;
+  const int64_t a = center - nf, b = center + nf;
+  lo = a >= 0 ? int(a / nc) + 1 : 0;
+  hi = int((b + nc - 1) / nc) - 1;
+  if (hi > nf) hi = nf;
+}
+
+// The FP64 sums of one (node, field), for results that are not finite: numerator x
+// value overflows in FP32 from values of 2^104 on, and its remainder makes NaN of an
+// infinite value. Rare, so out of line and with arguments that a kernel has at hand
+// anyway (passing the node indices kept registers for the call and cost a V-cycle on
+// 33^3 elements 1.1 per cent).
+inline __host__ __device__ __noinline__ float prolong_entry_f64(Grid f, Grid c, const float* xc, int64_t idx) {
+  const int64_t nnf = f.nn(), node = idx % nnf;
+  const Interp1 px = interp1(int(node % (f.nx + 1)), f.nx, c.nx),
+                py = interp1(int((node / (f.nx + 1)) % (f.ny + 1)), f.ny, c.ny),
+                pz = interp1(int(node / (int64_t(f.nx + 1) * (f.ny + 1))), f.nz, c.nz);
+  const double t[3] = {px.t, py.t, pz.t};
+  double w[8];
+  trilinear_weights(t, w);
+  const int64_t sy = c.nx + 1, sz = int64_t(c.nx + 1) * (c.ny + 1);
+  return float(trilinear(xc + (idx / nnf) * c.nn() + px.i0 + py.i0 * sy + pz.i0 * sz, sy, sz, w));
+}
+inline __host__ __device__ __noinline__ float restrict_entry_f64(Grid f, Grid c, const float* rf, const float* y,
+                                                                 int64_t idx) {
+  const int64_t nnc = c.nn(), node = idx % nnc, off = (idx / nnc) * f.nn();
+  const int Ic[3] = {int(node % (c.nx + 1)), int((node / (c.nx + 1)) % (c.ny + 1)),
+                     int(node / (int64_t(c.nx + 1) * (c.ny + 1)))};
+  const int nf[3] = {f.nx, f.ny, f.nz}, nc[3] = {c.nx, c.ny, c.nz};
+  int lo[3], hi[3];
+  for (int d = 0; d < 3; ++d) transfer_support(Ic[d], nf[d], nc[d], lo[d], hi[d]);
+  auto weight = [&](int d, int i) {
+    return 1.0 - fabs(double(int64_t(i) * nc[d] - int64_t(Ic[d]) * nf[d])) / nf[d];
+  };
+  double acc = 0.0;
+  for (int k = lo[2]; k <= hi[2]; ++k)
+    for (int j = lo[1]; j <= hi[1]; ++j)
+      for (int i = lo[0]; i <= hi[0]; ++i) {
+        const int64_t n = off + i + int64_t(f.nx + 1) * (j + int64_t(f.ny + 1) * k);
+        acc += weight(0, i) * weight(1, j) * weight(2, k) * double(y ? rf[n] - y[n] : rf[n]);
+      }
+  return float(acc);
+}
+inline __host__ __device__ bool transfer_finite(float v) { return fabsf(v) <= FLT_MAX; }
+
 // (P x)(i, j, k) of the coarse field x.
 __host__ __device__ __forceinline__ float prolong_value_int(const Grid& f, const Grid& c, const float* __restrict__ x,
                                                             int i, int j, int k) {
@@ -232,13 +280,7 @@ __host__ __device__ __forceinline__ float restrict_value_int(const Grid& f, cons
   const int Ic[3] = {I, J, K}, nf[3] = {f.nx, f.ny, f.nz}, nc[3] = {c.nx, c.ny, c.nz};
   int lo[3], hi[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int64_t center = int64_t(Ic[d]) * nf[d];  // |i nc - I nf| < nf
-    const int64_t a = center - nf[d], b = center + nf[d];
-    lo[d] = a >= 0 ? int(a / nc[d]) + 1 : 0;
-    hi[d] = int((b + nc[d] - 1) / nc[d]) - 1;
-    if (hi[d] > nf[d]) hi[d] = nf[d];
-  }
+  for (int d = 0; d < 3; ++d) transfer_support(Ic[d], nf[d], nc[d], lo[d], hi[d]);
   auto weight = [&](int d, int i) {
     const int64_t t = int64_t(i) * nc[d] - int64_t(Ic[d]) * nf[d];
     return nf[d] - int(t < 0 ? -t : t);
@@ -268,7 +310,9 @@ __host__ __device__ __forceinline__ void prolong_entry_int(const Grid& f, const 
   if ((mf[node] >> fld) & 1) return;
   const int nxp = f.nx + 1, nyp = f.ny + 1;
   const int64_t r = node / nxp;
-  xf[idx] += prolong_value_int(f, c, xc + fld * c.nn(), int(node - r * nxp), int(r % nyp), int(r / nyp));
+  float v = prolong_value_int(f, c, xc + fld * c.nn(), int(node - r * nxp), int(r % nyp), int(r / nyp));
+  if (!transfer_finite(v)) v = prolong_entry_f64(f, c, xc, idx);
+  xf[idx] += v;
 }
 __host__ __device__ __forceinline__ void restrict_entry_int(const Grid& f, const Grid& c, const float* __restrict__ rf,
                                                             const dmask_t* __restrict__ mc, float* __restrict__ rc,
@@ -278,10 +322,13 @@ __host__ __device__ __forceinline__ void restrict_entry_int(const Grid& f, const
   const int64_t node = idx - fld * nnc;
   const int nxp = c.nx + 1, nyp = c.ny + 1;
   const int64_t r = node / nxp;
-  rc[idx] = ((mc[node] >> fld) & 1)
-                ? 0.f
-                : restrict_value_int(f, c, rf + fld * f.nn(), y ? y + fld * f.nn() : nullptr, int(node - r * nxp),
-                                     int(r % nyp), int(r / nyp));
+  float v = 0.f;
+  if (!((mc[node] >> fld) & 1)) {
+    v = restrict_value_int(f, c, rf + fld * f.nn(), y ? y + fld * f.nn() : nullptr, int(node - r * nxp), int(r % nyp),
+                           int(r / nyp));
+    if (!transfer_finite(v)) v = restrict_entry_f64(f, c, rf, y, idx);
+  }
+  rc[idx] = v;
 }
 
 // Nested grids (nf = 2 nc on every axis), the case of every level of a
@@ -295,7 +342,16 @@ __host__ __device__ __forceinline__ void restrict_entry_int(const Grid& f, const
 // One (node, field) of the nested transfers, for one thread each. Prolongation
 // averages the coarse values at floor and ceil of half the index on every axis
 // (the same one twice at an even index: (a + a) / 2 = a exactly), so lanes at
-// odd and even nodes run the same instructions.
+// odd and even nodes run the same instructions. Values within a factor 8 of the
+// largest number overflow in those sums: then only the different ones are added.
+template <typename T>
+__host__ __device__ __noinline__ T prolong_value_nested_few(const T* X, int64_t sy, int64_t sz, int i, int j, int k) {
+  T s = T(0);
+  for (int a2 = 0; a2 <= (k & 1); ++a2)
+    for (int a1 = 0; a1 <= (j & 1); ++a1)
+      for (int a0 = 0; a0 <= (i & 1); ++a0) s += X[(i >> 1) + a0 + ((j >> 1) + a1) * sy + ((k >> 1) + a2) * sz];
+  return s * ((i & 1 ? T(0.5) : T(1)) * (j & 1 ? T(0.5) : T(1)) * (k & 1 ? T(0.5) : T(1)));
+}
 template <typename T>
 __host__ __device__ __forceinline__ T prolong_value_nested(const T* __restrict__ X, int64_t sy, int64_t sz, int i, int j,
                                                            int k) {
@@ -303,7 +359,8 @@ __host__ __device__ __forceinline__ T prolong_value_nested(const T* __restrict__
   const int64_t r0 = (j >> 1) * sy, r1 = ((j + 1) >> 1) * sy, p0 = (k >> 1) * sz, p1 = ((k + 1) >> 1) * sz;
   const T a = (X[p0 + r0 + i0] + X[p0 + r0 + i1]) + (X[p0 + r1 + i0] + X[p0 + r1 + i1]);
   const T b = (X[p1 + r0 + i0] + X[p1 + r0 + i1]) + (X[p1 + r1 + i0] + X[p1 + r1 + i1]);
-  return T(0.125) * (a + b);
+  const T v = T(0.125) * (a + b);
+  return v - v == T(0) ? v : prolong_value_nested_few<T>(X, sy, sz, i, j, k);
 }
 // P^T (r - y) at coarse node (I, J, K) of one field (y null: P^T r).
 template <typename T>

@@ -131,3 +131,51 @@ def test_entries_match_the_oracle(lib, fine, coarse, dtype, difference):
         keep = ((mc >> f) & 1) == 0
         ref, size = P.T @ d[f], P.T @ np.abs(d[f])
         assert (np.abs(got_c[f] - np.where(keep, ref, 0)) <= np.where(keep, 80 * eps * size, 0)).all()
+
+
+@pytest.mark.parametrize("fine, coarse", PAIRS)
+@pytest.mark.parametrize("power", [100, 108, 120, 126])
+def test_large_fp32_values_do_not_overflow_in_the_sums(lib, fine, coarse, power):
+    """The transfers are linear, and scaling by a power of two is exact: where the
+    scaled result is a number of FP32, it is the unscaled one times the power."""
+    rng, nnf, nnc, P, mf, mc = _setup(fine, coarse, 7)
+    s = np.float32(2.0) ** power
+    xc = rng.uniform(0.5, 1.9, (9, nnc)).astype(np.float32) * rng.choice([-1, 1], (9, nnc)).astype(np.float32)
+    r = rng.uniform(0.5, 1.9, (9, nnf)).astype(np.float32) * rng.choice([-1, 1], (9, nnf)).astype(np.float32)
+    zero = np.zeros(nnf, dtype=np.uint16)
+
+    def run(k):
+        of, oc = np.zeros((9, nnf), dtype=np.float32), np.empty((9, nnc), dtype=np.float32)
+        lib.prolong_f32(_n3(fine), _n3(coarse), _p(np.ascontiguousarray(xc * k)), _p(zero), _p(of))
+        lib.restrict_f32(_n3(fine), _n3(coarse), _p(np.ascontiguousarray(r * k)), None, _p(zero[:nnc].copy()), _p(oc))
+        return of.astype(np.float64), oc.astype(np.float64)
+
+    one, big = run(np.float32(1)), run(s)
+    nested = all(a == 2 * b for a, b in zip(fine, coarse))
+    # FP32 sums of up to 8 values on nested grids: at 2^126 only copies are in range
+    i, j, k = np.meshgrid(*[np.arange(n + 1) for n in fine[::-1]], indexing="ij")
+    copy = ((i % 2 == 0) & (j % 2 == 0) & (k % 2 == 0)).reshape(-1)
+    for to_fine, a, b in zip((True, False), one, big):
+        inside = np.abs(a) * float(s) < 2.0 ** 127.9
+        if nested and power == 126:
+            if not to_fine:
+                continue
+            inside &= copy
+        assert inside.any()
+        ulp = 2.0 ** -22 * np.maximum(np.abs(a), 2.0 ** -20) * float(s)  # the FP64 sums round differently
+        assert (np.abs(a * float(s) - b)[inside] <= ulp[inside]).all()
+
+
+def test_infinite_values_stay_infinite(lib):
+    fine, coarse = (9, 7, 6), (5, 4, 3)
+    rng, nnf, nnc, P, mf, mc = _setup(fine, coarse, 8)
+    xc, r = np.ones((9, nnc), dtype=np.float32), np.ones((9, nnf), dtype=np.float32)
+    xc[4, nnc // 2] = np.inf
+    r[2, nnf // 2] = -np.inf
+    of, oc = np.zeros((9, nnf), dtype=np.float32), np.empty((9, nnc), dtype=np.float32)
+    z = np.zeros(nnf, dtype=np.uint16)
+    lib.prolong_f32(_n3(fine), _n3(coarse), _p(xc), _p(z), _p(of))
+    lib.restrict_f32(_n3(fine), _n3(coarse), _p(r), None, _p(z), _p(oc))
+    assert (of[4] == np.where(P[:, nnc // 2] > 0, np.inf, of[4])).all() and np.isinf(of[4]).any()
+    assert (oc[2] == np.where(P[nnf // 2] > 0, -np.inf, oc[2])).all() and np.isinf(oc[2]).any()
+    assert np.isfinite(np.delete(of, 4, 0)).all() and np.isfinite(np.delete(oc, 2, 0)).all()
