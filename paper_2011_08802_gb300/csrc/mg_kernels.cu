@@ -265,9 +265,15 @@ __global__ void k_coarse_solve(int n, const double* __restrict__ Ainv, const T* 
 // flight together. Against the compiler's own choice (32 registers): V-cycle from
 // the binary16 store on 75^3 elements 3.14 against 3.31 ms, FP64 Newton step on 32^3
 // 171 against 175 ms, but 38.2 against 35.1 us per step on average over the levels
-// of 128^3 elements (bound by HBM there, about 470 bytes per node).
+// of 128^3 elements (bound by HBM there, about 470 bytes per node). In FP64 with twelve
+// variants a node's blocks are 960 bytes and 64 registers spill: 128 registers there, a
+// V-cycle on 24^3 elements 4100 -> 4058 us, on 36^3 10.09 -> 10.06 ms.
 template <typename T>
-__global__ void __launch_bounds__(256, 4) k_cheb_first(int64_t nn, const T* __restrict__ D, const T* __restrict__ b, const T* y, T c, bool zero_x,
+constexpr int cheb_minb() {
+  return NV > 6 && sizeof(T) == 8 ? 2 : 4;
+}
+template <typename T>
+__global__ void __launch_bounds__(256, (cheb_minb<T>())) k_cheb_first(int64_t nn, const T* __restrict__ D, const T* __restrict__ b, const T* y, T c, bool zero_x,
                              T* __restrict__ r, T* __restrict__ d, T* __restrict__ x, const dmask_t* __restrict__ mask,
                              T* yn) {
   for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn;
@@ -276,7 +282,7 @@ __global__ void __launch_bounds__(256, 4) k_cheb_first(int64_t nn, const T* __re
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256, 4) k_cheb_step(int64_t nn, const T* __restrict__ D, const T* y, T a, T c, T* __restrict__ r,
+__global__ void __launch_bounds__(256, (cheb_minb<T>())) k_cheb_step(int64_t nn, const T* __restrict__ D, const T* y, T a, T c, T* __restrict__ r,
                             T* __restrict__ d, T* __restrict__ x, const dmask_t* __restrict__ mask, T* yn) {
   for (int64_t node = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; node < nn;
        node += int64_t(gridDim.x) * blockDim.x)
