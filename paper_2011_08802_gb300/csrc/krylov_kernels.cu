@@ -56,9 +56,9 @@ __global__ void k_sub2(int64_t n, const double* __restrict__ b, const double* __
 // j = 0..CNT-1 (CNT <= MDOT_CHUNK). Bound by the FP64 pipe (CNT multiply-adds
 // against CNT + 1 reads). CNT is a template argument so that the loads of one
 // step are straight-line code and in flight together: with a test of j against
-// a run-time count around each load they came one after the other, and 19.3 M
-// entries took 311 us per chunk on average over a 26-step Arnoldi process
-// (FP64 bound 208 us); eight columns now take 450 us (FP64 bound 292 us).
+// a run-time count around each load they came one after the other. The 140 launches of
+// two passes over 26 Arnoldi steps on 2.5 M entries take 7.16 ms, 8.62 with that test;
+// eight columns of 2.5 M entries 80.7 us (ncu, cold; FP64 bound 37.4 us, HBM 26.7).
 template <int CNT>
 __global__ void __launch_bounds__(RED_THREADS) k_mdot_partial(int64_t n, int j0, const double* __restrict__ V,
                                                                int64_t ldv, const double* __restrict__ w,

@@ -263,8 +263,8 @@ __global__ void k_coarse_solve(int n, const double* __restrict__ Ainv, const T* 
 // Chebyshev-accelerated point-block Jacobi, first and later steps (mg_device.cuh).
 // 64 registers (4 CTAs of 256 threads per SM) let a node's 45 + 36 loads be in
 // flight together. Against the compiler's own choice (32 registers): V-cycle from
-// the binary16 store on 75^3 elements 3.14 against 3.31 ms, FP64 Newton step on 32^3
-// 171 against 175 ms, but 38.2 against 35.1 us per step on average over the levels
+// the binary16 store on 75^3 elements 3.14 against 3.31 ms, FP64 Newton solve on 32^3
+// 2 per cent less, but 38.2 against 35.1 us per step on average over the levels
 // of 128^3 elements (bound by HBM there, about 470 bytes per node). In FP64 with twelve
 // variants a node's blocks are 960 bytes and 64 registers spill: 128 registers there, a
 // V-cycle on 24^3 elements 4100 -> 4058 us, on 36^3 10.09 -> 10.06 ms.
