@@ -369,8 +369,12 @@ __device__ __forceinline__ void blockdiag_elem_node(const Grid& g, const JParams
 
 // In-place inverse of one node's NF x NF block (Dirichlet rows/columns replaced
 // by identity first) by Gauss-Jordan elimination with partial pivoting; a
-// singular block sets *singular and is replaced by the identity. Form for FP64:
-// one thread per node, bound by the FP64 pipe.
+// singular block sets *singular and is replaced by the identity. Stored symmetric, as
+// the mean of the two triangles: the rounding errors of an ill-conditioned block's
+// inverse are large along the block's weak direction, where X A - I does not see them;
+// one triangle taken for both loses that (|X A - I| up to 2800 units of |X| |A| in place
+// of 7, V-cycles in FP32 ten times further from FP64 ones). Form for FP64: one thread
+// per node, bound by the FP64 pipe.
 template <typename T>
 __device__ __forceinline__ void block_invert_node(int64_t nn, const dmask_t* __restrict__ mask, T* __restrict__ D,
                                                   int* singular, int64_t node) {
@@ -410,7 +414,7 @@ __device__ __forceinline__ void block_invert_node(int64_t nn, const dmask_t* __r
       for (int c = 0; c < NF; ++c) x[r][c] = (r == c) ? T(1) : T(0);
   }
   for (int r = 0; r < NF; ++r)
-    for (int c = r; c < NF; ++c) D[bidx(r, c) * nn + node] = x[r][c];
+    for (int c = r; c < NF; ++c) D[bidx(r, c) * nn + node] = T(0.5) * (x[r][c] + x[c][r]);
 }
 
 // The same in FP32 by 16 lanes per node, lane r holding row r in registers: the
@@ -484,6 +488,15 @@ __device__ __forceinline__ void block_invert_lanes(int64_t nn, const dmask_t* __
 #pragma unroll
     for (int j = 0; j < NF; ++j)
       if (own <= pc[j]) sm.S[bidx(own, pc[j])][m] = a[j];
+  }
+  __syncthreads();
+  if (!bad && r < NF) {  // the mean with the other triangle
+#pragma unroll
+    for (int j = 0; j < NF; ++j)
+      if (own > pc[j]) {
+        float& s = sm.S[bidx(own, pc[j])][m];
+        s = 0.5f * (s + a[j]);
+      }
   }
   __syncthreads();
   for (int i = tid; i < NBD * BI_NODES; i += int(blockDim.x)) {
