@@ -65,10 +65,12 @@ PFM_FX int fx_clz(uint64_t a) {
 // |v| < 2^(e - 1022) (e = 0: zero or below the normal numbers, read as zero)
 PFM_FX unsigned fx_top(double v) { return unsigned(fx_bits(v) >> 32) & 0x7fffffffu; }
 
-// Scales of a point's Hessian, a_F in the high and a_e in the low 16 bits, from
+constexpr int FX_TERMS = 16;  // products per sum
+
+// Scales of a point's Hessian, for a contraction that leaves the weak rows out of
+// account (host test only, see above): a_F in the high and a_e in the low 16 bits, from
 // the largest fx_top of its parts (F, F), (F, eta), (eta, eta); FX_NONE when an
 // entry is not finite or a scale is outside +-FX_RANGE.
-constexpr int FX_TERMS = 16;
 constexpr int FX_NONE = -2147483647 - 1;
 constexpr int FX_RANGE = 400;
 PFM_FX int fx_hess_scales(const unsigned top[3]) {
@@ -84,7 +86,7 @@ PFM_FX int fx_hess_scales(const unsigned top[3]) {
 PFM_FX int fx_scale_F(int hx) { return hx >> 16; }
 PFM_FX int fx_scale_eta(int hx) { return int(int16_t(uint16_t(unsigned(hx) & 0xffffu))); }
 
-// Z of the input from the largest fx_top of its two parts; false when the
+// Z of its input from the largest fx_top of its two parts; false when the
 // contraction does not take the point (then it goes through FP64).
 PFM_FX bool fx_input_scale(int hx, unsigned topF, unsigned tope, int& Z) {
   const int eF = int(topF >> 20), ee = int(tope >> 20);
